@@ -50,6 +50,9 @@ typedef enum {
 } prony_status;
 
 /* Arithmetic of the Toeplitz block products (the small steps are FP64 always).
+ * For d >= 2 and at least 2048 points a product may first diagonalise the leading axis by an FP32 DFT and
+ * run one product of d - 1 dimensions per frequency in the arithmetic below (a sample that is not
+ * finite then spoils every row of the product).
  *   PRONY_FP32   : complex64 operands, FP32 FMA on the CUDA cores.
  *   PRONY_BF16X3 : FP32 operands split into three BF16 parts, six tensor-core
  *                  products (tcgen05.mma kind::f16), FP32 accumulation.
@@ -253,8 +256,12 @@ typedef struct {
  *   PRONY_TC_TUNE=0      no autotuning: the smallest K split
  *   PRONY_TC_APPLY=0     the X M products of the tall blocks (CholeskyQR2, the final U and V) on
  *                        the FP32 CUDA cores instead of the tensor cores (three BF16 planes)
+ *   PRONY_AXIS=0 / 1     the products of every problem directly / through a DFT of the leading axis
+ *                        wherever that is possible (d >= 2, n <= 95; not PRONY_FFT32).  Default:
+ *                        the transform for problems of at least 2048 points (n+1)^d where it costs less
  * The first three change launch configurations only, never the arithmetic beyond FP32 summation
- * order; the fourth changes how the X M products are rounded (both are FP32-accurate).
+ * order; the fourth changes how the X M products are rounded (both are FP32-accurate), the fifth
+ * how the products are (FP32 transforms around shorter dot products in the chosen arithmetic).
  * For a given launch configuration every product is deterministic: split-K partial sums are
  * added in the order of their K ranges, whatever order the CTAs finish in. */
 int prony_set_profiling(prony_ctx* ctx, int enable);   /* also resets the statistics */

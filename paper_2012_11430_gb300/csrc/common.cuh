@@ -37,7 +37,10 @@ struct ProbDesc {
   long long toff;             // offset (words) of its split-plane tables in tabF / tabH
   int Gd4;                    // Gd rounded up to a multiple of 4 (length of one table)
   int fL;                     // FFT products: points per axis of the circulant embedding (0: dense)
-  long long foff;             // FFT products: offset (elements) of the problem's transform in fhat
+  long long foff;             // FFT products: offset (elements) of the problem's transform in fhat;
+                              // a sub-problem: offset of its axis twiddles
+  int st;                     // index of the problem's state (a sub-problem: of its parent's)
+  int sub;                    // index of the problem's first sub-problem (products by axis transform)
 };
 
 // Per-problem iteration state, device resident.
@@ -316,7 +319,8 @@ enum BufSel { BUF_V = 0, BUF_U = 1, BUF_B1 = 2, BUF_B2 = 3, BUF_Y = 4 };
 // Bytes of cross-block partials per problem that the tall kernels need for a batch of this
 // layout (D.nprob, D.maxN, D.maxGd, D.L set).
 long long red_bytes_per_problem(const Dev& D);
-void launch_prep(const Dev& D, cudaStream_t s);
+void launch_state_init(const Dev& D, cudaStream_t s);
+void launch_prep(const Dev& D, bool norms, cudaStream_t s);   // states, gF, gH; norms: ||T||_F, ||f||, finiteness
 void launch_init_v0(const Dev& D, unsigned long long seed, cudaStream_t s);
 void launch_zero_small(const Dev& D, long long off, long long bytes, cudaStream_t s);
 // out[a][b] (+)= sum_{r in I_n} conj(X[map(r), a]) Z[map(r), b]; X, Z buffers with row shifts
@@ -389,6 +393,15 @@ cudaError_t launch_gram_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int
 cudaError_t launch_apply_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int xbuf, int xw, int outw,
                             long long m_off, int m_double, int outbuf, int ntbox, int stages, void* xb,
                             long long prob_stride, int* err, cudaStream_t s);
+
+// kernels_axis.cu (products with the leading axis diagonalised by a DFT).  S: the Dev of the
+// sub-problems (S.P their descriptors, S.V / S.B2 / S.Y the transformed blocks).
+enum AxisMode { AX_FP32 = 0, AX_BF16X3 = 1, AX_TF32X3 = 2, AX_BF16X2 = 3 };   // the prony_precision of the products
+constexpr int AX_MAX_N = 95;          // largest n (twiddle table of (n + 3)/2 x (n + 1) float4 in shared memory)
+cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int trim, cudaStream_t s);
+cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int wsel, int maxw, void* xb,
+                           long long prob_stride, cudaStream_t s);
+cudaError_t launch_axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s);
 
 // kernels_refine.cu (Levenberg-Marquardt refinement of (t, c))
 long long lm_workspace_bytes(int m, int d);

@@ -57,7 +57,9 @@ __global__ void k_state_init(Dev D) {
 }
 
 // gF = f, gH(x) = conj f(-x) (zero where -x leaves the grid); ||T||_F^2 by the
-// multiplicity of each difference (prod_l (n+1-|x_l|)), ||f||^2 over I_n, finiteness.
+// multiplicity of each difference (prod_l (n+1-|x_l|)), ||f||^2 over I_n, finiteness.  A product on
+// its own needs the copies only (NORMS = false: no FP64 sums).
+template <bool NORMS>
 __global__ void k_prep(Dev D) {
   __shared__ double sh[32];
   const int pi = blockIdx.y;
@@ -89,13 +91,15 @@ __global__ void k_prep(Dev D) {
       h = make_float2((float)fm.x, -(float)fm.y);
     }
     D.gH[p.grid + i] = h;
+    if (!NORMS) continue;
     double a2 = f.x * f.x + f.y * f.y;
     if (inT) accT += w * a2;
     if (inI) accF += a2;
   }
+  if (bad) atomicOr(&D.st[pi].nonfinite, 1);
+  if (!NORMS) return;
   double sT = block_sum(accT, sh);
   double sF = block_sum(accF, sh);
-  if (bad) atomicOr(&D.st[pi].nonfinite, 1);
   // block sums in fixed block order
   double2* slot = (double2*)red_region(D, pi);
   if (threadIdx.x == 0 && ws_ok(D, 16LL * (blockIdx.x + 1) <= D.red_stride, 11)) slot[blockIdx.x] = make_double2(sT, sF);
@@ -783,12 +787,17 @@ inline int blocks_for(long long n, int per) { return (int)std::min<long long>((n
 
 #include <algorithm>
 
-void launch_prep(const Dev& D, cudaStream_t s) {
+void launch_state_init(const Dev& D, cudaStream_t s) {
   note_launch();
   k_state_init<<<(D.nprob + 127) / 128, 128, 0, s>>>(D);
-  dim3 g(blocks_per_problem(std::min((D.maxGd + 255) / 256, 64), D.nprob), D.nprob);
+}
+
+void launch_prep(const Dev& D, bool norms, cudaStream_t s) {
+  launch_state_init(D, s);
   note_launch();
-  k_prep<<<g, 256, 0, s>>>(D);
+  dim3 g(blocks_per_problem(std::min((D.maxGd + 255) / 256, 64), D.nprob), D.nprob);
+  if (norms) k_prep<true><<<g, 256, 0, s>>>(D);
+  else k_prep<false><<<g, 256, 0, s>>>(D);
 }
 
 void launch_init_v0(const Dev& D, unsigned long long seed, cudaStream_t s) {

@@ -78,33 +78,6 @@ __device__ inline int grid_of_h(int h, const ProbDesc& p) {
   return g;
 }
 
-// Split an FP32 pair into BF16x2 planes (exact for three planes).
-template <int NPL>
-__device__ __forceinline__ void split_pair(float a, float b, uint32_t* w) {
-  uint32_t h = pack_bf16x2(a, b);
-  w[0] = h;
-  float ra = a - bf16lo_to_f32(h), rb = b - bf16hi_to_f32(h);
-  uint32_t m = pack_bf16x2(ra, rb);
-  w[1] = m;
-  if (NPL == 3) {
-    ra -= bf16lo_to_f32(m);
-    rb -= bf16hi_to_f32(m);
-    w[2] = pack_bf16x2(ra, rb);
-  }
-}
-
-// Split an FP32 value into TF32 hi + lo (round to nearest, ties away; both exactly TF32).
-__device__ __forceinline__ float tf32_round(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-__device__ __forceinline__ void split_tf32(float x, uint32_t* w) {
-  const float hi = tf32_round(x);
-  w[0] = __float_as_uint(hi);
-  w[1] = __float_as_uint(tf32_round(x - hi));
-}
-
 // The three operand encodings.  Per 32-point K chunk (64 real K values) and plane:
 //   BF16X3 / BF16X2  32 TMEM columns (two BF16 per column), 4 MMAs of K = 16, B rows of 128 bytes
 //   TF32X3           64 TMEM columns (one TF32 per column), 8 MMAs of K = 8, B rows split into
@@ -349,7 +322,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   const ToeplitzJob job = jobs[blockIdx.x];
   const ProbDesc& p = D.P[job.prob];
-  const ProbState& st = D.st[job.prob];
+  const ProbState& st = D.st[p.st];
   if (st.done) return;
   const int w = tc_width(st, p, P.wsel);
   if (w <= 0) return;

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(256) k_toeplitz_simt(Dev D, const ToeplitzJob*
   __shared__ float2 Xs[TBK][NCOL];
   const ToeplitzJob job = jobs[blockIdx.x];
   const ProbDesc& p = D.P[job.prob];
-  const ProbState& st = D.st[job.prob];
+  const ProbState& st = D.st[p.st];
   if (st.done) return;
   const int w = twidth(st, p, wsel);
   if (w <= 0) return;

@@ -74,6 +74,9 @@ struct prony_ctx {
   DBuf red, rcnt;                       // fixed-order cross-block sums: partials and counters per problem
   DBuf oob;                             // first failed workspace bound check of a kernel (0: none)
   DBuf fhat, ftw;                       // FFT path: sample transforms, twiddles
+  // products by axis transform: sub-problem descriptors, twiddles, transformed blocks and samples
+  DBuf axP, axtw, axX, axY, axF, axH;
+  std::vector<int> ax_sig;              // (n, d, m, r0) of every problem axP was built for
   int* h_flag = nullptr;            // pinned
   std::vector<ProbState> h_st;
   // profiling of the Toeplitz launches
@@ -164,6 +167,17 @@ struct Batch {
   ToeplitzJob* jobs_ext = nullptr;
   ToeplitzJob* jobs_in = nullptr;
   int maxw = 0;
+  // Products with the leading axis diagonalised by a DFT (kernels_axis.cu).  rep[i]: the first of
+  // the P[i].G sub-problems of problem i (all of one shape); S: their device view.
+  struct AxisConf {
+    bool on = false;
+    std::vector<ProbDesc> rep;
+    Dev S{};
+  } ax;
+  // the problems the product kernels see: shapes, how many of each, index of the first
+  const std::vector<ProbDesc>& shapes() const { return ax.on ? ax.rep : P; }
+  int copies(size_t i) const { return ax.on ? P[i].G : 1; }
+  int first(size_t i) const { return ax.on ? P[i].sub : (int)i; }
   float2* part = nullptr;             // split K workspace of the products (FP32 path / tensor-core path)
   int* cnt = nullptr;
   long long part_jobs = 0;            // jobs the split K workspace holds
@@ -247,10 +261,11 @@ static int ensure_tcjobs(prony_ctx* ctx, size_t bytes) {
 int tc_set_jobs(prony_ctx* ctx, Batch& B, int nks) {
   TcConf& T = B.tc;
   std::vector<int> sig;
-  sig.reserve(3 + 2 * B.P.size());
+  sig.reserve(5 + 2 * B.P.size());
   sig.push_back(nks);
   sig.push_back(T.gram ? T.nks_gram : 0);
   sig.push_back(T.apply ? 1 : 0);
+  sig.push_back(B.ax.on ? 1 : 0);
   sig.push_back((int)B.P.size());
   for (const auto& p : B.P) {
     sig.push_back(p.n);
@@ -270,11 +285,13 @@ int tc_set_jobs(prony_ctx* ctx, Batch& B, int nks) {
   } else {
     std::vector<ToeplitzJob> jobs;
     auto add_jobs = [&](bool ext) {
-      for (int i = 0; i < (int)B.P.size(); ++i) {
-        const int tiles = ((ext ? B.P[i].Next : B.P[i].N) + 127) / 128;
-        const int nk = std::min(nks, std::max(1, (B.P[i].N + 31) / 32));
-        for (int mt = 0; mt < tiles; ++mt)
-          for (int ks = 0; ks < nk; ++ks) jobs.push_back({i, mt, ks, nk});
+      const std::vector<ProbDesc>& Q = B.shapes();
+      for (size_t i = 0; i < Q.size(); ++i) {
+        const int tiles = ((ext ? Q[i].Next : Q[i].N) + 127) / 128;
+        const int nk = std::min(nks, std::max(1, (Q[i].N + 31) / 32));
+        for (int c = 0; c < B.copies(i); ++c)
+          for (int mt = 0; mt < tiles; ++mt)
+            for (int ks = 0; ks < nk; ++ks) jobs.push_back({B.first(i) + c, mt, ks, nk});
       }
     };
     add_jobs(true);
@@ -317,11 +334,14 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   T.kind = prec;
   const int npl = tc_planes(prec);
   T.ntbox = ((2 * maxw + 15) / 16) * 16;
-  int maxnc = 0, tiles_ext = 0, tiles_in = 0;
-  for (const auto& p : B.P) {
-    maxnc = std::max(maxnc, (p.N + 31) / 32);
-    tiles_ext += (p.Next + 127) / 128;
-    tiles_in += (p.N + 127) / 128;
+  const std::vector<ProbDesc>& Q = B.shapes();
+  int maxnc = 0, maxrows = 0, tiles_ext = 0, tiles_in = 0, nprod = 0;
+  for (size_t i = 0; i < Q.size(); ++i) {
+    maxnc = std::max(maxnc, (Q[i].N + 31) / 32);
+    maxrows = std::max(maxrows, B.P[i].N);
+    tiles_ext += B.copies(i) * ((Q[i].Next + 127) / 128);
+    tiles_in += B.copies(i) * ((Q[i].N + 127) / 128);
+    nprod += B.copies(i);
   }
   const size_t stage = tc_stage_bytes(prec, T.ntbox);
   const size_t avail = 227 * 1024 - 2048 - 4608;   // static shared memory of the kernel (chunk table)
@@ -343,17 +363,19 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   // tolerance.  So at most 128 K chunks per CTA for BF16 planes, 64 for TF32.
   const int max_chunks = bf16 ? 128 : 64;
   int nks_lo = std::max(1, std::min(16, (2 * 152 + tiles_in - 1) / std::max(1, tiles_in)));
+  // sub-problems of an axis transform are many and short: no K range below eight chunks
+  if (B.ax.on) nks_lo = std::max(1, std::min(nks_lo, maxnc / 8));
   nks_lo = std::max(nks_lo, (maxnc + max_chunks - 1) / max_chunks);
   // largest window of a problem shape (it depends on n, d and the split only), computed once per
   // shape of the batch
   std::map<std::pair<int, int>, int> shapes;          // (n, d) -> a problem of that shape
-  for (int i = 0; i < (int)B.P.size(); ++i) shapes.emplace(std::make_pair(B.P[i].n, B.P[i].d), i);
+  for (int i = 0; i < (int)Q.size(); ++i) shapes.emplace(std::make_pair(Q[i].n, Q[i].d), i);
   std::map<std::tuple<int, int, int>, int> wmemo;      // (problem, nks, ext) -> window words
   auto window_of = [&](int i, int nks, int ext) {
     auto key = std::make_tuple(i, nks, ext);
     auto it = wmemo.find(key);
     if (it != wmemo.end()) return it->second;
-    const ProbDesc& p = B.P[i];
+    const ProbDesc& p = Q[i];
     const int wl = max_window(p, ext ? p.n + 2 : p.n + 1, nks, bf16);
     wmemo.emplace(key, wl);
     return wl;
@@ -363,7 +385,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     for (;; ++nks) {
       bool fits = true;
       for (const auto& sh : shapes) {
-        const ProbDesc& p = B.P[sh.second];
+        const ProbDesc& p = Q[sh.second];
         nks = std::min(nks, std::max(1, (p.N + 31) / 32));
         if (window_of(sh.second, nks, 1) > cap || window_of(sh.second, nks, 0) > cap) fits = false;
       }
@@ -404,11 +426,12 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     const char* e = getenv("PRONY_TC_GRAM");
     T.gram = e && atoi(e) == 1;
     const int np = (int)B.P.size();
-    T.nks_gram = std::max(1, std::min(maxnc, (2 * 152 + np - 1) / np));
-    T.nks_gram = std::max(T.nks_gram, (maxnc + 63) / 64);       // at most 64 K chunks per CTA
+    const int gnc = (maxrows + 31) / 32;
+    T.nks_gram = std::max(1, std::min(gnc, (2 * 152 + np - 1) / np));
+    T.nks_gram = std::max(T.nks_gram, (gnc + 63) / 64);         // at most 64 K chunks per CTA
     const size_t gstage = tc_stage_bytes(PRONY_BF16X3, T.ntbox);
     T.gram_stages = (int)std::max<size_t>(1, std::min<size_t>(4, (avail - 1024) / gstage));
-    T.gram_stride = tc_prob_stride(PRONY_BF16X3, T.ntbox, maxnc);
+    T.gram_stride = tc_prob_stride(PRONY_BF16X3, T.ntbox, gnc);
   }
   // X M products of the tall blocks (CholeskyQR2, the final U and V) on the tensor cores in three
   // BF16 planes, FP32-exact operands: the inner dimension is at most r0 <= 128 (four K chunks), so
@@ -426,7 +449,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     T.apply_stride = tc_prob_stride(PRONY_BF16X3, T.ntbox, maxac);
   }
   // batch shape signature for the tuning cache
-  T.key = std::to_string(prec) + ":" + std::to_string(B.P.size()) + ":" + std::to_string(maxw) + ":" +
+  T.key = std::to_string(prec) + (B.ax.on ? "a:" : ":") + std::to_string(B.P.size()) + ":" + std::to_string(maxw) + ":" +
           std::to_string(maxnc) + ":" + std::to_string(tiles_ext) + ":" + std::to_string(tiles_in) + ":" +
           std::to_string(nks);
   auto hit = ctx->tc_tuned.find(T.key);
@@ -439,14 +462,16 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   }
   int rc;
   long long twords = 64;                              // split-plane tables (+ slack for window rounding)
-  for (const auto& p : B.P) twords = std::max(twords, p.toff + 6LL * p.Gd4 + 64);
+  for (size_t i = 0; i < Q.size(); ++i) twords = std::max(twords, Q[i].toff + 6LL * Q[i].Gd4 * B.copies(i) + 64);
   if ((rc = ensure(ctx->tabF, 4 * (size_t)twords))) return rc;
   if ((rc = ensure(ctx->tabH, 4 * (size_t)twords))) return rc;
-  B.D.tabF = (uint32_t*)ctx->tabF.p;
-  B.D.tabH = (uint32_t*)ctx->tabH.p;
+  Dev& DT = B.ax.on ? B.ax.S : B.D;
+  DT.tabF = (uint32_t*)ctx->tabF.p;
+  DT.tabH = (uint32_t*)ctx->tabH.p;
   // B' tiles of the products and (three BF16 planes) of the Grams share one buffer
-  if ((rc = ensure(ctx->xb, (size_t)B.P.size() * (size_t)std::max(std::max(T.prob_stride, T.gram ? T.gram_stride : 0LL),
-                                                                    T.apply ? T.apply_stride : 0LL))))
+  if ((rc = ensure(ctx->xb, std::max((size_t)nprod * (size_t)T.prob_stride,
+                                     B.P.size() * (size_t)std::max(T.gram ? T.gram_stride : 0LL,
+                                                                   T.apply ? T.apply_stride : 0LL)))))
     return rc;
   if ((rc = ensure(ctx->tcerr, 256))) return rc;
   CK(cudaMemsetAsync(ctx->tcerr.p, 0, sizeof(int), ctx->stream));
@@ -493,6 +518,21 @@ void toeplitz_product(prony_ctx* ctx, const Batch& B, const Dev& D, int ext, int
   if (adjoint < 0) adjoint = ext ? 0 : 1;
   if (B.fft.on) {
     launch_toeplitz_fft(D, B.fft.maxpts, wsel == W_ONE ? 1 : B.maxw, adjoint, xbuf, wsel, ybuf, ext, s);
+  } else if (B.ax.on) {
+    // transform of the leading axis, one product per frequency, inverse transform
+    const TcConf& T = B.tc;
+    const Dev& S = B.ax.S;
+    const int sbuf = ext ? BUF_Y : BUF_B2;
+    cudaError_t e = launch_axis_in(D, S, prec, xbuf, wsel, B.maxw, ctx->xb.p, T.prob_stride, s);
+    if (e == cudaSuccess && T.on)
+      e = launch_toeplitz_tc(S, ext ? T.jobs_ext : T.jobs_in, ext ? T.njobs_ext : T.njobs_in, adjoint, wsel, sbuf, ext,
+                             T.kind, T.ntbox, T.win_cap, T.stages, ctx->xb.p, T.prob_stride, (float*)B.part, B.cnt,
+                             B.part_jobs, T.err, s);
+    else if (e == cudaSuccess)
+      launch_toeplitz(S, ext ? B.jobs_ext : B.jobs_in, ext ? B.njobs_ext : B.njobs_in, adjoint, BUF_V, wsel, sbuf, ext,
+                      B.maxw, B.part, B.cnt, B.part_jobs, s);
+    if (e == cudaSuccess) e = launch_axis_out(D, S, wsel, ybuf, ext, B.maxw, s);
+    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
   } else if (B.tc.on) {
     const TcConf& T = B.tc;
     launch_xb_prep(D, xbuf, -1, wsel, ctx->xb.p, T.kind, T.prob_stride, s);
@@ -516,7 +556,9 @@ int tc_autotune(prony_ctx* ctx, Batch& B, const Dev& D, int prec, cudaStream_t s
   if (2 * T.nks_min <= 16 && T.nks_min <= 8) cand.push_back(2 * T.nks_min);
   // room for the largest job list and split workspace first, so that no candidate reallocates them
   size_t maxjobs = 0;
-  for (const auto& p : B.P) maxjobs += (size_t)2 * T.nks_min * ((p.Next + 127) / 128 + (p.N + 127) / 128);
+  const std::vector<ProbDesc>& Q = B.shapes();
+  for (size_t i = 0; i < Q.size(); ++i)
+    maxjobs += (size_t)B.copies(i) * 2 * T.nks_min * ((Q[i].Next + 127) / 128 + (Q[i].N + 127) / 128);
   int rc;
   if ((rc = ensure_tcjobs(ctx, sizeof(ToeplitzJob) * maxjobs))) return rc;
   if ((rc = ensure_split_ws(ctx, B, maxjobs, sizeof(float) * tc_part_floats(T.ntbox)))) return rc;
@@ -591,12 +633,171 @@ int setup_fft(prony_ctx* ctx, Batch& B) {
   return PRONY_OK;
 }
 
+// Whether the products of a batch go through the transform of the leading axis: fewer
+// multiply-adds, for two more kernels and the traffic of the transformed blocks.  Costs in
+// units of one K chunk of a 128-row tile (about 1.1 us of an SM on the tensor cores): a CTA's
+// set-up and epilogue weigh about five chunks, the transforms 1e-3 per transformed value.
+// Below 2048 points the direct product's FP32 sums are short and round less than the transforms
+// do (relative error at N = 1331: 1.9e-7 direct, 2.4e-7 transformed; at N = 2601: 3.6e-7 and
+// 2.6e-7; at N = 8000: 3.4e-6 and 7e-7, BF16x3), so small problems keep it whatever the cost.
+// PRONY_AXIS=0 / 1 overrides the size and cost rules.
+bool axis_pays(const std::vector<ProbDesc>& P, int prec) {
+  if (prec != PRONY_FP32 && !is_tc(prec)) return false;
+  const char* e = getenv("PRONY_AXIS");
+  double dense = 0.0, axis = 0.0;
+  for (const auto& p : P) {
+    if (p.d < 2 || p.n > AX_MAX_N || (!e && p.N < 2048)) return false;
+    const double H = p.n + 1, Ns = p.N / H, Rs = p.Next / (H + 1);
+    dense += std::ceil(p.Next / 128.0) * (std::ceil(p.N / 32.0) + 5);
+    axis += 2 * H * (std::ceil(Rs / 128.0) * (std::ceil(Ns / 32.0) + 5) + 1e-3 * Ns * p.r0);
+  }
+  return e ? atoi(e) != 0 : axis < dense;
+}
+
+// Sub-problems of the products by axis transform: problem i's G frequencies, each a problem of
+// d - 1 dimensions on the same n, with its own sample tables and blocks.
+int setup_axis(prony_ctx* ctx, Batch& B, int prec) {
+  auto& A = B.ax;
+  A.rep.resize(B.P.size());
+  long long grid = 0, xoff = 0, yoff = 0, toff = 0, twoff = 0;
+  int sub = 0, maxn = 0, maxN = 0, maxNext = 0, maxGd = 0;
+  std::vector<int> sig;
+  for (size_t i = 0; i < B.P.size(); ++i) {
+    const ProbDesc& p = B.P[i];
+    ProbDesc& q = A.rep[i];
+    q = p;
+    q.d = p.d - 1;
+    q.N = p.N / (p.n + 1);
+    q.Next = p.Next / (p.n + 2);
+    q.Gd = p.Gd / p.G;
+    q.Gd4 = (q.Gd + 7) & ~7;
+    q.grid = grid;
+    q.xoff = xoff;
+    q.yoff = yoff;
+    q.toff = toff;
+    q.foff = twoff;
+    q.st = (int)i;
+    q.sub = -1;
+    sub += p.G;                                  // = p.sub of the next problem
+    grid += (long long)p.G * q.Gd;
+    xoff += (long long)p.G * q.N * q.r0;
+    yoff += (long long)p.G * q.Next * q.r0;
+    toff += 6LL * p.G * q.Gd4;
+    twoff += p.G;
+    maxn = std::max(maxn, p.n);
+    maxN = std::max(maxN, q.N);
+    maxNext = std::max(maxNext, q.Next);
+    maxGd = std::max(maxGd, q.Gd);
+    for (const int v : {p.n, p.d, p.m, p.r0}) sig.push_back(v);
+  }
+  int rc;
+  const size_t cap = ctx->axP.cap, tcap = ctx->axtw.cap;
+  if ((rc = ensure(ctx->axP, sizeof(ProbDesc) * sub))) return rc;
+  if ((rc = ensure(ctx->axtw, sizeof(float2) * twoff))) return rc;
+  if ((rc = ensure(ctx->axY, sizeof(float2) * std::max(xoff, yoff)))) return rc;
+  if (prec == PRONY_FP32) {
+    if ((rc = ensure(ctx->axX, sizeof(float2) * xoff))) return rc;
+    if ((rc = ensure(ctx->axF, sizeof(float2) * grid))) return rc;
+    if ((rc = ensure(ctx->axH, sizeof(float2) * grid))) return rc;
+  }
+  if (ctx->axP.cap != cap || ctx->axtw.cap != tcap || sig != ctx->ax_sig) {
+    ctx->ax_sig.clear();
+    // twiddles exp(2 pi i j / G) = (cos, sin), rounded from FP64
+    std::vector<float2> tw;
+    tw.reserve(twoff);
+    const double turn = 6.283185307179586;
+    for (const auto& p : B.P)
+      for (int j = 0; j < p.G; ++j) {
+        const double a = turn * j / p.G;
+        tw.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
+      }
+    CK(cudaMemcpyAsync(ctx->axtw.p, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice, ctx->stream));
+    std::vector<ProbDesc> all;
+    all.reserve(sub);
+    for (size_t i = 0; i < B.P.size(); ++i) {
+      ProbDesc q = A.rep[i];
+      for (int w = 0; w < B.P[i].G; ++w) {
+        all.push_back(q);
+        q.grid += q.Gd;
+        q.xoff += (long long)q.N * q.r0;
+        q.yoff += (long long)q.Next * q.r0;
+        q.toff += 6LL * q.Gd4;
+      }
+    }
+    // synchronous with respect to this host copy (pageable memory); stream-ordered on the device
+    CK(cudaMemcpyAsync(ctx->axP.p, all.data(), sizeof(ProbDesc) * all.size(), cudaMemcpyHostToDevice, ctx->stream));
+    ctx->ax_sig = std::move(sig);
+  }
+  Dev& S = A.S;
+  S = B.D;
+  S.P = (const ProbDesc*)ctx->axP.p;
+  S.nprob = sub;
+  S.maxN = maxN;
+  S.maxNext = maxNext;
+  S.maxGd = maxGd;
+  S.V = (float2*)ctx->axX.p;
+  S.Y = S.B2 = (float2*)ctx->axY.p;
+  S.gF = (float2*)ctx->axF.p;
+  S.gH = (float2*)ctx->axH.p;
+  S.ftw = (float2*)ctx->axtw.p;
+  S.fLT = maxn;
+  A.on = true;
+  return PRONY_OK;
+}
+
+// The sample tables of the products: split planes of the grid, or the transformed samples of the
+// sub-problems (`trim`: without the samples at x_0 = n + 1).
+void product_tables(prony_ctx* ctx, const Batch& B, int prec, int trim, cudaStream_t s) {
+  if (B.ax.on) {
+    const cudaError_t e = launch_axis_tables(B.D, B.ax.S, prec, trim, s);
+    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+  } else if (B.tc.on) {
+    launch_split_tables(B.D, B.tc.kind, s);
+  }
+}
+
+// Job lists and workspaces of the products: CUDA-core or tensor-core kernel.
+int setup_products(prony_ctx* ctx, Batch& B, int prec) {
+  if (is_tc(prec)) return setup_tc(ctx, B, prec, B.maxw);
+  const std::vector<ProbDesc>& Q = B.shapes();
+  long long tiles_in = 0;
+  int maxN = 0;
+  for (size_t i = 0; i < Q.size(); ++i) {
+    tiles_in += (long long)B.copies(i) * ((Q[i].N + 63) / 64);
+    maxN = std::max(maxN, Q[i].N);
+  }
+  // split K so that the smallest product still fills the GPU
+  int nks = (int)std::max<long long>(1, std::min<long long>(304 / std::max<long long>(1, tiles_in), 16));
+  nks = std::min(nks, std::max(1, maxN / 64));
+  B.nks = nks;
+  std::vector<ToeplitzJob> jobs;
+  auto add_jobs = [&](bool ext) {
+    for (size_t i = 0; i < Q.size(); ++i)
+      for (int c = 0; c < B.copies(i); ++c)
+        for (int mt = 0; mt < ((ext ? Q[i].Next : Q[i].N) + 63) / 64; ++mt)
+          for (int ks = 0; ks < nks; ++ks) jobs.push_back({B.first(i) + c, mt, ks, nks});
+  };
+  add_jobs(true);
+  B.njobs_ext = (int)jobs.size();
+  add_jobs(false);
+  B.njobs_in = (int)jobs.size() - B.njobs_ext;
+  int rc;
+  if ((rc = ensure(ctx->jobs, sizeof(ToeplitzJob) * jobs.size()))) return rc;
+  CK(cudaMemcpyAsync(ctx->jobs.p, jobs.data(), sizeof(ToeplitzJob) * jobs.size(), cudaMemcpyHostToDevice, ctx->stream));
+  B.jobs_ext = (ToeplitzJob*)ctx->jobs.p;
+  B.jobs_in = B.jobs_ext + B.njobs_ext;
+  if (nks > 1)
+    return ensure_split_ws(ctx, B, (size_t)std::max(B.njobs_ext, B.njobs_in), sizeof(float2) * simt_part_elems(B.maxw));
+  return PRONY_OK;
+}
+
 // Lay out a batch in the context workspace.  Grid samples are copied from `src`
 // (host or device, per problem sample_off) into the packed grid64 buffer.
 int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opts& o, Batch& B) {
   const int np = (int)hp.size();
   B.P.resize(np);
   long long goff = 0, xoff = 0, yoff = 0, toff = 0;
+  int sub = 0;
   int maxN = 0, maxNext = 0, maxGd = 0, maxR0 = 0, maxM = 0, maxD = 0;
   long long tiles_ext = 0, tiles_in = 0;
   for (int i = 0; i < np; ++i) {
@@ -616,6 +817,12 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
     p.xoff = xoff;
     p.yoff = yoff;
     p.ooff = h.out_off;
+    p.st = i;
+    p.sub = -1;
+    if (h.n <= AX_MAX_N) {                       // (products by axis transform: no larger n)
+      p.sub = sub;
+      sub += p.G;
+    }
     p.Gd4 = (p.Gd + 3) & ~3;
     p.toff = toff;
     toff += 6LL * p.Gd4;
@@ -633,21 +840,6 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   }
   SmallLay L = make_small_lay((maxR0 + 1) / 2 * 2, maxM, maxD);
   for (int i = 0; i < np; ++i) B.P[i].soff = (long long)i * L.bytes;
-  // split K so that the smallest product still fills the GPU
-  int nks = (int)std::max<long long>(1, std::min<long long>(304 / std::max<long long>(1, tiles_in), 16));
-  nks = std::min(nks, std::max(1, maxN / 64));
-  B.nks = nks;
-  // job list of the FP32 CUDA-core products (the tensor-core and FFT paths build their own)
-  std::vector<ToeplitzJob> jobs;
-  const bool simt = o.precision == PRONY_FP32;
-  for (int i = 0; simt && i < np; ++i)
-    for (int mt = 0; mt < (B.P[i].Next + 63) / 64; ++mt)
-      for (int ks = 0; ks < nks; ++ks) jobs.push_back({i, mt, ks, nks});
-  B.njobs_ext = (int)jobs.size();
-  for (int i = 0; simt && i < np; ++i)
-    for (int mt = 0; mt < (B.P[i].N + 63) / 64; ++mt)
-      for (int ks = 0; ks < nks; ++ks) jobs.push_back({i, mt, ks, nks});
-  B.njobs_in = (int)jobs.size() - B.njobs_ext;
   B.maxw = maxR0;
 
   int rc;
@@ -662,12 +854,8 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   if ((rc = ensure(ctx->small, (size_t)L.bytes * np))) return rc;
   if ((rc = ensure(ctx->P, sizeof(ProbDesc) * np))) return rc;
   if ((rc = ensure(ctx->st, sizeof(ProbState) * np))) return rc;
-  if ((rc = ensure(ctx->jobs, sizeof(ToeplitzJob) * jobs.size()))) return rc;
   if ((rc = ensure(ctx->flag, 256))) return rc;
   CK(cudaMemcpyAsync(ctx->P.p, B.P.data(), sizeof(ProbDesc) * np, cudaMemcpyHostToDevice, ctx->stream));
-  if (!jobs.empty())
-    CK(cudaMemcpyAsync(ctx->jobs.p, jobs.data(), sizeof(ToeplitzJob) * jobs.size(), cudaMemcpyHostToDevice,
-                       ctx->stream));
   CK(cudaMemsetAsync(ctx->small.p, 0, (size_t)L.bytes * np, ctx->stream));
   Dev& D = B.D;
   D.P = (const ProbDesc*)ctx->P.p;
@@ -701,13 +889,16 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   D.red = (char*)ctx->red.p;
   D.rcnt = (int*)ctx->rcnt.p;
   D.oob = (int*)ctx->oob.p;
-  B.jobs_ext = (ToeplitzJob*)ctx->jobs.p;
-  B.jobs_in = B.jobs_ext + B.njobs_ext;
-  if (simt && nks > 1 &&
-      (rc = ensure_split_ws(ctx, B, (size_t)std::max(B.njobs_ext, B.njobs_in), sizeof(float2) * simt_part_elems(B.maxw))))
-    return rc;
   if (o.precision == PRONY_FFT32) return setup_fft(ctx, B);
-  if (is_tc(o.precision) && (rc = setup_tc(ctx, B, o.precision, maxR0))) return rc;
+  // a batch whose transformed blocks do not fit the device keeps the direct products
+  if (axis_pays(B.P, o.precision)) {
+    rc = setup_axis(ctx, B, o.precision);
+    if (!rc) rc = setup_products(ctx, B, o.precision);
+    if (rc && rc != PRONY_ENOMEM) return rc;
+    B.ax.on = !rc;
+    if (rc) cudaGetLastError();
+  }
+  if (!B.ax.on && (rc = setup_products(ctx, B, o.precision))) return rc;
   if (o.svd_method == 1 && fft_fits(B)) {
     // The Lanczos steps multiply by one column at a time: a tensor-core or CUDA-core product
     // costs nearly as much for one column as for twenty (the tensor-core kernel is bound by its
@@ -752,7 +943,7 @@ struct RunOut {
 
 // Key of everything a captured loop graph bakes in: the device layout (pointers, sizes), the
 // problem descriptors, the product configuration and the loop's own parameters.
-std::string loop_graph_key(const Batch& B, const int* dflag, int cap, const double* params, int nparams) {
+std::string loop_graph_key(const Batch& B, const void* xb, const int* dflag, int cap, const double* params, int nparams) {
   std::string k;
   auto put = [&](const void* p, size_t n) { k.append((const char*)p, n); };
   put(&B.D, sizeof(Dev));
@@ -767,8 +958,12 @@ std::string loop_graph_key(const Batch& B, const int* dflag, int cap, const doub
                           // the Gram and X M modes of the tensor-core pipeline (environment switches)
                           T.gram, T.nks_gram, T.gram_stages, T.njobs_gram, T.gram_stride,
                           (long long)(size_t)T.jobs_gram, T.apply, T.apply_stages, T.njobs_apply,
-                          T.apply_stride, (long long)(size_t)T.jobs_apply};
+                          T.apply_stride, (long long)(size_t)T.jobs_apply, (long long)(size_t)xb};
   put(tc, sizeof(tc));
+  if (B.ax.on) {
+    put(&B.ax.S, sizeof(Dev));
+    put(B.ax.rep.data(), sizeof(ProbDesc) * B.ax.rep.size());
+  }
   put(params, sizeof(double) * nparams);
   return k;
 }
@@ -946,8 +1141,8 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
   // ---- the steps of a solve, each enqueued on the context stream
   // grid copies and tables, the Philox start block (Algorithm 3: V_0)
   auto prefix = [&]() -> int {
-    launch_prep(D, s);
-    if (B.tc.on) launch_split_tables(D, B.tc.kind, s);
+    launch_prep(D, true, s);
+    product_tables(ctx, B, prec, 0, s);
     if (B.fft.on || B.fft.lz) launch_fft_tables(D, B.fft.maxpts, s);
     launch_init_v0(D, o.seed, s);
     if (lanczos) launch_lz_start(D, s);
@@ -1037,7 +1232,7 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
   if (graph) {
     const double par[] = {tol_rank, tol_power, tol_drop, (double)max_iter, (double)prec, (double)o.svd_method,
                           (double)o.rank_mode, (double)o.vandermonde, (double)ro.want_S};
-    std::string key = loop_graph_key(B, dflag, max_iter, par, (int)(sizeof(par) / sizeof(par[0])));
+    std::string key = loop_graph_key(B, ctx->xb.p, dflag, max_iter, par, (int)(sizeof(par) / sizeof(par[0])));
     key.append((const char*)&o.seed, sizeof(o.seed));
     if (!ctx->solve_graph.exec || key != ctx->solve_graph.key) {
       std::vector<Seg> segs;
@@ -1101,6 +1296,12 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
                      std::pow((double)K, ax) * std::pow((double)L, q.d - 1 - ax);
           fl += w * (5.0 * L * lg * lines + 6.0 * std::pow((double)L, q.d));
           by += 8.0 * q.N * w + 8.0 * rows * w + 8.0 * (double)fft_points_host(q.n, q.d);
+        } else if (B.ax.on) {
+          // as computed: the sub-products, and 4 H flops per value of the transforms (H = n + 1)
+          const ProbDesc& r2 = B.ax.rep[p];
+          const double H = q.n + 1, sub_rows = r.ext ? r2.Next : r2.N;
+          fl += q.G * w * (8.0 * sub_rows * r2.N) + w * 4.0 * H * (r2.N * H + sub_rows * (rows / sub_rows));
+          by += 8.0 * q.Gd + 8.0 * q.N * w + 8.0 * rows * w;
         } else {
           fl += 8.0 * rows * q.N * w;
           by += 8.0 * q.Gd + 8.0 * q.N * w + 8.0 * rows * w;
@@ -1171,13 +1372,13 @@ int check_tc_error(prony_ctx* ctx, const Batch& B) {
     g_err = "internal workspace bound check failed at site " + std::to_string(oob);
     return PRONY_ECUDA;
   }
-  if (!B.tc.on) return PRONY_OK;
   if (ctx->launch_err != cudaSuccess) {
     const cudaError_t e = ctx->launch_err;
     ctx->launch_err = cudaSuccess;
-    g_err = std::string("tensor-core Toeplitz launch: ") + cudaGetErrorString(e);
+    g_err = std::string("Toeplitz product launch: ") + cudaGetErrorString(e);
     return PRONY_ECUDA;
   }
+  if (!B.tc.on) return PRONY_OK;
   int h = 0;
   CK(cudaMemcpyAsync(&h, B.tc.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
@@ -1270,7 +1471,7 @@ int prony_ctx_destroy(prony_ctx* c) {
   DBuf* bufs[] = {&c->grid64, &c->gF, &c->gH, &c->V, &c->U, &c->B1, &c->B2, &c->Y, &c->small, &c->P,
                   &c->st, &c->jobs, &c->flag, &c->tout, &c->cout, &c->misc, &c->misc2, &c->misc3,
                   &c->xb, &c->tabF, &c->tabH, &c->tcjobs, &c->tcerr, &c->lmws, &c->part, &c->cnt, &c->red,
-                  &c->rcnt, &c->oob};
+                  &c->rcnt, &c->oob, &c->fhat, &c->ftw, &c->axP, &c->axtw, &c->axX, &c->axY, &c->axF, &c->axH};
   if (c->lm_exec) cudaGraphExecDestroy(c->lm_exec);
   if (c->solve_graph.exec) cudaGraphExecDestroy(c->solve_graph.exec);
   for (DBuf* b : bufs)
@@ -1642,8 +1843,10 @@ int prony_toeplitz_mm_dev(prony_ctx* ctx, const prony_c128* grid_dev, int d, int
   B.P[0].r0 = r;
   CK(cudaMemcpyAsync(ctx->P.p, B.P.data(), sizeof(ProbDesc), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->grid64.p, grid_dev, sizeof(double2) * B.P[0].Gd, cudaMemcpyDeviceToDevice, ctx->stream));
-  launch_prep(B.D, ctx->stream);
-  if (B.tc.on) launch_split_tables(B.D, B.tc.kind, ctx->stream);
+  // (the transformed tables are made from the samples themselves)
+  if (B.ax.on) launch_state_init(B.D, ctx->stream);
+  else launch_prep(B.D, false, ctx->stream);
+  product_tables(ctx, B, precision, L == n + 1, ctx->stream);
   if (B.fft.on) launch_fft_tables(B.D, B.fft.maxpts, ctx->stream);
   // operate directly on the caller's buffers: X as V (ld N), Y as Y (ld L^d)
   Dev D = B.D;

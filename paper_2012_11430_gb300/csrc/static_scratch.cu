@@ -129,7 +129,7 @@ extern "C" int prony_toeplitz_mm_static(const prony_c128* grid_dev, int d, int n
   D.red_stride = 64 * 16;
   D.rcnt = (int*)(b + kOffRcnt);
   // state (widths, flags) is rewritten by the first kernel; gF / gH are overwritten whole
-  launch_prep(D, s);
+  launch_prep(D, false, s);
   const ToeplitzJob* jobs = (const ToeplitzJob*)(b + kOffJobs);
   const int ext = (L == n + 2);
   launch_toeplitz(D, jobs, tiles * nks, adjoint, BUF_V, W_R0, ext ? BUF_Y : BUF_B2, ext, r, nullptr, nullptr, 0, s);

@@ -173,3 +173,31 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 }
 __device__ __forceinline__ float bf16lo_to_f32(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16hi_to_f32(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
+
+// ----------------------------------------------------------------------------- operand splits
+// Split an FP32 pair into BF16x2 planes (exact for three planes).
+template <int NPL>
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t* w) {
+  uint32_t h = pack_bf16x2(a, b);
+  w[0] = h;
+  float ra = a - bf16lo_to_f32(h), rb = b - bf16hi_to_f32(h);
+  uint32_t m = pack_bf16x2(ra, rb);
+  w[1] = m;
+  if (NPL == 3) {
+    ra -= bf16lo_to_f32(m);
+    rb -= bf16hi_to_f32(m);
+    w[2] = pack_bf16x2(ra, rb);
+  }
+}
+
+// Split an FP32 value into TF32 hi + lo (round to nearest, ties away; both exactly TF32).
+__device__ __forceinline__ float tf32_round(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return __uint_as_float(r);
+}
+__device__ __forceinline__ void split_tf32(float x, uint32_t* w) {
+  const float hi = tf32_round(x);
+  w[0] = __float_as_uint(hi);
+  w[1] = __float_as_uint(tf32_round(x - hi));
+}
