@@ -340,8 +340,9 @@ void launch_expsum_fwd(const double* t, const float2* c, int m, int d, const int
 void launch_expsum_bwd(const double* t, const float2* c, int m, int d, const int* lo, const int* len,
                        long long K, const float2* g, double* acc, cudaStream_t s);
 void launch_expsum_bwd_finish(const double* acc, int m, int d, double* gt, float2* gc, cudaStream_t s);
-void launch_eval_points(const double* t, const double2* c, int m, int d, const int* k, int K, double2* f,
-                        cudaStream_t s);
+size_t eval_table_bytes(int m);
+cudaError_t launch_eval_points(const double* t, const double2* c, int m, int d, const int* k, int K, double2* f,
+                               double2* tab, cudaStream_t s);
 
 // kernels_toeplitz.cu
 // One CTA of a Toeplitz product: problem, row tile, K range ks of nks.  The K ranges of a row tile

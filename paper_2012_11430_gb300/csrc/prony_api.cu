@@ -1714,16 +1714,16 @@ int prony_eval(prony_ctx* ctx, const double* t, const prony_c128* c, int m, int 
   if (K == 0) return PRONY_OK;
   CK(cudaSetDevice(ctx->device));
   int rc;
-  if ((rc = ensure(ctx->misc, sizeof(double) * m * d + sizeof(double2) * m))) return rc;
+  const size_t tbytes = (sizeof(double) * m * d + 15) / 16 * 16;
+  if ((rc = ensure(ctx->misc, tbytes + sizeof(double2) * m + eval_table_bytes(m)))) return rc;
   if ((rc = ensure(ctx->misc2, sizeof(int) * (size_t)K * d))) return rc;
   if ((rc = ensure(ctx->misc3, sizeof(double2) * (size_t)K))) return rc;
   double* td = (double*)ctx->misc.p;
-  double2* cd = (double2*)((char*)ctx->misc.p + ((sizeof(double) * m * d + 15) / 16 * 16));
+  double2* cd = (double2*)((char*)ctx->misc.p + tbytes);
   CK(cudaMemcpyAsync(td, t, sizeof(double) * m * d, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(cd, c, sizeof(double2) * m, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->misc2.p, k, sizeof(int) * (size_t)K * d, cudaMemcpyHostToDevice, ctx->stream));
-  launch_eval_points(td, cd, m, d, (const int*)ctx->misc2.p, K, (double2*)ctx->misc3.p, ctx->stream);
-  CK(cudaGetLastError());
+  CK(launch_eval_points(td, cd, m, d, (const int*)ctx->misc2.p, K, (double2*)ctx->misc3.p, cd + m, ctx->stream));
   CK(cudaMemcpyAsync(f_out, ctx->misc3.p, sizeof(double2) * (size_t)K, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return PRONY_OK;
