@@ -187,11 +187,10 @@ int prony_expsum_bwd_dev(prony_ctx* ctx, const double* t_dev, const void* c_dev,
  * Eq. (1) of Section 1; the paper fits only c by least squares (Eq. ls_probl), this also moves t.
  * t_dev: m*d float64 (in/out, kept in [0,1)), c_dev: m complex128 (in/out),
  * y_dev: prod(len) complex64 samples, loss_dev: iters+1 float64 or NULL (the loss before each
- * step and after the last).  Each step: one pass over the points for J^* J and J^* r (FP32 per
- * block, FP64 accumulators), one FP32 Cholesky solve of the Jacobi-scaled damped system
- * (Marquardt damping lambda, initial value lambda0 > 0), one trial pass; the step is taken if
- * the loss decreased (lambda / 3), else refused (lambda * 4).  All steps run as one CUDA graph,
- * captured on the first call with a given argument set and reused while the set repeats.
+ * step and after the last).  Each step: one FP32 Cholesky solve of the Jacobi-scaled damped
+ * system (Marquardt damping lambda, initial value lambda0 > 0), one pass over the points at the
+ * candidate for its loss, J^* J and J^* r (FP32 per block, FP64 accumulators); the step is taken if
+ * the loss decreased (lambda / 3), else refused (lambda * 4).
  * m * (d + 2) <= 160, else PRONY_EINVAL.  Runs on `stream` (NULL: the context stream) and
  * returns when the refined (t, c) are written. */
 int prony_refine_lm_dev(prony_ctx* ctx, double* t_dev, prony_c128* c_dev, int m, int d,

@@ -406,11 +406,9 @@ cudaError_t launch_axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int 
 
 // kernels_refine.cu (Levenberg-Marquardt refinement of (t, c))
 long long lm_workspace_bytes(int m, int d);
-size_t lm_solve_smem(int m, int d);
 cudaError_t lm_set_attributes(int m, int d);
 void launch_refine_lm(double* t, double2* c, int m, int d, const int* lo, const int* len, long long K,
                       const float2* y, int iters, double lambda0, double* hist, void* ws, cudaStream_t s);
-constexpr int LM_LAUNCHES_PER_STEP = 4;
 
 // kernels_lanczos.cu (Algorithm 2, batched)
 // kernels_small.cu: condition node of the device-side power loop (CUDA graph WHILE node)

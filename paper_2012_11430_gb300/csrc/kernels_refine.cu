@@ -1,163 +1,53 @@
 // Least-squares refinement of the exponential-sum parameters (t_j, c_j) by damped Gauss-Newton
 // (Levenberg-Marquardt) steps on L(t, c) = sum_k |f(k; t, c) - y_k|^2, f from Eq. (1), over an
-// integer box of sample points.  Every step runs on the device:
-//   k_lm_normal  one pass over the points: residual r_k, L, and the weighted Grams
-//                M^{ll'}_{ab} = sum_k w_l(k) w_l'(k) conj(e_ak) e_bk  (w_0 = 1, w_l = k_l)
-//                V^{l}_a      = sum_k w_l(k) conj(e_ak) r_k,
-//                from which J^* J and J^* r of the real parameter vector follow in closed form
-//   k_lm_solve   one CTA: the real normal equations Re(J^*J) delta = -Re(J^*r) with Marquardt
-//                damping, Jacobi-scaled and solved by an FP32 Cholesky factorisation
-//   k_lm_trial   the loss at the candidate parameters
-//   k_lm_update  accept (loss decreased) or reject, adapt the damping, clear the accumulators
+// integer box of sample points.  Every step runs on the device, in two launches:
+//   k_lm_points  at the candidate parameters: one pass over the points for L and
+//                V^{l}_a      = sum_k w_l(k) conj(e_ak) r_k  (residual r_k, w_0 = 1, w_l = k_l),
+//                from which J^* r of the real parameters follows, and Re(J^* J) from the Grams
+//                M^{ll'}_{ab} = sum_k w_l(k) w_l'(k) conj(e_ak) e_bk
+//   k_lm_step    one CTA: accept the candidate (its loss is lower) or keep the old point, adapt the
+//                damping, then the next candidate from the normal equations Re(J^*J) delta = -Re(J^*r)
+//                with Marquardt damping, Jacobi-scaled and solved by an FP32 Cholesky factorisation
+// Two sets of (J^* J, V, L) alternate: the accepted point's and the candidate's, so a rejected
+// candidate costs no new pass and an accepted one needs none either.
+//
+// On a box the sum over k of M factorises over the axes: with q = conj(e_a) e_b of one axis,
+// M^{ll'}_{ab} is a product of the d one-dimensional sums of x^p q^x (p = 0, 1, 2 times the axis occurs
+// among l, l').  A CTA computes the sums of one pair (a >= b) directly, sum_l len_l terms in place of
+// prod_l len_l, and its (d + 2)^2 entries of J^* J; the rest of the pass is the residual and V, m (d + 1) sums over the points.
 // The exponentials are recomputed in every pass, never stored; phases <t_j, k> mod 1 are exact
-// 64-bit fixed-point sums, the exponentials and sums FP32 per CTA, the accumulators FP64.
+// 64-bit fixed-point sums, the sums FP32 over at most 128 terms, the accumulators FP64.
+// Near the minimum the decision compares losses that differ by less than FP32 rounding of the model
+// would leave, so the model is evaluated beyond FP32: exp(-2 pi i u) = T[round(32 u)] (1 + eps)
+// with |eps| < 0.1, the sum of c_j T in twice FP32 (error-free sums) from a table of the CTA, the sum of
+// c_j T eps in FP32, whose rounding is ten times smaller than that of the whole.
+// Measured at d = 2, n = 63 (16384 points), m = 20: a step took 195 us (143 in a one-CTA solve with three
+// barriers per column, 40 in the M sums over all points, 9 in a separate trial pass), now 41 us (k_lm_step
+// 23, k_lm_points 17): 50 steps 10.05 -> 2.15 ms.  Both kernels are latency chains on an almost idle GPU.
 #include "common.cuh"
 
 #include <algorithm>
 
 namespace {
 
-constexpr int LM_TILE = 128;            // points per CTA (= threads) in the point passes
+constexpr int LM_TILE = 128;            // points per CTA (= threads) in the point pass
+constexpr int LM_SEG_BITS = 5, LM_SEG = 1 << LM_SEG_BITS;   // table points of the unit circle
+constexpr int LM_EP = LM_TILE + 1;      // pitch of the exponentials (threads of different terms: different banks)
+constexpr int LM_NB = 16;               // column block of the Cholesky factorisation
+constexpr int LM_SOLVE_THREADS = 512;
 constexpr double TWO_PI = 6.283185307179586;
-
-__device__ inline int combo(int l, int lp, int d) {      // index of the pair l <= lp in {0..d}
-  if (l > lp) { int x = l; l = lp; lp = x; }
-  return l * (d + 1) - l * (l - 1) / 2 + (lp - l);
-}
-
-// Residual r_k = f(k) - y_k at the point of thread `i` of a tile, with its exponentials in E.
-__device__ inline float2 point_residual(const uint64_t* T, const float2* cs, int m, int d, const Box& B,
-                                        long long q, long long K, const float2* y, float2* E, int ldE, int* k) {
-  if (q >= K) {
-    for (int j = 0; j < m; ++j) E[j * ldE] = make_float2(0.f, 0.f);
-    for (int l = 0; l < d; ++l) k[l] = 0;
-    return make_float2(0.f, 0.f);
-  }
-  box_point(B, d, q, k);
-  float2 f = make_float2(0.f, 0.f);
-  for (int j = 0; j < m; ++j) {
-    const float u = centred_phase(T + j * d, k, d);
-    float sn, cn;
-    sincospif(2.0f * u, &sn, &cn);                 // e = exp(-2 pi i u) = cn - i sn
-    E[j * ldE] = make_float2(cn, -sn);
-    f.x += cs[j].x * cn + cs[j].y * sn;
-    f.y += cs[j].y * cn - cs[j].x * sn;
-  }
-  const float2 yk = y[q];
-  return make_float2(f.x - yk.x, f.y - yk.y);
-}
-
-__device__ inline float block_sum(float v, float* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float s = 0.f;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-  return s;
-}
-
-__device__ inline void load_params(const double* t, const double2* c, int m, int d, uint64_t* T, float2* cs) {
-  for (int q = threadIdx.x; q < m * d; q += blockDim.x) T[q] = frac64(t[q]);
-  for (int q = threadIdx.x; q < m; q += blockDim.x) cs[q] = make_float2((float)c[q].x, (float)c[q].y);
-}
-
-// acc layout (double2): M[NC][m][m], V[d+1][m]; then loss, loss_trial (double)
-template <int d>
-__global__ void __launch_bounds__(LM_TILE) k_lm_normal(const double* t, const double2* c, int m, Box B, long long K,
-                                                       const float2* y, double2* M, double2* V, double* loss) {
-  extern __shared__ float2 lm_smem[];
-  float2* E = lm_smem;                                   // m x LM_TILE
-  float2* R = E + m * LM_TILE;                           // LM_TILE
-  float* Wt = (float*)(R + LM_TILE);                     // d x LM_TILE
-  __shared__ uint64_t T[PRONY_MMAX * PRONY_DMAX];
-  __shared__ float2 cs[PRONY_MMAX];
-  __shared__ float red[LM_TILE / 32];
-  load_params(t, c, m, d, T, cs);
-  __syncthreads();
-  const int i = threadIdx.x;
-  const long long q = blockIdx.x * (long long)LM_TILE + i;
-  int k[PRONY_DMAX];
-  const float2 r = point_residual(T, cs, m, d, B, q, K, y, E + i, LM_TILE, k);
-  R[i] = r;
-  for (int l = 0; l < d; ++l) Wt[l * LM_TILE + i] = (float)k[l];
-  const float l2 = block_sum(r.x * r.x + r.y * r.y, red);
-  if (i == 0) atomicAdd(loss, (double)l2);
-  __syncthreads();
-  constexpr int NC = (d + 1) * (d + 2) / 2;
-  const long long left = K - blockIdx.x * (long long)LM_TILE;
-  const int npt = left < LM_TILE ? (int)left : LM_TILE;
-  for (int idx = i; idx < m * m; idx += LM_TILE) {
-    const int a = idx / m, b = idx % m;
-    float2 acc[NC];
-#pragma unroll
-    for (int x = 0; x < NC; ++x) acc[x] = make_float2(0.f, 0.f);
-    for (int p = 0; p < npt; ++p) {
-      const float2 ea = E[a * LM_TILE + p], eb = E[b * LM_TILE + p];
-      const float2 pr = make_float2(ea.x * eb.x + ea.y * eb.y, ea.x * eb.y - ea.y * eb.x);   // conj(ea) eb
-      acc[0].x += pr.x;
-      acc[0].y += pr.y;
-      float wk[d];
-#pragma unroll
-      for (int l = 0; l < d; ++l) wk[l] = Wt[l * LM_TILE + p];
-#pragma unroll
-      for (int l = 1; l <= d; ++l) {
-        acc[l].x += wk[l - 1] * pr.x;                      // (0, l)
-        acc[l].y += wk[l - 1] * pr.y;
-      }
-      int x = d + 1;
-#pragma unroll
-      for (int l = 1; l <= d; ++l)
-#pragma unroll
-        for (int lp = l; lp <= d; ++lp, ++x) {
-          const float w2 = wk[l - 1] * wk[lp - 1];
-          acc[x].x += w2 * pr.x;
-          acc[x].y += w2 * pr.y;
-        }
-    }
-    // accumulator order above: (0,0), (0,1..d), then (l, lp >= l) for l >= 1 -- the order of combo()
-#pragma unroll
-    for (int x = 0; x < NC; ++x) {
-      double2* dst = M + ((long long)x * m + a) * m + b;
-      atomicAdd(&dst->x, (double)acc[x].x);
-      atomicAdd(&dst->y, (double)acc[x].y);
-    }
-  }
-  for (int idx = i; idx < m * (d + 1); idx += LM_TILE) {
-    const int a = idx % m, l = idx / m;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int p = 0; p < npt; ++p) {
-      const float2 ea = E[a * LM_TILE + p], rp = R[p];
-      const float w = l == 0 ? 1.f : Wt[(l - 1) * LM_TILE + p];
-      acc.x += w * (ea.x * rp.x + ea.y * rp.y);            // conj(ea) r
-      acc.y += w * (ea.x * rp.y - ea.y * rp.x);
-    }
-    double2* dst = V + (long long)l * m + a;
-    atomicAdd(&dst->x, (double)acc.x);
-    atomicAdd(&dst->y, (double)acc.y);
-  }
-}
-
-__global__ void __launch_bounds__(LM_TILE) k_lm_trial(const double* t, const double2* c, int m, int d, Box B,
-                                                      long long K, const float2* y, double* loss) {
-  extern __shared__ float2 lm_smem[];
-  __shared__ uint64_t T[PRONY_MMAX * PRONY_DMAX];
-  __shared__ float2 cs[PRONY_MMAX];
-  __shared__ float red[LM_TILE / 32];
-  load_params(t, c, m, d, T, cs);
-  __syncthreads();
-  const long long q = blockIdx.x * (long long)LM_TILE + threadIdx.x;
-  int k[PRONY_DMAX];
-  const float2 r = point_residual(T, cs, m, d, B, q, K, y, lm_smem + threadIdx.x, LM_TILE, k);
-  const float l2 = block_sum(r.x * r.x + r.y * r.y, red);
-  if (threadIdx.x == 0) atomicAdd(loss, (double)l2);
-}
 
 struct LmState {
   double lambda;
   int accepted;
+  int cur;                              // set of the accepted point (the candidate's is 1 - cur)
 };
+
+// One set of accumulators (double): Re(J^* J) [P][P] (lower triangle), V[d+1][m] (complex), the loss.
+__host__ __device__ inline long long lm_set_elems(int m, int d) {
+  const long long P = (long long)m * (d + 2);
+  return P * P + 2LL * (d + 1) * m + 1;
+}
 
 // sigma_alpha(a): the factor of column (a, alpha) of J besides w_{lambda(alpha)}(k) e_ak.
 // alpha < d: t_a(alpha) -> -2 pi i c_a, weight index alpha + 1;  alpha = d: Re c_a -> 1;  d + 1: Im c_a -> i.
@@ -170,198 +60,470 @@ __device__ inline double2 sigma_of(int alpha, int d, double2 ca, int& widx) {
   return alpha == d ? make_double2(1.0, 0.0) : make_double2(0.0, 1.0);
 }
 
-// One CTA: damped normal equations -> candidate (tc, cc).  P = m (d + 2) real parameters.
-__global__ void __launch_bounds__(256) k_lm_solve(const double* t, const double2* c, int m, int d, const double2* M,
-                                                  const double2* V, const LmState* st, double* tc, double2* cc) {
-  extern __shared__ float lm_f[];
+// acc += b in FP32; returns the rounding error of the sum (Knuth).
+__device__ inline float two_sum(float& acc, float b) {
+  const float a = acc, s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  acc = s;
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// (a + al)(b + bl) + (c + cl)(e + el) as an FP32 value and its remainder (products exact by FMA, Dekker).
+__device__ inline void dot2(float a, float al, float b, float bl, float c, float cl, float e, float el, float& hi, float& lo) {
+  float s = __fmul_rn(a, b);
+  const float r1 = __fmaf_rn(a, b, -s), p = __fmul_rn(c, e), r2 = __fmaf_rn(c, e, -p);
+  const float r3 = two_sum(s, p);
+  hi = s;
+  lo = (r1 + r2) + (r3 + ((a * bl + al * b) + (c * el + cl * e)));
+}
+
+// Leading dimension of the P + 1 rows of the solve: whole 16-byte groups, an odd number of them (the
+// rows of eight lanes then start in different banks).
+__host__ __device__ inline int lm_ld(int P) {
+  const int g = (P + 4) / 4;
+  return 4 * (g | 1);
+}
+
+__device__ inline double block_sum(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+  return s;
+}
+
+// Blocks [0, npt_blocks): 128 points each.  The others: a pair (a >= b) each.
+__global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const double2* c, int m, int d, Box B,
+                                                       long long K, int npt_blocks, const float2* y,
+                                                       const LmState* st, const float4* circle, double* sets) {
+  extern __shared__ float4 lm_smem[];
+  __shared__ uint64_t T[PRONY_MMAX * PRONY_DMAX];
+  __shared__ float2 Tf[LM_SEG];
+  __shared__ double red[LM_TILE / 32];
   const int P = m * (d + 2);
-  float* A = lm_f;                                   // P x P (lower triangle used), Jacobi-scaled
-  float* g = A + P * P;                              // P
-  float* sc = g + P;                                 // P: 1 / sqrt(damped diagonal)
-  const double lam = st->lambda;
-  // diagonal first (for the scaling)
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const int a = p / (d + 2), al = p % (d + 2);
-    int wi;
-    const double2 s = sigma_of(al, d, c[a], wi);
-    const double2 Mv = M[((long long)combo(wi, wi, d) * m + a) * m + a];
-    const double diag = (s.x * s.x + s.y * s.y) * Mv.x;
-    const double dd = diag * (1.0 + lam) + 1e-30;
-    sc[p] = (float)(1.0 / sqrt(dd));
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < P * P; idx += blockDim.x) {
-    const int p = idx / P, q = idx % P;
-    if (q > p) continue;
-    const int a = p / (d + 2), al = p % (d + 2), b = q / (d + 2), be = q % (d + 2);
-    int wa, wb;
-    const double2 sa = sigma_of(al, d, c[a], wa), sb = sigma_of(be, d, c[b], wb);
-    const double2 Mv = M[((long long)combo(wa, wb, d) * m + a) * m + b];
-    // Re( conj(sa) sb M )
-    const double2 ss = make_double2(sa.x * sb.x + sa.y * sb.y, sa.x * sb.y - sa.y * sb.x);
-    double v = ss.x * Mv.x - ss.y * Mv.y;
-    if (p == q) v *= (1.0 + lam);
-    A[p * P + q] = (float)(v * (double)sc[p] * (double)sc[q]);
-  }
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const int a = p / (d + 2), al = p % (d + 2);
-    int wi;
-    const double2 s = sigma_of(al, d, c[a], wi);
-    const double2 v = V[(long long)wi * m + a];
-    const double re = s.x * v.x + s.y * v.y;          // Re( conj(s) v )
-    g[p] = (float)(-re * (double)sc[p]);
-  }
-  __syncthreads();
-  // Cholesky A = L L^T (lower, in place), right-looking
-  for (int j = 0; j < P; ++j) {
-    if (threadIdx.x == 0) A[j * P + j] = sqrtf(fmaxf(A[j * P + j], 1e-20f));
+  double* H = sets + (1 - st->cur) * lm_set_elems(m, d);
+  if ((int)blockIdx.x >= npt_blocks) {
+    __shared__ double axis_sum[LM_TILE / 32][PRONY_DMAX][6];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int pair = (int)blockIdx.x - npt_blocks;                // a (a + 1) / 2 + b
+    int a = (int)((sqrtf(8.f * pair + 1.f) - 1.f) * 0.5f);
+    while (a * (a + 1) / 2 > pair) --a;
+    while ((a + 1) * (a + 2) / 2 <= pair) ++a;
+    const int b = pair - a * (a + 1) / 2;
+    for (int l = threadIdx.x; l < d; l += LM_TILE)                // conj(e_a) e_b = exp(-2 pi i (t_b - t_a) x)
+      T[l] = frac64(t[b * d + l]) - frac64(t[a * d + l]);
     __syncthreads();
-    const float ljj = A[j * P + j];
-    for (int i = j + 1 + threadIdx.x; i < P; i += blockDim.x) A[i * P + j] /= ljj;
-    __syncthreads();
-    const int rem = P - j - 1;
-    for (int idx = threadIdx.x; idx < rem * rem; idx += blockDim.x) {
-      const int i = j + 1 + idx / rem, k2 = j + 1 + idx % rem;
-      if (k2 <= i) A[i * P + k2] -= A[i * P + j] * A[k2 * P + j];
+    for (int l = 0; l < d; ++l) {
+      const uint64_t dt = T[l];
+      double tot = 0.0;                                           // lane z < 6: the z-th sum of the warp
+      for (int i0 = 0; i0 < B.len[l]; i0 += 32 * LM_TILE) {       // at most 32 FP32 terms per thread, then FP64
+        float s[6] = {};
+        const int i1 = min(B.len[l], i0 + 32 * LM_TILE);
+        for (int i = i0 + threadIdx.x; i < i1; i += LM_TILE) {
+          const int x = B.lo[l] + i;
+          const float u = (float)(int)((dt * (uint64_t)(long long)x) >> 32) * 2.3283064365386963e-10f;
+          float sn, cn;
+          sincospif(2.0f * u, &sn, &cn);
+          const float xf = (float)x, x2 = xf * xf;
+          s[0] += cn;
+          s[1] -= sn;
+          s[2] += xf * cn;
+          s[3] -= xf * sn;
+          s[4] += x2 * cn;
+          s[5] -= x2 * sn;
+        }
+        float mine = 0.f;
+#pragma unroll
+        for (int z = 0; z < 6; ++z) {                             // FP32 over a warp, FP64 beyond
+          for (int o = 16; o > 0; o >>= 1) s[z] += __shfl_xor_sync(0xffffffffu, s[z], o);
+          if (lane == z) mine = s[z];
+        }
+        tot += (double)mine;
+      }
+      if (lane < 6) axis_sum[warp][l][lane] = tot;
     }
     __syncthreads();
+    const int al = threadIdx.x / (d + 2), be = threadIdx.x % (d + 2);
+    const int p = a * (d + 2) + al, q = b * (d + 2) + be;
+    for (int z = threadIdx.x; z < 6 * d; z += LM_TILE)            // the warps' sums, in order
+      axis_sum[0][z / 6][z % 6] += axis_sum[1][z / 6][z % 6] + axis_sum[2][z / 6][z % 6] + axis_sum[3][z / 6][z % 6];
+    __syncthreads();
+    if (al < d + 2 && q <= p) {
+      int wa, wb;
+      const double2 sa = sigma_of(al, d, c[a], wa), sb = sigma_of(be, d, c[b], wb);
+      double2 v = make_double2(sa.x * sb.x + sa.y * sb.y, sa.x * sb.y - sa.y * sb.x);   // conj(sa) sb M_ab
+      for (int l = 0; l < d; ++l) {
+        const int pw = 2 * ((wa == l + 1) + (wb == l + 1));
+        v = cmul(v, make_double2(axis_sum[0][l][pw], axis_sum[0][l][pw + 1]));
+      }
+      H[(long long)p * P + q] = v.x;
+    }
+    return;
   }
-  // triangular solves by one warp: L z = g, L^T x = z
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    for (int j = 0; j < P; ++j) {
-      const float zj = g[j] / A[j * P + j];
-      __syncwarp();
-      for (int i = j + 1 + lane; i < P; i += 32) g[i] -= A[i * P + j] * zj;
-      if (lane == 0) g[j] = zj;
-      __syncwarp();
-    }
-    for (int j = P - 1; j >= 0; --j) {
-      const float xj = g[j] / A[j * P + j];
-      __syncwarp();
-      for (int i = lane; i < j; i += 32) g[i] -= A[j * P + i] * xj;
-      if (lane == 0) g[j] = xj;
-      __syncwarp();
-    }
+  float4* CT = lm_smem;                                  // m x LM_SEG: c_j T as (Re, Im) + (Re, Im) 2^-24 below
+  float2* E = (float2*)(CT + m * LM_SEG);                // m x LM_EP: exponentials of this thread's point
+  float2* R = E + m * LM_EP;                             // LM_TILE: residuals
+  float2* part = R + LM_TILE;                            // LM_TILE partial sums of V
+  float* Wt = (float*)(part + LM_TILE);                  // d x LM_TILE
+  for (int q = threadIdx.x; q < m * d; q += blockDim.x) T[q] = frac64(t[q]);
+  for (int q = threadIdx.x; q < LM_SEG; q += blockDim.x) Tf[q] = make_float2(circle[q].x, circle[q].y);
+  for (int q = threadIdx.x; q < m * LM_SEG; q += blockDim.x) {
+    const double2 c2 = c[q / LM_SEG];
+    const float4 T2 = circle[q % LM_SEG];
+    const float cx = (float)c2.x, cy = (float)c2.y, cxl = (float)(c2.x - cx), cyl = (float)(c2.y - cy);
+    float4 v;
+    dot2(cx, cxl, T2.x, T2.z, -cy, -cyl, T2.y, T2.w, v.x, v.z);
+    dot2(cx, cxl, T2.y, T2.w, cy, cyl, T2.x, T2.z, v.y, v.w);
+    CT[q] = v;
   }
   __syncthreads();
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const int a = p / (d + 2), al = p % (d + 2);
-    const double delta = (double)g[p] * (double)sc[p];
-    if (al < d) {
-      double v = t[a * d + al] + delta;
-      v -= floor(v);                                   // f is 1-periodic in each t_a(l)
-      tc[a * d + al] = v;
-    } else if (al == d) {
-      cc[a].x = c[a].x + delta;
+  const int i = threadIdx.x;
+  const long long q = blockIdx.x * (long long)LM_TILE + i;
+  double2 rd = make_double2(0.0, 0.0);
+  int k[PRONY_DMAX] = {0, 0, 0, 0};
+  if (q < K) {
+    if (K <= 0xFFFFFFFFLL) {
+      unsigned rem = (unsigned)q;
+      for (int l = d - 1; l >= 0; --l) {
+        const unsigned len = (unsigned)B.len[l], nx = rem / len;
+        k[l] = B.lo[l] + (int)(rem - nx * len);
+        rem = nx;
+      }
     } else {
-      cc[a].y = c[a].y + delta;
+      box_point(B, d, q, k);
+    }
+    float2 fh = make_float2(0.f, 0.f), fe = fh;           // sum of c T, and of its remainders and c T eps
+    for (int j = 0; j < m; ++j) {
+      uint64_t ph = 0;
+      for (int l = 0; l < d; ++l) ph += T[j * d + l] * (uint64_t)(long long)k[l];
+      const int seg = (int)((ph + (1ull << (63 - LM_SEG_BITS))) >> (64 - LM_SEG_BITS));        // nearest table point
+      const int rem = (int)((long long)(ph - ((uint64_t)seg << (64 - LM_SEG_BITS))) >> 27);   // the rest in 2^-37 turns
+      const float x = (float)rem * 4.5716190e-11f, x2 = x * x;                                // 2 pi 2^-37; |x| <= pi / 32
+      // Taylor polynomials: the first terms left out are below 2e-11
+      const float sn = x * (1.f + x2 * (-1.f / 6.f + x2 * (1.f / 120.f)));
+      const float cm = x2 * (-0.5f + x2 * (1.f / 24.f - x2 * (1.f / 720.f)));                 // cos x - 1
+      const float4 ct = CT[j * LM_SEG + seg];
+      const float2 tf = Tf[seg];
+      fe.x += two_sum(fh.x, ct.x) + (ct.z + (ct.x * cm + ct.y * sn));     // c T (cm - i sn)
+      fe.y += two_sum(fh.y, ct.y) + (ct.w + (ct.y * cm - ct.x * sn));
+      E[j * LM_EP + i] = make_float2(tf.x + (tf.x * cm + tf.y * sn), tf.y + (tf.y * cm - tf.x * sn));
+    }
+    const float2 yk = y[q];
+    rd = make_double2((double)fh.x - (double)yk.x + (double)fe.x, (double)fh.y - (double)yk.y + (double)fe.y);
+  } else {
+    for (int j = 0; j < m; ++j) E[j * LM_EP + i] = make_float2(0.f, 0.f);
+  }
+  R[i] = make_float2((float)rd.x, (float)rd.y);
+  for (int l = 0; l < d; ++l) Wt[l * LM_TILE + i] = (float)k[l];
+  double* V = H + (long long)P * P;
+  const double l2 = block_sum(rd.x * rd.x + rd.y * rd.y, red);
+  if (i == 0) atomicAdd(&V[2 * (d + 1) * m], l2);
+  __syncthreads();
+  // V: one thread per (a, l) and slice of the points, the slices added in order
+  const int nv = m * (d + 1), slices = max(1, LM_TILE / nv), per = LM_TILE / slices;
+  for (int base = 0; base < nv; base += LM_TILE) {
+    const int idx = slices > 1 ? i % nv : base + i, sl = slices > 1 ? i / nv : 0;
+    float2 acc = make_float2(0.f, 0.f);
+    if (idx < nv && sl < slices) {
+      const int a = idx % m, l = idx / m;
+      const int p1 = sl + 1 == slices ? LM_TILE : (sl + 1) * per;
+      for (int p = sl * per; p < p1; ++p) {
+        const float2 ea = E[a * LM_EP + p], rp = R[p];
+        const float w = l == 0 ? 1.f : Wt[(l - 1) * LM_TILE + p];
+        acc.x += w * (ea.x * rp.x + ea.y * rp.y);          // conj(ea) r
+        acc.y += w * (ea.x * rp.y - ea.y * rp.x);
+      }
+    }
+    if (slices > 1) {
+      part[i] = acc;
+      __syncthreads();
+      if (sl == 0)
+        for (int s2 = 1; s2 < slices; ++s2) {
+          acc.x += part[i + s2 * nv].x;
+          acc.y += part[i + s2 * nv].y;
+        }
+    }
+    if (idx < nv && sl == 0) {
+      atomicAdd(&V[2 * idx], (double)acc.x);               // V[l][a] at l m + a = idx
+      atomicAdd(&V[2 * idx + 1], (double)acc.y);
     }
   }
 }
 
-// Accept or reject the candidate; record the loss; clear the accumulators of the next step.
-__global__ void k_lm_update(double* t, double2* c, const double* tc, const double2* cc, int m, int d,
-                            LmState* st, double2* acc, long long nacc, double* loss, double* hist, int it) {
-  __shared__ int ok;
+// GB300 does about two FP64 operations per clock and SM (an FP64 square root takes thousands of cycles,
+// and conversions share the pipe), so the scaling of the normal matrix works on the bits.
+__device__ inline int exponent_of(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF) - 1023; }
+// v 2^(-shift) in FP32 (rounded to nearest, ties away; below the FP32 range: zero; NaN for NaN and infinity)
+__device__ inline float scaled_float(double v, int shift) {
+  const uint64_t b = (uint64_t)__double_as_longlong(v);
+  const int e11 = (int)((b >> 52) & 0x7FF), e = e11 - 896 - shift;
+  const uint32_t sign = (uint32_t)(b >> 63) << 31;
+  uint32_t f = ((uint32_t)e << 23 | (uint32_t)((b >> 29) & 0x7FFFFF)) + (uint32_t)((b >> 28) & 1);
+  if (e <= 0) f = 0;
+  if (e11 == 0x7FF || e >= 255) f = 0x7FC00000u;
+  return __uint_as_float(f | sign);
+}
+
+// One CTA.  Decision on the candidate (step > 0; step 0 takes the starting point), then (solve) the
+// damped normal equations at the accepted point -> next candidate.  P = m (d + 2) real parameters.
+//
+// Cholesky in blocks of 16 columns, with the right-hand side as an extra row, so that the forward
+// substitution comes with the factorisation: the diagonal block by one warp (a row per lane, in
+// registers, columns by shuffles), the rows below it by one thread each (16 columns in registers),
+// the trailing block in 4 x 4 register tiles on and below the diagonal, 16 bytes per shared-memory
+// access.  Three barriers per block instead of three per column; bound by the chain of dependent
+// square roots and shuffles of the diagonal blocks.
+__global__ void __launch_bounds__(LM_SOLVE_THREADS) k_lm_step(double* t, double2* c, double* tc, double2* cc, int m,
+                                                              int d, LmState* st, double* sets, double* hist, int step,
+                                                              int solve) {
+  extern __shared__ __align__(16) float lm_f[];
+  __shared__ int s_ok, s_cur;
+  __shared__ float dinv[PRONY_LM_PMAX];
+  __shared__ __align__(16) float Ld[LM_NB][LM_NB];
+  __shared__ double2 cs[PRONY_MMAX];
+  const int P = m * (d + 2), ld = lm_ld(P);
+  const long long ns = lm_set_elems(m, d);
+  float* A = lm_f;                                   // ld x ld, lower triangle; row P: right-hand side
+  float* Pt = A + ld * ld;                           // LM_NB x ld: the rows below a diagonal block, transposed
+  float* sc = Pt + LM_NB * ld;                       // P: 1 / sqrt(damped diagonal) = sc 2^(-sh)
+  int* sh = (int*)(sc + ld);
   if (threadIdx.x == 0) {
-    const double l0 = loss[0], l1 = loss[1];
-    ok = (l1 < l0 && isfinite(l1)) ? 1 : 0;
-    if (hist) {
-      hist[it] = l0;
-      hist[it + 1] = ok ? l1 : l0;
+    const int cand = 1 - st->cur;
+    const double l0 = sets[(st->cur + 1) * ns - 1], l1 = sets[(cand + 1) * ns - 1];
+    const int ok = step == 0 || (l1 < l0 && isfinite(l1));
+    if (hist) hist[step] = ok ? l1 : l0;
+    if (step > 0) {
+      st->lambda = ok ? fmax(st->lambda * (1.0 / 3.0), 1e-12) : fmin(st->lambda * 4.0, 1e12);
+      st->accepted += ok;
     }
-    st->lambda = ok ? fmax(st->lambda * (1.0 / 3.0), 1e-12) : fmin(st->lambda * 4.0, 1e12);
-    st->accepted += ok;
+    if (ok) st->cur = cand;
+    s_ok = ok;
+    s_cur = st->cur;
   }
   __syncthreads();
-  if (ok) {
+  if (s_ok && step > 0) {
     for (int q = threadIdx.x; q < m * d; q += blockDim.x) t[q] = tc[q];
     for (int q = threadIdx.x; q < m; q += blockDim.x) c[q] = cc[q];
   }
-  for (long long q = threadIdx.x; q < nacc; q += blockDim.x) acc[q] = make_double2(0.0, 0.0);
-  if (threadIdx.x < 2) loss[threadIdx.x] = 0.0;
+  // the other set takes the next candidate: V and the loss are accumulated
+  for (int q = threadIdx.x; q < 2 * (d + 1) * m + 1; q += blockDim.x) sets[(2 - s_cur) * ns - 1 - q] = 0.0;
+  if (!solve) return;
+  const double lam = st->lambda;
+  const double* H = sets + s_cur * ns;
+  const double* V = H + (long long)P * P;
+  for (int q = threadIdx.x; q < m; q += blockDim.x) cs[q] = (s_ok && step > 0) ? cc[q] : c[q];
+  // the diagonal first (for the scaling)
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    const double v = H[(long long)p * P + p] * (1.0 + lam) + 1e-30;
+    const int h = exponent_of(v) >> 1;
+    const float f = scaled_float(v, 2 * h), r = rsqrtf(f);        // f in [1, 4)
+    sh[p] = h;
+    sc[p] = r;
+    A[p * ld + p] = f * r * r;
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < P * (P - 1) / 2; idx += LM_SOLVE_THREADS) {   // entries below the diagonal
+    int p = (int)((sqrtf(8.f * idx + 1.f) + 1.f) * 0.5f);
+    if (p * (p - 1) / 2 > idx) --p;
+    if (p * (p + 1) / 2 <= idx) ++p;
+    const int q = idx - p * (p - 1) / 2;
+    A[p * ld + q] = scaled_float(H[(long long)p * P + q], sh[p] + sh[q]) * sc[p] * sc[q];
+  }
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    const int a = p / (d + 2), al = p % (d + 2);
+    int wi;
+    const double2 s = sigma_of(al, d, cs[a], wi);
+    const double* v = V + 2 * (wi * m + a);
+    const double re = s.x * v[0] + s.y * v[1];        // Re( conj(s) v )
+    A[P * ld + p] = scaled_float(-re, sh[p]) * sc[p];
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int k0 = 0; k0 < P; k0 += LM_NB) {
+    const int nb = min(LM_NB, P - k0);
+    __syncthreads();
+    if (warp == 0) {
+      float row[LM_NB];
+#pragma unroll
+      for (int x = 0; x < LM_NB; ++x) row[x] = (lane < nb && x <= lane) ? A[(k0 + lane) * ld + k0 + x] : 0.f;
+#pragma unroll
+      for (int j = 0; j < LM_NB; ++j) {
+        const float dj = __shfl_sync(0xffffffffu, row[j], j);
+        const float dv = fmaxf(dj, 1e-20f), inv = rsqrtf(dv), root = dv * inv;
+        const float l = lane == j ? root : row[j] * inv;
+        row[j] = l;
+        if (lane == j && j < nb) dinv[k0 + j] = inv;
+#pragma unroll
+        for (int x = j + 1; x < LM_NB; ++x) row[x] -= l * __shfl_sync(0xffffffffu, l, x);
+      }
+      if (lane < LM_NB) {
+#pragma unroll
+        for (int x = 0; x < LM_NB; ++x) {
+          const float v = (lane < nb && x < nb && x <= lane) ? row[x] : 0.f;
+          Ld[lane][x] = v;
+          if (lane < nb && x <= lane) A[(k0 + lane) * ld + k0 + x] = v;
+        }
+      }
+    }
+    __syncthreads();
+    const int r0 = k0 + nb, nr = P + 1 - r0;         // rows below, the right-hand side among them
+    for (int i = threadIdx.x; i < nr; i += blockDim.x) {
+      float* Ai = A + (r0 + i) * ld + k0;
+      float x[LM_NB];
+#pragma unroll
+      for (int j = 0; j < LM_NB; j += 4) *(float4*)(x + j) = *(const float4*)(Ai + j);
+#pragma unroll
+      for (int j = 0; j < LM_NB; ++j) {
+        x[j] = j < nb ? x[j] * dinv[k0 + j] : 0.f;
+#pragma unroll
+        for (int e = j + 1; e < LM_NB; ++e) x[e] -= x[j] * Ld[e][j];
+        Pt[j * ld + i] = x[j];
+      }
+#pragma unroll
+      for (int j = 0; j < LM_NB; ++j)
+        if (j < nb) Ai[j] = x[j];
+    }
+    if (r0 >= P) break;
+    __syncthreads();
+    // trailing block: rows r0 + 4 ti .., columns r0 + 4 tj .., tj <= ti (what lies above the diagonal or
+    // past row P is never read)
+    const int nt = (nr + 3) / 4;
+    for (int tile = threadIdx.x; tile < nt * (nt + 1) / 2; tile += blockDim.x) {
+      int ti = (int)((sqrtf(8.f * tile + 1.f) - 1.f) * 0.5f);
+      if (ti * (ti + 1) / 2 > tile) --ti;
+      if ((ti + 1) * (ti + 2) / 2 <= tile) ++ti;
+      const int tj = tile - ti * (ti + 1) / 2;
+      float acc[4][4] = {};
+#pragma unroll 4
+      for (int j = 0; j < LM_NB; ++j) {
+        const float4 x4 = *(const float4*)(Pt + j * ld + 4 * ti), z4 = *(const float4*)(Pt + j * ld + 4 * tj);
+        const float x[4] = {x4.x, x4.y, x4.z, x4.w}, z[4] = {z4.x, z4.y, z4.z, z4.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] += x[u] * z[v];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float4* at = (float4*)(A + (r0 + 4 * ti + u) * ld + r0 + 4 * tj);
+        float4 o = *at;
+        o.x -= acc[u][0];
+        o.y -= acc[u][1];
+        o.z -= acc[u][2];
+        o.w -= acc[u][3];
+        *at = o;
+      }
+    }
+  }
+  __syncthreads();
+  // L^T x = z (row P) by one warp: lane l keeps the running residuals of the entries l + 32 q
+  if (warp == 0) {
+    constexpr int NQ = PRONY_LM_PMAX / 32;
+    float r[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) r[q] = lane + 32 * q < P ? A[P * ld + lane + 32 * q] : 0.f;
+#pragma unroll
+    for (int q = NQ - 1; q >= 0; --q)
+#pragma unroll 4
+      for (int jj = min(31, P - 1 - 32 * q); jj >= 0; --jj) {
+        const int j = 32 * q + jj;
+        const float xj = __shfl_sync(0xffffffffu, r[q], jj) * dinv[j];
+#pragma unroll
+        for (int e = 0; e <= q; ++e)
+          if (lane + 32 * e < j) r[e] -= A[j * ld + lane + 32 * e] * xj;
+        if (lane == jj) r[q] = xj;
+      }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+      if (lane + 32 * q < P) A[P * ld + lane + 32 * q] = r[q];
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < P; p += blockDim.x) {
+    const int a = p / (d + 2), al = p % (d + 2);
+    // sc 2^(-sh) in FP64
+    const double delta = (double)(A[P * ld + p] * sc[p]) * __longlong_as_double((long long)(1023 - sh[p]) << 52);
+    if (al < d) {
+      // tc holds the accepted point if the last candidate was taken, t always does
+      double v = ((s_ok && step > 0) ? tc[a * d + al] : t[a * d + al]) + delta;
+      v -= floor(v);                                   // f is 1-periodic in each t_a(l)
+      tc[a * d + al] = v;
+    } else if (al == d) {
+      cc[a].x = cs[a].x + delta;
+    } else {
+      cc[a].y = cs[a].y + delta;
+    }
+  }
 }
 
-__global__ void k_lm_init(LmState* st, double lambda0, double2* acc, long long nacc, double* loss, const double2* c,
-                          double2* cc, int m) {
+// The starting point as the first candidate, empty accumulators.
+__global__ void k_lm_init(LmState* st, double lambda0, double* sets, const double* t, const double2* c, double* tc,
+                          double2* cc, float4* circle, int m, int d) {
+  const long long ns = lm_set_elems(m, d);
   if (threadIdx.x == 0) {
     st->lambda = lambda0;
     st->accepted = 0;
+    st->cur = 1;
   }
-  for (long long q = threadIdx.x; q < nacc; q += blockDim.x) acc[q] = make_double2(0.0, 0.0);
+  for (int q = threadIdx.x; q < LM_SEG; q += blockDim.x) {     // exp(-2 pi i q / LM_SEG)
+    double sn, cn;
+    sincospi(2.0 * q / LM_SEG, &sn, &cn);
+    const float cf = (float)cn, sf = (float)-sn;
+    circle[q] = make_float4(cf, sf, (float)(cn - cf), (float)(-sn - sf));
+  }
+  for (int q = threadIdx.x; q < m * d; q += blockDim.x) tc[q] = t[q];
   for (int q = threadIdx.x; q < m; q += blockDim.x) cc[q] = c[q];
-  if (threadIdx.x < 2) loss[threadIdx.x] = 0.0;
+  for (int q = threadIdx.x; q < 2 * (d + 1) * m + 1; q += blockDim.x) sets[ns - 1 - q] = sets[2 * ns - 1 - q] = 0.0;
 }
 
-inline int lm_blocks(long long K) { return (int)((K + LM_TILE - 1) / LM_TILE); }
+size_t lm_points_smem(int m, int d) {
+  return sizeof(float4) * (size_t)m * LM_SEG + sizeof(float2) * ((size_t)m * LM_EP + 2 * LM_TILE) +
+         sizeof(float) * (size_t)d * LM_TILE;
+}
+size_t lm_step_smem(int m, int d) {
+  const size_t ld = lm_ld(m * (d + 2));
+  return sizeof(float) * (ld * ld + LM_NB * ld + 2 * ld);
+}
 
 }  // namespace
 
 // ----------------------------------------------------------------------------- host side
 long long lm_workspace_bytes(int m, int d) {
-  const int NC = (d + 1) * (d + 2) / 2;
-  const long long nacc = (long long)NC * m * m + (long long)(d + 1) * m;
-  return 16 * nacc + 16 * m + 8 * (long long)m * d + 16 + 64;
+  return 8 * (2 * lm_set_elems(m, d) + (long long)m * d) + 16LL * (m + LM_SEG) + sizeof(LmState) + 64;
 }
 
-size_t lm_solve_smem(int m, int d) {
-  const int P = m * (d + 2);
-  return sizeof(float) * ((size_t)P * P + 2 * P);
-}
-
-static size_t lm_normal_smem(int m, int d) {
-  return sizeof(float2) * (size_t)(m + 1) * LM_TILE + sizeof(float) * (size_t)d * LM_TILE;
-}
-
-// Dynamic shared-memory limits of the refinement kernels (outside any stream capture).
+// Dynamic shared-memory limits of the refinement kernels.
 cudaError_t lm_set_attributes(int m, int d) {
-  static size_t set_n[PRONY_DMAX + 1] = {0, 0, 0, 0, 0}, set_t = 0, set_s = 0;
-  void (*normal)(const double*, const double2*, int, Box, long long, const float2*, double2*, double2*, double*) =
-      d == 1 ? k_lm_normal<1> : d == 2 ? k_lm_normal<2> : d == 3 ? k_lm_normal<3> : k_lm_normal<4>;
-  const size_t sn = lm_normal_smem(m, d), st = sizeof(float2) * (size_t)m * LM_TILE, ss = lm_solve_smem(m, d);
+  static size_t set_p = 0, set_s = 0;
+  const size_t sp = lm_points_smem(m, d), ss = lm_step_smem(m, d);
   cudaError_t e = cudaSuccess;
-  if (sn > set_n[d] && (e = cudaFuncSetAttribute(normal, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sn)) ==
-                           cudaSuccess)
-    set_n[d] = sn;
-  if (e == cudaSuccess && st > set_t &&
-      (e = cudaFuncSetAttribute(k_lm_trial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st)) == cudaSuccess)
-    set_t = st;
+  if (sp > set_p &&
+      (e = cudaFuncSetAttribute(k_lm_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp)) == cudaSuccess)
+    set_p = sp;
   if (e == cudaSuccess && ss > set_s &&
-      (e = cudaFuncSetAttribute(k_lm_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss)) == cudaSuccess)
+      (e = cudaFuncSetAttribute(k_lm_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss)) == cudaSuccess)
     set_s = ss;
   return e;
 }
 
-// The whole refinement, enqueued on `s` (launches only: capturable in a CUDA graph; the
-// shared-memory attributes are set beforehand by lm_set_attributes).
+// The whole refinement, enqueued on `s`: 2 iters + 3 launches (the host stays ahead of the device,
+// so no graph is kept).
 void launch_refine_lm(double* t, double2* c, int m, int d, const int* lo, const int* len, long long K,
                       const float2* y, int iters, double lambda0, double* hist, void* ws, cudaStream_t s) {
-  const int NC = (d + 1) * (d + 2) / 2;
-  const long long nacc = (long long)NC * m * m + (long long)(d + 1) * m;
-  double2* acc = (double2*)ws;
-  double2* M = acc;
-  double2* V = acc + (long long)NC * m * m;
-  double2* cc = acc + nacc;
+  float4* circle = (float4*)ws;
+  double2* cc = (double2*)(circle + LM_SEG);
   double* tc = (double*)(cc + m);
-  double* loss = tc + m * d;                            // loss, loss_trial
-  LmState* st = (LmState*)(loss + 2);
+  double* sets = tc + m * d;
+  LmState* st = (LmState*)(sets + 2 * lm_set_elems(m, d));
   const Box B = make_box(d, lo, len);
-  const size_t sm_normal = lm_normal_smem(m, d);
-  const size_t sm_trial = sizeof(float2) * (size_t)m * LM_TILE;
-  const size_t sm_solve = lm_solve_smem(m, d);
-  void (*normal)(const double*, const double2*, int, Box, long long, const float2*, double2*, double2*, double*) =
-      d == 1 ? k_lm_normal<1> : d == 2 ? k_lm_normal<2> : d == 3 ? k_lm_normal<3> : k_lm_normal<4>;
+  const size_t sp = lm_points_smem(m, d), ss = lm_step_smem(m, d);
+  const int npt = (int)((K + LM_TILE - 1) / LM_TILE), npair = m * (m + 1) / 2;
   note_launch();
-  k_lm_init<<<1, 256, 0, s>>>(st, lambda0, acc, nacc, loss, c, cc, m);
-  for (int it = 0; it < iters; ++it) {
+  k_lm_init<<<1, 256, 0, s>>>(st, lambda0, sets, t, c, tc, cc, circle, m, d);
+  for (int it = 0; it <= iters; ++it) {
     note_launch();
-    normal<<<lm_blocks(K), LM_TILE, sm_normal, s>>>(t, c, m, B, K, y, M, V, loss);
+    k_lm_points<<<npt + npair, LM_TILE, sp, s>>>(tc, cc, m, d, B, K, npt, y, st, circle, sets);
     note_launch();
-    k_lm_solve<<<1, 256, sm_solve, s>>>(t, c, m, d, M, V, st, tc, cc);
-    note_launch();
-    k_lm_trial<<<lm_blocks(K), LM_TILE, sm_trial, s>>>(tc, cc, m, d, B, K, y, loss + 1);
-    note_launch();
-    k_lm_update<<<1, 256, 0, s>>>(t, c, tc, cc, m, d, st, acc, nacc, loss, hist, it);
+    k_lm_step<<<1, LM_SOLVE_THREADS, ss, s>>>(t, c, tc, cc, m, d, st, sets, hist, it, it < iters);
   }
 }

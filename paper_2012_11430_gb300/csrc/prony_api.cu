@@ -93,14 +93,7 @@ struct prony_ctx {
   // built for, and its ext / in counts (a repeated batch layout skips the rebuild and the upload)
   std::vector<int> tcjob_sig;
   int tcjob_next = 0, tcjob_nin = 0, tcjob_ngram = 0, tcjob_napply = 0;
-  // refinement: workspace and the CUDA graph of the last argument set
-  DBuf lmws;
-  struct LmKey {
-    const void *t, *c, *y, *loss, *ws;
-    int m, d, iters, lo[PRONY_DMAX], len[PRONY_DMAX];
-    double lambda0;
-  } lm_key{};
-  cudaGraphExec_t lm_exec = nullptr;
+  DBuf lmws;                            // refinement workspace
   // the whole solve as one CUDA graph, for the last batch layout and options
   struct SolveGraph {
     std::string key;
@@ -1472,7 +1465,6 @@ int prony_ctx_destroy(prony_ctx* c) {
                   &c->st, &c->jobs, &c->flag, &c->tout, &c->cout, &c->misc, &c->misc2, &c->misc3,
                   &c->xb, &c->tabF, &c->tabH, &c->tcjobs, &c->tcerr, &c->lmws, &c->part, &c->cnt, &c->red,
                   &c->rcnt, &c->oob, &c->fhat, &c->ftw, &c->axP, &c->axtw, &c->axX, &c->axY, &c->axF, &c->axH};
-  if (c->lm_exec) cudaGraphExecDestroy(c->lm_exec);
   if (c->solve_graph.exec) cudaGraphExecDestroy(c->solve_graph.exec);
   for (DBuf* b : bufs)
     if (b->p) cudaFree(b->p);
@@ -1765,31 +1757,10 @@ int prony_refine_lm_dev(prony_ctx* ctx, double* t_dev, prony_c128* c_dev, int m,
   if (iters == 0) return PRONY_OK;
   int rc;
   if ((rc = ensure(ctx->lmws, (size_t)lm_workspace_bytes(m, d)))) return rc;
-  prony_ctx::LmKey k{};
-  k.t = t_dev; k.c = c_dev; k.y = y_dev; k.loss = loss_dev; k.ws = ctx->lmws.p;
-  k.m = m; k.d = d; k.iters = iters; k.lambda0 = lambda0;
-  for (int l = 0; l < d; ++l) { k.lo[l] = lo[l]; k.len[l] = len[l]; }
-  if (!ctx->lm_exec || std::memcmp(&k, &ctx->lm_key, sizeof(k)) != 0) {
-    if (ctx->lm_exec) {
-      cudaGraphExecDestroy(ctx->lm_exec);
-      ctx->lm_exec = nullptr;
-    }
-    CK(lm_set_attributes(m, d));
-    // capture on the context stream (never the legacy default stream), launch on `s`
-    CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-    launch_refine_lm(t_dev, (double2*)c_dev, m, d, lo, len, K, (const float2*)y_dev, iters, lambda0, loss_dev,
-                     ctx->lmws.p, ctx->stream);
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamEndCapture(ctx->stream, &g));
-    cudaError_t e = cudaGraphInstantiate(&ctx->lm_exec, g, 0);
-    cudaGraphDestroy(g);
-    CK(e);
-    ctx->lm_key = k;
-  } else {
-    note_launches(1 + (long long)LM_LAUNCHES_PER_STEP * iters);
-  }
-  CK(cudaGraphLaunch(ctx->lm_exec, s));
+  CK(lm_set_attributes(m, d));
+  launch_refine_lm(t_dev, (double2*)c_dev, m, d, lo, len, K, (const float2*)y_dev, iters, lambda0, loss_dev,
+                   ctx->lmws.p, s);
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return PRONY_OK;
 }

@@ -6,7 +6,7 @@ backward the vector-Jacobian product for t (float64) and c (complex64).  Nothing
 for backward except the inputs: the exponentials are recomputed by the backward kernel.
 
 `refine_adam` runs a torch optimizer on L = sum_k |f(k) - y_k|^2 through ExpSumFn;
-`refine_lm` calls the library's on-device Levenberg-Marquardt steps (one CUDA graph).
+`refine_lm` calls the library's on-device Levenberg-Marquardt steps.
 Both are argument marshalling around libprony.so; there is no CPU fallback.
 """
 from __future__ import annotations

@@ -156,3 +156,57 @@ def test_adam_through_autograd_reduces_loss(ctx):
                                lr_t=2e-4, lr_c=1e-2)
     losses = losses.cpu().numpy()
     assert losses[-1] < 0.5 * losses[0]
+
+
+# ------------------------------------------------------------------ step kernels at their edges
+def _lm64(t, c, k, y, steps, lam=1e-3):
+    """The same damped Gauss-Newton iteration in FP64; returns (t, c, losses)."""
+    res = lambda t, c: O.expsum(t, c, k) - y  # noqa: E731
+    r = res(t, c)
+    L = float(np.sum(np.abs(r) ** 2))
+    losses = [L]
+    for _ in range(steps):
+        e = np.exp(-2j * np.pi * np.mod(k @ t.T, 1.0))
+        J = np.concatenate([e * c[None, :] * (-2j * np.pi) * k[:, l:l + 1] for l in range(t.shape[1])] + [e, 1j * e], 1)
+        J = np.concatenate([J.real, J.imag])
+        H = J.T @ J
+        step = np.linalg.solve(H + lam * np.diag(np.diag(H)), -(J.T @ np.concatenate([r.real, r.imag])))
+        step = step.reshape(t.shape[1] + 2, -1)
+        t1, c1 = np.mod(t + step[:-2].T, 1.0), c + step[-2] + 1j * step[-1]
+        r1 = res(t1, c1)
+        L1 = float(np.sum(np.abs(r1) ** 2))
+        if L1 < L:
+            t, c, r, L, lam = t1, c1, r1, L1, max(lam / 3, 1e-12)
+        else:
+            lam = min(lam * 4, 1e12)
+        losses.append(L)
+    return t, c, np.array(losses)
+
+
+@pytest.mark.parametrize("d,lo,length,m", [
+    (1, [0], [9], 1), (1, [-40], [300], 16), (1, [-5000], [9001], 2), (2, [-3, 2], [7, 129], 4), (2, [-15, -15], [32, 32], 17),
+    (2, [-20, -20], [42, 42], 40), (3, [-3, -2, 0], [8, 5, 11], 5), (4, [-2, -2, -2, -2], [6, 5, 6, 6], 3),
+    (1, [-100], [260], 53),
+])
+def test_lm_steps_match_fp64_iteration(ctx, d, lo, length, m):
+    """One to three steps from a perturbed start against the FP64 iteration: block edges of the Cholesky
+    solve (m (d + 2) from 3 to 160), boxes off centre, one axis longer than a CTA's FP32 sums, partial
+    tiles of points.  The candidate of a step carries FP32 rounding of its solve, amplified by the
+    scaled normal matrix; nodes lie at least 1 / (2 m) of a period of the longest axis apart."""
+    import torch
+    from paper_2012_11430_gb300.refine import refine_lm
+    rng = np.random.default_rng(40 + m)
+    k = O.box_set(length, d) + np.array(lo)
+    t = np.stack([(rng.permutation(m) + 0.5 + 0.2 * rng.uniform(-1, 1, m)) / m for _ in range(d)], 1)
+    c = (0.5 + rng.random(m)) * np.exp(2j * np.pi * rng.random(m))
+    y = (O.expsum(t, c, k) + 0.01 * (rng.standard_normal(len(k)) + 1j * rng.standard_normal(len(k)))).astype(np.complex64)
+    t0 = np.mod(t + 0.02 * rng.uniform(-1, 1, t.shape) / np.array(length), 1.0)
+    c0 = c * (1 + 0.02 * rng.standard_normal(m))
+    for steps in (1, 3):
+        tr, cr, Lr = _lm64(t0.copy(), c0.copy(), k, y.astype(np.complex128), steps)
+        tg, cg, Lg = refine_lm(_dev(t0, torch.float64), _dev(c0, torch.complex128), torch.from_numpy(y).cuda(), ctx, lo,
+                               length, steps=steps)
+        assert np.max(W.torus_dist(tg.cpu().numpy(), tr) * np.array(length)) <= 1e-5
+        assert np.linalg.norm(cg.cpu().numpy() - cr) <= 1e-4 * np.linalg.norm(cr)
+        # the loss of the starting point: exact parameters, so the rounding of the sums alone
+        assert abs(Lg[0].item() - Lr[0]) <= 1e-6 * Lr[0]
