@@ -144,6 +144,10 @@ struct Dev {
   // iteration caps of the small FP32 iterations (0: defaults, 30 Jacobi sweeps and 30 m + 30
   // shifted-QR steps); lowered only to exercise the PRONY_ENOCONV path
   int cap_jacobi, cap_eigqr;
+  // least-squares step: powers e^{2 pi i t x} per problem (k_powers), units of the largest problem
+  double2* zpow;
+  long long zpow_stride;
+  int maxUnits;
   // fixed-order sums over the blocks of one problem: `red_stride` bytes of partials per problem,
   // one arrival counter per problem (zero between launches)
   char* red;
@@ -332,6 +336,8 @@ void launch_gram(const Dev& D, int xbuf, int xshift, int xw, int zbuf, int zshif
 void launch_apply(const Dev& D, int xbuf, int xw, int outw, long long m_off, int m_double, int zbuf,
                   int outbuf, int norm_only, cudaStream_t s);
 void launch_argmax(const Dev& D, int buf, cudaStream_t s);
+void launch_powers(const Dev& D, cudaStream_t s);
+int rhs_units(const ProbDesc& p);
 void launch_rhs(const Dev& D, int resid, cudaStream_t s);
 void launch_gather_out(const Dev& D, double* t_out, double2* c_out, cudaStream_t s);
 void launch_copy_cols(const Dev& D, int buf, int w_sel, double2* out, cudaStream_t s);

@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(256) k_solve_c(Dev D) {
       zw[r * PRONY_DMAX + l] = zs[j * PRONY_DMAX + l];
     }
     cout[r] = cs_[j];
+    b[j] = cs_[j];                                   // for the residual, in the order of the powers
   }
   if (threadIdx.x == 0) st.ls_num2 = 0.0;
 }

@@ -550,116 +550,171 @@ __global__ void k_argmax(Dev D, int buf) {
   }
 }
 
-// ----------------------------------------------------------------------------- Vandermonde RHS / residual
-// rhs: b_i = sum_{k in I_n} conj(z_i^k) f(k);  resid: ||sum_j c_j z_j^k - f(k)||^2, all in FP64
-// (the normal equations square the condition of A: nodes closer than 1/n, as in the Section 5
-// workloads, need b to full FP64 accuracy).  z_i^k = prod_l E_l[i][k_l] with E_l[i][x] =
-// exp(-+2 pi i t_i(l) x) from an FP64 recurrence, built once per block of RHS_ROWS rows.  For b,
-// the threads split into m groups (one term each) that share the block's rows; for the
-// residual each thread takes rows.
-constexpr int RHS_ROWS = 1024;
-constexpr int RHS_TABLE_MAX = 6144;          // d m (n + 1) (checked when a problem is accepted)
+// ----------------------------------------------------------------------------- Vandermonde right-hand side
+// The sums of Eq. ls_probl factorise over the axes.  k_powers tabulates E_l[x][i] = e^{2 pi i t_i(l) x}
+// (or conj(z~_i(l))^x with the raw eigenvalues) for x in {0..n}, FP64, once per problem.  A unit of work
+// is a piece of at most RHS_SEG points of a line of the last axis:
+//   k_rhs<false>  conj(A) f: a thread sums f(k) E_{d-1}[k_{d-1}][i] over the points of a unit for one term i and
+//                 multiplies by the powers of the other axes once;
+//   k_rhs<true>   ||A^T c - f||: a block forms c_i times the conjugate powers of the other axes per unit, and a
+//                 thread sums the terms at one point.
+// Either way a point and term take four FP64 FMAs instead of 4 d (the FP64 pipe, two FMAs per clock and
+// SM, bounds both), and the powers come without a chain of n dependent products per block: 64 problems
+// d = 3, n = 19, m = 40: 0.69 ms each before, now 0.32 (floor of the FP64 operations 0.14); one problem of
+// n = 63, m = 20: 100 us each before, now 16.
+constexpr int RHS_SEG = 16;             // points of a unit
+constexpr int RHS_THREADS = 128;
 
-__global__ void __launch_bounds__(256) k_rhs(Dev D, int resid) {
-  extern __shared__ double2 tab[];   // [d][m][n+1] powers, then [d][RHS_ROWS] digits (16-bit)
-  __shared__ double2 part[256];
+__global__ void k_powers(Dev D) {
+  const int pi = blockIdx.y;
+  const ProbDesc& p = D.P[pi];
+  const ProbState& s = D.st[pi];
+  const int m = s.rank_used, n1 = p.n + 1;
+  if (s.done || m <= 0 || m > p.m) return;
+  double2* E = D.zpow + pi * D.zpow_stride;
+  if (D.vand) {
+    const double2* zr = (const double2*)(D.small + p.soff + D.L.zraw);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < p.d * m; q += gridDim.x * blockDim.x) {
+      const int l = q / m, i = q % m;
+      const double2 e1 = cconj(zr[i * PRONY_DMAX + l]);
+      double2 e = make_double2(1.0, 0.0);
+      for (int x = 0; x < n1; ++x) {
+        E[((size_t)l * n1 + x) * m + i] = e;
+        e = cmul(e, e1);
+      }
+    }
+    return;
+  }
+  const double* t = (const double*)(D.small + p.soff + D.L.t);
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < p.d * n1 * m; q += gridDim.x * blockDim.x) {
+    const int i = q % m, x = q / m % n1, l = q / m / n1;
+    double ph = t[i * PRONY_DMAX + l] * x, sn, cs;
+    ph = fma(t[i * PRONY_DMAX + l], (double)x, -rint(ph));       // reduced with one rounding
+    sincospi(2.0 * ph, &sn, &cs);
+    E[q] = make_double2(cs, sn);
+  }
+}
+
+// Unit u of a problem: line and first point of the last axis (nseg pieces per line).
+__device__ inline long long rhs_unit(const ProbDesc& p, int u, int nseg, int& line, int& x0) {
+  line = u / nseg;
+  x0 = (u - line * nseg) * RHS_SEG;
+  long long g = 0, mul = 1;
+  int rem = line;
+  g = x0 + p.n;
+  mul = p.G;
+  for (int l = p.d - 2; l >= 0; --l) {
+    g += (long long)(rem % (p.n + 1) + p.n) * mul;
+    rem /= p.n + 1;
+    mul *= p.G;
+  }
+  return p.grid + g;                                  // grid index of the unit's first sample
+}
+
+// `upb` units per block.
+template <bool RESID>
+__global__ void __launch_bounds__(RHS_THREADS) k_rhs(Dev D, int upb) {
+  __shared__ double2 sh[PRONY_MMAX * (RHS_THREADS / RHS_SEG) + RHS_THREADS];
   __shared__ double shr[32];
   const int pi = blockIdx.y;
   const ProbDesc& p = D.P[pi];
   ProbState& s = D.st[pi];
   const int m = s.rank_used;
   if (s.done || m <= 0 || m > p.m) return;
-  const int r0 = blockIdx.x * RHS_ROWS;
-  if (r0 >= p.N) return;
-  const int nrows = min(RHS_ROWS, p.N - r0);
-  const int n1 = p.n + 1;
-  short* kd = (short*)(tab + RHS_TABLE_MAX);       // kd[l * RHS_ROWS + rr]: digit l of row rr (n < 6144)
-  const double* t = (const double*)(D.small + p.soff + D.L.t);
-  const double2* c = (const double2*)(D.small + p.soff + D.L.c);
-  const double sign = resid ? -1.0 : 1.0;
-  const double2* zr = (const double2*)(D.small + p.soff + D.L.zraw);
-  for (int q = threadIdx.x; q < p.d * m; q += blockDim.x) {
-    int l = q / m, i = q % m;
-    double2 e1;
-    if (D.vand) {
-      // raw eigenvalue z~ (Section 4 reading): conj(z) for the right-hand side, z for the model
-      const double2 z = zr[i * PRONY_DMAX + l];
-      e1 = make_double2(z.x, -sign * z.y);
-    } else {
-      double sn, cs;
-      sincospi(2.0 * t[i * PRONY_DMAX + l], &sn, &cs);
-      e1 = make_double2(cs, sign * sn);
-    }
+  const int n1 = p.n + 1, nseg = (n1 + RHS_SEG - 1) / RHS_SEG, nunit = p.N / n1 * nseg;
+  const int u0 = blockIdx.x * upb, u1 = min(nunit, u0 + upb);
+  if (u0 >= nunit) return;
+  const int nblk = (nunit + upb - 1) / upb;
+  const double2* E = D.zpow + pi * D.zpow_stride;
+  const double2* last = E + (size_t)(p.d - 1) * n1 * m;
+  // product over the leading axes of the powers of term i at a line
+  auto lead = [&](int line, int i) {
     double2 e = make_double2(1.0, 0.0);
-    double2* row = tab + ((size_t)l * m + i) * n1;
-    for (int x = 0; x < n1; ++x) {
-      row[x] = e;
-      e = cmul(e, e1);
+    for (int l = p.d - 2; l >= 0; --l) {
+      const double2 v = E[((size_t)l * n1 + line % n1) * m + i];
+      e = l == p.d - 2 ? v : cmul(e, v);
+      line /= n1;
     }
-  }
-  for (int rr = threadIdx.x; rr < nrows; rr += blockDim.x) {
-    int rem = r0 + rr;
-    for (int l = p.d - 1; l >= 0; --l) {
-      kd[l * RHS_ROWS + rr] = (short)(rem % n1);
-      rem /= n1;
-    }
-  }
-  __syncthreads();
-  auto power = [&](int i, int rr) {
-    double2 e = tab[(size_t)i * n1 + kd[rr]];
-    for (int l = 1; l < p.d; ++l) e = cmul(e, tab[((size_t)l * m + i) * n1 + kd[l * RHS_ROWS + rr]]);
     return e;
   };
-  auto sample = [&](int rr) {
-    int gi = 0, mul = 1;
-    for (int l = p.d - 1; l >= 0; --l) {
-      gi += (kd[l * RHS_ROWS + rr] + p.n) * mul;
-      mul *= p.G;
-    }
-    return D.grid64[p.grid + gi];
-  };
-  if (!resid) {
-    const int tpi = blockDim.x / m;                 // threads per term (m <= 64: at least 4)
-    const int i = threadIdx.x / tpi, q = threadIdx.x % tpi;
-    // four interleaved partial sums (FP64 additions have a long dependent latency), fixed order
-    double2 a4[4] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
-    if (i < m) {
-      int u = 0;
-      for (int rr = q; rr < nrows; rr += tpi, u = (u + 1) & 3) a4[u] = cadd(a4[u], cmul(power(i, rr), sample(rr)));
-    }
-    part[threadIdx.x] = cadd(cadd(a4[0], a4[1]), cadd(a4[2], a4[3]));
-    __syncthreads();
-    double2* b = (double2*)(D.small + p.soff + D.L.rhs);
-    double2* slots = (double2*)red_region(D, pi);
-    if (i < m && q == 0 && ws_ok(D, 16LL * m * (blockIdx.x + 1) <= D.red_stride, 14)) {
-      double2 sum = make_double2(0.0, 0.0);
-      for (int u = 0; u < tpi; ++u) sum = cadd(sum, part[threadIdx.x + u]);
-      slots[(size_t)blockIdx.x * m + i] = sum;
-    }
-    // block sums of b in block order
-    const int nblk = (p.N + RHS_ROWS - 1) / RHS_ROWS;
-    if (red_arrive(D, pi, nblk))
-      for (int ii = threadIdx.x; ii < m; ii += blockDim.x) {
-        double2 sum = b[ii];
-        for (int k = 0; k < nblk; ++k) sum = cadd(sum, __ldcg(slots + (size_t)k * m + ii));
-        b[ii] = sum;
+  if (!RESID) {
+    const int groups = RHS_THREADS / m;               // m <= 64: at least two
+    const int i = threadIdx.x % m, grp = threadIdx.x / m;
+    double2 b = make_double2(0.0, 0.0);
+    if (grp < groups)
+      for (int u = u0 + grp; u < u1; u += groups) {
+        int line, x0;
+        const double2* f = D.grid64 + rhs_unit(p, u, nseg, line, x0);
+        const double2* w = last + (size_t)x0 * m + i;
+        const int nx = min(RHS_SEG, n1 - x0);
+        double2 a = make_double2(0.0, 0.0);
+#pragma unroll 4
+        for (int x = 0; x < nx; ++x) {
+          const double2 fv = f[x], wv = w[(size_t)x * m];
+          a.x = fma(fv.x, wv.x, fma(-fv.y, wv.y, a.x));
+          a.y = fma(fv.x, wv.y, fma(fv.y, wv.x, a.y));
+        }
+        b = cadd(b, p.d > 1 ? cmul(a, lead(line, i)) : a);
       }
-  } else {
-    double r2 = 0.0;
-    for (int rr = threadIdx.x; rr < nrows; rr += blockDim.x) {
-      const double2 f = sample(rr);
-      double2 v[2] = {make_double2(-f.x, -f.y), make_double2(0.0, 0.0)};   // two chains over the terms
-      for (int i = 0; i < m; ++i) v[i & 1] = cadd(v[i & 1], cmul(c[i], power(i, rr)));
-      r2 += cabs2(cadd(v[0], v[1]));
+    sh[threadIdx.x] = b;
+    __syncthreads();
+    double2* out = (double2*)(D.small + p.soff + D.L.rhs);
+    double2* slots = (double2*)red_region(D, pi);
+    if (grp == 0 && ws_ok(D, 16LL * m * (blockIdx.x + 1) <= D.red_stride, 14)) {
+      for (int g = 1; g < groups; ++g) b = cadd(b, sh[g * m + i]);
+      slots[(size_t)blockIdx.x * m + i] = b;
     }
-    double tot = block_sum(r2, shr);
+    // block sums in block order
+    if (red_arrive(D, pi, nblk) && threadIdx.x < m) {
+      double2 sum = make_double2(0.0, 0.0);
+#pragma unroll 4
+      for (int k = 0; k < nblk; ++k) sum = cadd(sum, __ldcg(slots + (size_t)k * m + threadIdx.x));
+      out[threadIdx.x] = sum;
+    }
+  } else {
+    const double2* c = (const double2*)(D.small + p.soff + D.L.rhs);   // in the order of the powers (k_solve_c)
+    constexpr int PER = RHS_THREADS / RHS_SEG;        // units at a time
+    double r2 = 0.0;
+    for (int v0 = u0; v0 < u1; v0 += PER) {
+      const int nv = min(PER, u1 - v0);
+      __syncthreads();
+      for (int q = threadIdx.x; q < nv * m; q += RHS_THREADS) {   // c_i conj(powers of the leading axes)
+        const int line = (v0 + q / m) / nseg, i = q % m;
+        sh[q] = p.d > 1 ? cmulc(lead(line, i), c[i]) : c[i];
+      }
+      __syncthreads();
+      const int v = threadIdx.x / RHS_SEG, dx = threadIdx.x % RHS_SEG;
+      if (v < nv) {
+        int line, x0;
+        const double2* f = D.grid64 + rhs_unit(p, v0 + v, nseg, line, x0);
+        if (x0 + dx < n1) {
+          const double2* w = last + (size_t)(x0 + dx) * m;
+          const double2* cu = sh + v * m;
+          const double2 fv = f[dx];
+          double2 a = make_double2(-fv.x, -fv.y), a1 = make_double2(0.0, 0.0);   // two chains over the terms
+#pragma unroll 2
+          for (int i = 0; i < m; i += 2) {
+            const double2 c0 = cu[i], w0 = w[i];
+            a.x = fma(c0.x, w0.x, fma(c0.y, w0.y, a.x));          // c conj(w)
+            a.y = fma(c0.y, w0.x, fma(-c0.x, w0.y, a.y));
+            if (i + 1 < m) {
+              const double2 c1 = cu[i + 1], w1 = w[i + 1];
+              a1.x = fma(c1.x, w1.x, fma(c1.y, w1.y, a1.x));
+              a1.y = fma(c1.y, w1.x, fma(-c1.x, w1.y, a1.y));
+            }
+          }
+          r2 += cabs2(cadd(a, a1));
+        }
+      }
+    }
+    const double tot = block_sum(r2, shr);
     double* slot = (double*)red_region(D, pi);
     if (threadIdx.x == 0 && ws_ok(D, 8LL * (blockIdx.x + 1) <= D.red_stride, 15)) slot[blockIdx.x] = tot;
-    const int nblk = (p.N + RHS_ROWS - 1) / RHS_ROWS;
-    if (red_arrive(D, pi, nblk) && threadIdx.x == 0) {
-      double sum = 0.0;
-      for (int k = 0; k < nblk; ++k) sum += __ldcg(slot + k);
-      s.ls_num2 = sum;
+    if (red_arrive(D, pi, nblk)) {
+      double sum = 0.0;                               // lane sums in lane order, then a fixed tree
+      for (int k = threadIdx.x; k < nblk; k += RHS_THREADS) sum += __ldcg(slot + k);
+      sum = block_sum(sum, shr);
+      if (threadIdx.x == 0) s.ls_num2 = sum;
     }
   }
 }
@@ -900,6 +955,15 @@ static void gram_geometry(const Dev& D, size_t& sm, int& chunk, int& nblk) {
   nblk = (D.maxN + chunk - 1) / chunk;
 }
 
+// Units of the largest problem, and units per block: about eight blocks per SM over the batch, at most
+// 256 blocks per problem (the last one adds their sums).
+static int rhs_units_per_block(const Dev& D) {
+  const long long total = (long long)D.maxUnits * D.nprob;
+  const long long want = std::max<long long>(1, total / (8 * 152));
+  return (int)std::max<long long>(std::max<long long>(RHS_THREADS / RHS_SEG, want), (D.maxUnits + 255) / 256);
+}
+int rhs_units(const ProbDesc& p) { return p.N / (p.n + 1) * ((p.n + RHS_SEG) / RHS_SEG); }
+
 long long red_bytes_per_problem(const Dev& D) {
   size_t sm;
   int chunk, nblk;
@@ -907,8 +971,8 @@ long long red_bytes_per_problem(const Dev& D) {
   long long b = (long long)nblk * D.L.LDR * D.L.LDR * (long long)sizeof(float2);           // k_gram
   b = std::max<long long>(b, 64LL * sizeof(double2));                                         // k_prep (<= 64 blocks)
   b = std::max<long long>(b, (D.maxN + 63) / 64 * (long long)sizeof(double));                // k_apply norms
-  b = std::max<long long>(b, (D.maxN + RHS_ROWS - 1) / RHS_ROWS * (long long)std::max(1, D.L.LDM) *
-                                 (long long)sizeof(double2));                                  // k_rhs
+  b = std::max<long long>(b, (D.maxUnits + rhs_units_per_block(D) - 1) / rhs_units_per_block(D) *
+                                 (long long)std::max(1, D.L.LDM) * (long long)sizeof(double2));   // k_rhs
   return (b + 255) / 256 * 256;
 }
 
@@ -943,16 +1007,17 @@ void launch_argmax(const Dev& D, int buf, cudaStream_t s) {
   k_argmax<<<g, 256, 0, s>>>(D, buf);
 }
 
-void launch_rhs(const Dev& D, int resid, cudaStream_t s) {
-  static bool attr = false;
-  const size_t sm = sizeof(double2) * RHS_TABLE_MAX + sizeof(short) * PRONY_DMAX * RHS_ROWS;
-  if (!attr) {
-    cudaFuncSetAttribute(k_rhs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
-  dim3 g((D.maxN + RHS_ROWS - 1) / RHS_ROWS, D.nprob);
+void launch_powers(const Dev& D, cudaStream_t s) {
   note_launch();
-  k_rhs<<<g, 256, sm, s>>>(D, resid);
+  const int want = D.vand ? 1 : (int)((D.zpow_stride + 127) / 128);
+  k_powers<<<dim3(blocks_per_problem(want, D.nprob), D.nprob), 128, 0, s>>>(D);
+}
+void launch_rhs(const Dev& D, int resid, cudaStream_t s) {
+  const int upb = rhs_units_per_block(D);
+  dim3 g((D.maxUnits + upb - 1) / upb, D.nprob);
+  note_launch();
+  if (resid) k_rhs<true><<<g, RHS_THREADS, 0, s>>>(D, upb);
+  else k_rhs<false><<<g, RHS_THREADS, 0, s>>>(D, upb);
 }
 
 void launch_gather_out(const Dev& D, double* t_out, double2* c_out, cudaStream_t s) {

@@ -71,6 +71,7 @@ struct prony_ctx {
   DBuf grid64, gF, gH, V, U, B1, B2, Y, small, P, st, jobs, flag, tout, cout, misc, misc2, misc3;
   DBuf xb, tabF, tabH, tcjobs, tcerr;   // tensor-core path: B' planes, split sample tables, jobs, error flag
   DBuf part, cnt;                       // split K products: partial tiles per job, arrival counters per tile
+  DBuf zpow;                            // powers of the least-squares step per problem
   DBuf red, rcnt;                       // fixed-order cross-block sums: partials and counters per problem
   DBuf oob;                             // first failed workspace bound check of a kernel (0: none)
   DBuf fhat, ftw;                       // FFT path: sample transforms, twiddles
@@ -871,6 +872,12 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   D.small = (char*)ctx->small.p;
   D.L = L;
   D.vand = o.vandermonde ? 1 : 0;
+  for (const auto& p : B.P) {
+    D.zpow_stride = std::max(D.zpow_stride, (long long)p.d * p.m * (p.n + 1));
+    D.maxUnits = std::max(D.maxUnits, rhs_units(p));
+  }
+  if ((rc = ensure(ctx->zpow, sizeof(double2) * (size_t)D.zpow_stride * np))) return rc;
+  D.zpow = (double2*)ctx->zpow.p;
   // partials of the cross-block sums (Grams, norms, right-hand sides), one region per problem
   D.red_stride = red_bytes_per_problem(D);
   if ((rc = ensure(ctx->red, (size_t)D.red_stride * np))) return rc;
@@ -1211,7 +1218,7 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
       apply(ctx, B, D, BUF_U, W_U, W_V, D.L.uq, 1, BUF_B2, s);   // U_final
     }
     launch_eig_t(D, o.seed, s);
-    launch_zero_small(D, D.L.rhs, 16LL * D.L.LDM, s);
+    launch_powers(D, s);
     launch_rhs(D, 0, s);
     launch_solve_c(D, s);
     launch_rhs(D, 1, s);
@@ -1464,7 +1471,7 @@ int prony_ctx_destroy(prony_ctx* c) {
   DBuf* bufs[] = {&c->grid64, &c->gF, &c->gH, &c->V, &c->U, &c->B1, &c->B2, &c->Y, &c->small, &c->P,
                   &c->st, &c->jobs, &c->flag, &c->tout, &c->cout, &c->misc, &c->misc2, &c->misc3,
                   &c->xb, &c->tabF, &c->tabH, &c->tcjobs, &c->tcerr, &c->lmws, &c->part, &c->cnt, &c->red,
-                  &c->rcnt, &c->oob, &c->fhat, &c->ftw, &c->axP, &c->axtw, &c->axX, &c->axY, &c->axF, &c->axH};
+                  &c->rcnt, &c->oob, &c->zpow, &c->fhat, &c->ftw, &c->axP, &c->axtw, &c->axX, &c->axY, &c->axF, &c->axH};
   if (c->solve_graph.exec) cudaGraphExecDestroy(c->solve_graph.exec);
   for (DBuf* b : bufs)
     if (b->p) cudaFree(b->p);
