@@ -327,7 +327,7 @@ void launch_state_init(const Dev& D, cudaStream_t s);
 void launch_prep(const Dev& D, bool norms, cudaStream_t s);   // states, gF, gH; norms: ||T||_F, ||f||, finiteness
 void launch_init_v0(const Dev& D, unsigned long long seed, cudaStream_t s);
 void launch_zero_small(const Dev& D, long long off, long long bytes, cudaStream_t s);
-// out[a][b] (+)= sum_{r in I_n} conj(X[map(r), a]) Z[map(r), b]; X, Z buffers with row shifts
+// out[a][b] = sum_{r in I_n} conj(X[map(r), a]) Z[map(r), b]; X, Z buffers with row shifts
 void launch_gram(const Dev& D, int xbuf, int xshift, int xw, int zbuf, int zshift, int zw,
                  long long out_off, int out_ld, cudaStream_t s);
 // OUT[r, j] = (zbuf >= 0 ? Z[r, j] : 0) - sum_a X[r, a] M[a][j] for r in I_n (without Z: + the sum); M in the small workspace

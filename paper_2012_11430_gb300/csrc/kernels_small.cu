@@ -42,36 +42,88 @@ __global__ void __launch_bounds__(256) k_chol(Dev D, int wsel, int target, int m
   const int mode = mode_in == QR_AUTO ? (st.iter == 0 ? QR_RANK : QR_PLAIN) : mode_in;
   const int w = swidth(st, p, wsel);
   const int LR = D.L.LDR;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const double2* G = (const double2*)(D.small + p.soff + D.L.gram);
-  for (int idx = threadIdx.x; idx < w * w; idx += blockDim.x) {
-    int i = idx / w, j = idx % w;
-    double2 g = G[i * LR + j];
-    A[i * LR + j] = make_float2((float)g.x, (float)g.y);
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < w * LR; idx += blockDim.x) {
+    const double2 g = G[idx];
+    T[idx] = make_float2((float)g.x, (float)g.y);
   }
-  for (int i = threadIdx.x; i < w; i += blockDim.x) perm[i] = i;
+  for (int j = threadIdx.x; j < w; j += blockDim.x) order[j] = w;
   __syncthreads();
+  const float tol2 = (float)(tol * tol);
+  int limit = w;  // columns that may be accepted (never more than m after the rank step)
+  if (mode == QR_RANK) limit = min(w, p.m);
+  // warp 0: the remaining diagonal (0 where eliminated or past w), start values of the tests
+  float d[NQ], trace0 = 0.f, maxd0 = 0.f;
+  int rank = -1;
+  // warp 0, before step i: choose its pivot or stop
+  auto choose = [&](int i) {
+    int pv = i;
+    float dp = 0.f;
+    bool stop = i >= w;
+    if (mode == QR_PLAIN) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q)
+        if (q == i >> 5) dp = d[q];
+      dp = __shfl_sync(0xffffffffu, dp, i & 31);
+    } else {
+      unsigned key = 0;                         // bits of a non-negative float are ordered as integers
+      int bi = PRONY_RMAX;
+      float tr = 0.f;
+#pragma unroll
+      for (int q = NQ - 1; q >= 0; --q) {
+        const int j = lane + 32 * q;
+        if (j < w && order[j] == w) {
+          const float dd = fmaxf(d[q], 0.f);
+          tr += dd;
+          if (bi == PRONY_RMAX || __float_as_uint(dd) >= key) {
+            key = __float_as_uint(dd);
+            bi = j;
+          }
+        }
+      }
+      const unsigned best = __reduce_max_sync(0xffffffffu, key);
+      pv = __reduce_min_sync(0xffffffffu, key == best ? bi : PRONY_RMAX);
+      if (mode == QR_RANK && rank < 0) {
+        for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+        if (!stop && tr <= tol2 * trace0) rank = i;
+      }
+      float mine = 0.f;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q)
+        if (q == pv >> 5) mine = d[q];
+      dp = __shfl_sync(0xffffffffu, mine, pv & 31);
+      if (mode == QR_DROP && dp <= tol2 * maxd0) stop = true;
+      if (i >= limit && (mode != QR_RANK || rank >= 0)) stop = true;
+      if (mode == QR_RANK && rank_mode == 1 && rank >= 0) stop = true;
+    }
+    if (!(dp > 1e-30f * maxd0) || !(dp > 0.f)) stop = true;                          // exhausted / not PD
+    if (lane == 0) {
+      s_piv[i & 1] = stop ? -1 : pv;
+      s_dp[i & 1] = dp;
+      if (stop) s_rho = min(i, limit);
+      s_rank = rank;
+    }
+  };
   if (warp == 0) {
-    float tr = 0.f, mx = 0.f;
     bool finite = true;
-    for (int i = lane; i < w; i += 32) {
-      const float dd = A[i * LR + i].x;
-      finite = finite && isfinite(dd);
-      tr += fmaxf(dd, 0.f);
-      mx = fmaxf(mx, dd);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int j = lane + 32 * q;
+      d[q] = j < w ? T[j * LR + j].x : 0.f;
+      finite = finite && isfinite(d[q]);
+      trace0 += fmaxf(d[q], 0.f);
+      maxd0 = fmaxf(maxd0, d[q]);
     }
     for (int o = 16; o > 0; o >>= 1) {
-      tr += __shfl_xor_sync(0xffffffffu, tr, o);
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      trace0 += __shfl_xor_sync(0xffffffffu, trace0, o);
+      maxd0 = fmaxf(maxd0, __shfl_xor_sync(0xffffffffu, maxd0, o));
     }
-    finite = __all_sync(0xffffffffu, finite);
+    const bool bad = !__all_sync(0xffffffffu, finite) || !isfinite(trace0);
     if (lane == 0) {
-      s_trace0 = tr;
-      s_maxd0 = mx;
-      s_rho = w;
-      s_rank = -1;
-      s_stop = finite && isfinite(tr) ? 0 : 2;
-      if (s_stop) {                     // non-finite block: the problem stops with ENAN
+      s_bad = bad;
+      if (bad) {                        // non-finite block: the problem stops with ENAN
         st.status = ST_ENAN;
         st.done = 1;
         st.w_in = w;

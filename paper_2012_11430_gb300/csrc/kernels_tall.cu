@@ -133,8 +133,7 @@ __global__ void k_init_v0(Dev D, unsigned long long seed) {
   }
 }
 
-// Clears a block of the small workspace of every problem still iterating (a stopped problem keeps
-// the Q and U^* T_l V of its last iteration).
+// Clears a block of the small workspace of every problem still iterating.
 __global__ void k_zero_small(Dev D, long long off, long long bytes) {
   if (D.st[blockIdx.y].done) return;
   const ProbDesc& p = D.P[blockIdx.y];
@@ -143,7 +142,7 @@ __global__ void k_zero_small(Dev D, long long off, long long bytes) {
 }
 
 // ----------------------------------------------------------------------------- tall-skinny Gram
-// out[a][b] += sum_r conj(X[r, a]) Z[r, b] over a block of `chunk` rows (chosen by the launcher
+// out[a][b] = sum_r conj(X[r, a]) Z[r, b] over a block of `chunk` rows (chosen by the launcher
 // so that the batch gives a few blocks per SM: few blocks per problem means few FP64 atomics on
 // the same output entries).
 //
@@ -158,7 +157,7 @@ __global__ void k_zero_small(Dev D, long long off, long long bytes) {
 // (broadcast).  When there are fewer 4x4 tiles than threads, threads split the staged rows into
 // row groups whose partial sums are added in shared memory; when there are more, the tiles are
 // processed in batches (every batch re-stages the rows).  Each block stores its partial Gram; the
-// last block of the problem adds the partials (FP32, a fixed order) into the FP64 output.
+// last block of the problem (or k_gram_sum) adds the partials (FP32, a fixed order) and writes the FP64 output.
 constexpr int GRAM_T = 4;           // register tile (GRAM_T x GRAM_T complex accumulators)
 constexpr int GRAM_KMAX = 10;       // staged values per thread and pass: (a + b) RS <= 256 GRAM_KMAX
 
@@ -189,7 +188,7 @@ __device__ __forceinline__ void ffma2(unsigned long long& acc, unsigned long lon
 }
 
 __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, int xw, int zbuf, int zshift, int zw,
-                                              long long out_off, int out_ld, int chunk) {
+                                              long long out_off, int out_ld, int chunk, int own_sum) {
   extern __shared__ float4 smem4[];
   const int pi = blockIdx.y;
   const ProbDesc& p = D.P[pi];
@@ -355,7 +354,7 @@ __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, in
   // additions, at a small fraction of the FP32 rate here, made this one block per problem the
   // longest part of the launch.)
   const int nblk = (p.N + chunk - 1) / chunk;
-  if (red_arrive(D, pi, nblk)) {
+  if (own_sum && red_arrive(D, pi, nblk)) {
     constexpr int GR = 2;
     const float2* slots = (const float2*)red_region(D, pi);
     const int ss = a * b;
@@ -401,12 +400,41 @@ __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, in
         if (e < ss) {
           const float tx = (acc[g][0].x + acc[g][1].x) + (acc[g][2].x + acc[g][3].x);
           const float ty = (acc[g][0].y + acc[g][1].y) + (acc[g][2].y + acc[g][3].y);
-          double2* o = &out[(e / b) * out_ld + e % b];
-          *o = make_double2(o->x + (double)tx, o->y + (double)ty);
+          out[(e / b) * out_ld + e % b] = make_double2((double)tx, (double)ty);
         }
       }
     }
   }
+}
+
+// The sum of the partial Grams as a launch of its own (k_gram without own_sum): one entry per thread,
+// the same order of additions.  With one problem on the GPU and 64 partials, one block took longer over
+// them than all blocks over the rows (w = 40: 20 of 28 us; now 3 us in 7 blocks).
+__global__ void __launch_bounds__(256) k_gram_sum(Dev D, int xw, int zw, long long out_off, int out_ld, int chunk) {
+  const int pi = blockIdx.y;
+  const ProbDesc& p = D.P[pi];
+  const ProbState& s = D.st[pi];
+  if (s.done) return;
+  const int a = width_of(s, p, xw), b = width_of(s, p, zw), ss = a * b;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (a <= 0 || b <= 0 || e >= ss) return;
+  const int nblk = (p.N + chunk - 1) / chunk;
+  const float2* slots = (const float2*)red_region(D, pi) + e;
+  float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  for (int k = 0; k < nblk; k += 16) {               // sixteen loads in flight
+    float2 v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = __ldcg(slots + (size_t)min(k + u, nblk - 1) * ss);
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (k + u < nblk) {
+        acc[u & 3].x += v[u].x;
+        acc[u & 3].y += v[u].y;
+      }
+  }
+  const float tx = (acc[0].x + acc[1].x) + (acc[2].x + acc[3].x);
+  const float ty = (acc[0].y + acc[1].y) + (acc[2].y + acc[3].y);
+  ((double2*)(D.small + p.soff + out_off))[(e / b) * out_ld + e % b] = make_double2((double)tx, (double)ty);
 }
 
 // ----------------------------------------------------------------------------- X M products
@@ -984,7 +1012,12 @@ void launch_gram(const Dev& D, int xbuf, int xshift, int xw, int zbuf, int zshif
   gram_attr(sm);
   dim3 g(nblk, D.nprob);
   note_launch();
-  k_gram<<<g, 256, sm, s>>>(D, xbuf, xshift, xw, zbuf, zshift, zw, out_off, out_ld, chunk);
+  const int own_sum = nblk <= 8;                 // few partials: the last block adds them
+  k_gram<<<g, 256, sm, s>>>(D, xbuf, xshift, xw, zbuf, zshift, zw, out_off, out_ld, chunk, own_sum);
+  if (!own_sum) {
+    note_launch();
+    k_gram_sum<<<dim3((D.L.LDR * D.L.LDR + 255) / 256, D.nprob), 256, 0, s>>>(D, xw, zw, out_off, out_ld, chunk);
+  }
 }
 
 void launch_apply(const Dev& D, int xbuf, int xw, int outw, long long m_off, int m_double, int zbuf, int outbuf,

@@ -918,7 +918,6 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
 // orthonormal to a few u32 after one pass).
 void tall_qr1(prony_ctx* ctx, const Batch& B, int xbuf, int xw, int target, cudaStream_t s) {
   const Dev& D = B.D;
-  launch_zero_small(D, D.L.gram, 16LL * D.L.LDR * D.L.LDR, s);
   gram(ctx, B, D, xbuf, -1, xw, xbuf, -1, xw, D.L.gram, D.L.LDR, s);
   launch_chol(D, xw, target, QR_PLAIN, 0.0, 0, s);
   apply(ctx, B, D, xbuf, W_IN, W_OUT, D.L.mapm, 0, xbuf, s);
@@ -927,11 +926,9 @@ void tall_qr1(prony_ctx* ctx, const Batch& B, int xbuf, int xw, int target, cuda
 void tall_qr(prony_ctx* ctx, const Batch& B, int xbuf, int xw, int target, int mode, double tol, int rank_mode,
              int outbuf, cudaStream_t s) {
   const Dev& D = B.D;
-  launch_zero_small(D, D.L.gram, 16LL * D.L.LDR * D.L.LDR, s);
   gram(ctx, B, D, xbuf, -1, xw, xbuf, -1, xw, D.L.gram, D.L.LDR, s);
   launch_chol(D, xw, target, mode, tol, rank_mode, s);
   apply(ctx, B, D, xbuf, W_IN, W_OUT, D.L.mapm, 0, BUF_B1, s);
-  launch_zero_small(D, D.L.gram, 16LL * D.L.LDR * D.L.LDR, s);
   gram(ctx, B, D, BUF_B1, -1, target, BUF_B1, -1, target, D.L.gram, D.L.LDR, s);
   launch_chol(D, target, target, QR_PLAIN, 0.0, 0, s);
   apply(ctx, B, D, BUF_B1, W_IN, W_OUT, D.L.mapm, 0, outbuf, s);
@@ -1152,7 +1149,6 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
   // Gram-Schmidt twice); its right vectors start the power loop
   auto reorth = [&](int basis, int wsel) {
     for (int pass = 0; pass < 2; ++pass) {
-      launch_zero_small(D, D.L.work1, 16LL * D.L.LDR * D.L.LDM, s);
       gram(ctx, B, D, basis, -1, wsel, BUF_B2, -1, W_ONE, D.L.work1, D.L.LDM, s);
       launch_apply(D, basis, wsel, W_ONE, D.L.work1, 1, BUF_B2, BUF_B2, 0, s);
     }
@@ -1193,7 +1189,6 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
     // Y = T V over the box {0..n+1}^d
     if ((rc = toeplitz(it, 1))) return rc;
     // Q = U^* (T V), ||T V - U Q||_F
-    launch_zero_small(D, D.L.q, 16LL * D.L.LDR * D.L.LDM, s);
     gram(ctx, B, D, BUF_U, -1, W_U, BUF_Y, -1, W_V, D.L.q, D.L.LDM, s);
     launch_apply(D, BUF_U, W_U, W_V, D.L.q, 1, BUF_Y, -1, 1, s);
     CK(cudaMemsetAsync(dflag, 0xFF, sizeof(int), s));
@@ -1204,7 +1199,6 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
   auto finish = [&]() -> int {
     launch_reset_done(D, s);
     // M_l = U^* Y_l  with Y_l the rows k + e_l of the last product Y = T V
-    launch_zero_small(D, D.L.mproj, 16LL * D.maxD * D.L.LDR * D.L.LDM, s);
     for (int l = 0; l < D.maxD; ++l)
       gram(ctx, B, D, BUF_U, -1, W_U, BUF_Y, l, W_V, D.L.mproj + 16LL * l * D.L.LDR * D.L.LDM, D.L.LDM, s);
     launch_svd_S(D, s);
