@@ -323,7 +323,6 @@ enum BufSel { BUF_V = 0, BUF_U = 1, BUF_B1 = 2, BUF_B2 = 3, BUF_Y = 4 };
 // Bytes of cross-block partials per problem that the tall kernels need for a batch of this
 // layout (D.nprob, D.maxN, D.maxGd, D.L set).
 long long red_bytes_per_problem(const Dev& D);
-void launch_state_init(const Dev& D, cudaStream_t s);
 void launch_prep(const Dev& D, bool norms, cudaStream_t s);   // states, gF, gH; norms: ||T||_F, ||f||, finiteness
 void launch_init_v0(const Dev& D, unsigned long long seed, cudaStream_t s);
 void launch_zero_small(const Dev& D, long long off, long long bytes, cudaStream_t s);

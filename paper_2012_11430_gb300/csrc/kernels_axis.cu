@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
   const long long total = (long long)Gs * groups;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total; q += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(q % Gs), w0 = 4 * (int)(q / Gs);
-    const double2* f = D.grid64 + p.grid + x;
+    const float2* f = D.gF + p.grid + x;
     float2 acc[2][4];                             // two interleaved partial sums per frequency
     int at[4], step[4];
 #pragma unroll
@@ -119,10 +119,7 @@ __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
     for (int i0 = 0; i0 < last; i0 += 8) {        // eight loads in flight
       float2 v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const double2 fv = i0 + e < last ? f[(long long)(i0 + e) * Gs] : make_double2(0.0, 0.0);
-        v[e] = make_float2((float)fv.x, (float)fv.y);
-      }
+      for (int e = 0; e < 8; ++e) v[e] = i0 + e < last ? f[(long long)(i0 + e) * Gs] : make_float2(0.f, 0.f);
 #pragma unroll
       for (int e = 0; e < 8; ++e)
 #pragma unroll

@@ -23,17 +23,26 @@ __device__ inline void set_status(ProbState& s, int st) {
 }
 
 // ----------------------------------------------------------------------------- pivoted Cholesky (FP32)
-// Step i: warp 0 finds the pivot (largest remaining diagonal entry, lowest index on ties) and the
-// trailing trace and decides whether to stop; rows and columns i, pv are swapped; the scaled
-// column l = A[:, i] / sqrt(A[i][i]) goes to shared memory and the trailing block takes the rank-1
-// update A[j][k] -= l_j conj(l_k).  R^{-1} (R = L^H) is formed by one warp per column with the
-// partial sums of the back substitution spread over the lanes.
-__global__ void __launch_bounds__(256) k_chol(Dev D, int wsel, int target, int mode_in, double tol, int rank_mode) {
-  extern __shared__ float2 A[];                 // [w][LDR]
+// P^T A P = L L^H and R^{-1} = L^{-H} by elimination in place: a step with pivot column pv takes, from
+// every row j that remains, T[j] -= (T[j][pv] / d) T[pv], where the columns that remain hold the Schur
+// complement of A and the eliminated ones the same row operations applied to the identity (column pv
+// becomes -T[j][pv] / d).  Row pv then holds row b of L^{-1} up to 1 / sqrt(d): no substitution follows, and
+// nothing is swapped or scaled on the way.
+// Warp 0 keeps the remaining diagonal in registers, updates it from row pv, and chooses the next pivot
+// (largest entry, lowest index on ties; without pivoting the next column) and whether to stop while the
+// other warps update the rows, four at a time so that their loads overlap: one barrier per step.
+// One CTA per problem, bound by the latency of its w dependent steps.  The version that searched, swapped
+// and scaled between barriers and then substituted back took 37 us at w = 40.
+template <int NQ>                              // 32-column groups: LDR <= 32 NQ
+__global__ void __launch_bounds__(NQ > 2 ? 512 : 256) k_chol(Dev D, int wsel, int target, int mode_in, double tol,
+                                                             int rank_mode) {
+  extern __shared__ float2 T[];                 // [w][LDR]
   __shared__ int perm[PRONY_RMAX];
-  __shared__ float2 lcol[PRONY_RMAX];
-  __shared__ int s_piv, s_stop, s_rho, s_rank;
-  __shared__ float s_trace0, s_maxd0;
+  __shared__ int order[PRONY_RMAX];             // step at which a column was eliminated (w: not)
+  __shared__ float dinv[PRONY_RMAX];            // 1 / sqrt of the pivots
+  __shared__ float s_dp[2];                     // pivot and its column, of this step and the next
+  __shared__ int s_piv[2];                      // (-1: stop)
+  __shared__ int s_bad, s_rho, s_rank;
   const ProbDesc& p = D.P[blockIdx.x];
   ProbState& st = D.st[blockIdx.x];
   if (st.done) return;
@@ -131,139 +140,82 @@ __global__ void __launch_bounds__(256) k_chol(Dev D, int wsel, int target, int m
         set_width(st, target, 0);
       }
     }
+    choose(0);
   }
   __syncthreads();
-  if (s_stop) return;
-  const float tol2 = (float)(tol * tol);
-  int limit = w;  // columns that may be accepted (never more than m after the rank step)
-  if (mode == QR_RANK) limit = min(w, p.m);
-  for (int i = 0; i < w; ++i) {
-    if (warp == 0) {                    // pivot search and trailing trace (no search without pivoting)
-      float best = -1.f, tr = 0.f;
-      int bi = i;
-      if (mode != QR_PLAIN) {
-        for (int j = i + lane; j < w; j += 32) {
-          const float dd = A[j * LR + j].x;
-          tr += fmaxf(dd, 0.f);
-          if (dd > best) {
-            best = dd;
-            bi = j;
-          }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          tr += __shfl_xor_sync(0xffffffffu, tr, o);
-          const float b2 = __shfl_xor_sync(0xffffffffu, best, o);
-          const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (b2 > best || (b2 == best && i2 < bi)) {
-            best = b2;
-            bi = i2;
-          }
-        }
-      }
+  if (s_bad) return;
+  for (int i = 0;; ++i) {
+    const int pv = s_piv[i & 1];
+    if (pv < 0) break;
+    const float inv = rsqrtf(s_dp[i & 1]), inv2 = inv * inv;
+    float2 lk[NQ];                              // row pv, 1 in the place of the pivot
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int k = lane + 32 * q;
+      lk[q] = k < w ? T[pv * LR + k] : make_float2(0.f, 0.f);
+    }
+    if (warp == 0) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) d[q] -= (lk[q].x * lk[q].x + lk[q].y * lk[q].y) * inv2;
       if (lane == 0) {
-        const int pv = (mode == QR_PLAIN) ? i : bi;
-        const float dp = A[pv * LR + pv].x;
-        if (mode == QR_RANK && s_rank < 0 && tr <= tol2 * s_trace0) s_rank = i;
-        bool stop = false;
-        if (!(dp > 1e-30f * s_maxd0) || !(dp > 0.f)) stop = true;                  // exhausted / not PD
-        if (mode == QR_DROP && dp <= tol2 * s_maxd0) stop = true;
-        if (i >= limit && (mode != QR_RANK || s_rank >= 0)) stop = true;
-        if (mode == QR_RANK && rank_mode == 1 && s_rank >= 0) stop = true;
-        if (stop) {
-          s_stop = 1;
-          s_rho = min(i, limit);
-        }
-        s_piv = pv;
+        perm[i] = pv;
+        dinv[i] = inv;
+        order[pv] = i;
       }
-    }
-    __syncthreads();
-    if (s_stop) break;
-    const int pv = s_piv;
-    if (pv != i) {
-      for (int j = threadIdx.x; j < w; j += blockDim.x) {  // swap rows i, pv
-        const float2 t = A[i * LR + j];
-        A[i * LR + j] = A[pv * LR + j];
-        A[pv * LR + j] = t;
-      }
-      __syncthreads();
-      for (int j = threadIdx.x; j < w; j += blockDim.x) {  // swap cols i, pv
-        const float2 t = A[j * LR + i];
-        A[j * LR + i] = A[j * LR + pv];
-        A[j * LR + pv] = t;
-      }
-      if (threadIdx.x == 0) {
-        const int t = perm[i];
-        perm[i] = perm[pv];
-        perm[pv] = t;
-      }
-      __syncthreads();
-    }
-    const float inv = rsqrtf(A[i * LR + i].x);
-    for (int j = i + threadIdx.x; j < w; j += blockDim.x) {
-      const float2 v = A[j * LR + i];
-      lcol[j] = make_float2(v.x * inv, v.y * inv);
-    }
-    __syncthreads();
-    for (int j = i + threadIdx.x; j < w; j += blockDim.x) A[j * LR + i] = lcol[j];   // column i of L
-    // rank-1 update of the trailing block: a warp per row (stepping by the warps), its lanes
-    // over the columns (no index division)
-    for (int j = i + 1 + warp; j < w; j += (int)(blockDim.x >> 5)) {
-      const float2 lj = lcol[j];
+      __syncwarp();
+      choose(i + 1);
+    } else {
 #pragma unroll
-      for (int q = 0; q < PRONY_RMAX / 32; ++q) {      // unrolled: the row's loads are issued together
-        const int k = i + 1 + lane + 32 * q;
-        if (k < w) {
-          const float2 lk = lcol[k];
-          float2 a = A[j * LR + k];
-          a.x -= lj.x * lk.x + lj.y * lk.y;          // lj * conj(lk)
-          a.y -= lj.y * lk.x - lj.x * lk.y;
-          A[j * LR + k] = a;
+      for (int q = 0; q < NQ; ++q)
+        if (lane + 32 * q == pv) lk[q] = make_float2(1.f, 0.f);
+      for (int j0 = warp - 1; j0 < w; j0 += 4 * (nwarp - 1)) {
+        float2 f[4], t[4][NQ];
+        bool go[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int j = j0 + r * (nwarp - 1);
+          // (order[pv] is written by warp 0 meanwhile: pv is excluded by its index)
+          go[r] = j < w && j != pv && order[j] == w;
+          const int jj = go[r] ? j : pv;
+          const float2 v = T[jj * LR + pv];
+          f[r] = make_float2(v.x * inv2, v.y * inv2);
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            const int k = lane + 32 * q;
+            t[r][q] = (k < w && k != pv) ? T[jj * LR + k] : make_float2(0.f, 0.f);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (!go[r]) continue;
+          float2* row = T + (j0 + r * (nwarp - 1)) * LR;
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            const int k = lane + 32 * q;
+            float2 v = t[r][q];
+            v.x -= f[r].x * lk[q].x - f[r].y * lk[q].y;
+            v.y -= f[r].x * lk[q].y + f[r].y * lk[q].x;
+            if (k < w) row[k] = v;
+          }
         }
       }
     }
     __syncthreads();
   }
-  __syncthreads();
   const int rho = min(s_rho, limit);
-  // R = L^H (rho x rho); M[perm[a]][b] = Rinv[a][b], column b by back substitution: x_b =
-  // 1 / r_bb, then for k = b .. 0: x_k = s_k / r_kk and s_a -= R[a][k] x_k for a < k, the s_a
-  // spread over the lanes of one warp (a = lane + 32 q).
+  // M[j][b] = R^{-1} in the original column order: conj(L^{-1}[b][j]) for the columns j eliminated up to step b
   float2* M = (float2*)(D.small + p.soff + D.L.mapm);
-  const int nwarp = blockDim.x >> 5;
-  // reciprocals of the diagonal once (each column's substitution would otherwise divide at every
-  // step of its dependent chain)
-  __shared__ float rinv[PRONY_RMAX];
-  for (int k = threadIdx.x; k < rho; k += blockDim.x) rinv[k] = 1.f / A[k * LR + k].x;
-  __syncthreads();
-  const int nq = (rho + 31) >> 5;
   for (int b = warp; b < rho; b += nwarp) {
-    float2 sv[PRONY_RMAX / 32];
+    const float s = dinv[b];
+    const float2* row = T + perm[b] * LR;
 #pragma unroll
-    for (int q = 0; q < PRONY_RMAX / 32; ++q) sv[q] = make_float2(lane + 32 * q == b ? 1.f : 0.f, 0.f);
-    for (int k = b; k >= 0; --k) {
-      const int ko = k & 31, kq = k >> 5;
-      float2 mine = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int q = 0; q < PRONY_RMAX / 32; ++q)
-        if (q == kq) mine = sv[q];
-      const float rk = rinv[k];
-      const float2 xk = make_float2(__shfl_sync(0xffffffffu, mine.x, ko) * rk, __shfl_sync(0xffffffffu, mine.y, ko) * rk);
-#pragma unroll
-      for (int q = 0; q < PRONY_RMAX / 32; ++q) {
-        if (q >= nq) break;
-        const int a = lane + 32 * q;
-        if (a == k) sv[q] = xk;
-        else if (a < k) {
-          const float2 l = A[k * LR + a];            // R[a][k] = conj(L[k][a])
-          sv[q].x -= l.x * xk.x + l.y * xk.y;
-          sv[q].y -= l.x * xk.y - l.y * xk.x;
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < PRONY_RMAX / 32; ++q) {
-      const int a = lane + 32 * q;
-      if (a < w) M[perm[a] * LR + b] = a <= b ? sv[q] : make_float2(0.f, 0.f);
+    for (int q = 0; q < NQ; ++q) {
+      const int j = lane + 32 * q;
+      if (j >= w) break;
+      float2 v = make_float2(0.f, 0.f);
+      if (order[j] < b) v = make_float2(row[j].x * s, -row[j].y * s);
+      else if (order[j] == b) v = make_float2(s, 0.f);
+      M[j * LR + b] = v;
     }
   }
   if (threadIdx.x == 0) {
@@ -473,15 +425,24 @@ __global__ void k_reset_done(Dev D) {
 
 void launch_reset_done(const Dev& D, cudaStream_t s) { note_launch(); k_reset_done<<<(D.nprob + 127) / 128, 128, 0, s>>>(D); }
 
-void launch_chol(const Dev& D, int wsel, int target, int mode, double tol, int rank_mode, cudaStream_t s) {
+template <int NQ>
+static void run_chol(const Dev& D, int wsel, int target, int mode, double tol, int rank_mode, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * PRONY_RMAX * PRONY_RMAX));
+    cudaFuncSetAttribute(k_chol<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * 1024 * NQ * NQ));
     attr = true;
   }
-  size_t sm = sizeof(float2) * D.L.LDR * D.L.LDR;
   note_launch();
-  k_chol<<<D.nprob, 256, sm, s>>>(D, wsel, target, mode, tol, rank_mode);
+  k_chol<NQ><<<D.nprob, NQ > 2 ? 512 : 256, sizeof(float2) * D.L.LDR * D.L.LDR, s>>>(D, wsel, target, mode, tol, rank_mode);
+}
+
+void launch_chol(const Dev& D, int wsel, int target, int mode, double tol, int rank_mode, cudaStream_t s) {
+  switch ((D.L.LDR + 31) / 32) {
+    case 1: return run_chol<1>(D, wsel, target, mode, tol, rank_mode, s);
+    case 2: return run_chol<2>(D, wsel, target, mode, tol, rank_mode, s);
+    case 3: return run_chol<3>(D, wsel, target, mode, tol, rank_mode, s);
+    default: return run_chol<4>(D, wsel, target, mode, tol, rank_mode, s);
+  }
 }
 
 void launch_solve_c(const Dev& D, cudaStream_t s) {

@@ -920,13 +920,9 @@ inline int blocks_for(long long n, int per) { return (int)std::min<long long>((n
 
 #include <algorithm>
 
-void launch_state_init(const Dev& D, cudaStream_t s) {
+void launch_prep(const Dev& D, bool norms, cudaStream_t s) {
   note_launch();
   k_state_init<<<(D.nprob + 127) / 128, 128, 0, s>>>(D);
-}
-
-void launch_prep(const Dev& D, bool norms, cudaStream_t s) {
-  launch_state_init(D, s);
   note_launch();
   dim3 g(blocks_per_problem(std::min((D.maxGd + 255) / 256, 64), D.nprob), D.nprob);
   if (norms) k_prep<true><<<g, 256, 0, s>>>(D);

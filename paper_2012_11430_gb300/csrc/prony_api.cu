@@ -1815,9 +1815,7 @@ int prony_toeplitz_mm_dev(prony_ctx* ctx, const prony_c128* grid_dev, int d, int
   B.P[0].r0 = r;
   CK(cudaMemcpyAsync(ctx->P.p, B.P.data(), sizeof(ProbDesc), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->grid64.p, grid_dev, sizeof(double2) * B.P[0].Gd, cudaMemcpyDeviceToDevice, ctx->stream));
-  // (the transformed tables are made from the samples themselves)
-  if (B.ax.on) launch_state_init(B.D, ctx->stream);
-  else launch_prep(B.D, false, ctx->stream);
+  launch_prep(B.D, false, ctx->stream);
   product_tables(ctx, B, precision, L == n + 1, ctx->stream);
   if (B.fft.on) launch_fft_tables(B.D, B.fft.maxpts, ctx->stream);
   // operate directly on the caller's buffers: X as V (ld N), Y as Y (ld L^d)
