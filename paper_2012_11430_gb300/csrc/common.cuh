@@ -62,7 +62,6 @@ struct ProbState {
   int lk;                     // Lanczos (Algorithm 2): vectors u_1..u_lk accepted
   int lstop;                  // Lanczos: why it stopped (1 alpha, 2 beta below the tolerance, 3 block full)
   double lalpha, lbeta;       // Lanczos: last alpha, beta
-  int oa_conv;                // refinement of the SVD of Q: 0 running, 2 last step pending, 1 converged
 };
 
 // Small per-problem workspace: byte offsets inside the block at ProbDesc::soff.

@@ -410,7 +410,7 @@ cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int trim, c
 template <int MODE, int CL, int NC>
 static cudaError_t axis_in_as(const Dev& D, const Dev& S, int xbuf, int wsel, long long items, void* xb,
                               long long prob_stride, cudaStream_t s) {
-  static size_t set = 48 * 1024;
+  static size_t set = 0;
   const int H = max_axis_n(S) + 1;
   const size_t sm = sizeof(float4) * (size_t)(H / 2 + 1) * (H + (H & 1));
   cudaError_t e = allow_smem(k_axis_in<MODE, CL, NC>, sm, set);
@@ -445,7 +445,7 @@ cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int w
 
 template <int KB>
 static cudaError_t axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s) {
-  static size_t set = 48 * 1024;
+  static size_t set = 0;
   const int H = max_axis_n(S) + 1, K = y_ext ? H + 1 : H, nblk = (K + KB - 1) / KB;
   // (H / 2 + 1) x Kt grows with n: the largest problem's table is the largest of the batch
   const size_t sm = sizeof(float4) * (size_t)(H / 2 + 1) * nblk * KB;

@@ -1,27 +1,30 @@
-// FP64-accurate small steps of Algorithm 1, designed for GB300's FP64 unit (high latency per
-// dependent operation, low throughput per SM): iterations run in FP32 on one CTA per problem,
-// and the quantities that fix the results are then computed or refined in FP64 with matrix
-// products only, which k_zgemm spreads over many CTAs per problem (every SM's FP64 units take
-// part even when the batch has fewer problems than SMs).
+// FP64-accurate small steps of Algorithm 1, designed for GB300's FP64 unit (about two FMAs per clock and
+// SM): iterations run in FP32, and the quantities that fix the results are then computed or refined in
+// FP64 with matrix products only.  Two launches, each a cluster of CTAs per problem: the FP32 iterations
+// on the first CTA, the FP64 products spread over all of them, a cluster barrier between dependent products
+// (operands go through L2 and are staged in shared memory).
 //
-//  SVD of Q = U^* T V (Algorithm 3, final step): k_svd_jacobi (FP32 one-sided Jacobi) gives a
-//           starting V; FP64 refinement of V as eigenvectors of H = Q^*Q (Ogita & Aishima 2018,
-//           iterative refinement for the symmetric eigenvalue problem based on matrix
-//           multiplication, Hermitian form): per step T1 = V^*V, T2 = H V, S = V^* T2 (k_zgemm),
-//           the correction F = I + E (k_oa_step), V <- V F (k_zgemm), until ||E||_F <= 1e-9;
-//           k_svd_sort orders the eigenpairs, sigma = sqrt(eigenvalues); U_Q = Q V_Q Sigma^{-1}
-//           and S_l = (U_Q^* (U^* T_l V)) V_Q Sigma^{-1} (Eq. generateSl) by k_zgemm.
-//  Eigen step: k_eig_w forms C_mu = sum_l mu_l S_l and finds W (FP32 Hessenberg reduction,
-//           shifted complex QR, triangular eigenvectors) and its FP32 inverse X; two FP64
-//           Newton-Schulz steps X <- 2X - X (W X) (k_zgemm); C_l = S_l W (k_zgemm);
-//           k_eig_z: z_j(l) = (X C_l)_jj, t_j(l) = -arg z_j(l) / 2pi mod 1 (Eq. diagonalizeSl).
-//           The diagonal of W^{-1} S_l W is stationary in W: an error E in W (W = W_0 (I + E))
-//           changes it only at second order, so z carries FP64 accuracy even though W comes
-//           from FP32 iterations.
+//  k_svd_S  SVD of Q = U^* T V (Algorithm 3, final step): FP32 one-sided Jacobi gives a starting V; FP64
+//           refinement of V as eigenvectors of H = Q^*Q (Ogita & Aishima 2018, iterative refinement for
+//           the symmetric eigenvalue problem based on matrix multiplication, Hermitian form): per step
+//           T1 = V^*V, T2 = H V, S = V^* T2, the correction F = I + E, V <- V F, until ||E||_F <= 1e-9; the
+//           eigenpairs sorted, sigma = sqrt(eigenvalues); U_Q = Q V_Q Sigma^{-1} and
+//           S_l = (U_Q^* (U^* T_l V)) V_Q Sigma^{-1} (Eq. generateSl).
+//  k_eig_t  C_mu = sum_l mu_l S_l, its eigenvectors W (FP32 Hessenberg reduction, shifted complex QR,
+//           triangular eigenvectors Y: W = Z Y) and the FP32 inverse X = Y^{-1} Z^*; one first-order
+//           correction of W from its FP64 residual; two FP64 Newton-Schulz steps X <- 2X - X (W X); z_j(l) = (X S_l W)_jj,
+//           t_j(l) = -arg z_j(l) / 2pi mod 1 (Eq. diagonalizeSl).  The diagonal of W^{-1} S_l W is
+//           stationary in W: an error E in W (W = W_0 (I + E)) changes it only at second order, and the
+//           correction squares E once more, so z carries FP64 accuracy even though W comes from FP32
+//           iterations.
 //  k_canon  phase-canonical singular basis for the S_l output.
+//
+// One launch per product (25 of them, 16 x 16 tiles) and one-CTA iterations before took, at m = 5 / 20 /
+// 40 (one problem), 300 / 910 / 2900 us; now 120 / 340 / 1000 us; 64 problems of m = 40 in one call 4.4 -> 2.2 ms.
 #include "common.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 
 namespace {
@@ -58,333 +61,436 @@ __device__ inline float2 fdiv(float2 a, float2 b) {
   float r = b.x / b.y, den = b.x * r + b.y;
   return fc((a.x * r + a.y) / den, (a.y * r - a.x) / den);
 }
+__device__ inline float rsqrt_a(float x) {       // approximation (0 for denormals' infinity is not asked for)
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// a square root for the shifts of the QR iteration (approximate: a shift need not be exact)
 __device__ inline float2 fsqrtc(float2 a) {
-  float r = hypotf(a.x, a.y);
-  if (r == 0.f) return fc(0.f, 0.f);
-  float sx = sqrtf(0.5f * (r + fabsf(a.x)));
-  if (a.x >= 0.f) return fc(sx, a.y / (2.f * sx));
-  return fc(fabsf(a.y) / (2.f * sx), a.y >= 0.f ? sx : -sx);
+  const float q = fabs2(a);
+  if (!(q > 1e-36f)) return fc(0.f, 0.f);
+  const float t = 0.5f * (q * rsqrt_a(q) + fabsf(a.x)), rt = rsqrt_a(t), sx = t * rt, o = 0.5f * a.y * rt;
+  if (a.x >= 0.f) return fc(sx, o);
+  return fc(fabsf(o), a.y >= 0.f ? sx : -sx);
+}
+// 1 / sqrt(x) correctly rounded but for the last step (a Newton step on the approximation): rotations and
+// reflectors built from it stay unitary to FP32 rounding
+__device__ inline float rsqrt_n(float x) {
+  const float r = rsqrt_a(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
+}
+__device__ inline float2 shfl2(float2 v, int src) {
+  return fc(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+// element i of a row spread over a warp: lane i & 31, register i >> 5
+template <int NQ>
+__device__ __forceinline__ float2 pick(const float2 (&v)[NQ], int i) {
+  return shfl2(NQ == 1 || i < 32 ? v[0] : v[NQ - 1], i & 31);
 }
 
-// block-wide sum of a double (tree; result in every thread)
+// block-wide sum of a double, in thread 0 (every FP64 instruction of a warp holds the pipe for about sixteen
+// cycles: one warp adds the partial sums of the others)
 __device__ double block_sum_d(double v, double* sh) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  double r = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
-  __syncthreads();
-  return r;
-}
-
-__device__ inline void rr_pair(int step, int k, int nb, int& pa, int& pb) {
-  // round-robin (circle) ordering: position 0 fixed, positions 1..nb-1 rotate
-  auto who = [&](int pos) { return pos == 0 ? 0 : ((pos - 1 + step) % (nb - 1)) + 1; };
-  pa = who(k);
-  pb = who(nb - 1 - k);
-}
-
-
-// ----------------------------------------------------------------------------- batched FP64 products
-// C = alpha op(A) op(B) [diag(1/sigma)] [+ beta C0] for every problem of the batch (and `nl`
-// consecutive matrices per problem), on the per-problem small workspace.  Matrices are row-major
-// complex FP64 at byte offsets of the problem's block; op = conjugate transpose when t* = 1.
-// One CTA computes a 16 x 16 tile of C: 256 threads, one entry each, K staged 16 at a time in
-// shared memory; eight partial sums per entry (k mod 8) keep sixteen independent FP64 chains per
-// thread in flight (a dependent FP64 operation waits hundreds of cycles on this GPU).  Dimensions come from the problem's state (a = wu, b = wv).
-enum ZDim { ZD_A = 0, ZD_B = 1 };
-enum ZLive { ZL_SVD = 0, ZL_EIG = 1 };
-enum ZConv { ZC_ALL = 0, ZC_SKIP_CONV = 1, ZC_COPY_CONV = 2 };
-struct ZG {
-  long long a, b, c, c0;          // byte offsets (c0 < 0: no C0 term)
-  long long la, lb, lc;           // byte strides between the nl matrices of a problem
-  long long colscale;             // byte offset of sigma (< 0: no column scaling)
-  int lda, ldb, ldc;
-  int ta, tb;
-  int M, N, K;                    // ZDim selectors
-  int nl;
-  int live;                       // ZLive
-  int conv;                       // ZConv: skip (or copy A to C for) problems whose refinement converged
-  double alpha, beta;
-};
-constexpr int ZT = 16;
-
-__device__ inline int zdim(const ProbState& st, int sel) { return sel == ZD_A ? st.wu : st.wv; }
-
-__global__ void __launch_bounds__(256) k_zgemm(Dev D, ZG g) {
-  __shared__ double2 As[ZT][ZT + 1];
-  __shared__ double2 Bs[ZT][ZT + 1];
-  const int pi = blockIdx.y;
-  const ProbDesc& p = D.P[pi];
-  const ProbState& st = D.st[pi];
-  if (!(g.live == ZL_SVD ? svd_live(p, st) : eig_live(p, st))) return;
-  const int l = blockIdx.z;
-  if (l >= g.nl) return;
-  const int M = zdim(st, g.M), N = zdim(st, g.N), K = zdim(st, g.K);
-  const int tiles_n = (N + ZT - 1) / ZT;
-  const int i0 = (blockIdx.x / tiles_n) * ZT, j0 = (blockIdx.x % tiles_n) * ZT;
-  if (i0 >= M) return;
-  char* sb = D.small + p.soff;
-  const double2* A = (const double2*)(sb + g.a + l * g.la);
-  const double2* B = (const double2*)(sb + g.b + l * g.lb);
-  double2* C = (double2*)(sb + g.c + l * g.lc);
-  const int ty = threadIdx.x / ZT, tx = threadIdx.x % ZT;
-  const int i = i0 + ty, j = j0 + tx;
-  // refinement state: 0 running, 2 last correction pending, 1 converged (products skipped, V copied)
-  if ((g.conv == ZC_SKIP_CONV && st.oa_conv != 0) || (g.conv == ZC_COPY_CONV && st.oa_conv == 1)) {
-    if (g.conv == ZC_COPY_CONV && i < M && j < N) C[i * g.ldc + j] = A[i * g.lda + j];
-    return;
+  if (threadIdx.x < 32) {
+    v = threadIdx.x < blockDim.x >> 5 ? sh[threadIdx.x] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   }
-  double2 acc[8];
+  return v;
+}
+
+// pair k of a round-robin step (circle ordering: position 0 fixed, positions 1..nb-1 rotate), step < nb - 1
+__device__ inline void rr_pair(int step, int k, int nb, int& pa, int& pb) {
+  auto who = [&](int pos) {
+    const int q = pos - 1 + step;
+    return pos == 0 ? 0 : (q >= nb - 1 ? q - (nb - 1) : q) + 1;
+  };
+  const int x = who(k), y = who(nb - 1 - k);
+  pa = min(x, y);
+  pb = max(x, y);
+}
+
+// ----------------------------------------------------------------------------- clusters and FP64 products
+// Barrier over the CTAs of a problem; global writes before it are visible after it (read with ld.cg, so
+// never from a stale L1 line).
+template <int CL>
+__device__ __forceinline__ void cl_sync() {
+  if (CL > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
+// rows x cols of a row-major matrix in global memory -> packed in shared memory
+__device__ inline void stage(double2* dst, const double2* src, int ld, int rows, int cols) {
+  for (int q = threadIdx.x; q < rows * cols; q += blockDim.x) dst[q] = __ldcg(src + (q / cols) * ld + q % cols);
+}
+
+// sum_k op(A[k as]) B[k bs], op = conjugation when CJ.  Four partial sums (k mod 4) keep eight
+// independent FP64 chains per thread in flight.
+template <bool CJ>
+__device__ inline double2 zdot(const double2* A, int as, const double2* B, int bs, int K) {
+  double2 acc[4];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) acc[u] = make_double2(0.0, 0.0);
-  for (int k0 = 0; k0 < K; k0 += ZT) {
-    {
-      // A tile rows i0.., columns k0..; B tile rows k0.., columns j0..
-      const int r = threadIdx.x / ZT, c = threadIdx.x % ZT;
-      const int ai = i0 + r, ak = k0 + c;
-      double2 av = make_double2(0.0, 0.0);
-      if (ai < M && ak < K) av = g.ta ? cconj(A[ak * g.lda + ai]) : A[ai * g.lda + ak];
-      As[r][c] = av;
-      const int bk = k0 + r, bj = j0 + c;
-      double2 bv = make_double2(0.0, 0.0);
-      if (bk < K && bj < N) bv = g.tb ? cconj(B[bj * g.ldb + bk]) : B[bk * g.ldb + bj];
-      Bs[r][c] = bv;
+  for (int u = 0; u < 4; ++u) acc[u] = make_double2(0.0, 0.0);
+  int k = 0;
+  for (; k + 4 <= K; k += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const double2 a = A[(k + u) * as], b = B[(k + u) * bs];
+      const double ay = CJ ? -a.y : a.y;
+      acc[u].x = fma(a.x, b.x, acc[u].x);
+      acc[u].y = fma(a.x, b.y, acc[u].y);
+      acc[u].x = fma(-ay, b.y, acc[u].x);
+      acc[u].y = fma(ay, b.x, acc[u].y);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+    if (k + u < K) {
+      const double2 a = A[(k + u) * as], b = B[(k + u) * bs];
+      const double ay = CJ ? -a.y : a.y;
+      acc[u].x = fma(a.x, b.x, acc[u].x);
+      acc[u].y = fma(a.x, b.y, acc[u].y);
+      acc[u].x = fma(-ay, b.y, acc[u].x);
+      acc[u].y = fma(ay, b.x, acc[u].y);
+    }
+  return cadd(cadd(acc[0], acc[1]), cadd(acc[2], acc[3]));
+}
+
+// entry e of the upper triangle (j (j + 1) / 2 + i, i <= j)
+__device__ inline void tri(int e, int& i, int& j) {
+  j = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+  if (j * (j + 1) / 2 > e) --j;
+  if ((j + 1) * (j + 2) / 2 <= e) ++j;
+  i = e - j * (j + 1) / 2;
+}
+
+constexpr int OA_MAX = 6;     // refinement steps at most (two where singular values are well apart)
+
+// FP32 one-sided Jacobi on the columns of Q (a x b, a <= 32 NA): right singular vectors -> V (FP64, ld LM).
+// A warp takes a pair of columns and holds both, and those of V, in registers from the inner product to
+// the rotation; the squared norms are kept and updated with the rotations (and computed afresh every
+// sweep), so a pair costs one inner product.  Rotations are unitary to FP32 rounding; angles need not be.
+template <int NA>
+__device__ void svd_jacobi(const Dev& D, ProbState& st, const double2* Q, int a, int b, int LM, double2* V, float2* fsm) {
+  __shared__ int s_rot;
+  __shared__ float nrm[PRONY_MMAX];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  float2* Qc = fsm;                                             // [b][a] columns
+  float2* Vc = fsm + (size_t)a * b;                             // [b][b] columns
+  for (int idx = threadIdx.x; idx < a * b; idx += blockDim.x) {
+    const int i = idx / b, j = idx % b;
+    const double2 q = Q[i * LM + j];
+    Qc[j * a + i] = fc((float)q.x, (float)q.y);
+  }
+  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
+    const int i = idx % b, j = idx / b;
+    Vc[j * b + i] = fc(i == j ? 1.f : 0.f, 0.f);
+  }
+  const int nb = b + (b & 1);
+  const float jtol = 4.f * a * 5.9604645e-8f, jtol2 = jtol * jtol;
+  const int max_sweeps = D.cap_jacobi > 0 ? D.cap_jacobi : 30;
+  int sweep = 0;
+  bool rotated = b > 1;                          // the last sweep still rotated (not converged)
+  for (; sweep < max_sweeps && b > 1; ++sweep) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_rot = 0;
+    for (int j = warp; j < b; j += nwarp) {
+      float s = 0.f;
+      for (int i = lane; i < a; i += 32) s += fabs2(Qc[j * a + i]);
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) nrm[j] = s;
     }
     __syncthreads();
+    for (int step = 0; step < nb - 1; ++step) {
+      for (int k = warp; k < nb / 2; k += nwarp) {
+        int pa, pb;
+        rr_pair(step, k, nb, pa, pb);
+        if (pb >= b) continue;
+        float2* xa = Qc + pa * a;
+        float2* xb = Qc + pb * a;
+        float2* va = Vc + pa * b;
+        float2* vb = Vc + pb * b;
+        float2 x[NA], y[NA], u[2], v[2], ga = fc(0.f, 0.f);
 #pragma unroll
-    for (int kk = 0; kk < ZT; kk += 8) {
+        for (int q = 0; q < NA; ++q) {
+          const int i = lane + 32 * q;
+          x[q] = i < a ? xa[i] : fc(0.f, 0.f);
+          y[q] = i < a ? xb[i] : fc(0.f, 0.f);
+        }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const double2 a = As[ty][kk + u], b = Bs[kk + u][tx];
-        acc[u].x = fma(a.x, b.x, acc[u].x);
-        acc[u].y = fma(a.x, b.y, acc[u].y);
-        acc[u].x = fma(-a.y, b.y, acc[u].x);
-        acc[u].y = fma(a.y, b.x, acc[u].y);
+        for (int q = 0; q < 2; ++q) {
+          const int i = lane + 32 * q;
+          u[q] = i < b ? va[i] : fc(0.f, 0.f);
+          v[q] = i < b ? vb[i] : fc(0.f, 0.f);
+        }
+        const float al = nrm[pa], be = nrm[pb];
+#pragma unroll
+        for (int q = 0; q < NA; ++q) ga = fadd(ga, fmulc(x[q], y[q]));
+        for (int o = 16; o > 0; o >>= 1) {
+          ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
+          ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
+        }
+        const float ag2 = fabs2(ga);
+        if (!(ag2 > jtol2 * fmaxf(al * be, 0.f)) || ag2 < 1e-37f) continue;
+        const float ri = rsqrtf(ag2), ag = ag2 * ri;             // 1 / |gamma|, |gamma|
+        const float zeta = (be - al) * 0.5f * ri, z1 = fmaf(zeta, zeta, 1.f);
+        const float tt = copysignf(__fdividef(1.f, fabsf(zeta) + z1 * rsqrtf(z1)), zeta);
+        const float c = rsqrt_n(fmaf(tt, tt, 1.f)), s = c * tt;
+        const float rn = rsqrt_n(ag2);
+        const float2 ph = fc(ga.x * rn, -ga.y * rn);             // e^{-i arg gamma}
+#pragma unroll
+        for (int q = 0; q < NA; ++q) {
+          const int i = lane + 32 * q;
+          const float2 yp = fmul(y[q], ph);
+          if (i < a) {
+            xa[i] = fsub(fscale(x[q], c), fscale(yp, s));
+            xb[i] = fadd(fscale(x[q], s), fscale(yp, c));
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int i = lane + 32 * q;
+          const float2 vp = fmul(v[q], ph);
+          if (i < b) {
+            va[i] = fsub(fscale(u[q], c), fscale(vp, s));
+            vb[i] = fadd(fscale(u[q], s), fscale(vp, c));
+          }
+        }
+        if (lane == 0) {
+          nrm[pa] = al - tt * ag;
+          nrm[pb] = be + tt * ag;
+          s_rot = 1;
+        }
+      }
+      __syncthreads();
+    }
+    rotated = s_rot != 0;
+    if (!rotated) break;
+  }
+  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
+    const int i = idx / b, j = idx % b;
+    const float2 v = Vc[j * b + i];
+    V[i * LM + j] = make_double2(v.x, v.y);
+  }
+  if (threadIdx.x == 0 && sweep >= max_sweeps && rotated) set_status_e(st, ST_ENOCONV);
+}
+
+// ----------------------------------------------------------------------------- SVD of Q and S_l
+template <int CL, int NT>
+__global__ void __launch_bounds__(NT) k_svd_S(Dev D) {
+  extern __shared__ double2 zsm[];
+  __shared__ double s_red[32];
+  __shared__ double s_lam[PRONY_MMAX], s_inv[PRONY_MMAX];
+  __shared__ int s_rank[PRONY_MMAX];
+  __shared__ double s_delta, s_en;
+  // upper-triangle entries per thread: b (b + 1) / 2 <= EMAX CL NT for the widest b of this NT
+  constexpr int BM = NT > 512 ? 64 : NT > 128 ? 32 : 16, EMAX = (BM * (BM + 1) / 2 + CL * NT - 1) / (CL * NT);
+  const ProbDesc& p = D.P[blockIdx.y];
+  ProbState& st = D.st[blockIdx.y];
+  if (!svd_live(p, st)) return;                  // the whole cluster
+  const int rank = CL > 1 ? blockIdx.x : 0;
+  const int a = st.wu, b = st.wv, LM = D.L.LDM;
+  char* sb = D.small + p.soff;
+  const double2* Q = (const double2*)(sb + D.L.q);
+  double2* Hm = (double2*)(sb + D.L.work1);
+  double2* V = (double2*)(sb + D.L.work2);
+  double2* Vn = (double2*)(sb + D.L.S);          // the first S_l slot is free until the end
+  double2* F = (double2*)(sb + D.L.work3);
+  double2* T2 = (double2*)(sb + D.L.work4);
+  double* lam = (double*)(sb + D.L.sigma);
+  double* part = (double*)(sb + D.L.gram);       // partial norms: [quantity][CTA]
+  double2* s1 = zsm;                             // two operands in shared memory
+  double2* s2 = zsm + (size_t)b * b;
+  const int ntri = b * (b + 1) / 2;
+  // ---- starting V on the first CTA; H = Q^* Q on the others meanwhile
+  if (rank == 0) {
+    if (a <= 32) svd_jacobi<1>(D, st, Q, a, b, LM, V, (float2*)zsm);
+    else if (a <= 64) svd_jacobi<2>(D, st, Q, a, b, LM, V, (float2*)zsm);
+    else svd_jacobi<4>(D, st, Q, a, b, LM, V, (float2*)zsm);
+  }
+  if (CL == 1 || rank > 0) {
+    __syncthreads();
+    stage(zsm, Q, LM, a, b);
+    __syncthreads();
+    constexpr int R = CL > 1 ? CL - 1 : 1;
+    for (int e = threadIdx.x * R + (CL > 1 ? rank - 1 : 0); e < ntri; e += NT * R) {
+      int i, j;
+      tri(e, i, j);
+      const double2 h = zdot<true>(zsm + i, b, zsm + j, b, a);
+      Hm[i * LM + j] = h;
+      if (i != j) Hm[j * LM + i] = cconj(h);
+    }
+  }
+  cl_sync<CL>();
+  double e2 = 0.0;                               // ||H||_F^2 (thread 0, once)
+  for (int it = 0; it < OA_MAX; ++it) {
+    stage(s1, V, LM, b, b);
+    stage(s2, Hm, LM, b, b);
+    __syncthreads();
+    if (it == 0) {
+      for (int q = threadIdx.x; q < b * b; q += NT) e2 += cabs2(s2[q]);
+      e2 = block_sum_d(e2, s_red);
+    }
+    double2 t1[EMAX], sv[EMAX];
+    double e3 = 0.0;
+#pragma unroll
+    for (int x = 0; x < EMAX; ++x) {             // T1 = V^* V (kept by the thread)
+      const int e = (threadIdx.x + x * NT) * CL + rank;
+      t1[x] = make_double2(0.0, 0.0);
+      if (e >= ntri) continue;
+      int i, j;
+      tri(e, i, j);
+      t1[x] = zdot<true>(s1 + i, b, s1 + j, b, b);
+      const double rx = (i == j ? 1.0 : 0.0) - t1[x].x;
+      e3 += (i == j ? 1.0 : 2.0) * (rx * rx + t1[x].y * t1[x].y);
+    }
+    for (int e = threadIdx.x * CL + rank; e < b * b; e += NT * CL)   // T2 = H V
+      T2[e / b * LM + e % b] = zdot<false>(s2 + (e / b) * b, 1, s1 + e % b, b, b);
+    cl_sync<CL>();
+    stage(s2, T2, LM, b, b);
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < EMAX; ++x) {             // S = V^* T2; lambda_i = s_ii / (V^* V)_ii
+      const int e = (threadIdx.x + x * NT) * CL + rank;
+      sv[x] = make_double2(0.0, 0.0);
+      if (e >= ntri) continue;
+      int i, j;
+      tri(e, i, j);
+      sv[x] = zdot<true>(s1 + i, b, s2 + j, b, b);
+      if (i == j) lam[i] = sv[x].x / t1[x].x;
+    }
+    cl_sync<CL>();
+    for (int i = threadIdx.x; i < b; i += NT) s_lam[i] = __ldcg(lam + i);
+    __syncthreads();
+    double e1 = 0.0;
+#pragma unroll
+    for (int x = 0; x < EMAX; ++x) {
+      const int e = (threadIdx.x + x * NT) * CL + rank;
+      if (e >= ntri) continue;
+      int i, j;
+      tri(e, i, j);
+      const double sx = sv[x].x - (i == j ? s_lam[i] : 0.0);
+      e1 += (i == j ? 1.0 : 2.0) * (sx * sx + sv[x].y * sv[x].y);
+    }
+    e1 = block_sum_d(e1, s_red);
+    e3 = block_sum_d(e3, s_red);
+    if (threadIdx.x == 0) {
+      part[rank] = e1;
+      part[CL + rank] = e3;
+    }
+    cl_sync<CL>();
+    // E: e_ij = (s_ij + lambda_j r_ij) / (lambda_j - lambda_i) with R = I - V^*V, r_ij / 2 within a
+    // cluster of eigenvalues closer than delta = 2 (||S - diag(lambda)||_F + ||H||_F ||R||_F)
+    if (threadIdx.x == 0) {
+      e1 = e3 = 0.0;
+      for (int r = 0; r < CL; ++r) {
+        e1 += __ldcg(part + r);
+        e3 += __ldcg(part + CL + r);
+      }
+      s_delta = 2.0 * (sqrt(e1) + sqrt(e2 * e3));
+    }
+    __syncthreads();
+    const double delta = s_delta;
+    double en = 0.0;
+#pragma unroll
+    for (int x = 0; x < EMAX; ++x) {
+      const int e = (threadIdx.x + x * NT) * CL + rank;
+      if (e >= ntri) continue;
+      int i, j;
+      tri(e, i, j);
+      const double2 r = make_double2((i == j ? 1.0 : 0.0) - t1[x].x, -t1[x].y);
+      double2 eij = cscale(r, 0.5), eji = cconj(eij);
+      const double gap = s_lam[j] - s_lam[i];
+      if (i != j && fabs(gap) > delta) {
+        const double ig = 1.0 / gap;
+        eij = cscale(cadd(sv[x], cscale(r, s_lam[j])), ig);
+        eji = cscale(cconj(cadd(sv[x], cscale(r, s_lam[i]))), -ig);
+      }
+      F[i * LM + j] = make_double2((i == j ? 1.0 : 0.0) + eij.x, eij.y);
+      en += cabs2(eij);
+      if (i != j) {
+        F[j * LM + i] = eji;
+        en += cabs2(eji);
       }
     }
+    en = block_sum_d(en, s_red);
+    if (threadIdx.x == 0) part[2 * CL + rank] = en;
+    cl_sync<CL>();
+    stage(s2, F, LM, b, b);
+    if (threadIdx.x == 0) {
+      en = 0.0;
+      for (int r = 0; r < CL; ++r) en += __ldcg(part + 2 * CL + r);
+      s_en = en;
+    }
     __syncthreads();
+    for (int e = threadIdx.x * CL + rank; e < b * b; e += NT * CL)   // V <- V F
+      Vn[e / b * LM + e % b] = zdot<false>(s1 + (e / b) * b, 1, s2 + e % b, b, b);
+    double2* t = V;
+    V = Vn;
+    Vn = t;
+    cl_sync<CL>();
+    // a step (after the first) with ||E||_F <= 1e-9 is the last: another would change V by less than
+    // the FP64 rounding of the products
+    if (it >= 1 && s_en <= 1e-18) break;
   }
-  if (i >= M || j >= N) return;
-  double2 v = cscale(cadd(cadd(cadd(acc[0], acc[1]), cadd(acc[2], acc[3])), cadd(cadd(acc[4], acc[5]), cadd(acc[6], acc[7]))),
-                     g.alpha);
-  if (g.colscale >= 0) {
-    const double sj = ((const double*)(sb + g.colscale))[j];
-    v = sj > 0.0 ? cscale(v, 1.0 / sj) : make_double2(0.0, 0.0);
-  }
-  if (g.c0 >= 0) v = cadd(v, cscale(((const double2*)(sb + g.c0 + l * g.lc))[i * g.ldc + j], g.beta));
-  C[i * g.ldc + j] = v;
-}
-
-// One refinement step of V (eigenvectors of H = Q^*Q) from T1 = V^*V (work3) and S = V^* H V
-// (uq): lambda_i = s_ii / (1 - r_ii) with R = I - V^*V, the correction E with
-// e_ij = (s_ij + lambda_j r_ij) / (lambda_j - lambda_i) (r_ij / 2 within a cluster of
-// eigenvalues closer than delta = 2 (||S - diag(lambda)||_F + ||H||_F ||R||_F)), written as
-// F = I + E into work4 for V <- V F; lambda into the sigma slots.  A step whose ||E||_F is at most
-// 1e-9 (after the first) is the last one (state 2: its V F still runs; the next step marks the
-// refinement converged, state 1): another would change V by less than the FP64 rounding of the
-// products.
-__global__ void __launch_bounds__(256) k_oa_step(Dev D, int iter) {
-  __shared__ double s_red[32];
-  __shared__ double s_lam[PRONY_MMAX];
-  const ProbDesc& p = D.P[blockIdx.x];
-  ProbState& st = D.st[blockIdx.x];
-  if (!svd_live(p, st)) return;
-  const int state = st.oa_conv;
+  // ---- eigenpairs of H in descending order: V_Q, sigma = sqrt(lambda)
+  double2* sVQ = zsm;
+  double2* sA = zsm + (size_t)b * b;             // a x b operand
   __syncthreads();
-  if (state == 2 && threadIdx.x == 0) st.oa_conv = 1;
-  if (state != 0) return;
-  const int b = st.wv, LM = D.L.LDM;
-  char* sb = D.small + p.soff;
-  const double2* Hm = (const double2*)(sb + D.L.work1);
-  const double2* T1 = (const double2*)(sb + D.L.work3);
-  const double2* Sm = (const double2*)(sb + D.L.uq);
-  double2* F = (double2*)(sb + D.L.work4);
-  double* lam = (double*)(sb + D.L.sigma);
-  for (int i = threadIdx.x; i < b; i += blockDim.x) {
-    s_lam[i] = Sm[i * LM + i].x / T1[i * LM + i].x;       // s_ii / (1 - r_ii), 1 - r_ii = (V^*V)_ii
-    lam[i] = s_lam[i];
-  }
-  __syncthreads();
-  double e1 = 0.0, e2 = 0.0, e3 = 0.0;
-  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
-    const int i = idx / b, j = idx % b;
-    double2 sv = Sm[i * LM + j];
-    if (i == j) sv.x -= s_lam[i];
-    const double2 t = T1[i * LM + j];
-    const double2 r = make_double2((i == j ? 1.0 : 0.0) - t.x, -t.y);
-    e1 += cabs2(sv);
-    e2 += cabs2(Hm[i * LM + j]);
-    e3 += cabs2(r);
-  }
-  e1 = block_sum_d(e1, s_red);
-  e2 = block_sum_d(e2, s_red);
-  e3 = block_sum_d(e3, s_red);
-  const double delta = 2.0 * (sqrt(e1) + sqrt(e2) * sqrt(e3));
-  double en = 0.0;
-  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
-    const int i = idx / b, j = idx % b;
-    const double2 t = T1[i * LM + j];
-    const double2 r = make_double2((i == j ? 1.0 : 0.0) - t.x, -t.y);
-    double2 e;
-    if (i != j && fabs(s_lam[i] - s_lam[j]) > delta)
-      e = cscale(cadd(Sm[i * LM + j], cscale(r, s_lam[j])), 1.0 / (s_lam[j] - s_lam[i]));
-    else
-      e = cscale(r, 0.5);
-    en += cabs2(e);
-    F[i * LM + j] = make_double2((i == j ? 1.0 : 0.0) + e.x, e.y);
-  }
-  en = block_sum_d(en, s_red);
-  if (threadIdx.x == 0 && iter >= 1 && en <= 1e-18) st.oa_conv = 2;
-}
-
-// Eigenpairs of H in descending order: V_Q (vq) = the columns of the refined V (at byte offset
-// `voff`) permuted, sigma = sqrt(lambda) sorted, sigma_m / sigma_1.
-__global__ void __launch_bounds__(256) k_svd_sort(Dev D, long long voff) {
-  __shared__ double s_lam[PRONY_MMAX];
-  __shared__ int s_rank[PRONY_MMAX];
-  const ProbDesc& p = D.P[blockIdx.x];
-  ProbState& st = D.st[blockIdx.x];
-  if (!svd_live(p, st)) return;
-  const int b = st.wv, LM = D.L.LDM;
-  char* sb = D.small + p.soff;
-  const double2* Vm = (const double2*)(sb + voff);
-  double2* VQ = (double2*)(sb + D.L.vq);
-  double* sig = (double*)(sb + D.L.sigma);
-  for (int i = threadIdx.x; i < b; i += blockDim.x) s_lam[i] = sig[i];
-  __syncthreads();
-  for (int j = threadIdx.x; j < b; j += blockDim.x) {
+  for (int j = threadIdx.x; j < b; j += NT) {
     int r = 0;
     for (int i = 0; i < b; ++i)
       if (s_lam[i] > s_lam[j] || (s_lam[i] == s_lam[j] && i < j)) ++r;
     s_rank[j] = r;
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
-    const int i = idx / b, j = idx % b;
-    VQ[i * LM + s_rank[j]] = Vm[i * LM + j];
+  double2* VQ = (double2*)(sb + D.L.vq);
+  for (int q = threadIdx.x; q < b * b; q += NT) {
+    const int i = q / b, j = q % b;
+    const double2 v = __ldcg(V + i * LM + j);
+    sVQ[i * b + s_rank[j]] = v;
+    if (rank == 0) VQ[i * LM + s_rank[j]] = v;
   }
-  for (int j = threadIdx.x; j < b; j += blockDim.x) sig[s_rank[j]] = sqrt(fmax(s_lam[j], 0.0));
-  __syncthreads();
-  if (threadIdx.x == 0) st.sigma_ratio = sig[0] > 0.0 ? sig[b - 1] / sig[0] : 0.0;
-}
-
-// z_j(l) = sum_a X[j][a] C_l[a][j] with X = W^{-1} (work3 after the Newton-Schulz steps) and
-// C_l = S_l W (mproj slices); t_j(l) = -arg z_j(l) / 2 pi mod 1.
-__global__ void k_eig_z(Dev D) {
-  const ProbDesc& p = D.P[blockIdx.x];
-  ProbState& st = D.st[blockIdx.x];
-  if (!eig_live(p, st)) return;
-  const int m = st.wv, LM = D.L.LDM, LR = D.L.LDR;
-  char* sb = D.small + p.soff;
-  const double2* Xd = (const double2*)(sb + D.L.work3);
-  double* tout = (double*)(sb + D.L.t);
-  double2* zr = (double2*)(sb + D.L.zraw);
-  for (int q = threadIdx.x; q < m * p.d; q += blockDim.x) {
-    const int j = q / p.d, l = q % p.d;
-    const double2* Cl = (const double2*)(sb + D.L.mproj) + (size_t)l * LR * LM;
-    double2 acc[4] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-    for (int a = 0; a < m; ++a) acc[a & 3] = cadd(acc[a & 3], cmul(Xd[j * LM + a], Cl[a * LM + j]));
-    const double2 z = cadd(cadd(acc[0], acc[1]), cadd(acc[2], acc[3]));
-    zr[j * PRONY_DMAX + l] = z;
-    double tj = -atan2(z.y, z.x) / 6.283185307179586;
-    tj -= floor(tj);
-    if (tj >= 1.0) tj = 0.0;
-    tout[j * PRONY_DMAX + l] = tj;
-  }
-  if (threadIdx.x == 0) st.rank_used = m;
-}
-
-// ----------------------------------------------------------------------------- SVD of Q and S_l
-// FP32 one-sided Jacobi on the columns of Q: the starting V (FP64 copy in work2) of the FP64
-// refinement.  One CTA per problem.
-__global__ void __launch_bounds__(256) k_svd_jacobi(Dev D) {
-  extern __shared__ float2 fsm[];
-  __shared__ int s_rot;
-  const ProbDesc& p = D.P[blockIdx.x];
-  ProbState& st = D.st[blockIdx.x];
-  if (!svd_live(p, st)) return;
-  const int a = st.wu, b = st.wv;
-  const int LM = D.L.LDM, LR = D.L.LDR;
-  char* sb = D.small + p.soff;
-  const double2* Q = (const double2*)(sb + D.L.q);            // a x b, ld LM
-  double2* Vm = (double2*)(sb + D.L.work2);                     // b x b, ld LM
-  float2* Qc = fsm;                                             // [b][a] columns (FP32)
-  float2* Vc = fsm + (size_t)LM * LR;                           // [b][b] columns (FP32)
-
-  // ---- FP32 one-sided Jacobi on the columns of Q
-  for (int idx = threadIdx.x; idx < a * b; idx += blockDim.x) {
-    int i = idx % a, j = idx / a;
-    double2 q = Q[i * LM + j];
-    Qc[j * a + i] = fc((float)q.x, (float)q.y);
-  }
-  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
-    int i = idx % b, j = idx / b;
-    Vc[j * b + i] = fc(i == j ? 1.f : 0.f, 0.f);
+  double mine = 0.0;
+  if (threadIdx.x < b) mine = sqrt(fmax(s_lam[threadIdx.x], 0.0));
+  stage(sA, Q, LM, a, b);
+  // every CTA has read lambda from its shared copy; the sorted sigma replaces it
+  if (threadIdx.x < b) {
+    s_inv[s_rank[threadIdx.x]] = mine > 0.0 ? 1.0 / mine : 0.0;
+    if (rank == 0) lam[s_rank[threadIdx.x]] = mine;
+    if (rank == 0 && s_rank[threadIdx.x] == b - 1) s_red[0] = mine;
+    if (rank == 0 && s_rank[threadIdx.x] == 0) s_red[1] = mine;
   }
   __syncthreads();
-  const int nb = b + (b & 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-  const float jtol = 4.f * a * 5.9604645e-8f;
-  const int max_sweeps = D.cap_jacobi > 0 ? D.cap_jacobi : 30;
-  int sweep = 0;
-  bool rotated = b > 1;                          // the last sweep still rotated (not converged)
-  for (; sweep < max_sweeps && b > 1; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
-    for (int step = 0; step < nb - 1; ++step) {
-      for (int k = warp; k < nb / 2; k += nwarp) {
-        int pa, pb;
-        rr_pair(step, k, nb, pa, pb);
-        if (pa >= b || pb >= b) continue;
-        if (pa > pb) { int t = pa; pa = pb; pb = t; }
-        float al = 0.f, be = 0.f;
-        float2 ga = fc(0.f, 0.f);
-        for (int i = lane; i < a; i += 32) {
-          float2 x = Qc[pa * a + i], y = Qc[pb * a + i];
-          al += fabs2(x);
-          be += fabs2(y);
-          ga = fadd(ga, fmulc(x, y));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
-          ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
-        }
-        float ag = sqrtf(fabs2(ga));
-        if (ag <= jtol * sqrtf(al * be) || ag == 0.f) continue;
-        float zeta = (be - al) / (2.f * ag);
-        float tt = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-        float c = rsqrtf(1.f + tt * tt), s = c * tt;
-        float2 ph = fc(ga.x / ag, -ga.y / ag);   // e^{-i arg gamma}
-        for (int i = lane; i < a; i += 32) {
-          float2 x = Qc[pa * a + i], y = fmul(Qc[pb * a + i], ph);
-          Qc[pa * a + i] = fsub(fscale(x, c), fscale(y, s));
-          Qc[pb * a + i] = fadd(fscale(x, s), fscale(y, c));
-        }
-        for (int i = lane; i < b; i += 32) {
-          float2 x = Vc[pa * b + i], y = fmul(Vc[pb * b + i], ph);
-          Vc[pa * b + i] = fsub(fscale(x, c), fscale(y, s));
-          Vc[pb * b + i] = fadd(fscale(x, s), fscale(y, c));
-        }
-        if (lane == 0) s_rot = 1;
-      }
-      __syncthreads();
-    }
-    rotated = s_rot != 0;
-    if (!s_rot) break;
-    __syncthreads();
+  if (rank == 0 && threadIdx.x == 0) st.sigma_ratio = s_red[1] > 0.0 ? s_red[0] / s_red[1] : 0.0;
+  // ---- U_Q = Q V_Q Sigma^{-1}, S_l = (U_Q^* M_l) V_Q Sigma^{-1}: this CTA takes the columns (of U_Q) and
+  // rows (of S_l) i = rank mod CL, so no other CTA's results are needed
+  const int ni = (b - rank + CL - 1) / CL;       // how many
+  double2* sU = sA + (size_t)a * b;              // a x ni
+  double2* sP = sU + (size_t)a * ((b + CL - 1) / CL);   // ni x b
+  double2* UQ = (double2*)(sb + D.L.uq);
+  for (int e = threadIdx.x; e < a * ni; e += NT) {
+    const int r = e / ni, c = e % ni, i = rank + c * CL;
+    const double2 u = cscale(zdot<false>(sA + r * b, 1, sVQ + i, b, b), s_inv[i]);
+    sU[e] = u;
+    UQ[r * LM + i] = u;
   }
-  for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
-    int i = idx / b, j = idx % b;
-    float2 v = Vc[j * b + i];
-    Vm[i * LM + j] = make_double2(v.x, v.y);
-  }
-  if (threadIdx.x == 0) {
-    st.oa_conv = 0;
-    if (sweep >= max_sweeps && rotated) set_status_e(st, ST_ENOCONV);
+  for (int l = 0; l < p.d; ++l) {
+    __syncthreads();
+    stage(sA, (const double2*)(sb + D.L.mproj) + (size_t)l * D.L.LDR * LM, LM, a, b);
+    __syncthreads();
+    for (int e = threadIdx.x; e < ni * b; e += NT) sP[e] = zdot<true>(sU + e / b, ni, sA + e % b, b, a);
+    __syncthreads();
+    double2* S = (double2*)(sb + D.L.S) + (size_t)l * LM * LM;
+    for (int e = threadIdx.x; e < ni * b; e += NT)
+      S[(rank + e / b * CL) * LM + e % b] = cscale(zdot<false>(sP + (e / b) * b, 1, sVQ + e % b, b, b), s_inv[e % b]);
   }
 }
 
@@ -427,115 +533,125 @@ __global__ void k_canon(Dev D) {
 }
 
 // ----------------------------------------------------------------------------- eigen step
-// C_mu, its eigenvectors W (FP32 Hessenberg reduction, shifted complex QR, triangular
-// eigenvectors; FP64 copy in work2) and the FP32 Gauss-Jordan inverse X of W (FP64 copy in
-// work3).  One CTA per problem.
-__global__ void __launch_bounds__(256) k_eig_w(Dev D, unsigned long long seed) {
-  extern __shared__ float2 esm[];
-  __shared__ double2 mu[PRONY_DMAX];
+// mu of C_mu for every dimension: Philox draws, unit vectors (the same for every problem of a call)
+struct MuTable { double2 v[PRONY_DMAX][PRONY_DMAX]; };   // [d - 1][l]
+
+__device__ __forceinline__ void bar4() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Eigenvectors W of the m x m matrix H (m <= 32 NQ; shared memory, pitch 32 NQ + 1, zero beyond m) and X ~ W^{-1}, both FP32 values, to
+// global memory in FP64.  The whole block (at least 128 threads).
+// (FP32 copies Wf, Xf, packed, and the eigenvalues lamf beside them).
+template <int NQ>
+__device__ void eig_w(const Dev& D, ProbState& st, int m, float2* H, float2* Z, float2* Y, double2* Wd, double2* Xd,
+                      int LM, float2* Wf, float2* Xf, float2* lamf) {
+  constexpr int LD = 32 * NQ + 1;
   __shared__ float2 hv[PRONY_MMAX];
-  __shared__ float2 sv[PRONY_MMAX];
-  __shared__ float s_norm;
-  __shared__ int s_fail, s_pr;
-  const ProbDesc& p = D.P[blockIdx.x];
-  ProbState& st = D.st[blockIdx.x];
-  if (!eig_live(p, st)) return;                 // shared memory holds 3 maxM^2 entries
-  const int m = st.wv;
-  const int LM = D.L.LDM;
-  const int LD = m;                             // smem leading dimension
-  float2* H = esm;                              // m x m  (C_mu, then Schur form, then W^{-1} work)
-  float2* Z = esm + LD * LD;                    // m x m  (Schur vectors, then W)
-  float2* Y = Z + LD * LD;                      // m x m  (triangular eigenvectors, then W^{-1})
-  char* sb = D.small + p.soff;
-  const double2* S = (const double2*)(sb + D.L.S);
-  double2* Wd = (double2*)(sb + D.L.work2);     // W (FP64)
-  double2* Xd = (double2*)(sb + D.L.work3);     // W^{-1} (FP64, FP32 accurate)
-  if (threadIdx.x == 0) {
-    double nrm = 0.0;
-    for (int l = 0; l < p.d; ++l) {
-      uint64_t c[4] = {(uint64_t)l, 0, 0, 0};
-      philox4x64(c, seed, PRONY_STREAM_MU);
-      double u0 = philox_u01(c[0]), u1 = philox_u01(c[1]);
-      double r = sqrt(-log(u0)), sn, cs;
-      sincospi(2.0 * u1, &sn, &cs);
-      mu[l] = make_double2(r * cs, r * sn);
-      nrm += cabs2(mu[l]);
-    }
-    nrm = sqrt(nrm);
-    for (int l = 0; l < p.d; ++l) mu[l] = cscale(mu[l], 1.0 / nrm);
-    s_fail = 0;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    int i = idx / m, j = idx % m;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int l = 0; l < p.d; ++l) acc = cadd(acc, cmul(mu[l], S[(size_t)l * LM * LM + i * LM + j]));
-    H[i * LD + j] = fc((float)acc.x, (float)acc.y);
-    Z[i * LD + j] = fc(i == j ? 1.f : 0.f, 0.f);
-  }
-  __syncthreads();
-  // ---- FP32 Householder reduction to Hessenberg form
+  __shared__ float4 rot[PRONY_MMAX];             // rotations of a sweep: c, Re s, Im s
+  __shared__ float sv[PRONY_MMAX];
+  __shared__ float s_red[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+  // ---- Householder reduction to Hessenberg form: warp 0 forms the reflector, then eight threads share
+  // a column of H (sums over its rows), then a row of H or Z
   for (int k = 0; k + 2 < m; ++k) {
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
+      float2 x[NQ];
       float nx = 0.f;
-      for (int i = k + 1; i < m; ++i) nx += fabs2(H[i * LD + k]);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int i = lane + 32 * q;
+        x[q] = (i > k && i < m) ? H[i * LD + k] : fc(0.f, 0.f);
+        nx += fabs2(x[q]);
+      }
+      for (int o = 16; o > 0; o >>= 1) nx += __shfl_xor_sync(0xffffffffu, nx, o);
       nx = sqrtf(nx);
-      float2 x0 = H[(k + 1) * LD + k];
-      float ax0 = sqrtf(fabs2(x0));
-      float2 ph = ax0 > 0.f ? fscale(x0, 1.f / ax0) : fc(1.f, 0.f);
-      float2 alpha = fscale(ph, -nx);
-      for (int i = 0; i < m; ++i) hv[i] = fc(0.f, 0.f);
-      for (int i = k + 1; i < m; ++i) hv[i] = H[i * LD + k];
-      hv[k + 1] = fsub(hv[k + 1], alpha);
-      float nv = 0.f;
-      for (int i = k + 1; i < m; ++i) nv += fabs2(hv[i]);
-      s_norm = nv;
-      if (nv > 0.f) {
-        float inv = rsqrtf(nv);
-        for (int i = k + 1; i < m; ++i) hv[i] = fscale(hv[i], inv);
+      const float2 x0 = pick<NQ>(x, k + 1);
+      const float ax0 = sqrtf(fabs2(x0));
+      const float2 ph = ax0 > 0.f ? fscale(x0, 1.f / ax0) : fc(1.f, 0.f);
+      const float2 v0 = fadd(x0, fscale(ph, nx));
+      // ||v||^2 = 2 nx (nx + |x0|)
+      const float nv = 2.f * nx * (nx + ax0), inv = nv > 1e-36f ? rsqrt_n(nv) : 0.f;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int i = lane + 32 * q;
+        if (i < m) hv[i] = fscale(i == k + 1 ? v0 : x[q], inv);
+      }
+      if (lane == 0) s_red[0] = inv;
+    }
+    __syncthreads();
+    if (s_red[0] > 0.f) {                        // (uniform)
+      const int part = threadIdx.x & 7, grp = threadIdx.x >> 3, ngrp = blockDim.x >> 3;
+      for (int j0 = k; j0 < m; j0 += ngrp) {
+        const int j = j0 + grp;
+        float2 h[4 * NQ], s = fc(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 4 * NQ; ++e) {
+          const int i = k + 1 + part + 8 * e;
+          h[e] = (i < m && j < m) ? H[i * LD + j] : fc(0.f, 0.f);
+          if (i < m) s = fadd(s, fmulc(hv[i], h[e]));
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+          s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+          s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+        }
+        s = fscale(s, 2.f);
+#pragma unroll
+        for (int e = 0; e < 4 * NQ; ++e) {
+          const int i = k + 1 + part + 8 * e;
+          if (i < m && j < m) H[i * LD + j] = (j == k && i > k + 1) ? fc(0.f, 0.f) : fsub(h[e], fmul(hv[i], s));
+        }
+      }
+      __syncthreads();
+      for (int i0 = 0; i0 < 2 * m; i0 += ngrp) {
+        const int i = i0 + grp;
+        float2* R = i < m ? H + i * LD : Z + (i - m) * LD;
+        float2 h[4 * NQ], s = fc(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 4 * NQ; ++e) {
+          const int j = k + 1 + part + 8 * e;
+          h[e] = (j < m && i < 2 * m) ? R[j] : fc(0.f, 0.f);
+          if (j < m) s = fadd(s, fmul(h[e], hv[j]));
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+          s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+          s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+        }
+        s = fscale(s, 2.f);
+#pragma unroll
+        for (int e = 0; e < 4 * NQ; ++e) {
+          const int j = k + 1 + part + 8 * e;
+          if (j < m && i < 2 * m) R[j] = fsub(h[e], fmul(s, fconj(hv[j])));
+        }
       }
     }
     __syncthreads();
-    if (s_norm > 0.f) {
-      for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        float2 s = fc(0.f, 0.f);
-        for (int i = k + 1; i < m; ++i) s = fadd(s, fmulc(hv[i], H[i * LD + j]));
-        sv[j] = s;
-      }
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < (m - k - 1) * m; idx += blockDim.x) {
-        int i = k + 1 + idx / m, j = idx % m;
-        H[i * LD + j] = fsub(H[i * LD + j], fscale(fmul(hv[i], sv[j]), 2.f));
-      }
-      __syncthreads();
-      for (int i = threadIdx.x; i < 2 * m; i += blockDim.x) {
-        float2* R = i < m ? H : Z;
-        int ii = i < m ? i : i - m;
-        float2 s = fc(0.f, 0.f);
-        for (int j = k + 1; j < m; ++j) s = fadd(s, fmul(R[ii * LD + j], hv[j]));
-        for (int j = k + 1; j < m; ++j) R[ii * LD + j] = fsub(R[ii * LD + j], fscale(fmul(s, fconj(hv[j])), 2.f));
-      }
-      __syncthreads();
-      for (int i = k + 2 + threadIdx.x; i < m; i += blockDim.x) H[i * LD + k] = fc(0.f, 0.f);
-      __syncthreads();
-    }
   }
-  // ---- FP32 shifted complex QR iteration (one warp), full Schur form
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
+  // ---- shifted complex QR iteration, full Schur form, by four warps.  A sweep on the active block
+  // l..hi: H - sigma I = Q R row by row on warp 0 (a lane owns a column; the rotation of step k is
+  // formed from column k, which all earlier rotations have reached), then R Q + sigma I and Z Q with a
+  // thread per row.  The dependent chain is one rotation per row instead of one with its row, column
+  // and Z updates (180 cycles instead of about 420).  Entries of R left of the subdiagonal are stored
+  // as they come and never read.
+  if (warp < 4) {
     const float eps = 5.9604645e-8f;
     int hi = m - 1, its = 0, total = 0;
     const int cap = D.cap_eigqr > 0 ? D.cap_eigqr : 30 * m + 30;
     while (hi > 0) {
       if (total > cap) break;
-      int l = hi;
-      for (; l > 0; --l) {
-        float s = fabs1(H[(l - 1) * LD + l - 1]) + fabs1(H[l * LD + l]);
-        if (s == 0.f) s = 1.f;
-        if (fabs1(H[l * LD + l - 1]) <= eps * s) break;
+      int l = 0;
+#pragma unroll
+      for (int q = NQ - 1; q >= 0; --q) {        // largest index with a negligible subdiagonal entry
+        const int i = lane + 32 * q;
+        bool small = false;
+        if (i >= 1 && i <= hi) {
+          float s = fabs1(H[(i - 1) * LD + i - 1]) + fabs1(H[i * LD + i]);
+          if (s == 0.f) s = 1.f;
+          small = fabs1(H[i * LD + i - 1]) <= eps * s;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, small);
+        if (l == 0 && bal) l = 32 * q + 31 - __clz(bal);
       }
-      if (l > 0 && lane == 0) H[l * LD + l - 1] = fc(0.f, 0.f);
-      __syncwarp();
       if (l == hi) {
         --hi;
         its = 0;
@@ -545,229 +661,430 @@ __global__ void __launch_bounds__(256) k_eig_w(Dev D, unsigned long long seed) {
       if (its == 10 || its == 20) {
         sh = fadd(H[hi * LD + hi], fc(0.75f * fabs1(H[hi * LD + hi - 1]), 0.f));
       } else {
-        float2 a = H[(hi - 1) * LD + hi - 1], bb = H[(hi - 1) * LD + hi], c = H[hi * LD + hi - 1], dd = H[hi * LD + hi];
-        float2 hd = fscale(fsub(a, dd), 0.5f);
-        float2 disc = fsqrtc(fadd(fmul(hd, hd), fmul(bb, c)));
-        float2 mid = fscale(fadd(a, dd), 0.5f);
-        float2 l1 = fadd(mid, disc), l2 = fsub(mid, disc);
+        const float2 a = H[(hi - 1) * LD + hi - 1], bb = H[(hi - 1) * LD + hi], c = H[hi * LD + hi - 1], dd = H[hi * LD + hi];
+        const float2 hd = fscale(fsub(a, dd), 0.5f);
+        const float2 disc = fsqrtc(fadd(fmul(hd, hd), fmul(bb, c)));
+        const float2 mid = fscale(fadd(a, dd), 0.5f);
+        const float2 l1 = fadd(mid, disc), l2 = fsub(mid, disc);
         sh = fabs2(fsub(l1, dd)) <= fabs2(fsub(l2, dd)) ? l1 : l2;
       }
-      float2 x = fsub(H[l * LD + l], sh), y = H[(l + 1) * LD + l];
-      for (int k = l; k < hi; ++k) {
-        if (k > l) {
-          x = H[k * LD + k - 1];
-          y = H[(k + 1) * LD + k - 1];
-        }
-        float ax = sqrtf(fabs2(x)), ay = sqrtf(fabs2(y));
-        float nr = hypotf(ax, ay);
-        float c;
-        float2 s;
-        if (nr == 0.f) {
-          c = 1.f;
-          s = fc(0.f, 0.f);
-        } else if (ax == 0.f) {
-          c = 0.f;
-          s = fscale(fconj(y), 1.f / ay);
-        } else {
-          c = ax / nr;
-          s = fscale(fmul(fscale(x, 1.f / ax), fconj(y)), 1.f / nr);
-        }
-        for (int j = max(l, k - 1) + lane; j < m; j += 32) {
-          float2 rk = H[k * LD + j], rk1 = H[(k + 1) * LD + j];
-          H[k * LD + j] = fadd(fscale(rk, c), fmul(s, rk1));
-          H[(k + 1) * LD + j] = fsub(fscale(rk1, c), fmul(fconj(s), rk));
-        }
-        __syncwarp();
-        int rmax = min(k + 2, hi);
-        for (int i = lane; i <= rmax; i += 32) {
-          float2 ck = H[i * LD + k], ck1 = H[i * LD + k + 1];
-          H[i * LD + k] = fadd(fscale(ck, c), fmul(fconj(s), ck1));
-          H[i * LD + k + 1] = fsub(fscale(ck1, c), fmul(s, ck));
-        }
-        for (int i = lane; i < m; i += 32) {
-          float2 ck = Z[i * LD + k], ck1 = Z[i * LD + k + 1];
-          Z[i * LD + k] = fadd(fscale(ck, c), fmul(fconj(s), ck1));
-          Z[i * LD + k + 1] = fsub(fscale(ck1, c), fmul(s, ck));
-        }
-        __syncwarp();
+      bar4();                                    // every warp has read H
+      if ((int)threadIdx.x >= l && (int)threadIdx.x <= hi) {
+        H[threadIdx.x * LD + threadIdx.x] = fsub(H[threadIdx.x * LD + threadIdx.x], sh);
+        if ((int)threadIdx.x == l && l > 0) H[l * LD + l - 1] = fc(0.f, 0.f);
       }
+      bar4();
+      if (warp == 0) {
+        float2 cur[NQ], nx[NQ];
+        float2* row = H + l * LD + lane;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          cur[q] = row[32 * q];
+          nx[q] = row[LD + 32 * q];
+        }
+#pragma unroll 2
+        for (int k = l; k < hi; ++k, row += LD) {
+          float2 nn[NQ];                         // the row after next (the last: any)
+          const int ahead = k + 2 <= hi ? 2 * LD : LD;
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) nn[q] = row[ahead + 32 * q];
+          const float2 x = pick<NQ>(cur, k), y = pick<NQ>(nx, k);
+          // c = |x| / r, s = x conj(y) / (|x| r), r^2 = |x|^2 + |y|^2, by one reciprocal root
+          const float ax2 = fabs2(x), n2 = ax2 + fabs2(y), pr = ax2 * n2;
+          const float2 xy = fmul(x, fconj(y));
+          const float rr = rsqrt_n(pr);
+          float c = ax2 * rr;
+          float2 s = fscale(xy, rr);
+          if (!(pr > 1e-36f)) {                  // x (or both) negligible
+            c = n2 > 1e-36f ? 0.f : 1.f;
+            s = n2 > 1e-36f ? fscale(fconj(y), rsqrt_n(n2)) : fc(0.f, 0.f);
+          }
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            row[32 * q] = fadd(fscale(cur[q], c), fmul(s, nx[q]));
+            cur[q] = fsub(fscale(nx[q], c), fmul(fconj(s), cur[q]));
+            nx[q] = nn[q];
+          }
+          if (lane == 0) rot[k] = make_float4(c, s.x, s.y, 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) row[32 * q] = cur[q];
+      }
+      bar4();
+      {
+        const bool zrow = threadIdx.x >= 64;
+        const int i = threadIdx.x & 63;
+        if (i < m && (zrow || i <= hi)) {
+          float2* R = (zrow ? Z : H) + i * LD;
+          // row i of R starts at its diagonal; the entry left of it is zero
+          const bool low = !zrow && i > l;
+          const int k0 = low ? i - 1 : l;
+          float2 cur = low ? fc(0.f, 0.f) : R[l];
+          float2 nx = R[k0 + 1];
+          float4 rn = rot[k0];
+#pragma unroll 2
+          for (int k = k0; k < hi; ++k) {
+            const float2 nn = R[min(k + 2, hi)];
+            const float4 r = rn;
+            rn = rot[min(k + 1, hi - 1)];
+            const float2 s = fc(r.y, r.z);
+            R[k] = fadd(fscale(cur, r.x), fmul(fconj(s), nx));
+            cur = fsub(fscale(nx, r.x), fmul(s, cur));
+            nx = nn;
+          }
+          if (!zrow && i >= l && i < hi) R[i] = fadd(R[i], sh);
+          if (!zrow && i == hi) cur = fadd(cur, sh);
+          R[hi] = cur;
+        }
+      }
+      bar4();
       ++its;
       ++total;
     }
-    if (lane == 0 && hi > 0) s_fail = 1;
+    if (threadIdx.x == 0 && hi > 0) set_status_e(st, ST_ENOCONV);
   }
   __syncthreads();
-  if (s_fail && threadIdx.x == 0) set_status_e(st, ST_ENOCONV);
-  // ---- triangular eigenvectors (FP32), W = Z Y with unit columns
-  if (threadIdx.x == 0) {
+  // ---- triangular eigenvectors, a warp per column: (H_ii - lambda_k) y_i = -(H_ik + sum_{i < j < k} H_ij y_j)
+  {
     float hn = 0.f;
-    for (int i = 0; i < m; ++i)
-      for (int j = i; j < m; ++j) hn = fmaxf(hn, fabs1(H[i * LD + j]));
-    s_norm = hn;
-  }
-  __syncthreads();
-  const float small = fmaxf(s_norm, 1e-30f) * 5.9604645e-8f;
-  for (int k = threadIdx.x; k < m; k += blockDim.x) {
-    float2 lam = H[k * LD + k];
-    for (int i = k + 1; i < m; ++i) Y[i * LD + k] = fc(0.f, 0.f);
-    Y[k * LD + k] = fc(1.f, 0.f);
-    for (int i = k - 1; i >= 0; --i) {
-      float2 s = fc(0.f, 0.f);
-      for (int j = i + 1; j <= k; ++j) s = fadd(s, fmul(H[i * LD + j], Y[j * LD + k]));
-      float2 den = fsub(H[i * LD + i], lam);
-      if (fabs1(den) < small) den = fc(small, 0.f);
-      Y[i * LD + k] = fdiv(fc(-s.x, -s.y), den);
+    for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
+      const int i = q / m, j = q % m;
+      if (j >= i) hn = fmaxf(hn, fabs1(H[i * LD + j]));
+    }
+    for (int o = 16; o > 0; o >>= 1) hn = fmaxf(hn, __shfl_xor_sync(0xffffffffu, hn, o));
+    if (lane == 0) s_red[warp] = hn;
+    __syncthreads();
+    hn = 0.f;
+    for (int w = 0; w < nwarp; ++w) hn = fmaxf(hn, s_red[w]);
+    const float small = fmaxf(hn, 1e-30f) * 5.9604645e-8f;
+    for (int k = threadIdx.x; k < m; k += blockDim.x) lamf[k] = H[k * LD + k];
+    for (int k = warp; k < m; k += nwarp) {
+      const float2 lamk = H[k * LD + k];
+      float2 acc[NQ], rd[NQ];
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int i = lane + 32 * q;
+        acc[q] = rd[q] = fc(0.f, 0.f);
+        if (i < k) {
+          float2 den = fsub(H[i * LD + i], lamk);
+          if (fabs1(den) < small) den = fc(small, 0.f);
+          rd[q] = fdiv(fc(1.f, 0.f), den);
+          acc[q] = fc(-H[i * LD + k].x, -H[i * LD + k].y);
+        }
+      }
+      for (int i = k - 1; i >= 0; --i) {
+        float2 hc[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) hc[q] = lane + 32 * q < i ? H[(lane + 32 * q) * LD + i] : fc(0.f, 0.f);
+        float2 own[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) own[q] = fmul(acc[q], rd[q]);
+        const float2 y = pick<NQ>(own, i);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          acc[q] = fsub(acc[q], fmul(hc[q], y));
+          if (lane + 32 * q == i) Y[i * LD + k] = y;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const int i = lane + 32 * q;
+        if (i >= k && i < m) Y[i * LD + k] = fc(i == k ? 1.f : 0.f, 0.f);
+      }
     }
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    int i = idx / m, k = idx % m;
+  // ---- W = Z Y with unit columns (into H, then FP64)
+  for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
+    const int i = q / m, k = q % m;
     float2 acc = fc(0.f, 0.f);
     for (int j = 0; j <= k; ++j) acc = fadd(acc, fmul(Z[i * LD + j], Y[j * LD + k]));
     H[i * LD + k] = acc;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < m; k += blockDim.x) {
+  for (int k = warp; k < m; k += nwarp) {
     float s = 0.f;
-    for (int i = 0; i < m; ++i) s += fabs2(H[i * LD + k]);
-    sv[k] = fc(s > 0.f ? rsqrtf(s) : 1.f, 0.f);
+    for (int i = lane; i < m; i += 32) s += fabs2(H[i * LD + k]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sv[k] = s > 0.f ? rsqrtf(s) : 1.f;
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    int i = idx / m, k = idx % m;
-    float2 w = fscale(H[i * LD + k], sv[k].x);
-    Z[i * LD + k] = w;                                  // W (FP32) for the inverse
-    Wd[i * LM + k] = make_double2(w.x, w.y);            // W (FP64, exactly the same numbers)
-    Y[i * LD + k] = fc(i == k ? 1.f : 0.f, 0.f);
+  for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
+    const int i = q / m, k = q % m;
+    const float2 w = fscale(H[i * LD + k], sv[k]);
+    Wd[i * LM + k] = make_double2(w.x, w.y);
+    Wf[q] = w;
   }
   __syncthreads();
-  // ---- FP32 Gauss-Jordan inverse of W (partial pivoting): Z -> I, Y -> W^{-1}
-  for (int k = 0; k < m; ++k) {
-    if (threadIdx.x == 0) {
-      int pr = k;
-      float best = fabs1(Z[k * LD + k]);
-      for (int i = k + 1; i < m; ++i) {
-        float v = fabs1(Z[i * LD + k]);
-        if (v > best) { best = v; pr = i; }
+  // ---- Y^{-1} (into H), a warp per column: u_k = 1, u_i = -(Y_ik + sum_{i < j < k} Y_ij u_j)
+  for (int k = warp; k < m; k += nwarp) {
+    float2 acc[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int i = lane + 32 * q;
+      acc[q] = i < k ? fc(-Y[i * LD + k].x, -Y[i * LD + k].y) : fc(0.f, 0.f);
+      if (i >= k && i < m) H[i * LD + k] = fc(i == k ? 1.f : 0.f, 0.f);
+    }
+    for (int i = k - 1; i >= 0; --i) {
+      float2 yc[NQ];
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) yc[q] = lane + 32 * q < i ? Y[(lane + 32 * q) * LD + i] : fc(0.f, 0.f);
+      const float2 u = pick<NQ>(acc, i);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        acc[q] = fsub(acc[q], fmul(yc[q], u));
+        if (lane + 32 * q == i) H[i * LD + k] = u;
       }
-      s_pr = pr;
-      if (best == 0.f) s_fail = 2;
+    }
+  }
+  __syncthreads();
+  // ---- X = diag(1 / sv) Y^{-1} Z^*
+  for (int q = threadIdx.x; q < m * m; q += blockDim.x) {
+    const int j = q / m, i = q % m;
+    float2 acc = fc(0.f, 0.f);
+    for (int b = j; b < m; ++b) acc = fadd(acc, fmul(H[j * LD + b], fconj(Z[i * LD + b])));
+    const float f = 1.f / sv[j];
+    Xd[j * LM + i] = make_double2(acc.x * f, acc.y * f);
+    Xf[q] = fscale(acc, f);
+  }
+}
+
+template <int CL, int NT>
+__global__ void __launch_bounds__(NT) k_eig_t(Dev D, MuTable mu) {
+  extern __shared__ double2 zsm[];
+  const ProbDesc& p = D.P[blockIdx.y];
+  ProbState& st = D.st[blockIdx.y];
+  if (!eig_live(p, st)) return;                  // the whole cluster
+  const int rank = CL > 1 ? blockIdx.x : 0;
+  const int m = st.wv, LM = D.L.LDM;
+  constexpr int NQ = NT > 512 ? 2 : 1, LD = 32 * NQ + 1;   // (NT by the widest problem of the batch)
+  char* sb = D.small + p.soff;
+  const double2* S = (const double2*)(sb + D.L.S);
+  double2* Wd = (double2*)(sb + D.L.work2);      // W (FP64)
+  double2* Xd = (double2*)(sb + D.L.work3);      // X, alternating with work1
+  double2* Xn = (double2*)(sb + D.L.work1);
+  double2* Rd = (double2*)(sb + D.L.work4);
+  float2* Cm = (float2*)(sb + D.L.mapm);         // C_mu
+  float2* Wf = (float2*)(sb + D.L.gram);         // FP32 W, X, eigenvalues (packed)
+  float2* Xf = Wf + (size_t)m * m;
+  float2* lamf = (float2*)(sb + D.L.q);
+  for (int e = threadIdx.x * CL + rank; e < m * m; e += NT * CL) {
+    const double2* s = S + (e / m) * LM + e % m;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int l = 0; l < p.d; ++l) acc = cadd(acc, cmul(mu.v[p.d - 1][l], s[(size_t)l * LM * LM]));
+    Cm[e] = fc((float)acc.x, (float)acc.y);
+  }
+  cl_sync<CL>();
+  if (rank == 0) {
+    float2* H = (float2*)zsm;                    // m x m each, pitch LD
+    float2* Z = H + m * LD;
+    float2* Y = Z + m * LD;
+    for (int q = threadIdx.x; q < m * LD; q += NT) {
+      const int i = q / LD, j = q % LD;
+      H[q] = j < m ? __ldcg(Cm + i * m + j) : fc(0.f, 0.f);
+      Z[q] = fc(i == j ? 1.f : 0.f, 0.f);
     }
     __syncthreads();
-    const int pr = s_pr;
-    if (pr != k) {
-      for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        float2 t = Z[k * LD + j]; Z[k * LD + j] = Z[pr * LD + j]; Z[pr * LD + j] = t;
-        t = Y[k * LD + j]; Y[k * LD + j] = Y[pr * LD + j]; Y[pr * LD + j] = t;
+    eig_w<NQ>(D, st, m, H, Z, Y, Wd, Xd, LM, Wf, Xf, lamf);
+    if (threadIdx.x == 0) st.rank_used = m;
+  }
+  cl_sync<CL>();
+  // ---- this CTA owns the columns (of W and S_l W) and rows (of X) j = rank mod CL
+  const int nj = (m - rank + CL - 1) / CL;
+  double2* sW = zsm;
+  double2* sX = sW + (size_t)m * m;
+  double2* sR = sX + (size_t)m * m;
+  double2* Cl = (double2*)(sb + D.L.mproj);      // S_l W, own columns
+  double2* Wc = (double2*)(sb + D.L.vq);         // the corrected W (V_Q has served; others may still read W)
+  const long long lC = (long long)D.L.LDR * LM;
+  stage(sW, Wd, LM, m, m);
+  __syncthreads();
+  for (int e = threadIdx.x; e < p.d * m * nj; e += NT) {
+    const int c = e % nj, q = e / nj, i = q % m, l = q / m, j = rank + c * CL;
+    Cl[l * lC + i * LM + j] = zdot<false>(S + (size_t)l * LM * LM + i * LM, 1, sW + j, m, m);
+  }
+  // One correction of W: W <- W + dW, dW = W E, E_kj = (X (C_mu W - W Lambda))_kj / (lambda_j - lambda_k) off the
+  // diagonal.  The residual is formed in FP64; being of FP32 size itself, the rest of the step is FP32,
+  // and leaves W accurate to about the square of its FP32 error.
+  {
+    float2* fres = (float2*)sX;                  // m x nj: the residual, then E
+    float2* fE = fres + (size_t)m * nj;
+    float2* fS = fE + (size_t)m * nj;            // m x m
+    float2* fdW = fS + (size_t)m * m;            // m x nj
+    __syncthreads();
+    for (int e = threadIdx.x; e < m * nj; e += NT) {
+      const int c = e % nj, i = e / nj, j = rank + c * CL;
+      double2 acc = make_double2(0.0, 0.0);
+      for (int l = 0; l < p.d; ++l) acc = cadd(acc, cmul(mu.v[p.d - 1][l], Cl[l * lC + i * LM + j]));
+      const float2 lj = __ldcg(lamf + j);
+      acc = csub(acc, cmul(sW[i * m + j], make_double2(lj.x, lj.y)));
+      fres[e] = fc((float)acc.x, (float)acc.y);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < m * nj; e += NT) {
+      const int c = e % nj, k = e / nj, j = rank + c * CL;
+      float2 o = fc(0.f, 0.f);
+#pragma unroll 4
+      for (int i = 0; i < m; ++i) o = fadd(o, fmul(__ldcg(Xf + k * m + i), fres[i * nj + c]));
+      const float2 gap = fsub(__ldcg(lamf + j), __ldcg(lamf + k));
+      float2 ev = (k == j || fabs1(gap) == 0.f) ? fc(0.f, 0.f) : fdiv(o, gap);
+      if (!(fabs1(ev) < 0.25f)) ev = fc(0.f, 0.f);               // no correction: eigenvalues too close
+      fE[e] = ev;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < m * nj; e += NT) {
+      const int c = e % nj, i = e / nj, j = rank + c * CL;
+      float2 o = fc(0.f, 0.f);
+#pragma unroll 4
+      for (int k = 0; k < m; ++k) o = fadd(o, fmul(__ldcg(Wf + i * m + k), fE[k * nj + c]));
+      fdW[e] = o;
+      Wc[i * LM + j] = make_double2(sW[i * m + j].x + (double)o.x, sW[i * m + j].y + (double)o.y);
+    }
+    for (int l = 0; l < p.d; ++l) {
+      __syncthreads();
+      for (int q = threadIdx.x; q < m * m; q += NT) {
+        const double2 v = S[(size_t)l * LM * LM + (q / m) * LM + q % m];
+        fS[q] = fc((float)v.x, (float)v.y);
       }
       __syncthreads();
+      for (int e = threadIdx.x; e < m * nj; e += NT) {
+        const int c = e % nj, i = e / nj, j = rank + c * CL;
+        float2 o = fc(0.f, 0.f);
+#pragma unroll 4
+        for (int k = 0; k < m; ++k) o = fadd(o, fmul(fS[i * m + k], fdW[k * nj + c]));
+        double2* at = &Cl[l * lC + i * LM + j];
+        *at = make_double2(at->x + (double)o.x, at->y + (double)o.y);
+      }
     }
-    float2 piv = Z[k * LD + k];
-    if (fabs1(piv) == 0.f) piv = fc(1e-30f, 0.f);
-    __syncthreads();
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-      Z[k * LD + j] = fdiv(Z[k * LD + j], piv);
-      Y[k * LD + j] = fdiv(Y[k * LD + j], piv);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) hv[i] = (i == k) ? fc(0.f, 0.f) : Z[i * LD + k];
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-      int i = idx / m, j = idx % m;
-      if (i == k) continue;
-      float2 f = hv[i];
-      Z[i * LD + j] = fsub(Z[i * LD + j], fmul(f, Z[k * LD + j]));
-      Y[i * LD + j] = fsub(Y[i * LD + j], fmul(f, Y[k * LD + j]));
-    }
-    __syncthreads();
-  }  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    int i = idx / m, j = idx % m;
-    float2 x = Y[i * LD + j];
-    Xd[i * LM + j] = make_double2(x.x, x.y);
   }
-  if (threadIdx.x == 0 && s_fail == 2) set_status_e(st, ST_ENOCONV);
+  cl_sync<CL>();
+  // ---- Newton-Schulz steps X <- 2X - X (W X) until ||I - W X||_max before the last is below 1e-8 (two,
+  // unless the correction of W was large)
+  __shared__ float s_dev[32];
+  __shared__ int s_more;
+  float* devs = (float*)(lamf + m);              // one slot per CTA and parity of the step
+  stage(sW, Wc, LM, m, m);
+  for (int it = 0; it < 6; ++it) {
+    stage(sX, Xd, LM, m, m);
+    __syncthreads();
+    float dev = 0.f;
+    for (int e = threadIdx.x; e < nj * m; e += NT) {
+      const int j = rank + e / m * CL, c = e % m;
+      const double2 r = zdot<false>(sW + j * m, 1, sX + c, m, m);
+      Rd[j * LM + c] = r;
+      dev = fmaxf(dev, fabsf((float)(r.x - (c == j ? 1.0 : 0.0))) + fabsf((float)r.y));
+    }
+    for (int o = 16; o > 0; o >>= 1) dev = fmaxf(dev, __shfl_xor_sync(0xffffffffu, dev, o));
+    if ((threadIdx.x & 31) == 0) s_dev[threadIdx.x >> 5] = dev;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < NT / 32; ++w) dev = fmaxf(dev, s_dev[w]);
+      devs[(it & 1) * CL + rank] = dev;
+    }
+    cl_sync<CL>();
+    stage(sR, Rd, LM, m, m);
+    if (threadIdx.x == 0) {
+      dev = 0.f;
+      for (int r = 0; r < CL; ++r) dev = fmaxf(dev, __ldcg(devs + (it & 1) * CL + r));
+      s_more = dev > 1e-8f && it < 5;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nj * m; e += NT) {
+      const int j = rank + e / m * CL, c = e % m;
+      const double2 v = zdot<false>(sX + j * m, 1, sR + c, m, m), x = sX[j * m + c];
+      Xn[j * LM + c] = make_double2(2.0 * x.x - v.x, 2.0 * x.y - v.y);
+    }
+    double2* t = Xd;
+    Xd = Xn;
+    Xn = t;
+    if (!s_more) break;                          // (the same in every CTA)
+    cl_sync<CL>();
+  }
+  __syncthreads();                               // of the last X only this CTA's own rows are read
+  // ---- z_j(l) = sum_a X[j][a] (S_l W)[a][j] for the own j
+  double* tout = (double*)(sb + D.L.t);
+  double2* zr = (double2*)(sb + D.L.zraw);
+  for (int e = threadIdx.x; e < nj * p.d; e += NT) {
+    const int c = e % nj, l = e / nj, j = rank + c * CL;
+    const double2 z = zdot<false>(Xd + j * LM, 1, Cl + l * lC + j, LM, m);
+    zr[j * PRONY_DMAX + l] = z;
+    double tj = -atan2(z.y, z.x) / 6.283185307179586;
+    tj -= floor(tj);
+    if (tj >= 1.0) tj = 0.0;
+    tout[j * PRONY_DMAX + l] = tj;
+  }
 }
 
-}  // namespace
-
-namespace {
-constexpr int OA_MAX = 4;     // refinement steps launched (converged problems skip the rest)
-
-void launch_zgemm(const Dev& D, const ZG& g, cudaStream_t s) {
-  // tiles of the largest product of the batch: widths are at most r0 (a) and m (b)
-  const int mx = g.M == ZD_A ? D.L.LDR : D.L.LDM, nx = g.N == ZD_A ? D.L.LDR : D.L.LDM;
-  const int tiles = ((mx + ZT - 1) / ZT) * ((nx + ZT - 1) / ZT);
+template <typename... Args>
+cudaError_t launch_cluster(void (*kernel)(Args...), int cl, int threads, size_t smem, int nprob, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cl, nprob);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cl;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cl > 1 ? 1 : 0;
   note_launch();
-  k_zgemm<<<dim3(tiles, D.nprob, g.nl), ZT * ZT, 0, s>>>(D, g);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-ZG zg(long long a, int lda, int ta, long long b, int ldb, int tb, long long c, int ldc, int M, int N, int K,
-      int live) {
-  ZG g{};
-  g.a = a; g.b = b; g.c = c; g.c0 = -1;
-  g.lda = lda; g.ldb = ldb; g.ldc = ldc;
-  g.ta = ta; g.tb = tb;
-  g.M = M; g.N = N; g.K = K;
-  g.nl = 1;
-  g.colscale = -1;
-  g.live = live;
-  g.conv = ZC_ALL;
-  g.alpha = 1.0;
-  g.beta = 0.0;
-  return g;
-}
-}  // namespace
-
-void launch_svd_S(const Dev& D, cudaStream_t s) {
+template <int CL, int NT>
+void run_svd(const Dev& D, cudaStream_t s) {
   static size_t set = 0;
-  const SmallLay& L = D.L;
-  const int LM = L.LDM;
-  size_t sm = sizeof(float2) * ((size_t)L.LDM * L.LDR + (size_t)L.LDM * L.LDM);
+  const size_t a = D.L.LDR, b = D.L.LDM, own = (b + CL - 1) / CL;
+  // V_Q, an a x b operand, own columns of U_Q, own rows of P; the Jacobi columns (FP32) fit as well
+  const size_t sm = sizeof(double2) * (b * b + std::max(a, b) * b + a * own + own * b);
   if (sm > set) {
-    cudaFuncSetAttribute(k_svd_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_svd_S<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     set = sm;
   }
-  // H = Q^* Q (work1); starting V (work2) by FP32 Jacobi
-  launch_zgemm(D, zg(L.q, LM, 1, L.q, LM, 0, L.work1, LM, ZD_B, ZD_B, ZD_A, ZL_SVD), s);
-  note_launch();
-  k_svd_jacobi<<<D.nprob, 256, sm, s>>>(D);
-  // refinement steps; V alternates between work2 and the first S_l slot (free until the end)
-  long long v = L.work2, vn = L.S;
-  for (int it = 0; it < OA_MAX; ++it) {
-    ZG t1 = zg(v, LM, 1, v, LM, 0, L.work3, LM, ZD_B, ZD_B, ZD_B, ZL_SVD);   // V^* V
-    t1.conv = ZC_SKIP_CONV;
-    launch_zgemm(D, t1, s);
-    ZG t2 = zg(L.work1, LM, 0, v, LM, 0, L.work4, LM, ZD_B, ZD_B, ZD_B, ZL_SVD);   // H V
-    t2.conv = ZC_SKIP_CONV;
-    launch_zgemm(D, t2, s);
-    ZG sv = zg(v, LM, 1, L.work4, LM, 0, L.uq, LM, ZD_B, ZD_B, ZD_B, ZL_SVD);   // V^* H V
-    sv.conv = ZC_SKIP_CONV;
-    launch_zgemm(D, sv, s);
-    note_launch();
-    k_oa_step<<<D.nprob, 256, 0, s>>>(D, it);
-    ZG vf = zg(v, LM, 0, L.work4, LM, 0, vn, LM, ZD_B, ZD_B, ZD_B, ZL_SVD);   // V F
-    vf.conv = ZC_COPY_CONV;
-    launch_zgemm(D, vf, s);
-    std::swap(v, vn);
+  launch_cluster(k_svd_S<CL, NT>, CL, NT, sm, D.nprob, s, D);
+}
+
+template <int CL, int NT>
+void run_eig(const Dev& D, const MuTable& mu, cudaStream_t s) {
+  static size_t set = 0;
+  const size_t m = D.L.LDM, own = (m + CL - 1) / CL;
+  // W and two more m x m operands (the correction's FP32 blocks fit in those); the FP32 iterations' three
+  const size_t sm = std::max(sizeof(double2) * (m * m + std::max(2 * m * m, (m * m + 3 * m * own + 1) / 2)),
+                             sizeof(float2) * 3 * m * (NT > 512 ? 65 : 33));
+  if (sm > set) {
+    cudaFuncSetAttribute(k_eig_t<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    set = sm;
   }
-  note_launch();
-  k_svd_sort<<<D.nprob, 256, 0, s>>>(D, v);
-  // U_Q = Q V_Q Sigma^{-1} (a x b)
-  ZG uq = zg(L.q, LM, 0, L.vq, LM, 0, L.uq, LM, ZD_A, ZD_B, ZD_B, ZL_SVD);
-  uq.colscale = L.sigma;
-  launch_zgemm(D, uq, s);
-  // P_l = U_Q^* M_l (b x b, into work1 + l (work2 - work1)); S_l = P_l V_Q Sigma^{-1}
-  ZG pl = zg(L.uq, LM, 1, L.mproj, LM, 0, L.work1, LM, ZD_B, ZD_B, ZD_A, ZL_SVD);
-  pl.nl = D.maxD;
-  pl.lb = 16LL * L.LDR * L.LDM;
-  pl.lc = L.work2 - L.work1;
-  launch_zgemm(D, pl, s);
-  ZG sl = zg(L.work1, LM, 0, L.vq, LM, 0, L.S, LM, ZD_B, ZD_B, ZD_B, ZL_SVD);
-  sl.nl = D.maxD;
-  sl.la = L.work2 - L.work1;
-  sl.lc = 16LL * L.LDM * L.LDM;
-  sl.colscale = L.sigma;
-  launch_zgemm(D, sl, s);
+  launch_cluster(k_eig_t<CL, NT>, CL, NT, sm, D.nprob, s, D, mu);
+}
+}  // namespace
+
+// The widest cluster whose CTAs are all resident at once (two per SM): a problem's FP32 iterations run on one
+// CTA, so a second wave of problems would wait for whole iterations of the first.
+static int cluster_of(const Dev& D) {
+  const int m = D.L.LDM, fit = 2 * 152 / std::max(1, D.nprob);
+  const int want = m > 32 ? 8 : m > 8 ? 4 : 1;
+  return want >= 8 && fit >= 8 ? 8 : want >= 4 && fit >= 4 ? 4 : want >= 4 && fit >= 2 ? 2 : 1;
+}
+
+void launch_svd_S(const Dev& D, cudaStream_t s) {
+  const int cl = cluster_of(D);
+  if (D.L.LDM > 32) {
+    if (cl == 8) run_svd<8, 640>(D, s);
+    else if (cl == 4) run_svd<4, 640>(D, s);
+    else if (cl == 2) run_svd<2, 640>(D, s);
+    else run_svd<1, 640>(D, s);
+  } else if (D.L.LDM > 16) {
+    if (cl == 4) run_svd<4, 512>(D, s);
+    else if (cl == 2) run_svd<2, 512>(D, s);
+    else run_svd<1, 512>(D, s);
+  } else {
+    if (cl == 4) run_svd<4, 128>(D, s);
+    else if (cl == 2) run_svd<2, 128>(D, s);
+    else run_svd<1, 128>(D, s);
+  }
 }
 
 void launch_canon(const Dev& D, cudaStream_t s) {
@@ -776,33 +1093,32 @@ void launch_canon(const Dev& D, cudaStream_t s) {
 }
 
 void launch_eig_t(const Dev& D, unsigned long long seed, cudaStream_t s) {
-  static size_t set = 0;
-  const SmallLay& L = D.L;
-  const int LM = L.LDM;
-  size_t sm = sizeof(float2) * 3 * (size_t)D.maxM * D.maxM;
-  if (sm > set) {
-    cudaFuncSetAttribute(k_eig_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(sm, 1024));
-    set = sm;
+  double2 g[PRONY_DMAX];                         // complex normals (the draw convention of Philox above)
+  for (int l = 0; l < PRONY_DMAX; ++l) {
+    uint64_t c[4] = {(uint64_t)l, 0, 0, 0};
+    philox4x64(c, seed, PRONY_STREAM_MU);
+    const double r = std::sqrt(-std::log(philox_u01(c[0]))), u = 6.283185307179586 * philox_u01(c[1]);
+    g[l] = make_double2(r * std::cos(u), r * std::sin(u));
   }
-  note_launch();
-  k_eig_w<<<D.nprob, 256, std::max<size_t>(sm, 16), s>>>(D, seed);
-  // two Newton-Schulz steps X <- 2X - X (W X): W in work2, X in work3 -> work1 -> work3
-  long long x = L.work3, xn = L.work1;
-  for (int it = 0; it < 2; ++it) {
-    launch_zgemm(D, zg(L.work2, LM, 0, x, LM, 0, L.work4, LM, ZD_B, ZD_B, ZD_B, ZL_EIG), s);   // R = W X
-    ZG ns = zg(x, LM, 0, L.work4, LM, 0, xn, LM, ZD_B, ZD_B, ZD_B, ZL_EIG);                  // 2X - X R
-    ns.alpha = -1.0;
-    ns.c0 = x;
-    ns.beta = 2.0;
-    launch_zgemm(D, ns, s);
-    std::swap(x, xn);
+  MuTable mu = {};
+  double nrm = 0.0;
+  for (int d = 1; d <= PRONY_DMAX; ++d) {
+    nrm += cabs2(g[d - 1]);
+    for (int l = 0; l < d; ++l) mu.v[d - 1][l] = cscale(g[l], 1.0 / std::sqrt(nrm));
   }
-  // C_l = S_l W into the mproj slices, then z and t
-  ZG cl = zg(L.S, LM, 0, L.work2, LM, 0, L.mproj, LM, ZD_B, ZD_B, ZD_B, ZL_EIG);
-  cl.nl = D.maxD;
-  cl.la = 16LL * L.LDM * L.LDM;
-  cl.lc = 16LL * L.LDR * L.LDM;
-  launch_zgemm(D, cl, s);
-  note_launch();
-  k_eig_z<<<D.nprob, 128, 0, s>>>(D);
+  const int cl = cluster_of(D);
+  if (D.L.LDM > 32) {
+    if (cl == 8) run_eig<8, 640>(D, mu, s);
+    else if (cl == 4) run_eig<4, 640>(D, mu, s);
+    else if (cl == 2) run_eig<2, 640>(D, mu, s);
+    else run_eig<1, 640>(D, mu, s);
+  } else if (D.L.LDM > 16) {
+    if (cl == 4) run_eig<4, 512>(D, mu, s);
+    else if (cl == 2) run_eig<2, 512>(D, mu, s);
+    else run_eig<1, 512>(D, mu, s);
+  } else {
+    if (cl == 4) run_eig<4, 128>(D, mu, s);
+    else if (cl == 2) run_eig<2, 128>(D, mu, s);
+    else run_eig<1, 128>(D, mu, s);
+  }
 }

@@ -1089,7 +1089,7 @@ cudaError_t launch_eval_points(const double* t, const double2* c, int m, int d, 
     return cudaGetLastError();
   }
   const size_t sm = eval_table_bytes(m);
-  static size_t set = 48 * 1024;
+  static size_t set = 0;
   if (sm > set) {
     const cudaError_t e = cudaFuncSetAttribute(k_eval_many, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;

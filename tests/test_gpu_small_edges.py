@@ -1,0 +1,57 @@
+"""The clustered small steps at the edges of their sizes: block widths at which the number of CTAs, threads
+and column groups change, U wider than V, and batches large enough for the narrower clusters."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2012_11430_gb300 import Context
+    with Context(0) as c:
+        yield c
+
+
+@pytest.mark.parametrize("d,m,a", [(1, 1, 1), (2, 2, 5), (1, 8, 8), (3, 9, 16), (2, 16, 128), (2, 17, 17), (4, 32, 33),
+                                   (2, 33, 64), (3, 63, 65), (4, 64, 128)])
+def test_small_steps_sizes(ctx, d, m, a):
+    """Q = U_0 diag(sigma) V_0^* and M_l = Q V_0 S_l V_0^* with S_l = W diag(z(l)) W^{-1}: sigma to FP64 rounding,
+    z and t to the second order of the FP32 eigenvectors (1e-11; kappa(W) is below 20 here)."""
+    rng = np.random.Generator(np.random.PCG64(500 + 10 * m + d))
+    gauss = lambda *s: rng.standard_normal(s) + 1j * rng.standard_normal(s)  # noqa: E731
+    U0 = np.linalg.qr(gauss(a, m))[0]
+    V0 = np.linalg.qr(gauss(m, m))[0]
+    sigma = np.sort(1.0 + 4.0 * rng.random(m))[::-1]
+    Wm = np.linalg.qr(gauss(m, m))[0] + 0.3 * gauss(m, m) / np.sqrt(m)
+    t = np.stack([(rng.permutation(m) + 0.5 + 0.2 * rng.uniform(-1, 1, m)) / m for _ in range(d)], 1)
+    S = [Wm @ np.diag(np.exp(-2j * np.pi * t[:, l])) @ np.linalg.inv(Wm) for l in range(d)]
+    Q = U0 @ np.diag(sigma) @ V0.conj().T
+    # U^* T_l V = U_0 (S_l Sigma) V_0^* for the singular pairs (U_0, V_0)
+    M = np.array([U0 @ S[l] @ np.diag(sigma) @ V0.conj().T for l in range(d)])
+    sig, Sg, z, tg, status = ctx.small_steps(Q, M)
+    assert status == 0
+    assert np.max(np.abs(sig - sigma) / sigma) <= 64 * 2.0 ** -53 * m
+    o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
+    assert np.max(np.abs(z[og] - np.exp(-2j * np.pi * t[o]))) <= 1e-11
+    assert np.max(W.torus_dist(tg[og], t[o])) <= 2e-12
+    for l in range(d):                                 # S_l up to the phases of the singular vectors
+        assert np.max(np.abs(np.abs(Sg[l]) - np.abs(S[l]))) <= 1e-9
+
+
+@pytest.mark.parametrize("count,n,m", [(60, 15, 36), (100, 15, 36), (310, 13, 34), (100, 11, 18), (310, 11, 18), (100, 9, 12)])
+def test_batches_of_every_cluster_width(ctx, count, n, m):
+    """Noise-free problems in batches for which a problem gets four, two or one CTAs."""
+    probs = [W.make_problem(f"cw{i}", 2, n, m, 7000 + i) for i in range(5)]
+    idx = [i % 5 for i in range(count)]
+    outs, rc = ctx.solve_batched([probs[i].grid for i in idx], [2] * count, [n] * count, [m] * count)
+    assert rc == 0
+    for k, i in enumerate(idx):
+        te, ce = W.match_to_truth(outs[k].t, outs[k].c, probs[i].t, probs[i].c)
+        assert te <= 1e-6 and ce <= 1e-5, (k, te, ce)
+        assert np.array_equal(outs[k].t, outs[i].t) and np.array_equal(outs[k].c, outs[i].c)
