@@ -53,6 +53,12 @@ class PronyInfo(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+def _info_dicts(infos) -> list:
+    """The dicts of PronyInfo.as_dict for an array of them, in one pass over its memory."""
+    names = [k for k, _ in PronyInfo._fields_]
+    return [dict(zip(names, row)) for row in np.ctypeslib.as_array(infos).tolist()]
+
+
 class PronyError(RuntimeError):
     def __init__(self, code: int, what: str):
         super().__init__(f"{what}: status {code} ({status_string(code)}) {last_error()}")
@@ -262,11 +268,11 @@ class Context:
                                            ctypes.byref(opts) if opts else None)
         if rc in (PRONY_EINVAL, PRONY_ECUDA, PRONY_ENOMEM):
             raise PronyError(rc, "prony_solve_batched")
-        out = []
+        out, dicts = [], _info_dicts(infos)
         for i in range(P):
             d, m, o = int(ds[i]), int(ms[i]), int(ooff[i])
             out.append(SolveResult(t[o * dmax:(o + m) * dmax].reshape(m, dmax)[:, :d].copy(), c[o:o + m].copy(),
-                                   infos[i].as_dict()))
+                                   dicts[i]))
         return out, rc
 
     # ---------------------------------------------------------------- device-pointer calls (torch tensors)
@@ -288,7 +294,7 @@ class Context:
                                            ctypes.byref(opts) if opts else None)
         if rc in (PRONY_EINVAL, PRONY_ECUDA, PRONY_ENOMEM):
             raise PronyError(rc, "prony_solve_batched")
-        return [i.as_dict() for i in infos], rc
+        return _info_dicts(infos), rc
 
     def solve_batched_dev(self, samples_dev, ds, ns, ms, soff, ooff, t_out_dev, c_out_dev,
                           opts: PronyOpts | None = None, stream: int = 0):
@@ -306,7 +312,7 @@ class Context:
                                                ctypes.byref(opts) if opts else None, ctypes.c_void_p(stream))
         if rc in (PRONY_EINVAL, PRONY_ECUDA, PRONY_ENOMEM):
             raise PronyError(rc, "prony_solve_batched_dev")
-        return [infos[i].as_dict() for i in range(P)], rc
+        return _info_dicts(infos), rc
 
     def expsum_fwd_dev(self, t_dev, c_dev, lo, length, f_dev, stream: int = 0):
         m, d = t_dev.shape

@@ -78,8 +78,12 @@ struct prony_ctx {
   // products by axis transform: sub-problem descriptors, twiddles, transformed blocks and samples
   DBuf axP, axtw, axX, axY, axF, axH;
   std::vector<int> ax_sig;              // (n, d, m, r0) of every problem axP was built for
-  int* h_flag = nullptr;            // pinned
-  std::vector<ProbState> h_st;
+  int* h_flag = nullptr;            // pinned: loop flag, body counters, error flags (see queue_flags)
+  void* pin = nullptr;              // pinned staging of a call's results, grown on demand
+  size_t pin_cap = 0;
+  cudaEvent_t order = nullptr;      // orders the context stream after a caller's stream
+  std::vector<ProbDesc> lastP;      // what the device descriptors hold (empty: unknown)
+  const ProbState* h_st = nullptr;  // states of the last call, in `pin`
   // profiling of the Toeplitz launches
   bool prof = false;
   struct TRec { int ev; int iter; int ext; int wsel; };
@@ -101,6 +105,7 @@ struct prony_ctx {
     cudaGraphExec_t exec = nullptr;
     long long fixed_launches = 0, body_launches[2] = {0, 0};
     bool has_loop[2] = {false, false};
+    bool pending = false;             // a replay whose launches are not counted yet
   } solve_graph;
 };
 
@@ -226,6 +231,36 @@ int max_window(const ProbDesc& p, int L, int nks, bool bf16) {
     }
   }
   return mx;
+}
+
+// Problem descriptors to the device, unless it holds these already (a repeated batch layout).
+int upload_problems(prony_ctx* ctx, const std::vector<ProbDesc>& P) {
+  const size_t bytes = sizeof(ProbDesc) * P.size();
+  if (ctx->lastP.size() == P.size() && std::memcmp(ctx->lastP.data(), P.data(), bytes) == 0) return PRONY_OK;
+  ctx->lastP.clear();
+  CK(cudaMemcpyAsync(ctx->P.p, P.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
+  ctx->lastP = P;
+  return PRONY_OK;
+}
+
+// The context stream waits for the work queued on a caller's stream so far.
+int wait_for(prony_ctx* ctx, cudaStream_t user) {
+  if (!user) return PRONY_OK;
+  CK(cudaEventRecord(ctx->order, user));
+  CK(cudaStreamWaitEvent(ctx->stream, ctx->order, 0));
+  return PRONY_OK;
+}
+
+int ensure_pinned(prony_ctx* ctx, size_t bytes) {
+  if (ctx->pin_cap >= bytes) return PRONY_OK;
+  if (ctx->pin) cudaFreeHost(ctx->pin);
+  ctx->pin = nullptr;
+  ctx->pin_cap = 0;
+  const size_t want = bytes + bytes / 4;
+  const cudaError_t e = cudaMallocHost(&ctx->pin, want);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
+  ctx->pin_cap = want;
+  return PRONY_OK;
 }
 
 // Split K workspace for `njobs` jobs of `slot_bytes` each: partial tiles and zeroed arrival
@@ -467,14 +502,16 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
                                      B.P.size() * (size_t)std::max(T.gram ? T.gram_stride : 0LL,
                                                                    T.apply ? T.apply_stride : 0LL)))))
     return rc;
-  if ((rc = ensure(ctx->tcerr, 256))) return rc;
-  CK(cudaMemsetAsync(ctx->tcerr.p, 0, sizeof(int), ctx->stream));
+  // (zeroed when allocated and after an error)
+  if (!ctx->tcerr.p) {
+    if ((rc = ensure(ctx->tcerr, 256))) return rc;
+    CK(cudaMemsetAsync(ctx->tcerr.p, 0, sizeof(int), ctx->stream));
+  }
   T.err = (int*)ctx->tcerr.p;
   return tc_set_jobs(ctx, B, nks0);
 }
 
 // One Toeplitz block product for every live problem of the batch.
-int check_tc_error(prony_ctx* ctx, const Batch& B);
 
 // The Gram X^* Z of two tall blocks (N rows) for every live problem: out (FP64, small workspace at
 // out_off, leading dimension out_ld) = sum over the rows r in I_n of conj(X[r, a]) Z[r, b]; on the
@@ -618,7 +655,6 @@ int setup_fft(prony_ctx* ctx, Batch& B) {
   int rc;
   if ((rc = ensure(ctx->fhat, sizeof(float2) * foff))) return rc;
   if ((rc = ensure(ctx->ftw, sizeof(float2) * LT))) return rc;
-  CK(cudaMemcpyAsync(ctx->P.p, B.P.data(), sizeof(ProbDesc) * B.P.size(), cudaMemcpyHostToDevice, ctx->stream));
   B.D.fhat = (float2*)ctx->fhat.p;
   B.D.ftw = (float2*)ctx->ftw.p;
   B.D.fLT = LT;
@@ -787,7 +823,7 @@ int setup_products(prony_ctx* ctx, Batch& B, int prec) {
 
 // Lay out a batch in the context workspace.  Grid samples are copied from `src`
 // (host or device, per problem sample_off) into the packed grid64 buffer.
-int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opts& o, Batch& B) {
+int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opts& o, Batch& B, bool product_only = false) {
   const int np = (int)hp.size();
   B.P.resize(np);
   long long goff = 0, xoff = 0, yoff = 0, toff = 0;
@@ -846,11 +882,14 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   if ((rc = ensure(ctx->B2, sizeof(float2) * xoff))) return rc;
   if ((rc = ensure(ctx->Y, sizeof(float2) * yoff))) return rc;
   if ((rc = ensure(ctx->small, (size_t)L.bytes * np))) return rc;
-  if ((rc = ensure(ctx->P, sizeof(ProbDesc) * np))) return rc;
+  {
+    const size_t cap = ctx->P.cap;
+    if ((rc = ensure(ctx->P, sizeof(ProbDesc) * np))) return rc;
+    if (ctx->P.cap != cap) ctx->lastP.clear();
+  }
   if ((rc = ensure(ctx->st, sizeof(ProbState) * np))) return rc;
   if ((rc = ensure(ctx->flag, 256))) return rc;
-  CK(cudaMemcpyAsync(ctx->P.p, B.P.data(), sizeof(ProbDesc) * np, cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaMemsetAsync(ctx->small.p, 0, (size_t)L.bytes * np, ctx->stream));
+  if (!product_only) CK(cudaMemsetAsync(ctx->small.p, 0, (size_t)L.bytes * np, ctx->stream));
   Dev& D = B.D;
   D.P = (const ProbDesc*)ctx->P.p;
   D.st = (ProbState*)ctx->st.p;
@@ -889,7 +928,10 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   D.red = (char*)ctx->red.p;
   D.rcnt = (int*)ctx->rcnt.p;
   D.oob = (int*)ctx->oob.p;
-  if (o.precision == PRONY_FFT32) return setup_fft(ctx, B);
+  if (o.precision == PRONY_FFT32) {
+    if ((rc = setup_fft(ctx, B))) return rc;
+    return upload_problems(ctx, B.P);
+  }
   // a batch whose transformed blocks do not fit the device keeps the direct products
   if (axis_pays(B.P, o.precision)) {
     rc = setup_axis(ctx, B, o.precision);
@@ -908,7 +950,7 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
     B.fft.on = false;
     B.fft.lz = true;
   }
-  return PRONY_OK;
+  return upload_problems(ctx, B.P);
 }
 
 // CholeskyQR2 of the tall block in `xbuf` (width selector xw) into `outbuf`, through B1.
@@ -1080,18 +1122,24 @@ int build_solve_graph(prony_ctx* ctx, const std::vector<Seg>& segs, int* dflag, 
   return PRONY_OK;
 }
 
-// One replay of the solve graph; the launch statistics count its bodies as they ran.
+// One replay of the solve graph; its launches are counted once its body counters are on the host
+// (count_graph_launches, after the call's synchronisation).
 int launch_solve_graph(prony_ctx* ctx) {
   auto& G = ctx->solve_graph;
   cudaStream_t s = ctx->stream;
   CK(cudaGraphLaunch(G.exec, s));
   CK(cudaMemcpyAsync(ctx->h_flag + 1, (int*)ctx->flag.p + 1, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  G.pending = true;
+  return PRONY_OK;
+}
+void count_graph_launches(prony_ctx* ctx) {
+  auto& G = ctx->solve_graph;
+  if (!G.pending) return;
+  G.pending = false;
   long long n = G.fixed_launches;
   for (int k = 0; k < 2; ++k)
     if (G.has_loop[k]) n += (long long)ctx->h_flag[1 + k] * G.body_launches[k];
   note_launches(n);
-  return PRONY_OK;
 }
 
 int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
@@ -1239,7 +1287,7 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
     }
     if ((rc = launch_solve_graph(ctx))) return rc;
     CK(cudaGetLastError());
-    return check_tc_error(ctx, B);
+    return PRONY_OK;
   }
   prefix();
   if (lanczos) {
@@ -1311,14 +1359,12 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
   }
   finish();
   CK(cudaGetLastError());
-  return check_tc_error(ctx, B);
+  return PRONY_OK;
 }
 
-int read_states(prony_ctx* ctx, const Batch& B, prony_info* infos, int* worst) {
+// Per-problem outcomes from the states on the host (queue_results, after the synchronisation).
+void read_states(prony_ctx* ctx, const Batch& B, prony_info* infos, int* worst) {
   const int np = B.D.nprob;
-  ctx->h_st.resize(np);
-  CK(cudaMemcpyAsync(ctx->h_st.data(), B.D.st, sizeof(ProbState) * np, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
   int w = PRONY_OK;
   for (int i = 0; i < np; ++i) {
     const ProbState& s = ctx->h_st[i];
@@ -1337,7 +1383,6 @@ int read_states(prony_ctx* ctx, const Batch& B, prony_info* infos, int* worst) {
     if (s.status != PRONY_OK && (w == PRONY_OK || s.status < w)) w = s.status;
   }
   *worst = w;
-  return PRONY_OK;
 }
 
 prony_opts resolve_opts(const prony_opts* o) {
@@ -1351,14 +1396,34 @@ int check_precision(int prec) {
   return (prec == PRONY_FP32 || prec == PRONY_FFT32 || is_tc(prec)) ? PRONY_OK : PRONY_EINVAL;
 }
 
-// Error flags of the kernels: a failed workspace bound check (any kernel; the access was skipped,
+// Error flags of the kernels to pinned host memory (with the next synchronisation).
+int queue_flags(prony_ctx* ctx, const Batch& B) {
+  ctx->h_flag[3] = ctx->h_flag[4] = 0;
+  CK(cudaMemcpyAsync(ctx->h_flag + 3, ctx->oob.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  if (B.tc.on) CK(cudaMemcpyAsync(ctx->h_flag + 4, B.tc.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  return PRONY_OK;
+}
+
+// States, error flags and (copy_out) packed results of a solve: queued behind its kernels and
+// waited for once.  Layout of `pin`: states, then t, then c.
+int queue_results(prony_ctx* ctx, const Batch& B, const double* tdev, const double2* cdev, long long t_count, long long c_count) {
+  const size_t sb = (sizeof(ProbState) * B.D.nprob + 15) / 16 * 16, tb = (sizeof(double) * (size_t)t_count + 15) / 16 * 16;
+  int rc;
+  if ((rc = ensure_pinned(ctx, sb + tb + sizeof(double2) * (size_t)c_count))) return rc;
+  char* h = (char*)ctx->pin;
+  ctx->h_st = (const ProbState*)h;
+  CK(cudaMemcpyAsync(h, B.D.st, sizeof(ProbState) * B.D.nprob, cudaMemcpyDeviceToHost, ctx->stream));
+  if (t_count) CK(cudaMemcpyAsync(h + sb, tdev, sizeof(double) * t_count, cudaMemcpyDeviceToHost, ctx->stream));
+  if (c_count) CK(cudaMemcpyAsync(h + sb + tb, cdev, sizeof(double2) * c_count, cudaMemcpyDeviceToHost, ctx->stream));
+  return queue_flags(ctx, B);
+}
+
+// After the synchronisation: a failed workspace bound check (any kernel; the access was skipped,
 // the split-K and cross-block counters are cleared for the next call) and the tensor-core kernels'
 // bounded waits or window overflow.
-int check_tc_error(prony_ctx* ctx, const Batch& B) {
-  int oob = 0;
-  CK(cudaMemcpyAsync(&oob, ctx->oob.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
-  if (oob) {
+int check_flags(prony_ctx* ctx) {
+  count_graph_launches(ctx);
+  if (const int oob = ctx->h_flag[3]) {
     CK(cudaMemsetAsync(ctx->oob.p, 0, sizeof(int), ctx->stream));
     if (ctx->cnt.p) CK(cudaMemsetAsync(ctx->cnt.p, 0, ctx->cnt.cap, ctx->stream));
     if (ctx->rcnt.p) CK(cudaMemsetAsync(ctx->rcnt.p, 0, ctx->rcnt.cap, ctx->stream));
@@ -1372,11 +1437,9 @@ int check_tc_error(prony_ctx* ctx, const Batch& B) {
     g_err = std::string("Toeplitz product launch: ") + cudaGetErrorString(e);
     return PRONY_ECUDA;
   }
-  if (!B.tc.on) return PRONY_OK;
-  int h = 0;
-  CK(cudaMemcpyAsync(&h, B.tc.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
-  if (h) {
+  if (const int h = ctx->h_flag[4]) {
+    CK(cudaMemsetAsync(ctx->tcerr.p, 0, sizeof(int), ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     g_err = "tensor-core Toeplitz kernel reported error " + std::to_string(h);
     return PRONY_ECUDA;
   }
@@ -1445,11 +1508,20 @@ int prony_ctx_create(prony_ctx** out, int device) {
   c->device = device;
   e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
   if (e != cudaSuccess) { delete c; return cuda_fail(e, "cudaStreamCreate"); }
+  e = cudaEventCreateWithFlags(&c->order, cudaEventDisableTiming);
+  if (e != cudaSuccess) { cudaStreamDestroy(c->stream); delete c; return cuda_fail(e, "cudaEventCreate"); }
   e = cudaMallocHost(&c->h_flag, 256);
-  if (e != cudaSuccess) { cudaStreamDestroy(c->stream); delete c; return cuda_fail(e, "cudaMallocHost"); }
+  if (e != cudaSuccess) {
+    cudaEventDestroy(c->order);
+    cudaStreamDestroy(c->stream);
+    delete c;
+    return cuda_fail(e, "cudaMallocHost");
+  }
+  std::memset(c->h_flag, 0, 256);
   if (ensure(c->oob, 256) != PRONY_OK || cudaMemsetAsync(c->oob.p, 0, 256, c->stream) != cudaSuccess) {
     if (c->oob.p) cudaFree(c->oob.p);
     cudaFreeHost(c->h_flag);
+    cudaEventDestroy(c->order);
     cudaStreamDestroy(c->stream);
     delete c;
     return PRONY_ENOMEM;
@@ -1470,6 +1542,8 @@ int prony_ctx_destroy(prony_ctx* c) {
   for (DBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   if (c->h_flag) cudaFreeHost(c->h_flag);
+  if (c->pin) cudaFreeHost(c->pin);
+  cudaEventDestroy(c->order);
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
   cudaStreamDestroy(c->stream);
   delete c;
@@ -1507,16 +1581,10 @@ static int solve_batched_impl(prony_ctx* ctx, int P, const int* d, const int* n,
     if (validate(hp[i])) return PRONY_EINVAL;
     total_terms = std::max(total_terms, out_off[i] + m[i]);
   }
-  if (user_stream) {
-    cudaEvent_t ev;
-    CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    CK(cudaEventRecord(ev, user_stream));
-    CK(cudaStreamWaitEvent(ctx->stream, ev, 0));
-    cudaEventDestroy(ev);
-  }
-  Batch B;
-  int rc = setup_batch(ctx, hp, o, B);
+  int rc = wait_for(ctx, user_stream);
   if (rc) return rc;
+  Batch B;
+  if ((rc = setup_batch(ctx, hp, o, B))) return rc;
   if ((rc = load_grids(ctx, B, hp, samples, dev_samples))) return rc;
   RunOut ro;
   if ((rc = run_batch(ctx, B, o, ro))) return rc;
@@ -1531,25 +1599,23 @@ static int solve_batched_impl(prony_ctx* ctx, int P, const int* d, const int* n,
   }
   launch_gather_out(B.D, tdev, cdev, ctx->stream);
   CK(cudaGetLastError());
+  const long long tc = dev_out ? 0 : total_terms * maxd, cc = dev_out ? 0 : total_terms;
+  if ((rc = queue_results(ctx, B, tdev, cdev, tc, cc))) return rc;
+  CK(cudaStreamSynchronize(ctx->stream));
+  if ((rc = check_flags(ctx))) return rc;
   int worst = PRONY_OK;
-  if ((rc = read_states(ctx, B, infos, &worst))) return rc;
+  read_states(ctx, B, infos, &worst);
   if (!dev_out) {
     // rows of maxd entries; a problem writes its first d of each row only
-    std::vector<double> th(total_terms * maxd);
-    std::vector<double2> ch(total_terms);
-    CK(cudaMemcpy(th.data(), tdev, sizeof(double) * total_terms * maxd, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(ch.data(), cdev, sizeof(double2) * total_terms, cudaMemcpyDeviceToHost));
+    const char* h = (const char*)ctx->pin + (sizeof(ProbState) * P + 15) / 16 * 16;
+    const double* th = (const double*)h;
+    const double2* ch = (const double2*)(h + (sizeof(double) * (size_t)tc + 15) / 16 * 16);
     for (int i = 0; i < P; ++i) {
       for (int j = 0; j < m[i]; ++j)
-        std::memcpy(t_out + (out_off[i] + j) * maxd, th.data() + (out_off[i] + j) * maxd, sizeof(double) * d[i]);
-      std::memcpy(c_out + out_off[i], ch.data() + out_off[i], sizeof(double2) * m[i]);
+        std::memcpy(t_out + (out_off[i] + j) * maxd, th + (out_off[i] + j) * maxd, sizeof(double) * d[i]);
+      std::memcpy(c_out + out_off[i], ch + out_off[i], sizeof(double2) * m[i]);
     }
   } else if (user_stream) {
-    cudaEvent_t ev;
-    CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    CK(cudaEventRecord(ev, ctx->stream));
-    CK(cudaStreamWaitEvent(user_stream, ev, 0));
-    cudaEventDestroy(ev);
     CK(cudaStreamSynchronize(user_stream));
   }
   return worst;
@@ -1609,8 +1675,11 @@ int prony_build_S(prony_ctx* ctx, const prony_c128* samples, int d, int n, int m
       CK(cudaMemcpyAsync(V_out, ctx->misc.p, sizeof(double2) * N * m, cudaMemcpyDeviceToHost, ctx->stream));
     }
   }
+  if ((rc = queue_results(ctx, B, nullptr, nullptr, 0, 0))) return rc;
+  CK(cudaStreamSynchronize(ctx->stream));
+  if ((rc = check_flags(ctx))) return rc;
   int worst = PRONY_OK;
-  if ((rc = read_states(ctx, B, info, &worst))) return rc;
+  read_states(ctx, B, info, &worst);
   const int w = ctx->h_st[0].wv;
   const double2* S = (const double2*)(small.data() + L.S);
   const double* sg = (const double*)(small.data() + L.sigma);
@@ -1649,6 +1718,7 @@ int prony_small_steps(prony_ctx* ctx, int d, int m, int a, const prony_c128* Q, 
   int rc;
   if ((rc = ensure(ctx->small, (size_t)L.bytes))) return rc;
   if ((rc = ensure(ctx->P, sizeof(ProbDesc)))) return rc;
+  ctx->lastP.clear();
   if ((rc = ensure(ctx->st, sizeof(ProbState)))) return rc;
   CK(cudaMemsetAsync(ctx->small.p, 0, (size_t)L.bytes, s));
   CK(cudaMemcpyAsync(ctx->P.p, &pd, sizeof(ProbDesc), cudaMemcpyHostToDevice, s));
@@ -1794,7 +1864,6 @@ int prony_toeplitz_mm_dev(prony_ctx* ctx, const prony_c128* grid_dev, int d, int
   if (adjoint && L != n + 1) return PRONY_EINVAL;
   if (check_precision(precision)) return PRONY_EINVAL;
   CK(cudaSetDevice(ctx->device));
-  cudaStream_t s = stream ? (cudaStream_t)stream : ctx->stream;
   std::vector<HostProb> hp = {{d, n, 1, 0, 0}};
   if (std::pow((double)(n + 1), d) > 2.0e8 || r > (long long)ipow(n + 1, d)) return PRONY_EINVAL;
   prony_opts o;
@@ -1802,18 +1871,9 @@ int prony_toeplitz_mm_dev(prony_ctx* ctx, const prony_c128* grid_dev, int d, int
   o.oversample_p = r - 1;
   o.precision = precision;
   Batch B;
-  // ensure the stream order: ctx work after the caller's stream
-  if (stream) {
-    cudaEvent_t ev;
-    CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    CK(cudaEventRecord(ev, s));
-    CK(cudaStreamWaitEvent(ctx->stream, ev, 0));
-    cudaEventDestroy(ev);
-  }
-  int rc = setup_batch(ctx, hp, o, B);
+  int rc = wait_for(ctx, (cudaStream_t)stream);
+  if (!rc) rc = setup_batch(ctx, hp, o, B, true);
   if (rc) return rc;
-  B.P[0].r0 = r;
-  CK(cudaMemcpyAsync(ctx->P.p, B.P.data(), sizeof(ProbDesc), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->grid64.p, grid_dev, sizeof(double2) * B.P[0].Gd, cudaMemcpyDeviceToDevice, ctx->stream));
   launch_prep(B.D, false, ctx->stream);
   product_tables(ctx, B, precision, L == n + 1, ctx->stream);
@@ -1826,8 +1886,9 @@ int prony_toeplitz_mm_dev(prony_ctx* ctx, const prony_c128* grid_dev, int d, int
   const int y_ext = (L == n + 2);
   toeplitz_product(ctx, B, D, y_ext, BUF_V, W_R0, y_ext ? BUF_Y : BUF_B2, precision, ctx->stream, adjoint);
   CK(cudaGetLastError());
+  if ((rc = queue_flags(ctx, B))) return rc;
   CK(cudaStreamSynchronize(ctx->stream));
-  return check_tc_error(ctx, B);
+  return check_flags(ctx);
 }
 
 }  // extern "C"
