@@ -16,7 +16,8 @@
 // among l, l').  A CTA computes the sums of one pair (a >= b) directly, sum_l len_l terms in place of
 // prod_l len_l, and its (d + 2)^2 entries of J^* J; the rest of the pass is the residual and V, m (d + 1) sums over the points.
 // The exponentials are recomputed in every pass, never stored; phases <t_j, k> mod 1 are exact
-// 64-bit fixed-point sums, the sums FP32 over at most 128 terms, the accumulators FP64.
+// 64-bit fixed-point sums, the sums FP32 over at most 128 terms, then FP64 over the tiles of a CTA and twice FP32
+// (error-free sums) over the CTAs' FP32 results, in a fixed order: a refinement is reproducible.
 // Near the minimum the decision compares losses that differ by less than FP32 rounding of the model
 // would leave, so the model is evaluated beyond FP32: exp(-2 pi i u) = T[round(32 u)] (1 + eps)
 // with |eps| < 0.1, the sum of c_j T in twice FP32 (error-free sums) from a table of the CTA, the sum of
@@ -32,6 +33,7 @@ namespace {
 
 constexpr int LM_TILE = 128;            // points per CTA (= threads) in the point pass
 constexpr int LM_SEG_BITS = 5, LM_SEG = 1 << LM_SEG_BITS;   // table points of the unit circle
+constexpr int LM_MAXCTA = 304;          // point CTAs at most (two per SM)
 constexpr int LM_EP = LM_TILE + 1;      // pitch of the exponentials (threads of different terms: different banks)
 constexpr int LM_NB = 16;               // column block of the Cholesky factorisation
 constexpr int LM_SOLVE_THREADS = 512;
@@ -93,10 +95,12 @@ __device__ inline double block_sum(double v, double* red) {
   return s;
 }
 
-// Blocks [0, npt_blocks): 128 points each.  The others: a pair (a >= b) each.
+// Blocks [0, npt_blocks): tiles of 128 points.  The others: a pair (a >= b) each.  vs: V[d+1][m]
+// of every point block, ls: its loss.
 __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const double2* c, int m, int d, Box B,
                                                        long long K, int npt_blocks, const float2* y,
-                                                       const LmState* st, const float4* circle, double* sets) {
+                                                       const LmState* st, const float4* circle, double* sets,
+                                                       float2* vs, double* ls) {
   extern __shared__ float4 lm_smem[];
   __shared__ uint64_t T[PRONY_MMAX * PRONY_DMAX];
   __shared__ float2 Tf[LM_SEG];
@@ -179,76 +183,85 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
   }
   __syncthreads();
   const int i = threadIdx.x;
-  const long long q = blockIdx.x * (long long)LM_TILE + i;
-  double2 rd = make_double2(0.0, 0.0);
-  int k[PRONY_DMAX] = {0, 0, 0, 0};
-  if (q < K) {
-    if (K <= 0xFFFFFFFFLL) {
-      unsigned rem = (unsigned)q;
-      for (int l = d - 1; l >= 0; --l) {
-        const unsigned len = (unsigned)B.len[l], nx = rem / len;
-        k[l] = B.lo[l] + (int)(rem - nx * len);
-        rem = nx;
-      }
-    } else {
-      box_point(B, d, q, k);
-    }
-    float2 fh = make_float2(0.f, 0.f), fe = fh;           // sum of c T, and of its remainders and c T eps
-    for (int j = 0; j < m; ++j) {
-      uint64_t ph = 0;
-      for (int l = 0; l < d; ++l) ph += T[j * d + l] * (uint64_t)(long long)k[l];
-      const int seg = (int)((ph + (1ull << (63 - LM_SEG_BITS))) >> (64 - LM_SEG_BITS));        // nearest table point
-      const int rem = (int)((long long)(ph - ((uint64_t)seg << (64 - LM_SEG_BITS))) >> 27);   // the rest in 2^-37 turns
-      const float x = (float)rem * 4.5716190e-11f, x2 = x * x;                                // 2 pi 2^-37; |x| <= pi / 32
-      // Taylor polynomials: the first terms left out are below 2e-11
-      const float sn = x * (1.f + x2 * (-1.f / 6.f + x2 * (1.f / 120.f)));
-      const float cm = x2 * (-0.5f + x2 * (1.f / 24.f - x2 * (1.f / 720.f)));                 // cos x - 1
-      const float4 ct = CT[j * LM_SEG + seg];
-      const float2 tf = Tf[seg];
-      fe.x += two_sum(fh.x, ct.x) + (ct.z + (ct.x * cm + ct.y * sn));     // c T (cm - i sn)
-      fe.y += two_sum(fh.y, ct.y) + (ct.w + (ct.y * cm - ct.x * sn));
-      E[j * LM_EP + i] = make_float2(tf.x + (tf.x * cm + tf.y * sn), tf.y + (tf.y * cm - tf.x * sn));
-    }
-    const float2 yk = y[q];
-    rd = make_double2((double)fh.x - (double)yk.x + (double)fe.x, (double)fh.y - (double)yk.y + (double)fe.y);
-  } else {
-    for (int j = 0; j < m; ++j) E[j * LM_EP + i] = make_float2(0.f, 0.f);
-  }
-  R[i] = make_float2((float)rd.x, (float)rd.y);
-  for (int l = 0; l < d; ++l) Wt[l * LM_TILE + i] = (float)k[l];
-  double* V = H + (long long)P * P;
-  const double l2 = block_sum(rd.x * rd.x + rd.y * rd.y, red);
-  if (i == 0) atomicAdd(&V[2 * (d + 1) * m], l2);
-  __syncthreads();
-  // V: one thread per (a, l) and slice of the points, the slices added in order
   const int nv = m * (d + 1), slices = max(1, LM_TILE / nv), per = LM_TILE / slices;
-  for (int base = 0; base < nv; base += LM_TILE) {
-    const int idx = slices > 1 ? i % nv : base + i, sl = slices > 1 ? i / nv : 0;
-    float2 acc = make_float2(0.f, 0.f);
-    if (idx < nv && sl < slices) {
-      const int a = idx % m, l = idx / m;
-      const int p1 = sl + 1 == slices ? LM_TILE : (sl + 1) * per;
-      for (int p = sl * per; p < p1; ++p) {
-        const float2 ea = E[a * LM_EP + p], rp = R[p];
-        const float w = l == 0 ? 1.f : Wt[(l - 1) * LM_TILE + p];
-        acc.x += w * (ea.x * rp.x + ea.y * rp.y);          // conj(ea) r
-        acc.y += w * (ea.x * rp.y - ea.y * rp.x);
+  double2 vsum[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};   // V entries i, i + 128 (nv <= 256)
+  double lsum = 0.0;
+  for (long long tile = blockIdx.x; tile * LM_TILE < K; tile += npt_blocks) {
+    const long long q = tile * LM_TILE + i;
+    double2 rd = make_double2(0.0, 0.0);
+    int k[PRONY_DMAX] = {0, 0, 0, 0};
+    if (q < K) {
+      if (K <= 0xFFFFFFFFLL) {
+        unsigned rem = (unsigned)q;
+        for (int l = d - 1; l >= 0; --l) {
+          const unsigned len = (unsigned)B.len[l], nx = rem / len;
+          k[l] = B.lo[l] + (int)(rem - nx * len);
+          rem = nx;
+        }
+      } else {
+        box_point(B, d, q, k);
+      }
+      float2 fh = make_float2(0.f, 0.f), fe = fh;           // sum of c T, and of its remainders and c T eps
+      for (int j = 0; j < m; ++j) {
+        uint64_t ph = 0;
+        for (int l = 0; l < d; ++l) ph += T[j * d + l] * (uint64_t)(long long)k[l];
+        const int seg = (int)((ph + (1ull << (63 - LM_SEG_BITS))) >> (64 - LM_SEG_BITS));        // nearest table point
+        const int rem = (int)((long long)(ph - ((uint64_t)seg << (64 - LM_SEG_BITS))) >> 27);   // the rest in 2^-37 turns
+        const float x = (float)rem * 4.5716190e-11f, x2 = x * x;                                // 2 pi 2^-37; |x| <= pi / 32
+        // Taylor polynomials: the first terms left out are below 2e-11
+        const float sn = x * (1.f + x2 * (-1.f / 6.f + x2 * (1.f / 120.f)));
+        const float cm = x2 * (-0.5f + x2 * (1.f / 24.f - x2 * (1.f / 720.f)));                 // cos x - 1
+        const float4 ct = CT[j * LM_SEG + seg];
+        const float2 tf = Tf[seg];
+        fe.x += two_sum(fh.x, ct.x) + (ct.z + (ct.x * cm + ct.y * sn));     // c T (cm - i sn)
+        fe.y += two_sum(fh.y, ct.y) + (ct.w + (ct.y * cm - ct.x * sn));
+        E[j * LM_EP + i] = make_float2(tf.x + (tf.x * cm + tf.y * sn), tf.y + (tf.y * cm - tf.x * sn));
+      }
+      const float2 yk = y[q];
+      rd = make_double2((double)fh.x - (double)yk.x + (double)fe.x, (double)fh.y - (double)yk.y + (double)fe.y);
+    } else {
+      for (int j = 0; j < m; ++j) E[j * LM_EP + i] = make_float2(0.f, 0.f);
+    }
+    R[i] = make_float2((float)rd.x, (float)rd.y);
+    for (int l = 0; l < d; ++l) Wt[l * LM_TILE + i] = (float)k[l];
+    lsum += block_sum(rd.x * rd.x + rd.y * rd.y, red);      // (thread 0)
+    __syncthreads();
+    // V: one thread per (a, l) and slice of the points, the slices added in order
+#pragma unroll
+    for (int base = 0; base < 2 * LM_TILE; base += LM_TILE) {
+      if (base >= nv) break;
+      const int idx = slices > 1 ? i % nv : base + i, sl = slices > 1 ? i / nv : 0;
+      float2 acc = make_float2(0.f, 0.f);
+      if (idx < nv && sl < slices) {
+        const int a = idx % m, l = idx / m;
+        const int p1 = sl + 1 == slices ? LM_TILE : (sl + 1) * per;
+        for (int p = sl * per; p < p1; ++p) {
+          const float2 ea = E[a * LM_EP + p], rp = R[p];
+          const float w = l == 0 ? 1.f : Wt[(l - 1) * LM_TILE + p];
+          acc.x += w * (ea.x * rp.x + ea.y * rp.y);          // conj(ea) r
+          acc.y += w * (ea.x * rp.y - ea.y * rp.x);
+        }
+      }
+      if (slices > 1) {
+        part[i] = acc;
+        __syncthreads();
+        if (sl == 0)
+          for (int s2 = 1; s2 < slices; ++s2) {
+            acc.x += part[i + s2 * nv].x;
+            acc.y += part[i + s2 * nv].y;
+          }
+      }
+      if (idx < nv && sl == 0) {
+        vsum[base / LM_TILE].x += (double)acc.x;
+        vsum[base / LM_TILE].y += (double)acc.y;
       }
     }
-    if (slices > 1) {
-      part[i] = acc;
-      __syncthreads();
-      if (sl == 0)
-        for (int s2 = 1; s2 < slices; ++s2) {
-          acc.x += part[i + s2 * nv].x;
-          acc.y += part[i + s2 * nv].y;
-        }
-    }
-    if (idx < nv && sl == 0) {
-      atomicAdd(&V[2 * idx], (double)acc.x);               // V[l][a] at l m + a = idx
-      atomicAdd(&V[2 * idx + 1], (double)acc.y);
-    }
+    __syncthreads();                                       // E, R and part are reused by the next tile
   }
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (i + u * LM_TILE < nv) vs[(long long)blockIdx.x * nv + i + u * LM_TILE] = make_float2((float)vsum[u].x, (float)vsum[u].y);
+  if (i == 0) ls[blockIdx.x] = lsum;
 }
 
 // GB300 does about two FP64 operations per clock and SM (an FP64 square root takes thousands of cycles,
@@ -275,7 +288,8 @@ __device__ inline float scaled_float(double v, int shift) {
 // access.  Three barriers per block instead of three per column; bound by the chain of dependent
 // square roots and shuffles of the diagonal blocks.
 __global__ void __launch_bounds__(LM_SOLVE_THREADS) k_lm_step(double* t, double2* c, double* tc, double2* cc, int m,
-                                                              int d, LmState* st, double* sets, double* hist, int step,
+                                                              int d, LmState* st, double* sets, const float2* vs, const double* ls, int nblk,
+                                                              double* hist, int step,
                                                               int solve) {
   extern __shared__ __align__(16) float lm_f[];
   __shared__ int s_ok, s_cur;
@@ -288,6 +302,42 @@ __global__ void __launch_bounds__(LM_SOLVE_THREADS) k_lm_step(double* t, double2
   float* Pt = A + ld * ld;                           // LM_NB x ld: the rows below a diagonal block, transposed
   float* sc = Pt + LM_NB * ld;                       // P: 1 / sqrt(damped diagonal) = sc 2^(-sh)
   int* sh = (int*)(sc + ld);
+  {                                                  // V and the loss of the candidate: eight threads per entry
+    const int nv = m * (d + 1), sub = threadIdx.x & 7;
+    double* Vc = sets + (1 - st->cur) * ns + (long long)P * P;
+    for (int v0 = 0; v0 < nv; v0 += LM_SOLVE_THREADS / 8) {
+      const int v = v0 + (threadIdx.x >> 3);
+      float2 hi = make_float2(0.f, 0.f), lo = hi;
+      for (int k0 = sub; k0 < nblk; k0 += 64) {      // eight loads in flight
+        float2 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          x[u] = (v < nv && k0 + 8 * u < nblk) ? vs[(long long)(k0 + 8 * u) * nv + v] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          lo.x += two_sum(hi.x, x[u].x);
+          lo.y += two_sum(hi.y, x[u].y);
+        }
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        const float hx = __shfl_down_sync(0xffffffffu, hi.x, o), hy = __shfl_down_sync(0xffffffffu, hi.y, o);
+        lo.x += __shfl_down_sync(0xffffffffu, lo.x, o) + two_sum(hi.x, hx);
+        lo.y += __shfl_down_sync(0xffffffffu, lo.y, o) + two_sum(hi.y, hy);
+      }
+      if (sub == 0 && v < nv) {
+        Vc[2 * v] = (double)hi.x + (double)lo.x;
+        Vc[2 * v + 1] = (double)hi.y + (double)lo.y;
+      }
+    }
+    if (threadIdx.x >= LM_SOLVE_THREADS - 32) {
+      double l = 0.0;
+      for (int k = threadIdx.x & 31; k < nblk; k += 32) l += ls[k];
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if ((threadIdx.x & 31) == 0) Vc[2 * nv] = l;
+    }
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     const int cand = 1 - st->cur;
     const double l0 = sets[(st->cur + 1) * ns - 1], l1 = sets[(cand + 1) * ns - 1];
@@ -306,8 +356,6 @@ __global__ void __launch_bounds__(LM_SOLVE_THREADS) k_lm_step(double* t, double2
     for (int q = threadIdx.x; q < m * d; q += blockDim.x) t[q] = tc[q];
     for (int q = threadIdx.x; q < m; q += blockDim.x) c[q] = cc[q];
   }
-  // the other set takes the next candidate: V and the loss are accumulated
-  for (int q = threadIdx.x; q < 2 * (d + 1) * m + 1; q += blockDim.x) sets[(2 - s_cur) * ns - 1 - q] = 0.0;
   if (!solve) return;
   const double lam = st->lambda;
   const double* H = sets + s_cur * ns;
@@ -457,9 +505,8 @@ __global__ void __launch_bounds__(LM_SOLVE_THREADS) k_lm_step(double* t, double2
 }
 
 // The starting point as the first candidate, empty accumulators.
-__global__ void k_lm_init(LmState* st, double lambda0, double* sets, const double* t, const double2* c, double* tc,
+__global__ void k_lm_init(LmState* st, double lambda0, const double* t, const double2* c, double* tc,
                           double2* cc, float4* circle, int m, int d) {
-  const long long ns = lm_set_elems(m, d);
   if (threadIdx.x == 0) {
     st->lambda = lambda0;
     st->accepted = 0;
@@ -473,7 +520,6 @@ __global__ void k_lm_init(LmState* st, double lambda0, double* sets, const doubl
   }
   for (int q = threadIdx.x; q < m * d; q += blockDim.x) tc[q] = t[q];
   for (int q = threadIdx.x; q < m; q += blockDim.x) cc[q] = c[q];
-  for (int q = threadIdx.x; q < 2 * (d + 1) * m + 1; q += blockDim.x) sets[ns - 1 - q] = sets[2 * ns - 1 - q] = 0.0;
 }
 
 size_t lm_points_smem(int m, int d) {
@@ -489,7 +535,8 @@ size_t lm_step_smem(int m, int d) {
 
 // ----------------------------------------------------------------------------- host side
 long long lm_workspace_bytes(int m, int d) {
-  return 8 * (2 * lm_set_elems(m, d) + (long long)m * d) + 16LL * (m + LM_SEG) + sizeof(LmState) + 64;
+  return 16LL * (LM_SEG + m) + 8LL * LM_MAXCTA * ((long long)m * (d + 1) + 1) +
+         8 * (2 * lm_set_elems(m, d) + (long long)m * d) + sizeof(LmState) + 64;
 }
 
 // Dynamic shared-memory limits of the refinement kernels.
@@ -513,17 +560,19 @@ void launch_refine_lm(double* t, double2* c, int m, int d, const int* lo, const 
   float4* circle = (float4*)ws;
   double2* cc = (double2*)(circle + LM_SEG);
   double* tc = (double*)(cc + m);
-  double* sets = tc + m * d;
+  double* ls = tc + m * d;
+  float2* vs = (float2*)(ls + LM_MAXCTA);
+  double* sets = (double*)(vs + (long long)LM_MAXCTA * m * (d + 1));
   LmState* st = (LmState*)(sets + 2 * lm_set_elems(m, d));
   const Box B = make_box(d, lo, len);
   const size_t sp = lm_points_smem(m, d), ss = lm_step_smem(m, d);
-  const int npt = (int)((K + LM_TILE - 1) / LM_TILE), npair = m * (m + 1) / 2;
+  const int npt = (int)std::min<long long>(LM_MAXCTA, (K + LM_TILE - 1) / LM_TILE), npair = m * (m + 1) / 2;
   note_launch();
-  k_lm_init<<<1, 256, 0, s>>>(st, lambda0, sets, t, c, tc, cc, circle, m, d);
+  k_lm_init<<<1, 256, 0, s>>>(st, lambda0, t, c, tc, cc, circle, m, d);
   for (int it = 0; it <= iters; ++it) {
     note_launch();
-    k_lm_points<<<npt + npair, LM_TILE, sp, s>>>(tc, cc, m, d, B, K, npt, y, st, circle, sets);
+    k_lm_points<<<npt + npair, LM_TILE, sp, s>>>(tc, cc, m, d, B, K, npt, y, st, circle, sets, vs, ls);
     note_launch();
-    k_lm_step<<<1, LM_SOLVE_THREADS, ss, s>>>(t, c, tc, cc, m, d, st, sets, hist, it, it < iters);
+    k_lm_step<<<1, LM_SOLVE_THREADS, ss, s>>>(t, c, tc, cc, m, d, st, sets, vs, ls, npt, hist, it, it < iters);
   }
 }

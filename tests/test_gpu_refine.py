@@ -210,3 +210,17 @@ def test_lm_steps_match_fp64_iteration(ctx, d, lo, length, m):
         assert np.linalg.norm(cg.cpu().numpy() - cr) <= 1e-4 * np.linalg.norm(cr)
         # the loss of the starting point: exact parameters, so the rounding of the sums alone
         assert abs(Lg[0].item() - Lr[0]) <= 1e-6 * Lr[0]
+
+
+def test_lm_reproducible(ctx):
+    """Every sum of a refinement has a fixed order: repeated runs give the same bits, in one tile of points
+    per CTA, in several, and with the last group of CTAs not full."""
+    import torch
+    from paper_2012_11430_gb300.refine import refine_lm
+    for d, n, m in ((2, 15, 5), (2, 63, 20), (2, 120, 4), (1, 40, 3)):
+        P = _noisy(d, n, m, 850 + n, 20.0)
+        lo, length, _ = _box(n, d)
+        args = (_dev(P.t, torch.float64), _dev(P.c, torch.complex128), _dev(P.grid.reshape(-1), torch.complex64))
+        a = refine_lm(*args, ctx, lo, length, steps=8)
+        b = refine_lm(*args, ctx, lo, length, steps=8)
+        assert all(torch.equal(x, y) for x, y in zip(a, b)), (d, n)
