@@ -359,37 +359,48 @@ void launch_toeplitz(const Dev& D, const ToeplitzJob* jobs, int njobs, int adjoi
                      int y_ext, int maxw, float2* part, int* cnt, long long part_jobs, cudaStream_t s);
 
 // kernels_tc.cu (tensor-core Toeplitz products: split BF16 planes or TF32 hi + lo)
-// Window of a product CTA in its split-plane tables, [lo, lo + len) in table entries, for the grid
-// indices [f_lo, f_hi] it reads.  TF32 tables hold one 32-bit entry per grid index x; BF16
-// tables hold 16-bit entries in reverse order (entry Gd4 - 1 - x holds sample x), so that two
-// consecutive input points on a grid line are two ascending entries (one 32-bit word, or two
-// joined by a funnel shift).  Starts are 16-byte aligned; a BF16 window carries 8 spare entries
-// (the word pairs of a line read up to two entries past its last point).
-__host__ __device__ inline void tc_window(bool bf16, int Gd4, int f_lo, int f_hi, int& lo, int& len) {
-  if (bf16) {
-    const int r_lo = (Gd4 - 1 - f_hi) & ~7, r_hi = Gd4 - 1 - f_lo;
-    lo = r_lo;
-    len = ((r_hi - r_lo + 1 + 7) & ~7) + 8;
-  } else {
+// Formats of the split-plane tables.  TF32: one 32-bit word per grid index x.  BF16: in reverse order (entry
+// Gd4 - 1 - x holds sample x, so consecutive input points on a grid line are ascending entries), either
+// wide -- a 32-bit word holds an entry and the one after it, so that two input points of a line are one
+// load -- or compact, 16 bits per entry (two points from two words by a funnel shift), for windows
+// that would not fit shared memory in the wide form.
+enum TcTable { TT_TF32 = 0, TT_COMPACT = 1, TT_WIDE = 2 };
+__host__ __device__ inline int tc_entry_bytes(int fmt) { return fmt == TT_COMPACT ? 2 : 4; }
+// Window of a product CTA in its tables, [lo, lo + len) in entries, for the grid indices [f_lo, f_hi] it
+// reads.  Starts and lengths are multiples of 16 bytes; a compact window carries 8 spare entries (the
+// word pairs of a line read up to two entries past its last point).
+__host__ __device__ inline void tc_window(int fmt, int Gd4, int f_lo, int f_hi, int& lo, int& len) {
+  if (fmt == TT_TF32) {
     lo = f_lo & ~3;
     len = ((f_hi - lo + 1) + 3) & ~3;
+    return;
+  }
+  const int r_lo = Gd4 - 1 - f_hi, r_hi = Gd4 - 1 - f_lo;
+  if (fmt == TT_COMPACT) {
+    lo = r_lo & ~7;
+    len = ((r_hi - lo + 1 + 7) & ~7) + 8;
+  } else {
+    lo = r_lo & ~3;
+    len = (r_hi - lo + 1 + 3) & ~3;
   }
 }
 int tc_planes(int kind);
 size_t tc_stage_bytes(int kind, int ntbox);
-size_t tc_elem_bytes(int kind);
-size_t tc_smem_bytes(int kind, int ntbox, int stages, int win_cap);
+size_t tc_smem_bytes(int kind, int fmt, int ntbox, int stages, int win_cap);
 long long tc_prob_stride(int kind, int ntbox, int maxnc);
 // Split K workspace of the tensor-core products: tc_part_floats(ntbox) floats per job, one zeroed
 // counter per job.
 size_t tc_part_floats(int ntbox);
-void launch_split_tables(const Dev& D, int kind, cudaStream_t s);
+void launch_split_tables(const Dev& D, int fmt, cudaStream_t s);
 void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long prob_stride,
                     cudaStream_t s);
 cudaError_t launch_toeplitz_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int adjoint, int wsel, int ybuf,
-                               int y_ext, int kind, int ntbox, int win_cap, int stages, const void* xb,
+                               int y_ext, int kind, int fmt, int ntbox, int win_cap, int stages, int half, const void* xb,
                                long long prob_stride, float* part, int* cnt, long long part_jobs, int* err,
                                cudaStream_t s);
+// A stages of a product CTA that shares its SM with a second one (half: 256 columns of tensor memory);
+// 0: the stacked accumulator of ntbox columns per plane leaves no room
+int tc_half_stages(int kind, int ntbox);
 cudaError_t launch_gram_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int xbuf, int xshift, int xw, int zw,
                            long long out_off, int out_ld, int ntbox, int stages, const void* xb, long long prob_stride,
                            float* part, int* cnt, long long part_jobs, int* err, cudaStream_t s);
@@ -403,7 +414,7 @@ cudaError_t launch_apply_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, in
 // sub-problems (S.P their descriptors, S.V / S.B2 / S.Y the transformed blocks).
 enum AxisMode { AX_FP32 = 0, AX_BF16X3 = 1, AX_TF32X3 = 2, AX_BF16X2 = 3 };   // the prony_precision of the products
 constexpr int AX_MAX_N = 95;          // largest n (twiddle table of (n + 3)/2 x (n + 1) float4 in shared memory)
-cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int trim, cudaStream_t s);
+cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int fmt, int trim, cudaStream_t s);
 cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int wsel, int maxw, void* xb,
                            long long prob_stride, cudaStream_t s);
 cudaError_t launch_axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s);

@@ -58,8 +58,8 @@ __device__ __forceinline__ uint16_t ax_bf16(float a) { return (uint16_t)(pack_bf
 
 // Entry x of a sub-problem's sample table (both sides share the format): complex64 for the FP32
 // products, else the split planes of Re and Im as the tensor-core kernel reads them (TF32: word x
-// of each table; BF16: 16-bit entries in reverse order).
-template <int MODE>
+// of each table; BF16: entries in reverse order, wide or compact).
+template <int MODE, int FMT>
 __device__ __forceinline__ void ax_put(float2* grid, uint32_t* tab, int Gd4, int x, float2 v) {
   if (MODE == AX_FP32) {
     grid[x] = v;
@@ -81,7 +81,14 @@ __device__ __forceinline__ void ax_put(float2* grid, uint32_t* tab, int Gd4, int
 #pragma unroll
       for (int pl = 0; pl < 3; ++pl) {
         const uint16_t h = ax_bf16(rest);
-        t16[2LL * (part * 3 + pl) * Gd4 + (Gd4 - 1 - x)] = h;
+        const int r = Gd4 - 1 - x;
+        uint16_t* t = t16 + 2LL * (part * 3 + pl) * Gd4;
+        if (FMT == TT_WIDE) {                     // low half of word r, high half of the word before
+          t[2 * r] = h;
+          if (r > 0) t[2 * r - 1] = h;
+        } else {
+          t[r] = h;
+        }
         rest -= __uint_as_float((uint32_t)h << 16);
       }
     }
@@ -92,7 +99,7 @@ __device__ __forceinline__ void ax_put(float2* grid, uint32_t* tab, int Gd4, int
 // transform to conj F^(w; -x'), zero where -x' leaves the grid.  The difference x_0 = n + 1 occurs
 // in the products over the row box {0..n+1}^d only; `trim` leaves those samples out where a caller
 // asks for a product over I_n alone (whatever they hold, they do not enter it).
-template <int MODE>
+template <int MODE, int FMT>
 __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
   extern __shared__ float2 ax_tw[];
   const ProbDesc& p = D.P[blockIdx.y];
@@ -147,13 +154,13 @@ __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
       if (w0 + u >= G) break;
       const ProbDesc& ps = S.P[p.sub + w0 + u];
       const float2 v = make_float2(acc[0][u].x + acc[1][u].x, acc[0][u].y + acc[1][u].y);
-      ax_put<MODE>(S.gF + ps.grid, S.tabF + ps.toff, ps.Gd4, x, v);
-      ax_put<MODE>(S.gH + ps.grid, S.tabH + ps.toff, ps.Gd4, mvalid ? mir : x,
+      ax_put<MODE, FMT>(S.gF + ps.grid, S.tabF + ps.toff, ps.Gd4, x, v);
+      ax_put<MODE, FMT>(S.gH + ps.grid, S.tabH + ps.toff, ps.Gd4, mvalid ? mir : x,
                    mvalid ? make_float2(v.x, -v.y) : make_float2(0.f, 0.f));
       if (MODE != AX_FP32 && x == Gs - 1)                         // padding of the tables
         for (int y = Gs; y < ps.Gd4; ++y) {
-          ax_put<MODE>(nullptr, S.tabF + ps.toff, ps.Gd4, y, make_float2(0.f, 0.f));
-          ax_put<MODE>(nullptr, S.tabH + ps.toff, ps.Gd4, y, make_float2(0.f, 0.f));
+          ax_put<MODE, FMT>(nullptr, S.tabF + ps.toff, ps.Gd4, y, make_float2(0.f, 0.f));
+          ax_put<MODE, FMT>(nullptr, S.tabH + ps.toff, ps.Gd4, y, make_float2(0.f, 0.f));
         }
     }
   }
@@ -390,21 +397,20 @@ cudaError_t allow_smem(F* kernel, size_t bytes, size_t& set) {
 
 }  // namespace
 
-template <int MODE>
+template <int MODE, int FMT>
 static cudaError_t axis_tables(const Dev& D, const Dev& S, int trim, cudaStream_t s) {
   const int G = 2 * max_axis_n(S) + 2;
   const long long items = (long long)S.maxGd * ((G + 3) / 4);
   note_launch();
-  k_axis_tables<MODE><<<dim3(blocks_per_problem((items + 63) / 64, D.nprob), D.nprob), 64, sizeof(float2) * G, s>>>(D, S, trim);
+  k_axis_tables<MODE, FMT><<<dim3(blocks_per_problem((items + 63) / 64, D.nprob), D.nprob), 64, sizeof(float2) * G, s>>>(D, S, trim);
   return cudaGetLastError();
 }
 
-cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int trim, cudaStream_t s) {
-  switch (mode) {
-    case AX_FP32: return axis_tables<AX_FP32>(D, S, trim, s);
-    case AX_TF32X3: return axis_tables<AX_TF32X3>(D, S, trim, s);
-    default: return axis_tables<AX_BF16X3>(D, S, trim, s);         // three planes written, two or three read
-  }
+cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int fmt, int trim, cudaStream_t s) {
+  if (mode == AX_FP32) return axis_tables<AX_FP32, TT_TF32>(D, S, trim, s);
+  if (mode == AX_TF32X3) return axis_tables<AX_TF32X3, TT_TF32>(D, S, trim, s);
+  return fmt == TT_WIDE ? axis_tables<AX_BF16X3, TT_WIDE>(D, S, trim, s)              // three planes written, two or three read
+                        : axis_tables<AX_BF16X3, TT_COMPACT>(D, S, trim, s);
 }
 
 template <int MODE, int CL, int NC>

@@ -41,8 +41,10 @@ namespace {
 constexpr int TC_BM = 128;
 constexpr uint32_t TC_SPIN = 1u << 24;      // bounded mbarrier polls (~seconds)
 constexpr int TC_MAXSTAGE = 8;
-constexpr int TC_APROD = 8;                 // A' warps (two per TMEM lane quadrant)
-constexpr int TC_THREADS = 32 * (2 + TC_APROD);
+// A' warps: eight (two per TMEM lane quadrant, each taking half of a chunk's points) in a CTA that has the
+// SM to itself; four, each taking both halves in turn, where two CTAs share the SM (256 columns of
+// tensor memory and half of the shared memory each)
+constexpr int TC_APROD = 8, TC_APROD2 = 4;
 constexpr int TC_MAXCH = 512;               // K chunks per CTA (host splits K to stay below)
 enum TcMode { TC_PRODUCT = 0, TC_GRAM = 1, TC_APPLY = 2 };
 
@@ -191,11 +193,10 @@ __global__ void k_xb_prep(Dev D, int xbuf, int xshift, int wsel, unsigned char* 
 }
 
 // Split planes of the sample grid, table a = part * NPL + plane (part 0: Re, 1: Im), at word
-// offset toff + a * Gd4 of the problem.  TF32: one 32-bit word per grid index x.  BF16: 16-bit
-// entries in reverse order (entry Gd4 - 1 - x holds sample x; see tc_window), in the first half of
-// the table's word range.  One pass per solve.
+// offset toff + a * Gd4 of the problem, in one of the formats of TcTable (compact: in the first half of the
+// table's word range).  One pass per solve.
 __device__ __forceinline__ uint16_t bf16_bits(float a) { return (uint16_t)(pack_bf16x2(a, 0.f) & 0xFFFFu); }
-__global__ void k_split_tables(Dev D, int tf32) {
+__global__ void k_split_tables(Dev D, int fmt) {
   const int pi = blockIdx.y;
   const ProbDesc& p = D.P[pi];
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < p.Gd4; j += gridDim.x * blockDim.x) {
@@ -203,9 +204,9 @@ __global__ void k_split_tables(Dev D, int tf32) {
     for (int side = 0; side < 2; ++side) {
       const float2* F = (side ? D.gH : D.gF) + p.grid;
       uint32_t* tab = (side ? D.tabH : D.tabF) + p.toff;
-      const int x = tf32 ? j : p.Gd4 - 1 - j;
+      const int x = fmt == TT_TF32 ? j : p.Gd4 - 1 - j;
       const float2 v = x < p.Gd ? F[x] : make_float2(0.f, 0.f);
-      if (tf32) {
+      if (fmt == TT_TF32) {
         uint32_t wr[2], wi[2];
         split_tf32(v.x, wr);
         split_tf32(v.y, wi);
@@ -213,6 +214,16 @@ __global__ void k_split_tables(Dev D, int tf32) {
         for (int pl = 0; pl < 2; ++pl) {
           tab[(long long)pl * p.Gd4 + x] = wr[pl];
           tab[(long long)(2 + pl) * p.Gd4 + x] = wi[pl];
+        }
+      } else if (fmt == TT_WIDE) {
+        const float2 u = x > 0 && x - 1 < p.Gd ? F[x - 1] : make_float2(0.f, 0.f);   // the entry after
+        uint32_t wr[3], wi[3];
+        split_pair<3>(v.x, u.x, wr);
+        split_pair<3>(v.y, u.y, wi);
+#pragma unroll
+        for (int pl = 0; pl < 3; ++pl) {
+          tab[(long long)pl * p.Gd4 + j] = wr[pl];
+          tab[(long long)(3 + pl) * p.Gd4 + j] = wi[pl];
         }
       } else {
         uint16_t* t16 = (uint16_t*)tab;
@@ -263,13 +274,14 @@ struct TcLayout {
   int dcols, acol0, sa;
 };
 template <int KIND>
-__device__ inline TcLayout tc_layout(int NT) {
+__host__ __device__ inline TcLayout tc_layout(int NT, int columns) {
   using K = TcKind<KIND>;
   TcLayout t;
   t.stacked = K::NPL * NT <= 256;
   t.dcols = t.stacked ? K::NPL * NT : NT;
-  t.acol0 = max(32, (t.dcols + 31) / 32 * 32);
-  t.sa = min(TC_MAXSTAGE, (512 - t.acol0) / (K::NPL * K::PCOLS));   // whole-chunk A stages
+  t.acol0 = (t.dcols + 31) / 32 * 32;
+  const int sa = (columns - t.acol0) / (K::NPL * K::PCOLS);         // whole-chunk A stages
+  t.sa = sa < TC_MAXSTAGE ? sa : TC_MAXSTAGE;
   return t;
 }
 
@@ -302,9 +314,10 @@ __device__ __forceinline__ void tc_load_acc(uint32_t taddr, bool stacked, int NT
 //               and an a x b matrix M of the small workspace: A' row r = X[r, :] read from HBM
 //               ([Re x | Im x] per chunk of 32 columns), B' = M by k_xb_prep, one CTA per row tile
 //               and the whole K range (no split), OUT stored like a product.
-template <int KIND, int MODE>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+template <int KIND, int MODE, int AW, int FMT>
+__global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
     k_toeplitz_tc(Dev D, const ToeplitzJob* jobs, TcParams P, int* err) {
+  constexpr uint32_t TMEM_COLS = AW == TC_APROD ? 512 : 256;
   using K = TcKind<KIND>;
   constexpr bool GRAM = MODE == TC_GRAM, APPLY = MODE == TC_APPLY;
   constexpr bool HBMA = GRAM || APPLY;              // A' read from a tall block in HBM, no window
@@ -344,7 +357,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int c_begin = job.ks * cper, c_end = min(nc, c_begin + cper);
   const int nchunks = max(0, c_end - c_begin);
   const int NT = ((2 * w + 15) / 16) * 16;
-  const TcLayout lay = tc_layout<KIND>(NT);
+  const TcLayout lay = tc_layout<KIND>(NT, TMEM_COLS);
   // One pipeline stage = one K chunk: its B' tile in shared memory and its A' tile in tensor
   // memory, filled together (full barrier: eight A' warps + the loader's byte count) and
   // released together by one commit of the MMAs that read them.
@@ -356,7 +369,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   // window of grid indices needed by this CTA: [gk(first row) - gh(last h), gk(last row) - gh(first h)],
   // as table entries [wlo, wlo + wlen)
-  constexpr int EB = K::TF32 ? 4 : 2;           // bytes per table entry
+  constexpr int EB = FMT == TT_COMPACT ? 2 : 4;  // bytes per table entry
   int wlo = 0, wlen = 0;
   bool idle = nchunks == 0;                     // an empty K range (a split wider than the problem)
   if (!idle && !HBMA) {
@@ -364,7 +377,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int h_first = 32 * c_begin, h_last = min(p.N, 32 * c_end) - 1;
     const int f_lo = grid_of_row(row0, L, p) - grid_of_h(h_last, p);
     const int f_hi = grid_of_row(last_row, L, p) - grid_of_h(h_first, p);
-    tc_window(!K::TF32, p.Gd4, f_lo, f_hi, wlo, wlen);
+    tc_window(FMT, p.Gd4, f_lo, f_hi, wlo, wlen);
     if (wlen > P.win_cap) {
       if (threadIdx.x == 0) atomicExch(err, 3);
       idle = true;
@@ -387,14 +400,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0) {
-    tmem_alloc(&s_tmem, 512);
+    tmem_alloc(&s_tmem, TMEM_COLS);
     tmem_relinquish();
   }
   if (threadIdx.x == 32) {
     mbar_init(&bar_win, 1);
     mbar_init(&bar_d, 1);
     for (int i = 0; i < S; ++i) {
-      mbar_init(&bar_full[i], TC_APROD + 1);    // eight A' warps + the loader (with the byte count)
+      mbar_init(&bar_full[i], AW + 1);          // the A' warps + the loader (with the byte count)
       mbar_init(&bar_empty[i], 1);              // the commit of the stage's MMAs
     }
     s_err = 0;
@@ -497,16 +510,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
   } else {
     // ------------------------------------------------------------- A' producers + epilogue
-    // Warps 2..9: quadrant q = warp & 3 (TMEM lanes 32q..32q+31 = tile rows), half hh of every
-    // K chunk (input points 32c + 16hh .. +15).
+    // Warps 2..: quadrant q = warp & 3 (TMEM lanes 32q..32q+31 = tile rows), half hh of every
+    // K chunk (input points 32c + 16hh .. +15), or both halves in turn.
     const int q = warp & 3;
-    const int hh = (warp - 2) >> 2;
+    constexpr int HALVES = TC_APROD / AW;         // halves of a chunk per warp
+    const int hh0 = HALVES == 1 ? (warp - 2) >> 2 : 0;
     const int i = 32 * q + lane;                // row within the tile
     const int row = row0 + i;
     const bool vrow = row < rows_total;
-    // window entry of grid index 0 for this row: TF32 entry of grid index g is gk - g... (descending
-    // with the input point), BF16 entry is gk + g (ascending, reversed tables)
-    const int gk = (HBMA || !vrow) ? 0 : K::TF32 ? grid_of_row(row, L, p) - wlo : p.Gd4 - 1 - grid_of_row(row, L, p) - wlo;
+    // window entry of grid index 0 for this row: TF32 entry of grid index g is gk - g (descending with
+    // the input point), BF16 entry is gk + g (ascending, reversed tables).  Rows past the end take the last
+    // row's samples (their results are not stored).
+    const int grow = HBMA ? 0 : grid_of_row(vrow ? row : rows_total - 1, L, p);
+    const int gk = HBMA ? 0 : K::TF32 ? grow - wlo : p.Gd4 - 1 - grow - wlo;
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
     bool ok = idle || HBMA || __all_sync(0xffffffffu, mbar_wait(&bar_win, 0, TC_SPIN));
     if (!ok) s_err = 1;
@@ -525,7 +541,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         s_err = 1;
         break;
       }
-      {
+#pragma unroll 1
+      for (int hh = hh0; hh < hh0 + HALVES; ++hh) {
         const int g0 = HBMA ? 0 : ghalf[2 * it + hh];
         // TMEM column of (plane pl, part, point j of this half): BF16 two points per column at
         // pl * 32 + part * 16 + hh * 8 + j / 2; TF32 one point per column at pl * 64 + part * 32 + hh * 16 + j
@@ -602,62 +619,76 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
               }
             }
           }
-        } else if (g0 >= 0 && K::TF32) {
-          // the 16 points lie on one grid line: F(k - h_j) sits at window entry x - j
-          const int x = vrow ? gk - g0 : 16;      // rows past the end read nothing (any in-range x)
-#pragma unroll
-          for (int part = 0; part < 2; ++part)
-#pragma unroll
-            for (int pl = 0; pl < NPL; ++pl) {
-              const uint32_t* T = (const uint32_t*)(wtab + (size_t)(part * NPL + pl) * P.win_cap * EB) + x;
-#pragma unroll
-              for (int e = 0; e < NW; ++e) wv[part][pl][e] = vrow ? T[-e] : 0u;
-            }
         } else if (g0 >= 0) {
-          // the 16 points lie on one grid line: point j at window entry x + j (ascending), so the
-          // word of the points (2e, 2e + 1) is the 32-bit pair at entry x + 2e -- aligned when x is
-          // even, else joined from two aligned words by a 16-bit funnel shift
-          const int x = vrow ? gk + g0 : 0;
-          const int wb = x >> 1;
+          // the 16 points lie on one grid line
+          const int x = K::TF32 ? gk - g0 : gk + g0;
           const uint32_t sh = (uint32_t)(x & 1) << 4;
 #pragma unroll
           for (int part = 0; part < 2; ++part)
 #pragma unroll
             for (int pl = 0; pl < NPL; ++pl) {
-              const uint32_t* T = (const uint32_t*)(wtab + (size_t)(part * NPL + pl) * P.win_cap * EB) + wb;
-              uint32_t w[NW + 1];
-#pragma unroll
-              for (int e = 0; e <= NW; ++e) w[e] = vrow ? T[e] : 0u;
-#pragma unroll
-              for (int e = 0; e < NW; ++e) wv[part][pl][e] = __funnelshift_r(w[e], w[e + 1], sh);
-            }
-        } else {
-          // points on several grid lines: each point from its own table entry
-          const int h = 32 * (c_begin + it) + 16 * hh + (lane & 15);
-          const int ghl = h < p.N ? grid_of_h(h, p) : INT_MIN;
-          int xs[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int g = __shfl_sync(0xffffffffu, ghl, j);
-            xs[j] = (vrow && g != INT_MIN) ? (K::TF32 ? gk - g : gk + g) : -1;
-          }
-#pragma unroll
-          for (int part = 0; part < 2; ++part)
-#pragma unroll
-            for (int pl = 0; pl < NPL; ++pl) {
               const unsigned char* Tb = wtab + (size_t)(part * NPL + pl) * P.win_cap * EB;
+              if (FMT == TT_TF32) {              // point j at entry x - j
 #pragma unroll
-              for (int e = 0; e < NW; ++e) {
-                if (K::TF32) {
-                  wv[part][pl][e] = xs[e] >= 0 ? ((const uint32_t*)Tb)[xs[e]] : 0u;
-                } else {
-                  const uint16_t* T = (const uint16_t*)Tb;
-                  const uint32_t lo = xs[2 * e] >= 0 ? (uint32_t)T[xs[2 * e]] : 0u;
-                  const uint32_t hi = xs[2 * e + 1] >= 0 ? (uint32_t)T[xs[2 * e + 1]] << 16 : 0u;
-                  wv[part][pl][e] = lo | hi;
-                }
+                for (int e = 0; e < NW; ++e) wv[part][pl][e] = ((const uint32_t*)Tb)[x - e];
+              } else if (FMT == TT_WIDE) {       // points (2e, 2e + 1): the word at entry x + 2e
+#pragma unroll
+                for (int e = 0; e < NW; ++e) wv[part][pl][e] = ((const uint32_t*)Tb)[x + 2 * e];
+              } else {                           // joined from two aligned words by a 16-bit funnel shift
+                const uint32_t* T = (const uint32_t*)Tb + (x >> 1);
+                uint32_t w[NW + 1];
+#pragma unroll
+                for (int e = 0; e <= NW; ++e) w[e] = T[e];
+#pragma unroll
+                for (int e = 0; e < NW; ++e) wv[part][pl][e] = __funnelshift_r(w[e], w[e + 1], sh);
               }
             }
+        } else {
+          // points on several grid lines: each point from its own entry; points past N take the last
+          // one's samples (B' is zero there)
+          const int h = min(32 * (c_begin + it) + 16 * hh + (lane & 15), p.N - 1);
+          const int ghl = grid_of_h(h, p);
+          if (FMT == TT_WIDE) {
+#pragma unroll
+            for (int e = 0; e < NW; ++e) {
+              const int ga = __shfl_sync(0xffffffffu, ghl, 2 * e), gb = __shfl_sync(0xffffffffu, ghl, 2 * e + 1);
+              const uint32_t* T = (const uint32_t*)wtab + gk + ga;
+              if (gb == ga + 1) {                // both on one line (the same for every row)
+#pragma unroll
+                for (int part = 0; part < 2; ++part)
+#pragma unroll
+                  for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = T[(part * NPL + pl) * P.win_cap];
+              } else {
+#pragma unroll
+                for (int part = 0; part < 2; ++part)
+#pragma unroll
+                  for (int pl = 0; pl < NPL; ++pl)
+                    wv[part][pl][e] = __byte_perm(T[(part * NPL + pl) * P.win_cap], T[(part * NPL + pl) * P.win_cap + gb - ga], 0x5410);
+              }
+            }
+          } else {
+            int xs[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int g = __shfl_sync(0xffffffffu, ghl, j);
+              xs[j] = K::TF32 ? gk - g : gk + g;
+            }
+#pragma unroll
+            for (int part = 0; part < 2; ++part)
+#pragma unroll
+              for (int pl = 0; pl < NPL; ++pl) {
+                const unsigned char* Tb = wtab + (size_t)(part * NPL + pl) * P.win_cap * EB;
+#pragma unroll
+                for (int e = 0; e < NW; ++e) {
+                  if (FMT == TT_TF32) {
+                    wv[part][pl][e] = ((const uint32_t*)Tb)[xs[e]];
+                  } else {
+                    const uint16_t* T = (const uint16_t*)Tb;
+                    wv[part][pl][e] = (uint32_t)T[xs[2 * e]] | (uint32_t)T[xs[2 * e + 1]] << 16;
+                  }
+                }
+              }
+          }
         }
 #pragma unroll
         for (int part = 0; part < 2; ++part)
@@ -667,14 +698,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (K::TF32) tmem_st_x16(col, wv[part][pl]);
             else tmem_st_x8(col, wv[part][pl]);
           }
-        tmem_st_wait();
       }
+      tmem_st_wait();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_full[s]);
       if (++s == S) { s = 0; ph ^= 1u; }
     }
-    // epilogue: D (TMEM) -> Y; the two warps of a quadrant take alternate 16-column groups
+    // epilogue: D (TMEM) -> Y; the warps of a quadrant take alternate 16-column groups
+    constexpr int CSTEP = HALVES == 1 ? 32 : 16;
     const bool dready = idle || __all_sync(0xffffffffu, mbar_wait(&bar_d, 0, TC_SPIN));
     if (!dready) s_err = 1;
     int ldy;
@@ -688,7 +720,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (job.nks == 1) {
       if (dready && !s_err) {
         tc_fence_after();
-        for (int c0 = 16 * hh; c0 < NT; c0 += 32) {
+        for (int c0 = 16 * hh0; c0 < NT; c0 += CSTEP) {
           float v[16];
           tc_load_acc<NPL>(tb + lane_off + c0, lay.stacked, NT, v);
           if (vrow) {
@@ -707,7 +739,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       float* mine = P.part + (size_t)blockIdx.x * slot;
       const bool mine_ok = ws_ok(D, (long long)blockIdx.x - job.ks + job.nks <= P.part_jobs && job.ks < job.nks, 21);
       if (dready && !s_err && !idle) tc_fence_after();
-      for (int c0 = 16 * hh; c0 < NT; c0 += 32) {
+      for (int c0 = 16 * hh0; c0 < NT; c0 += CSTEP) {
         float v[16];
         if (dready && !s_err && !idle) {
           tc_load_acc<NPL>(tb + lane_off + c0, lay.stacked, NT, v);
@@ -721,10 +753,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
       }
       __threadfence();
-      named_bar_sync(1, 32 * TC_APROD);
+      named_bar_sync(1, 32 * AW);
       const int first_job = blockIdx.x - job.ks;  // the tile's CTAs are consecutive jobs
       if (warp == 2 && lane == 0) s_last = mine_ok && atomicAdd(&P.cnt[first_job], 1) == job.nks - 1;
-      named_bar_sync(1, 32 * TC_APROD);
+      named_bar_sync(1, 32 * AW);
       if (s_last) {
         // every other CTA of the tile has stored its partial (fence before its arrival): add the
         // partials in the order of their K ranges -- in FP32 for a product (at most 16 ranges;
@@ -732,7 +764,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         __threadfence();
         const float* base = P.part + (size_t)first_job * slot;
         using Acc = typename std::conditional<GRAM, double, float>::type;
-        for (int c0 = 16 * hh; c0 < NT; c0 += 32) {
+        for (int c0 = 16 * hh0; c0 < NT; c0 += CSTEP) {
           Acc v[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) v[e] = (Acc)__ldcg(base + (size_t)(c0 + e) * TC_BM + i);
@@ -763,7 +795,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_after();
     // on an error path, let the MMAs already issued finish before the columns are released
     if (s_err && !idle) mbar_wait(&bar_d, 0, TC_SPIN);
-    tmem_dealloc(tb, 512);
+    tmem_dealloc(tb, TMEM_COLS);
   }
 }
 
@@ -772,17 +804,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // ----------------------------------------------------------------------------- host side
 int tc_planes(int kind) { return kind == PRONY_BF16X3 ? 3 : 2; }
 size_t tc_stage_bytes(int kind, int ntbox) { return (size_t)(kind == PRONY_TF32X3 ? 2 : 1) * tc_planes(kind) * ntbox * 128; }
-size_t tc_elem_bytes(int kind) { return kind == PRONY_TF32X3 ? 4 : 2; }
-
-size_t tc_entry_bytes(int kind) { return kind == PRONY_TF32X3 ? 4 : 2; }
-size_t tc_smem_bytes(int kind, int ntbox, int stages, int win_cap) {
-  return 1024 + (size_t)stages * tc_stage_bytes(kind, ntbox) + (size_t)2 * tc_planes(kind) * win_cap * tc_entry_bytes(kind);
+size_t tc_smem_bytes(int kind, int fmt, int ntbox, int stages, int win_cap) {
+  return 1024 + (size_t)stages * tc_stage_bytes(kind, ntbox) + (size_t)2 * tc_planes(kind) * win_cap * tc_entry_bytes(fmt);
 }
 
-void launch_split_tables(const Dev& D, int kind, cudaStream_t s) {
+void launch_split_tables(const Dev& D, int fmt, cudaStream_t s) {
   note_launch();
   dim3 g(blocks_per_problem(std::min((D.maxGd + 3) / 4 / 256 + 1, 64), D.nprob), D.nprob);
-  k_split_tables<<<g, 256, 0, s>>>(D, kind == PRONY_TF32X3 ? 1 : 0);
+  k_split_tables<<<g, 256, 0, s>>>(D, fmt);
 }
 
 // Bytes of B' tiles reserved per problem: every chunk at the widest tile of the batch.
@@ -813,36 +842,49 @@ void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int 
   xb_prep(D, xbuf, xshift, wsel, xb, kind, prob_stride, -1, 0, 0, D.maxN, s);
 }
 
-template <int KIND, int MODE>
+template <int KIND, int MODE, int FMT = TT_TF32, int AW = TC_APROD>
 static cudaError_t launch_tc_kind(const Dev& D, const ToeplitzJob* jobs, int njobs, const TcParams& P, int* err,
                                   size_t sm, cudaStream_t s) {
   static size_t set = 0;
   if (sm > set) {
     // the attribute must cover this launch's dynamic shared memory (static + dynamic <= 227 KB)
     cudaError_t e =
-        cudaFuncSetAttribute(k_toeplitz_tc<KIND, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(k_toeplitz_tc<KIND, MODE, AW, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     set = sm;
   }
-  k_toeplitz_tc<KIND, MODE><<<njobs, TC_THREADS, sm, s>>>(D, jobs, P, err);
+  k_toeplitz_tc<KIND, MODE, AW, FMT><<<njobs, 32 * (2 + AW), sm, s>>>(D, jobs, P, err);
   return cudaGetLastError();
+}
+
+int tc_half_stages(int kind, int ntbox) {
+  const TcLayout t = kind == PRONY_BF16X3   ? tc_layout<PRONY_BF16X3>(ntbox, 256)
+                     : kind == PRONY_BF16X2 ? tc_layout<PRONY_BF16X2>(ntbox, 256)
+                                            : tc_layout<PRONY_TF32X3>(ntbox, 256);
+  return t.stacked && t.sa > 0 ? t.sa : 0;
 }
 
 size_t tc_part_floats(int ntbox) { return (size_t)ntbox * TC_BM; }
 
 cudaError_t launch_toeplitz_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int adjoint, int wsel, int ybuf,
-                               int y_ext, int kind, int ntbox, int win_cap, int stages, const void* xb,
+                               int y_ext, int kind, int fmt, int ntbox, int win_cap, int stages, int half, const void* xb,
                                long long prob_stride, float* part, int* cnt, long long part_jobs, int* err,
                                cudaStream_t s) {
   TcParams P{(const unsigned char*)xb, prob_stride, adjoint, wsel, ybuf, y_ext, ntbox, win_cap, stages, part, cnt,
              part_jobs, 0, -1, 0, 0, 0};
-  const size_t sm = tc_smem_bytes(kind, ntbox, stages, win_cap);
+  const size_t sm = tc_smem_bytes(kind, fmt, ntbox, stages, win_cap);
   note_launch();
-  switch (kind) {
-    case PRONY_BF16X3: return launch_tc_kind<PRONY_BF16X3, TC_PRODUCT>(D, jobs, njobs, P, err, sm, s);
-    case PRONY_BF16X2: return launch_tc_kind<PRONY_BF16X2, TC_PRODUCT>(D, jobs, njobs, P, err, sm, s);
-    default: return launch_tc_kind<PRONY_TF32X3, TC_PRODUCT>(D, jobs, njobs, P, err, sm, s);
-  }
+  constexpr int TCP = TC_PRODUCT;
+  if (kind == PRONY_TF32X3)
+    return half ? launch_tc_kind<PRONY_TF32X3, TCP, TT_TF32, TC_APROD2>(D, jobs, njobs, P, err, sm, s)
+                : launch_tc_kind<PRONY_TF32X3, TCP, TT_TF32>(D, jobs, njobs, P, err, sm, s);
+  if (kind == PRONY_BF16X3)
+    return half ? launch_tc_kind<PRONY_BF16X3, TCP, TT_WIDE, TC_APROD2>(D, jobs, njobs, P, err, sm, s)
+           : fmt == TT_WIDE ? launch_tc_kind<PRONY_BF16X3, TCP, TT_WIDE>(D, jobs, njobs, P, err, sm, s)
+                            : launch_tc_kind<PRONY_BF16X3, TCP, TT_COMPACT>(D, jobs, njobs, P, err, sm, s);
+  return half ? launch_tc_kind<PRONY_BF16X2, TCP, TT_WIDE, TC_APROD2>(D, jobs, njobs, P, err, sm, s)
+         : fmt == TT_WIDE ? launch_tc_kind<PRONY_BF16X2, TCP, TT_WIDE>(D, jobs, njobs, P, err, sm, s)
+                          : launch_tc_kind<PRONY_BF16X2, TCP, TT_COMPACT>(D, jobs, njobs, P, err, sm, s);
 }
 
 // The Gram X^* Z of two tall blocks on the tensor cores in three BF16 planes (B' tiles of Z from
@@ -852,7 +894,7 @@ cudaError_t launch_gram_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int
                            float* part, int* cnt, long long part_jobs, int* err, cudaStream_t s) {
   TcParams P{(const unsigned char*)xb, prob_stride, 0, zw, 0, 0, ntbox, 0, stages, part, cnt, part_jobs,
              xbuf, xshift, xw, out_off, out_ld};
-  const size_t sm = tc_smem_bytes(PRONY_BF16X3, ntbox, stages, 0);
+  const size_t sm = tc_smem_bytes(PRONY_BF16X3, TT_WIDE, ntbox, stages, 0);
   note_launch();
   return launch_tc_kind<PRONY_BF16X3, TC_GRAM>(D, jobs, njobs, P, err, sm, s);
 }
@@ -867,7 +909,7 @@ cudaError_t launch_apply_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, in
              xbuf, -1, xw, 0, 0};
   // at least half the shared memory of an SM, so that one CTA holds an SM (and all of its tensor
   // memory) at a time
-  const size_t sm = std::max<size_t>(tc_smem_bytes(PRONY_BF16X3, ntbox, stages, 0), 116 * 1024);
+  const size_t sm = std::max<size_t>(tc_smem_bytes(PRONY_BF16X3, TT_WIDE, ntbox, stages, 0), 116 * 1024);
   note_launch();
   return launch_tc_kind<PRONY_BF16X3, TC_APPLY>(D, jobs, njobs, P, err, sm, s);
 }

@@ -142,6 +142,8 @@ struct TcConf {
   int nks_min = 1;                    // tuning range: nks_min, 2 nks_min
   std::string key;                    // batch shape signature
   int kind = PRONY_BF16X3, ntbox = 16, stages = 2, win_cap = 0, nks = 1;
+  int half = 0;                       // two CTAs per SM
+  int fmt = 0;                        // TcTable format of the sample tables
   long long prob_stride = 0;          // bytes of B' tiles per problem
   int njobs_ext = 0, njobs_in = 0;
   ToeplitzJob* jobs_ext = nullptr;
@@ -214,7 +216,7 @@ int h_grid_of_h(int h, const ProbDesc& p) {
 }
 // largest window (table entries, as the kernel sizes it: tc_window) over the CTAs of a problem
 // for a K split into nks ranges
-int max_window(const ProbDesc& p, int L, int nks, bool bf16) {
+int max_window(const ProbDesc& p, int L, int nks, int fmt) {
   const int rows = ipow(L, p.d) > 0 ? (int)ipow(L, p.d) : 0;
   const int nc = (p.N + 31) / 32, cper = (nc + nks - 1) / nks;
   int mx = 0;
@@ -225,7 +227,7 @@ int max_window(const ProbDesc& p, int L, int nks, bool bf16) {
       if (cb >= ce) continue;
       int hf = 32 * cb, hl = std::min(p.N, 32 * ce) - 1;
       int lo = 0, len = 0;
-      tc_window(bf16, p.Gd4, h_grid_of_row(r0, L, p) - h_grid_of_h(hl, p), h_grid_of_row(last, L, p) - h_grid_of_h(hf, p),
+      tc_window(fmt, p.Gd4, h_grid_of_row(r0, L, p) - h_grid_of_h(hl, p), h_grid_of_row(last, L, p) - h_grid_of_h(hf, p),
                 lo, len);
       mx = std::max(mx, len);
     }
@@ -380,10 +382,10 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   if (T.ntbox > 256) return PRONY_EINVAL;
   int st_max = 4;
   while (st_max > 1 && 1024 + st_max * stage + 64 * 1024 > avail) --st_max;
-  // window entries per table: BF16 tables hold 2-byte entries (multiples of 8), TF32 4-byte (of 4)
   const bool bf16 = prec != PRONY_TF32X3;
-  auto win_cap_for = [&](int st) {
-    return (int)((avail - 1024 - st * stage) / (2 * npl * (bf16 ? 2 : 4))) & (bf16 ? ~7 : ~3);
+  // window entries per table (16-byte multiples)
+  auto win_cap_for = [&](int st, int fmt) {
+    return (int)((avail - 1024 - st * stage) / (2 * npl * tc_entry_bytes(fmt))) & (fmt == TT_COMPACT ? ~7 : ~3);
   };
   // split K: enough CTAs to fill the GPU, every window within the shared-memory capacity, and at
   // most 512 roundings of the leading accumulator block per CTA: the FP32 accumulator in tensor
@@ -399,24 +401,24 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   // shape of the batch
   std::map<std::pair<int, int>, int> shapes;          // (n, d) -> a problem of that shape
   for (int i = 0; i < (int)Q.size(); ++i) shapes.emplace(std::make_pair(Q[i].n, Q[i].d), i);
-  std::map<std::tuple<int, int, int>, int> wmemo;      // (problem, nks, ext) -> window words
-  auto window_of = [&](int i, int nks, int ext) {
-    auto key = std::make_tuple(i, nks, ext);
+  std::map<std::tuple<int, int, int, int>, int> wmemo;   // (problem, nks, ext, format) -> window entries
+  auto window_of = [&](int i, int nks, int ext, int fmt) {
+    auto key = std::make_tuple(i, nks, ext, fmt);
     auto it = wmemo.find(key);
     if (it != wmemo.end()) return it->second;
     const ProbDesc& p = Q[i];
-    const int wl = max_window(p, ext ? p.n + 2 : p.n + 1, nks, bf16);
+    const int wl = max_window(p, ext ? p.n + 2 : p.n + 1, nks, fmt);
     wmemo.emplace(key, wl);
     return wl;
   };
-  auto split_for = [&](int cap) {
+  auto split_for = [&](int cap, int fmt) {
     int nks = nks_lo;
     for (;; ++nks) {
       bool fits = true;
       for (const auto& sh : shapes) {
         const ProbDesc& p = Q[sh.second];
         nks = std::min(nks, std::max(1, (p.N + 31) / 32));
-        if (window_of(sh.second, nks, 1) > cap || window_of(sh.second, nks, 0) > cap) fits = false;
+        if (window_of(sh.second, nks, 1, fmt) > cap || window_of(sh.second, nks, 0, fmt) > cap) fits = false;
       }
       if (fits || nks >= maxnc) break;
     }
@@ -432,16 +434,49 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   }
   int nks = INT_MAX;
   T.stages = st_max;
+  T.fmt = bf16 ? TT_COMPACT : TT_TF32;
   for (int st = st_max; st >= st_min; --st) {
-    if (win_cap_for(st) < 256) continue;
-    const int k = split_for(win_cap_for(st));
+    if (win_cap_for(st, T.fmt) < 256) continue;
+    const int k = split_for(win_cap_for(st, T.fmt), T.fmt);
     if (k < nks) {
       nks = k;
       T.stages = st;
     }
   }
   if (nks == INT_MAX) return PRONY_EINVAL;
-  T.win_cap = win_cap_for(T.stages);
+  auto longest = [&](int fmt) {
+    int need = 0;
+    for (const auto& sh : shapes)
+      need = std::max(need, std::max(window_of(sh.second, nks, 1, fmt), window_of(sh.second, nks, 0, fmt)));
+    return need;
+  };
+  // wide tables where their windows fit at the same split (with the stages given, or two)
+  if (bf16)
+    for (int st = T.stages; st >= st_min; --st)
+      if (win_cap_for(st, TT_WIDE) >= std::max(256, longest(TT_WIDE))) {
+        T.stages = st;
+        T.fmt = TT_WIDE;
+        break;
+      }
+  T.win_cap = win_cap_for(T.stages, T.fmt);
+  // Narrow blocks (at most 24 columns in BF16x3) of problems whose windows are short: two CTAs per SM, each with
+  // half of its memories, so that one's set-up, window load and epilogue run under the other's
+  // chunks.  Wider accumulators leave no tensor memory for it, longer windows no shared memory.
+  {
+    const size_t per = 228 * 1024 / 2 - 1024 - 6144;   // (1 KB reserved per CTA, static shared memory)
+    const int need = longest(T.fmt);
+    const int sa = tc_half_stages(prec, T.ntbox);
+    // (narrower problems of the batch have room for more A stages than the widest)
+    int st = std::min(T.stages, 3);
+    while (st > std::max(1, sa) && tc_smem_bytes(prec, T.fmt, T.ntbox, st, need) > per) --st;
+    const char* e = getenv("PRONY_TC_HALF");
+    if (sa > 0 && T.fmt != TT_COMPACT && !getenv("PRONY_TC_BSTAGES") && !(e && atoi(e) == 0) &&
+        (long long)tiles_in * nks >= 4 * 152 && tc_smem_bytes(prec, T.fmt, T.ntbox, st, need) <= per) {
+      T.half = 1;
+      T.stages = st;
+      T.win_cap = need;
+    }
+  }
   T.nks_min = nks;
   T.prob_stride = tc_prob_stride(prec, T.ntbox, maxnc);
   // Grams of the tall blocks on the tensor cores, on request only (PRONY_TC_GRAM=1): the FP32
@@ -478,7 +513,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     T.apply_stride = tc_prob_stride(PRONY_BF16X3, T.ntbox, maxac);
   }
   // batch shape signature for the tuning cache
-  T.key = std::to_string(prec) + (B.ax.on ? "a:" : ":") + std::to_string(B.P.size()) + ":" + std::to_string(maxw) + ":" +
+  T.key = std::to_string(prec) + (B.ax.on ? "a" : "") + (T.half ? "h" : "") + std::to_string(T.fmt) + ":" + std::to_string(B.P.size()) + ":" + std::to_string(maxw) + ":" +
           std::to_string(maxnc) + ":" + std::to_string(tiles_ext) + ":" + std::to_string(tiles_in) + ":" +
           std::to_string(nks);
   auto hit = ctx->tc_tuned.find(T.key);
@@ -557,7 +592,7 @@ void toeplitz_product(prony_ctx* ctx, const Batch& B, const Dev& D, int ext, int
     cudaError_t e = launch_axis_in(D, S, prec, xbuf, wsel, B.maxw, ctx->xb.p, T.prob_stride, s);
     if (e == cudaSuccess && T.on)
       e = launch_toeplitz_tc(S, ext ? T.jobs_ext : T.jobs_in, ext ? T.njobs_ext : T.njobs_in, adjoint, wsel, sbuf, ext,
-                             T.kind, T.ntbox, T.win_cap, T.stages, ctx->xb.p, T.prob_stride, (float*)B.part, B.cnt,
+                             T.kind, T.fmt, T.ntbox, T.win_cap, T.stages, T.half, ctx->xb.p, T.prob_stride, (float*)B.part, B.cnt,
                              B.part_jobs, T.err, s);
     else if (e == cudaSuccess)
       launch_toeplitz(S, ext ? B.jobs_ext : B.jobs_in, ext ? B.njobs_ext : B.njobs_in, adjoint, BUF_V, wsel, sbuf, ext,
@@ -568,7 +603,7 @@ void toeplitz_product(prony_ctx* ctx, const Batch& B, const Dev& D, int ext, int
     const TcConf& T = B.tc;
     launch_xb_prep(D, xbuf, -1, wsel, ctx->xb.p, T.kind, T.prob_stride, s);
     cudaError_t e = launch_toeplitz_tc(D, ext ? T.jobs_ext : T.jobs_in, ext ? T.njobs_ext : T.njobs_in, adjoint,
-                                       wsel, ybuf, ext, T.kind, T.ntbox, T.win_cap, T.stages, ctx->xb.p,
+                                       wsel, ybuf, ext, T.kind, T.fmt, T.ntbox, T.win_cap, T.stages, T.half, ctx->xb.p,
                                        T.prob_stride, (float*)B.part, B.cnt, B.part_jobs, T.err, s);
     if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
   } else {
@@ -779,10 +814,10 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec) {
 // sub-problems (`trim`: without the samples at x_0 = n + 1).
 void product_tables(prony_ctx* ctx, const Batch& B, int prec, int trim, cudaStream_t s) {
   if (B.ax.on) {
-    const cudaError_t e = launch_axis_tables(B.D, B.ax.S, prec, trim, s);
+    const cudaError_t e = launch_axis_tables(B.D, B.ax.S, prec, B.tc.fmt, trim, s);
     if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
   } else if (B.tc.on) {
-    launch_split_tables(B.D, B.tc.kind, s);
+    launch_split_tables(B.D, B.tc.fmt, s);
   }
 }
 
@@ -988,7 +1023,7 @@ std::string loop_graph_key(const Batch& B, const void* xb, const int* dflag, int
   put(&B.D, sizeof(Dev));
   put(B.P.data(), sizeof(ProbDesc) * B.P.size());
   const TcConf& T = B.tc;
-  const long long tc[] = {T.on, T.kind, T.ntbox, T.stages, T.win_cap, T.nks, (long long)(size_t)B.part,
+  const long long tc[] = {T.on, T.half, T.fmt, T.kind, T.ntbox, T.stages, T.win_cap, T.nks, (long long)(size_t)B.part,
                           (long long)(size_t)B.cnt, B.part_jobs, T.prob_stride, T.njobs_ext,
                           T.njobs_in, (long long)(size_t)T.jobs_ext, (long long)(size_t)T.jobs_in,
                           (long long)(size_t)T.err, B.fft.on, B.fft.lz, B.fft.maxpts, B.njobs_ext, B.njobs_in, B.nks,
