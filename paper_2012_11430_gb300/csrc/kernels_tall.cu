@@ -126,7 +126,10 @@ __global__ void k_init_v0(Dev D, unsigned long long seed) {
     const long long q = (long long)row * p.r0 + col;
     uint64_t c[4] = {(uint64_t)q, 0, 0, 0};
     philox4x64(c, seed, PRONY_STREAM_V0);
-    float u0 = (float)philox_u01(c[0]), u1 = (float)philox_u01(c[1]);
+    // u = ((w >> 11) + 1/2) 2^-53 rounded to FP32 without FP64 operations (they took most of this kernel:
+    // 0.61 ms for 64 blocks of 8000 x 80, now 0.48; 0.41 -> 0.34 for 4096 blocks of d=2, n 7..31)
+    float u0 = __ull2float_rn((c[0] >> 11) * 2 + 1) * 5.5511151231257827e-17f;      // 2^-54
+    float u1 = __ull2float_rn((c[1] >> 11) * 2 + 1) * 5.5511151231257827e-17f;
     float r = sqrtf(-logf(u0)), sn, cs;
     sincospif(2.0f * u1, &sn, &cs);
     D.V[p.xoff + (long long)col * p.N + row] = make_float2(r * cs, r * sn);
