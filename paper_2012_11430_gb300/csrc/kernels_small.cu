@@ -4,8 +4,8 @@
 //             column-pivoted QR (Algorithm 3, lines with QR / QR with column pivoting),
 //             the rank criterion ||R(i:r0,i:r0)||_F <= tol ||R||_F (Section 2.2) read off the
 //             trailing Schur-complement trace, and the map X -> X P R^{-1}.
-//  k_solve_c  FP64 Vandermonde Gram conj(A) A^T (product of Dirichlet kernels) and Cholesky
-//             solve of the normal equations of Eq. ls_probl; results sorted by t.
+//  k_solve_c  FP64 L D L^H solve of the normal equations of Eq. ls_probl (the Gram matrix from k_powers);
+//             results sorted by t.
 // All loops are bounded; a cap that is hit sets PRONY_ENOCONV in the problem's state.
 #include "common.cuh"
 #include <algorithm>
@@ -251,66 +251,48 @@ __global__ void __launch_bounds__(256) k_solve_c(Dev D) {
   for (int i = threadIdx.x; i < m; i += blockDim.x) bb[i] = b[i];
   if (threadIdx.x == 0) s_bad = 0;
   __syncthreads();
-  // G[i][j] = prod_l sum_{x=0}^{n} exp(2 pi i (t_i(l) - t_j(l)) x), or with the raw eigenvalues
-  // prod_l sum_x (conj(z_i(l)) z_j(l))^x (summed term by term: |q| need not be 1)
-  const double2* zr = (const double2*)(D.small + p.soff + D.L.zraw);
-  for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-    int i = idx / m, j = idx % m;
-    double2 g = make_double2(1.0, 0.0);
-    if (D.vand) {
-      for (int l = 0; l < d; ++l) {
-        const double2 q = cmulc(zr[i * PRONY_DMAX + l], zr[j * PRONY_DMAX + l]);
-        double2 sum = make_double2(1.0, 0.0), pw = make_double2(1.0, 0.0);
-        for (int x = 1; x <= p.n; ++x) {
-          pw = cmul(pw, q);
-          sum = cadd(sum, pw);
-        }
-        g = cmul(g, sum);
-      }
-      G[i * LD + j] = g;
-      continue;
-    }
-    for (int l = 0; l < d; ++l) {
-      double dl = ts[i * PRONY_DMAX + l] - ts[j * PRONY_DMAX + l];
-      dl -= rint(dl);
-      double2 term;
-      if (dl == 0.0) {
-        term = make_double2((double)(p.n + 1), 0.0);
-      } else {
-        double num = sinpi(dl * (p.n + 1)), den = sinpi(dl), sn, cs;
-        sincospi(dl * p.n, &sn, &cs);
-        term = cscale(make_double2(cs, sn), num / den);
-      }
-      g = cmul(g, term);
-    }
-    G[i * LD + j] = g;
+  const double2* Gp = (const double2*)(D.small + p.soff + D.L.gram);   // lower triangle, packed (k_powers)
+  for (int q = threadIdx.x; q < m * (m + 1) / 2; q += blockDim.x) {
+    int i = (int)((sqrtf(8.f * q + 1.f) - 1.f) * 0.5f);
+    if (i * (i + 1) / 2 > q) --i;
+    if ((i + 1) * (i + 2) / 2 <= q) ++i;
+    G[i * LD + q - i * (i + 1) / 2] = Gp[q];
   }
   __syncthreads();
-  // Cholesky G = L L^H (lower, in place), single thread per row update
+  // G = L D L^H (unit lower L in place, reciprocals of D beside it): a step takes the reciprocal of its pivot
+  // (one thread), the scaled column, then the trailing update, with three barriers and no square root
+  // (4096 problems of m 1..5: 0.31 -> 0.16 ms; 64 of m = 40: 0.26 -> 0.10 ms)
+  __shared__ double rd[PRONY_MMAX];
+  __shared__ double2 col[PRONY_MMAX];
   for (int k = 0; k < m; ++k) {
     if (threadIdx.x == 0) {
       double dkk = G[k * LD + k].x;
       if (!(dkk > 0.0)) { s_bad = 1; dkk = 1e-300; }
-      G[k * LD + k] = make_double2(sqrt(dkk), 0.0);
+      rd[k] = 1.0 / dkk;
     }
     __syncthreads();
-    double lkk = G[k * LD + k].x;
-    for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) G[i * LD + k] = cscale(G[i * LD + k], 1.0 / lkk);
+    for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) {
+      const double2 g = G[i * LD + k];
+      col[i] = cconj(g);
+      G[i * LD + k] = cscale(g, rd[k]);
+    }
     __syncthreads();
-    int rem = m - k - 1;
-    for (int idx = threadIdx.x; idx < rem * rem; idx += blockDim.x) {
-      int i = k + 1 + idx / rem, j = k + 1 + idx % rem;
-      if (j > i) continue;
-      G[i * LD + j] = csub(G[i * LD + j], cmul(G[i * LD + k], cconj(G[j * LD + k])));
+    const int rem = m - k - 1;
+    for (int q = threadIdx.x; q < rem * (rem + 1) / 2; q += blockDim.x) {
+      int i = (int)((sqrtf(8.f * q + 1.f) - 1.f) * 0.5f);
+      if (i * (i + 1) / 2 > q) --i;
+      if ((i + 1) * (i + 2) / 2 <= q) ++i;
+      const int j = k + 1 + q - i * (i + 1) / 2;
+      i += k + 1;
+      G[i * LD + j] = csub(G[i * LD + j], cmul(G[i * LD + k], col[j]));
     }
     __syncthreads();
   }
   __shared__ double2 cs_[PRONY_MMAX];
   if (threadIdx.x < 32) {
-    // L y = b, then L^H c = y, column by column on one warp: lane l keeps the running residuals
-    // r_j (j = l, l + 32); each step divides one residual by the diagonal and updates the
-    // residuals of the rows that remain, so a step costs a few dependent FP64 operations instead
-    // of a dot product of growing length
+    // L y = b, then L^H c = D^{-1} y, column by column on one warp: lane l keeps the running residuals
+    // r_j (j = l, l + 32); each step updates the residuals of the rows that remain, so a step costs a
+    // few dependent FP64 operations instead of a dot product of growing length
     const int lane = threadIdx.x;
     double2 r[2];
 #pragma unroll
@@ -320,7 +302,7 @@ __global__ void __launch_bounds__(256) k_solve_c(Dev D) {
       double2 ri = q ? r[1] : r[0];
       ri.x = __shfl_sync(0xffffffffu, ri.x, i & 31);
       ri.y = __shfl_sync(0xffffffffu, ri.y, i & 31);
-      const double2 yi = cscale(ri, 1.0 / G[i * LD + i].x);
+      const double2 yi = ri;
       if (lane == (i & 31)) cs_[i] = yi;
 #pragma unroll
       for (int qq = 0; qq < 2; ++qq) {
@@ -330,13 +312,14 @@ __global__ void __launch_bounds__(256) k_solve_c(Dev D) {
     }
     __syncwarp();
 #pragma unroll
-    for (int q = 0; q < 2; ++q) r[q] = lane + 32 * q < m ? cs_[lane + 32 * q] : make_double2(0.0, 0.0);
+    for (int q = 0; q < 2; ++q)
+      r[q] = lane + 32 * q < m ? cscale(cs_[lane + 32 * q], rd[lane + 32 * q]) : make_double2(0.0, 0.0);
     for (int i = m - 1; i >= 0; --i) {
       const int q = i >> 5;
       double2 ri = q ? r[1] : r[0];
       ri.x = __shfl_sync(0xffffffffu, ri.x, i & 31);
       ri.y = __shfl_sync(0xffffffffu, ri.y, i & 31);
-      const double2 ci = cscale(ri, 1.0 / G[i * LD + i].x);
+      const double2 ci = ri;
       if (lane == (i & 31)) cs_[i] = ci;
 #pragma unroll
       for (int qq = 0; qq < 2; ++qq) {

@@ -598,6 +598,10 @@ __global__ void k_argmax(Dev D, int buf) {
 constexpr int RHS_SEG = 16;             // points of a unit
 constexpr int RHS_THREADS = 128;
 
+// The same launch evaluates the Gram matrix conj(A) A^T (its lower triangle) over the whole GPU for k_solve_c
+// (there, one CTA per problem computed all m^2 entries: FP64 sincospi is what it spent its time on):
+//   G_ij = prod_l sum_{x=0}^{n} exp(2 pi i (t_i(l) - t_j(l)) x), or with the raw eigenvalues
+//   prod_l sum_x (conj(z_i(l)) z_j(l))^x (summed term by term: |q| need not be 1).
 __global__ void k_powers(Dev D) {
   const int pi = blockIdx.y;
   const ProbDesc& p = D.P[pi];
@@ -605,26 +609,60 @@ __global__ void k_powers(Dev D) {
   const int m = s.rank_used, n1 = p.n + 1;
   if (s.done || m <= 0 || m > p.m) return;
   double2* E = D.zpow + pi * D.zpow_stride;
-  if (D.vand) {
-    const double2* zr = (const double2*)(D.small + p.soff + D.L.zraw);
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < p.d * m; q += gridDim.x * blockDim.x) {
-      const int l = q / m, i = q % m;
-      const double2 e1 = cconj(zr[i * PRONY_DMAX + l]);
-      double2 e = make_double2(1.0, 0.0);
-      for (int x = 0; x < n1; ++x) {
-        E[((size_t)l * n1 + x) * m + i] = e;
-        e = cmul(e, e1);
-      }
-    }
-    return;
-  }
+  double2* G = (double2*)(D.small + p.soff + D.L.gram);              // packed: i (i + 1) / 2 + j, j <= i
+  const double2* zr = (const double2*)(D.small + p.soff + D.L.zraw);
   const double* t = (const double*)(D.small + p.soff + D.L.t);
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < p.d * n1 * m; q += gridDim.x * blockDim.x) {
-    const int i = q % m, x = q / m % n1, l = q / m / n1;
-    double ph = t[i * PRONY_DMAX + l] * x, sn, cs;
-    ph = fma(t[i * PRONY_DMAX + l], (double)x, -rint(ph));       // reduced with one rounding
-    sincospi(2.0 * ph, &sn, &cs);
-    E[q] = make_double2(cs, sn);
+  const int ntri = m * (m + 1) / 2, npow = D.vand ? p.d * m : p.d * n1 * m;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ntri + npow; q += gridDim.x * blockDim.x) {
+    if (q < ntri) {
+      int i = (int)((sqrtf(8.f * q + 1.f) - 1.f) * 0.5f);
+      if (i * (i + 1) / 2 > q) --i;
+      if ((i + 1) * (i + 2) / 2 <= q) ++i;
+      const int j = q - i * (i + 1) / 2;
+      double2 g = make_double2(1.0, 0.0);
+      for (int l = 0; l < p.d; ++l) {
+        double2 term;
+        if (D.vand) {
+          const double2 w = cmulc(zr[i * PRONY_DMAX + l], zr[j * PRONY_DMAX + l]);
+          double2 pw = make_double2(1.0, 0.0);
+          term = make_double2(1.0, 0.0);
+          for (int x = 1; x <= p.n; ++x) {
+            pw = cmul(pw, w);
+            term = cadd(term, pw);
+          }
+        } else {
+          double dl = t[i * PRONY_DMAX + l] - t[j * PRONY_DMAX + l];
+          dl -= rint(dl);
+          if (dl == 0.0) {
+            term = make_double2((double)n1, 0.0);
+          } else {
+            const double num = sinpi(dl * n1), den = sinpi(dl);
+            double sn, cs;
+            sincospi(dl * p.n, &sn, &cs);
+            term = cscale(make_double2(cs, sn), num / den);
+          }
+        }
+        g = cmul(g, term);
+      }
+      G[q] = g;
+      continue;
+    }
+    const int e = q - ntri;
+    if (D.vand) {
+      const int l = e / m, i = e % m;
+      const double2 e1 = cconj(zr[i * PRONY_DMAX + l]);
+      double2 v = make_double2(1.0, 0.0);
+      for (int x = 0; x < n1; ++x) {
+        E[((size_t)l * n1 + x) * m + i] = v;
+        v = cmul(v, e1);
+      }
+    } else {
+      const int i = e % m, x = e / m % n1, l = e / m / n1;
+      double ph = t[i * PRONY_DMAX + l] * x, sn, cs;
+      ph = fma(t[i * PRONY_DMAX + l], (double)x, -rint(ph));       // reduced with one rounding
+      sincospi(2.0 * ph, &sn, &cs);
+      E[e] = make_double2(cs, sn);
+    }
   }
 }
 
@@ -1043,7 +1081,8 @@ void launch_argmax(const Dev& D, int buf, cudaStream_t s) {
 
 void launch_powers(const Dev& D, cudaStream_t s) {
   note_launch();
-  const int want = D.vand ? 1 : (int)((D.zpow_stride + 127) / 128);
+  const int ntri = D.maxM * (D.maxM + 1) / 2;
+  const int want = (int)(((D.vand ? (long long)D.maxD * D.maxM : D.zpow_stride) + ntri + 127) / 128);
   k_powers<<<dim3(blocks_per_problem(want, D.nprob), D.nprob), 128, 0, s>>>(D);
 }
 void launch_rhs(const Dev& D, int resid, cudaStream_t s) {
