@@ -149,34 +149,36 @@ __global__ void k_zero_small(Dev D, long long off, long long bytes) {
 // so that the batch gives a few blocks per SM: few blocks per problem means few FP64 atomics on
 // the same output entries).
 //
-// Rows are staged RS at a time in two alternating shared-memory buffers (RS = 128 down to 8: the
-// most that the staged columns of this problem leave room for): each thread loads the next rows'
-// values into registers while the current ones are multiplied, then stores them.  A thread stages one row (its row index is computed once per
-// pass) and several columns; the values are stored column-major with a row pitch of RS + 1 and
-// pre-arranged for paired FP32 FMAs (fma.rn.f32x2): x as (Re x, Re x, Im x, Im x) and z as
-// (Re z, Im z, Im z, -Re z), so that conj(x) z is two paired FMAs on (re, im) accumulators.
+// Rows are staged RS at a time through three shared-memory buffers filled by cp.async (two passes in flight while
+// one is multiplied; rows past the end are zeros).  A buffer holds the values as they are in memory, column-major,
+// with a row pitch of RS + 2: a pair of rows is one 16-byte load, and consecutive columns lie in different banks.
+// The products are paired FP32 FMAs on whole values: acc1 += (Re x Re z, Im x Im z) and
+// acc2 += (Re x Im z, Im x Re z), with conj(x) z = (acc1.lo + acc1.hi) + i (acc2.lo - acc2.hi) at the end, so that
+// nothing but a swap of z is rearranged.  What bounds a 4 x 4 tile is then shared memory and the FP32 pipe about
+// equally; values stored as the four floats of two paired operands took twice the loads (64 blocks of 8000 x 80:
+// 0.69 ms, now 0.45; a solve of 4096 problems with n 7..31: 5.3 -> 1.9 ms of Gram sums, with blocks of 128 threads).
 // Output ownership is interleaved: thread (ti, tj) owns the entries (ti + NA i, tj + NB j),
 // i, j < 4, so the threads of a warp read consecutive columns (different banks) or the same one
-// (broadcast).  When there are fewer 4x4 tiles than threads, threads split the staged rows into
+// (broadcast).  When there are fewer 4x4 tiles than threads, threads split the staged row pairs into
 // row groups whose partial sums are added in shared memory; when there are more, the tiles are
 // processed in batches (every batch re-stages the rows).  Each block stores its partial Gram; the
 // last block of the problem (or k_gram_sum) adds the partials (FP32, a fixed order) and writes the FP64 output.
-constexpr int GRAM_T = 4;           // register tile (GRAM_T x GRAM_T complex accumulators)
-constexpr int GRAM_KMAX = 10;       // staged values per thread and pass: (a + b) RS <= 256 GRAM_KMAX
+constexpr int GRAM_T = 4;           // register tile (GRAM_T x GRAM_T entries, two packed sums each)
+constexpr int GRAM_STAGES = 3;      // staging buffers
+constexpr int GRAM_RED = GRAM_T * GRAM_T + 1;        // pitch of a thread's sums in the group reduction
 
-// Narrow blocks: more rows per pass, fewer passes of one load latency each (4096 problems of up to 20 columns,
-// N up to 1024: 6.0 -> 5.3 ms a solve).
-__host__ __device__ inline int gram_rows(int LR) { return LR <= 24 ? 64 : LR <= 40 ? 32 : LR <= 80 ? 16 : 8; }
-// float4 entries of one staging buffer (sized by the widest blocks of the batch, LR columns)
-__host__ __device__ inline int gram_buf_elems(int LR) { return 2 * LR * (gram_rows(LR) + 1); }
-// Rows staged per pass for a block of `cols` staged columns (float4 each) of which `loaded` are
-// read from HBM: the most (128 down to 8) that fit the buffer and the staging registers.
-__device__ inline int gram_rows_for(int cols, int loaded, int LR) {
+__host__ __device__ inline int gram_rows(int LR) { return LR <= 40 ? 32 : 16; }
+// float2 entries of one staging buffer (sized by the widest blocks of the batch, LR columns)
+__host__ __device__ inline int gram_buf_elems(int LR) { return 2 * LR * (gram_rows(LR) + 2); }
+// Rows staged per pass for a block of `cols` staged columns: the most (128 down to 8) that fit the buffer.
+__device__ inline int gram_rows_for(int cols, int LR) {
   const int cap = gram_buf_elems(LR);
   int rs = 128;
-  while (rs > 8 && (cols * (rs + 1) > cap || loaded * rs > 256 * 10)) rs >>= 1;
+  while (rs > 8 && cols * (rs + 2) > cap) rs >>= 1;
   return rs;
 }
+// Threads of a block: narrow blocks have few tiles and are bound by latency, so more and smaller blocks per SM
+inline int gram_threads(int LR) { return LR <= 24 ? 128 : 256; }
 
 __device__ __forceinline__ unsigned long long pk2(float lo, float hi) {
   unsigned long long r;
@@ -188,8 +190,18 @@ __device__ __forceinline__ float2 upk2(unsigned long long v) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
   return make_float2(lo, hi);
 }
+__device__ __forceinline__ unsigned long long swap2(unsigned long long v) {
+  unsigned long long r;
+  asm("{ .reg .b32 lo, hi; mov.b64 {lo, hi}, %1; mov.b64 %0, {hi, lo}; }" : "=l"(r) : "l"(v));
+  return r;
+}
 __device__ __forceinline__ void ffma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool valid) {   // (zeros when not valid)
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;"
+               ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 8 : 0)
+               : "memory");
 }
 
 __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, int xw, int zbuf, int zshift, int zw,
@@ -204,15 +216,14 @@ __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, in
   if (r_begin >= p.N || a <= 0 || b <= 0) return;
   const int r_end = min(p.N, r_begin + chunk);
   const int LR = D.L.LDR;
-  // X^* X (same buffer, shift and width): the rows are loaded once and only the tiles on and
+  // X^* X (same buffer, shift and width): the rows are staged once and only the tiles on and
   // above the diagonal are computed, the others written as their conjugate mirrors
   const bool sym = xbuf == zbuf && xshift == zshift && a == b;
-  // staged columns: a of X, then b of Z (for X^* X the second form of the same a columns)
-  const int ZC = a;                                // first staged column of Z
-  const int RS = gram_rows_for(a + b, sym ? a : a + b, LR), PR = RS + 1;
-  const size_t buf_elems = (size_t)gram_buf_elems(LR);   // X then Z, column-major with row pitch PR
-  // [RG-1][per_batch][16] packed partial sums, over the staging buffers once the rows are done
-  unsigned long long* red = (unsigned long long*)smem4;
+  const int ncols = sym ? a : a + b, ZC = sym ? 0 : a;   // staged columns: of X, then of Z
+  const int RS = gram_rows_for(ncols, LR), PR = RS + 2;
+  const int buf_elems = gram_buf_elems(LR);
+  float2* stage = (float2*)smem4;
+  float2* red = (float2*)smem4;                    // [RG][per_batch][GRAM_RED], over the buffers once the rows are done
   int ldx, ldz;
   const float2* X = buf_base(D, xbuf, p, ldx);
   const float2* Z = buf_base(D, zbuf, p, ldz);
@@ -220,44 +231,27 @@ __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, in
   const int ntile = sym ? NA * (NA + 1) / 2 : NA * NB;
   const int nthr = blockDim.x;
   const int per_batch = min(ntile, nthr);
-  const int RG = max(1, min(RS, nthr / per_batch));    // row groups (1 when tiles >= threads)
+  const int RG = max(1, min(RS / 2, nthr / per_batch));   // row groups (1 when tiles >= threads)
   const int nbatch = (ntile + per_batch - 1) / per_batch;
   double2* out = (double2*)(D.small + p.soff + out_off);
   float2* mine = (float2*)red_region(D, pi) + (size_t)blockIdx.x * a * b;   // this block's partial Gram
   const bool mine_ok = ws_ok(D, 8LL * a * b * (blockIdx.x + 1) <= D.red_stride, 12);
-  // staging role: one row, columns c0, c0 + cstep, ... (k-th: X column if below a, else Z)
+  // staging role: one row, columns c0, c0 + cstep, ...
   const int my_rr = threadIdx.x % RS, c0 = threadIdx.x / RS, cstep = nthr / RS;
-  float2 held[GRAM_KMAX];
-  auto load_rows = [&](int r0) {
-    const int r = r0 + my_rr;
-    const bool ok = r < r_end;
-    const int gx = ok ? buf_row(xbuf, p, r, xshift) : 0, gz = ok ? buf_row(zbuf, p, r, zshift) : 0;
-    const int ncols = sym ? a : a + b;
-#pragma unroll
-    for (int k = 0; k < GRAM_KMAX; ++k) {
-      const int col = c0 + k * cstep;
-      float2 v = make_float2(0.f, 0.f);
-      if (ok && col < ncols) v = col < a ? X[(long long)col * ldx + gx] : Z[(long long)(col - a) * ldz + gz];
-      held[k] = v;
+  auto issue = [&](int r0, int buf) {
+    if (r0 < r_end) {
+      const int r = r0 + my_rr;
+      const bool ok = r < r_end;
+      const float2* x = X + (ok ? buf_row(xbuf, p, r, xshift) : 0);
+      const float2* z = Z + (ok && !sym ? buf_row(zbuf, p, r, zshift) : 0);
+      float2* dst = stage + (size_t)buf * buf_elems + my_rr;
+      for (int col = c0; col < ncols; col += cstep)
+        cp_async8(dst + col * PR, col < a ? x + (long long)col * ldx : z + (long long)(col - a) * ldz, ok);
     }
-  };
-  auto store_rows = [&](int buf) {
-    float4* Xs = smem4 + (size_t)buf * buf_elems;
-#pragma unroll
-    for (int k = 0; k < GRAM_KMAX; ++k) {
-      const int col = c0 + k * cstep;
-      const float2 v = held[k];
-      // X and Z regions are contiguous: Z column c sits at column ZC + c of the buffer
-      if (col < a) {
-        Xs[col * PR + my_rr] = make_float4(v.x, v.x, v.y, v.y);
-        if (sym) Xs[(col + ZC) * PR + my_rr] = make_float4(v.x, v.y, v.y, -v.x);
-      } else if (!sym && col < a + b) {
-        Xs[(col - a + ZC) * PR + my_rr] = make_float4(v.x, v.y, v.y, -v.x);
-      }
-    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
   for (int batch = 0; batch < nbatch; ++batch) {
-    const int tile = batch * per_batch + threadIdx.x % per_batch, grp = threadIdx.x / per_batch;
+    const int tl = threadIdx.x % per_batch, tile = batch * per_batch + tl, grp = threadIdx.x / per_batch;
     const bool active = grp < RG && tile < ntile;
     int ti = tile / NB, tj = tile % NB;
     if (sym) {                                    // tile -> (ti, tj), ti <= tj, row by row
@@ -277,79 +271,86 @@ __global__ void __launch_bounds__(256, 2) k_gram(Dev D, int xbuf, int xshift, in
       xo[i] = min(ti + NA * i, a - 1) * PR;
       zo[i] = (min(tj + NB * i, b - 1) + ZC) * PR;
     }
-    unsigned long long acc[GRAM_T][GRAM_T];
+    unsigned long long acc1[GRAM_T][GRAM_T], acc2[GRAM_T][GRAM_T];
 #pragma unroll
     for (int i = 0; i < GRAM_T; ++i)
 #pragma unroll
-      for (int j = 0; j < GRAM_T; ++j) acc[i][j] = 0ull;
+      for (int j = 0; j < GRAM_T; ++j) acc1[i][j] = acc2[i][j] = 0ull;
     __syncthreads();                              // the buffers are free (previous batch done)
-    load_rows(r_begin);
-    store_rows(0);
-    int k = 0;
-    for (int r0 = r_begin; r0 < r_end; r0 += RS, k ^= 1) {
-      const bool more = r0 + RS < r_end;
-      if (more) load_rows(r0 + RS);               // in flight while these rows are multiplied
-      __syncthreads();
-      // each staged value is 16 bytes read as two packed pairs: x = ((Re x, Re x), (Im x, Im x)),
-      // z = ((Re z, Im z), (Im z, -Re z))
-      const ulonglong2* Bs = (const ulonglong2*)(smem4 + (size_t)k * buf_elems);
+    issue(r_begin, 0);
+    issue(r_begin + RS, 1);
+    int buf = 0;
+    for (int r0 = r_begin; r0 < r_end; r0 += RS) {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();                            // these rows are there; the buffer of the pass before is free
+      issue(r0 + 2 * RS, buf == 0 ? 2 : buf - 1);
+      const float2* Bs = stage + (size_t)buf * buf_elems;
       if (active) {
-        const int nrows = min(RS, r_end - r0);
-        for (int rr = grp; rr < nrows; rr += RG) {
+        const int npair = (min(RS, r_end - r0) + 1) / 2;
+        for (int rp = grp; rp < npair; rp += RG) {
           ulonglong2 xa[GRAM_T], zb[GRAM_T];
 #pragma unroll
-          for (int i = 0; i < GRAM_T; ++i) xa[i] = Bs[xo[i] + rr];
+          for (int i = 0; i < GRAM_T; ++i) xa[i] = *(const ulonglong2*)(Bs + xo[i] + 2 * rp);
 #pragma unroll
-          for (int j = 0; j < GRAM_T; ++j) zb[j] = Bs[zo[j] + rr];
+          for (int j = 0; j < GRAM_T; ++j) zb[j] = *(const ulonglong2*)(Bs + zo[j] + 2 * rp);
 #pragma unroll
-          for (int i = 0; i < GRAM_T; ++i)
+          for (int j = 0; j < GRAM_T; ++j) {
+            const unsigned long long s0 = swap2(zb[j].x), s1 = swap2(zb[j].y);
 #pragma unroll
-            for (int j = 0; j < GRAM_T; ++j) {
-              ffma2(acc[i][j], xa[i].x, zb[j].x);   // (Re x Re z, Re x Im z)
-              ffma2(acc[i][j], xa[i].y, zb[j].y);   // + (Im x Im z, -Im x Re z)
-            }
-        }
-      }
-      if (more) store_rows(k ^ 1);                // the other buffer was released by the sync above
-    }
-    // row groups: partial sums meet in shared memory, group 0 adds them (fixed order)
-    if (RG > 1) {
-      __syncthreads();                            // every group is done with the staged rows
-      if (active && grp > 0) {
-        unsigned long long* dst = red + ((size_t)(grp - 1) * per_batch + (tile - batch * per_batch)) * 16;
-#pragma unroll
-        for (int i = 0; i < GRAM_T; ++i)
-#pragma unroll
-          for (int j = 0; j < GRAM_T; ++j) dst[i * GRAM_T + j] = acc[i][j];
-      }
-      __syncthreads();
-      if (active && grp == 0) {
-        for (int g = 1; g < RG; ++g) {
-          const unsigned long long* src = red + ((size_t)(g - 1) * per_batch + (tile - batch * per_batch)) * 16;
-#pragma unroll
-          for (int i = 0; i < GRAM_T; ++i)
-#pragma unroll
-            for (int j = 0; j < GRAM_T; ++j) {
-              const float2 u = upk2(acc[i][j]), v = upk2(src[i * GRAM_T + j]);
-              acc[i][j] = pk2(u.x + v.x, u.y + v.y);
-            }
-        }
-      }
-    }
-    if (active && grp == 0) {
-#pragma unroll
-      for (int i = 0; i < GRAM_T; ++i)
-#pragma unroll
-        for (int j = 0; j < GRAM_T; ++j) {
-          const int ia = ti + NA * i, jb = tj + NB * j;
-          if (ia < a && jb < b) {
-            const float2 v = upk2(acc[i][j]);
-            if (mine_ok) {
-              mine[ia * b + jb] = v;
-              if (sym && ti != tj) mine[jb * b + ia] = make_float2(v.x, -v.y);   // mirror of a tile above the diagonal
+            for (int i = 0; i < GRAM_T; ++i) {
+              ffma2(acc1[i][j], xa[i].x, zb[j].x);
+              ffma2(acc2[i][j], xa[i].x, s0);
+              ffma2(acc1[i][j], xa[i].y, zb[j].y);
+              ffma2(acc2[i][j], xa[i].y, s1);
             }
           }
         }
+      }
+      buf = buf == GRAM_STAGES - 1 ? 0 : buf + 1;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // one entry of the block's sums: the tile's (i, j)-th
+    auto put = [&](int ti, int tj, int i, int j, float2 v) {
+      const int ia = ti + NA * i, jb = tj + NB * j;
+      if (mine_ok && ia < a && jb < b) {
+        mine[ia * b + jb] = v;
+        if (sym && ti != tj) mine[jb * b + ia] = make_float2(v.x, -v.y);   // mirror of a tile above the diagonal
+      }
+    };
+    auto sum_of = [&](int i, int j) {
+      const float2 u = upk2(acc1[i][j]), v = upk2(acc2[i][j]);
+      return make_float2(u.x + u.y, v.x - v.y);
+    };
+    if (RG == 1) {
+      if (active)
+#pragma unroll
+        for (int i = 0; i < GRAM_T; ++i)
+#pragma unroll
+          for (int j = 0; j < GRAM_T; ++j) put(ti, tj, i, j, sum_of(i, j));
+    } else {
+      // row groups: their sums meet in shared memory and are added in the order of the groups, an entry per
+      // thread (there is one batch then)
+      __shared__ int s_tile[256];
+      __syncthreads();                            // every group is done with the staged rows
+      if (active) {
+        if (grp == 0) s_tile[tl] = ti | tj << 16;
+        float2* dst = red + (size_t)(grp * per_batch + tl) * GRAM_RED;
+#pragma unroll
+        for (int i = 0; i < GRAM_T; ++i)
+#pragma unroll
+          for (int j = 0; j < GRAM_T; ++j) dst[i * GRAM_T + j] = sum_of(i, j);
+      }
+      __syncthreads();
+      for (int q = threadIdx.x; q < per_batch * 16; q += nthr) {
+        const int t = q >> 4, e = q & 15;
+        float2 v = red[(size_t)t * GRAM_RED + e];
+        for (int g = 1; g < RG; ++g) {
+          const float2 u = red[(size_t)(g * per_batch + t) * GRAM_RED + e];
+          v.x += u.x;
+          v.y += u.y;
+        }
+        put(s_tile[t] & 0xffff, s_tile[t] >> 16, e >> 2, e & 3, v);
+      }
     }
   }
   // The blocks' partial Grams (one slot of a x b each) added in FP32 in a fixed order: slot k
@@ -995,28 +996,30 @@ static void gram_attr(size_t sm) {
 }
 
 // Launch geometry of k_gram for a batch: dynamic shared memory, rows per block and blocks per
-// problem (the batch fills the resident blocks once, at least RS rows per block).
+// problem (the batch fills the resident blocks once or twice, at least RS rows per block).
 static void gram_geometry(const Dev& D, size_t& sm, int& chunk, int& nblk) {
   static std::map<size_t, int> slots_for;      // shared memory size -> resident blocks on the GPU
-  // two buffers of staged rows of X and Z (float4 per value); afterwards the same space holds the
-  // row-group partial sums, (RG - 1) x tiles x 16 packed entries with RG = min(RS, 256 / tiles):
-  // fewer than 256 x 16
-  const int RS = gram_rows(D.L.LDR);
-  sm = std::max(sizeof(float4) * (4 * (size_t)D.L.LDR * (RS + 1)), sizeof(unsigned long long) * 256 * 16);
+  // the staging buffers (float2 per value); afterwards the same space holds the sums of the row groups, at most
+  // one thread's per thread
+  const int RS = gram_rows(D.L.LDR), nthr = gram_threads(D.L.LDR);
+  sm = sizeof(float2) * std::max<size_t>((size_t)GRAM_STAGES * gram_buf_elems(D.L.LDR), (size_t)nthr * GRAM_RED);
   auto it = slots_for.find(sm);
   if (it == slots_for.end()) {
     int occ = 1, dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     gram_attr(sm);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gram, 256, sm) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gram, nthr, sm) != cudaSuccess) {
       cudaGetLastError();
       occ = 2;
     }
     it = slots_for.emplace(sm, std::max(1, occ) * sms).first;
   }
   // at most 64 blocks per problem: the last block of a problem adds every block's partial Gram
-  const int per_prob = std::max(1, std::min(64, it->second / std::max(1, D.nprob)));
+  const int np = std::max(1, D.nprob), slots = it->second;
+  int per_prob = std::max(1, std::min(64, slots / np));
+  // (a whole number per problem that leaves over a tenth of the resident blocks empty: two rounds of half the rows)
+  if ((long long)np * per_prob * 10 < 9LL * slots && per_prob < 64) per_prob = std::min(64, 2 * slots / np);
   chunk = std::max(RS, (D.maxN + per_prob - 1) / per_prob);
   chunk = (chunk + RS - 1) / RS * RS;
   nblk = (D.maxN + chunk - 1) / chunk;
@@ -1052,7 +1055,7 @@ void launch_gram(const Dev& D, int xbuf, int xshift, int xw, int zbuf, int zshif
   dim3 g(nblk, D.nprob);
   note_launch();
   const int own_sum = nblk <= 8;                 // few partials: the last block adds them
-  k_gram<<<g, 256, sm, s>>>(D, xbuf, xshift, xw, zbuf, zshift, zw, out_off, out_ld, chunk, own_sum);
+  k_gram<<<g, gram_threads(D.L.LDR), sm, s>>>(D, xbuf, xshift, xw, zbuf, zshift, zw, out_off, out_ld, chunk, own_sum);
   if (!own_sum) {
     note_launch();
     k_gram_sum<<<dim3((D.L.LDR * D.L.LDR + 255) / 256, D.nprob), 256, 0, s>>>(D, xw, zw, out_off, out_ld, chunk);
