@@ -21,8 +21,8 @@
 //               written straight into tensor memory (tcgen05.st); two warps per TMEM
 //               lane quadrant, each taking half of the chunk's input points; then the epilogue
 // The Toeplitz matrix is never formed in HBM: each A' element is F at grid index gk(k) - gh(h).
-// A pipeline stage is one K chunk (its B' tile in shared memory and its A' tile in tensor
-// memory); one full and one empty mbarrier per stage; every wait is bounded.
+// A pipeline stage is one K chunk: a ring of B' tiles in shared memory and one of A' tiles in tensor memory,
+// each with one full and one empty mbarrier per stage; every wait is bounded.
 // Split K: the CTAs of one row tile (consecutive jobs) each store their FP32 partial tile in a
 // workspace slot; the last of them to finish (a per-tile arrival counter) adds the partials in
 // the order of their K ranges and writes Y, so results do not depend on which CTA ends first.
@@ -41,10 +41,10 @@ namespace {
 constexpr int TC_BM = 128;
 constexpr uint32_t TC_SPIN = 1u << 24;      // bounded mbarrier polls (~seconds)
 constexpr int TC_MAXSTAGE = 8;
-// A' warps: eight (two per TMEM lane quadrant, each taking half of a chunk's points) in a CTA that has the
-// SM to itself; four, each taking both halves in turn, where two CTAs share the SM (256 columns of
-// tensor memory and half of the shared memory each)
-constexpr int TC_APROD = 8, TC_APROD2 = 4;
+// A' warps: two per TMEM lane quadrant, each taking half of a chunk's points, also where two CTAs share the SM
+// (256 columns of tensor memory and half of the shared memory each): four warps there, each taking both halves in
+// turn, left the schedulers idle two cycles in three (products of 4096 problems, n 7..31: 13.7 ms, eight 12.8 ms)
+constexpr int TC_APROD = 8;
 constexpr int TC_MAXCH = 512;               // K chunks per CTA (host splits K to stay below)
 enum TcMode { TC_PRODUCT = 0, TC_GRAM = 1, TC_APPLY = 2 };
 
@@ -314,10 +314,11 @@ __device__ __forceinline__ void tc_load_acc(uint32_t taddr, bool stacked, int NT
 //               and an a x b matrix M of the small workspace: A' row r = X[r, :] read from HBM
 //               ([Re x | Im x] per chunk of 32 columns), B' = M by k_xb_prep, one CTA per row tile
 //               and the whole K range (no split), OUT stored like a product.
-template <int KIND, int MODE, int AW, int FMT>
-__global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
+template <int KIND, int MODE, int FMT, bool HALF>
+__global__ void __launch_bounds__(32 * (2 + TC_APROD), HALF ? 2 : 1)
     k_toeplitz_tc(Dev D, const ToeplitzJob* jobs, TcParams P, int* err) {
-  constexpr uint32_t TMEM_COLS = AW == TC_APROD ? 512 : 256;
+  constexpr int AW = TC_APROD;
+  constexpr uint32_t TMEM_COLS = HALF ? 256 : 512;
   using K = TcKind<KIND>;
   constexpr bool GRAM = MODE == TC_GRAM, APPLY = MODE == TC_APPLY;
   constexpr bool HBMA = GRAM || APPLY;              // A' read from a tall block in HBM, no window
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
   constexpr int GPL = K::TF32 ? 2 : 3;            // planes per part in the global tables
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint64_t bar_win, bar_d;
-  __shared__ uint64_t bar_full[TC_MAXSTAGE], bar_empty[TC_MAXSTAGE];
+  __shared__ uint64_t bar_bfull[TC_MAXSTAGE], bar_bempty[TC_MAXSTAGE], bar_afull[TC_MAXSTAGE], bar_aempty[TC_MAXSTAGE];
   __shared__ uint32_t s_tmem;
   __shared__ int s_err, s_last;
   __shared__ int ghalf[2 * TC_MAXCH];   // grid offset of each half chunk on one grid line, else -1
@@ -358,11 +359,13 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
   const int nchunks = max(0, c_end - c_begin);
   const int NT = ((2 * w + 15) / 16) * 16;
   const TcLayout lay = tc_layout<KIND>(NT, TMEM_COLS);
-  // One pipeline stage = one K chunk: its B' tile in shared memory and its A' tile in tensor
-  // memory, filled together (full barrier: eight A' warps + the loader's byte count) and
-  // released together by one commit of the MMAs that read them.
-  const int S = min(P.stages, lay.sa);
-  if (nchunks > TC_MAXCH || NT > P.ntbox || S < 1) {   // host sizing rules these out
+  // Two rings of K chunks: B' tiles in shared memory (filled by the loader's bulk copies) and A' tiles in
+  // tensor memory (filled by the eight A' warps), each stage released by a commit of the MMAs that read it.
+  // The accumulator may leave tensor memory for one A' stage only; the B' tiles then still arrive ahead (with
+  // one ring of the smaller count, each chunk waited for its copy
+  // from L2: 12.8 ms for the products of 4096 problems with n 7..31, now 10.9).
+  const int SB = P.stages, SA = lay.sa;
+  if (nchunks > TC_MAXCH || NT > P.ntbox || SB < 1 || SB > TC_MAXSTAGE || SA < 1) {   // host sizing rules these out
     if (threadIdx.x == 0) atomicExch(err, 3);
     return;
   }
@@ -406,9 +409,13 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
   if (threadIdx.x == 32) {
     mbar_init(&bar_win, 1);
     mbar_init(&bar_d, 1);
-    for (int i = 0; i < S; ++i) {
-      mbar_init(&bar_full[i], AW + 1);          // the A' warps + the loader (with the byte count)
-      mbar_init(&bar_empty[i], 1);              // the commit of the stage's MMAs
+    for (int i = 0; i < SB; ++i) {
+      mbar_init(&bar_bfull[i], 1);              // the loader (with the byte count)
+      mbar_init(&bar_bempty[i], 1);             // the commit of the stage's MMAs
+    }
+    for (int i = 0; i < SA; ++i) {
+      mbar_init(&bar_afull[i], AW);             // the A' warps
+      mbar_init(&bar_aempty[i], 1);
     }
     s_err = 0;
     s_last = 0;
@@ -444,17 +451,19 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
       uint32_t ph = 0;                            // stage and round parity (no divisions in the loop)
       for (int it = 0; it < nchunks; ++it) {
         // stage s is free once the MMAs that read its previous contents have completed
-        if (it >= S && !mbar_wait_spin(&bar_empty[s], ph ^ 1u, TC_SPIN)) { s_err = 1; break; }
-        mbar_arrive_expect_tx(&bar_full[s], tile_bytes);
-        tma_load_1d(Bs + (size_t)s * stage_bytes, src0 + (size_t)it * tile_bytes, tile_bytes, &bar_full[s]);
+        if (it >= SB && !mbar_wait_spin(&bar_bempty[s], ph ^ 1u, TC_SPIN)) { s_err = 1; break; }
+        mbar_arrive_expect_tx(&bar_bfull[s], tile_bytes);
+        tma_load_1d(Bs + (size_t)s * stage_bytes, src0 + (size_t)it * tile_bytes, tile_bytes, &bar_bfull[s]);
         ++issued;
-        if (++s == S) { s = 0; ph ^= 1u; }
+        if (++s == SB) { s = 0; ph ^= 1u; }
       }
       // Tail: the last stages are released by the MMAs that read them, so every copy into this
       // CTA has landed before it exits.
       if (!s_err)
-        for (int it = max(0, issued - S); it < issued; ++it)
-          if (!mbar_wait_spin(&bar_empty[it % S], (it / S) & 1, TC_SPIN)) { s_err = 1; break; }
+        for (int it = max(0, issued - SB); it < issued; ++it)
+          if (!mbar_wait_spin(&bar_bempty[it % SB], (it / SB) & 1, TC_SPIN)) { s_err = 1; break; }
+      if (s_err)                                  // without those MMAs: the copies themselves
+        for (int it = max(0, issued - SB); it < issued; ++it) mbar_wait(&bar_bfull[it % SB], (it / SB) & 1, TC_SPIN);
       if (!HBMA && !mbar_wait(&bar_win, 0, TC_SPIN)) s_err = 1;
     }
   } else if (warp == 1) {
@@ -466,16 +475,16 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
         const int n = lay.stacked ? (NPL - a) * NT : NT;
         idesc[a] = K::TF32 ? idesc_tf32_f32(TC_BM, n) : idesc_bf16_f32(TC_BM, n);
       }
-      int s = 0;
-      uint32_t ph = 0;
+      int sb = 0, sa = 0;
+      uint32_t phb = 0, pha = 0;
       for (int it = 0; it < nchunks; ++it) {
-        if (!mbar_wait_spin(&bar_full[s], ph, TC_SPIN)) {
+        if (!mbar_wait_spin(&bar_bfull[sb], phb, TC_SPIN) || !mbar_wait_spin(&bar_afull[sa], pha, TC_SPIN)) {
           s_err = 1;
           break;
         }
         tc_fence_after();
-        const uint32_t a0 = tb + lay.acol0 + (uint32_t)s * NPL * K::PCOLS;
-        const uint32_t bsm = smem_u32(Bs + (size_t)s * stage_bytes);
+        const uint32_t a0 = tb + lay.acol0 + (uint32_t)sa * NPL * K::PCOLS;
+        const uint32_t bsm = smem_u32(Bs + (size_t)sb * stage_bytes);
         // Operand-major order: all K steps of one MMA shape and operand pair before the next, so
         // consecutive MMAs share their instruction descriptor and operand planes (issuing them
         // K step by K step, with the descriptor or plane changing every MMA, was 2-7 % slower on
@@ -503,8 +512,10 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
               mma_ts(K::TF32, tb, a0 + PA[pr] * K::PCOLS + 8 * kk, bd, idesc[0], acc);
             }
         }
-        tc_commit(&bar_empty[s]);                 // releases the stage once these MMAs are done
-        if (++s == S) { s = 0; ph ^= 1u; }
+        tc_commit(&bar_aempty[sa]);               // release the stages once these MMAs are done
+        tc_commit(&bar_bempty[sb]);
+        if (++sa == SA) { sa = 0; pha ^= 1u; }
+        if (++sb == SB) { sb = 0; phb ^= 1u; }
       }
       tc_commit(&bar_d);                          // arrives when every MMA issued above has completed
     }
@@ -513,8 +524,7 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
     // Warps 2..: quadrant q = warp & 3 (TMEM lanes 32q..32q+31 = tile rows), half hh of every
     // K chunk (input points 32c + 16hh .. +15), or both halves in turn.
     const int q = warp & 3;
-    constexpr int HALVES = TC_APROD / AW;         // halves of a chunk per warp
-    const int hh0 = HALVES == 1 ? (warp - 2) >> 2 : 0;
+    const int hh = (warp - 2) >> 2;
     const int i = 32 * q + lane;                // row within the tile
     const int row = row0 + i;
     const bool vrow = row < rows_total;
@@ -524,6 +534,8 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
     const int grow = HBMA ? 0 : grid_of_row(vrow ? row : rows_total - 1, L, p);
     const int gk = HBMA ? 0 : K::TF32 ? grow - wlo : p.Gd4 - 1 - grow - wlo;
     const uint32_t lane_off = (uint32_t)(32 * q) << 16;
+    // floor(2^32 / (n + 1)): floor(x inv / 2^32) is floor(x / (n + 1)) or one less
+    const unsigned n1 = p.n + 1, inv_n1 = (unsigned)((1ull << 32) / n1);
     bool ok = idle || HBMA || __all_sync(0xffffffffu, mbar_wait(&bar_win, 0, TC_SPIN));
     if (!ok) s_err = 1;
     constexpr int NW = K::TF32 ? 16 : 8;          // words per part and plane: 16 points
@@ -537,176 +549,186 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
     int s = 0;
     uint32_t ph = 0;
     for (int it = 0; ok && it < nchunks; ++it) {
-      if (it >= S && !__all_sync(0xffffffffu, mbar_wait_spin(&bar_empty[s], ph ^ 1u, TC_SPIN))) {
-        s_err = 1;
-        break;
-      }
-#pragma unroll 1
-      for (int hh = hh0; hh < hh0 + HALVES; ++hh) {
-        const int g0 = HBMA ? 0 : ghalf[2 * it + hh];
-        // TMEM column of (plane pl, part, point j of this half): BF16 two points per column at
-        // pl * 32 + part * 16 + hh * 8 + j / 2; TF32 one point per column at pl * 64 + part * 32 + hh * 16 + j
-        const uint32_t a0 = tb + lane_off + lay.acol0 + (uint32_t)s * NPL * K::PCOLS + hh * NW;
-        // all table words of the chunk are loaded before the first tensor-memory store (the
-        // stores are compiler barriers), so the loads overlap
-        uint32_t wv[2][NPL][NW];
-        if (APPLY) {
-          // A'(r, i) = X[r, i] for the 16 columns i of this half chunk: parts Re x and Im x
-          const int i0 = 32 * (c_begin + it) + 16 * hh;
-          float v[2][16];
+      const int g0 = HBMA ? 0 : ghalf[2 * it + hh];
+      // TMEM column of (plane pl, part, point j of this half): BF16 two points per column at
+      // pl * 32 + part * 16 + hh * 8 + j / 2; TF32 one point per column at pl * 64 + part * 32 + hh * 16 + j
+      const uint32_t a0 = tb + lane_off + lay.acol0 + (uint32_t)s * NPL * K::PCOLS + hh * NW;
+      // all table words of the chunk are loaded before the first tensor-memory store (the
+      // stores are compiler barriers), so the loads overlap
+      uint32_t wv[2][NPL][NW];
+      if (APPLY) {
+        // A'(r, i) = X[r, i] for the 16 columns i of this half chunk: parts Re x and Im x
+        const int i0 = 32 * (c_begin + it) + 16 * hh;
+        float v[2][16];
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const float2 x = (vrow && i0 + jj < aw) ? xrow[(long long)(i0 + jj) * ldx_a] : make_float2(0.f, 0.f);
-            v[0][jj] = x.x;
-            v[1][jj] = x.y;
-          }
+        for (int jj = 0; jj < 16; ++jj) {
+          const float2 x = (vrow && i0 + jj < aw) ? xrow[(long long)(i0 + jj) * ldx_a] : make_float2(0.f, 0.f);
+          v[0][jj] = x.x;
+          v[1][jj] = x.y;
+        }
 #pragma unroll
-          for (int part = 0; part < 2; ++part) {
-            if (K::TF32) {
+        for (int part = 0; part < 2; ++part) {
+          if (K::TF32) {
 #pragma unroll
-              for (int e = 0; e < NW; ++e) {
-                uint32_t w2[2];
-                split_tf32(v[part][e], w2);
-                wv[part][0][e] = w2[0];
-                wv[part][NPL - 1][e] = w2[1];
-              }
-            } else {
+            for (int e = 0; e < NW; ++e) {
+              uint32_t w2[2];
+              split_tf32(v[part][e], w2);
+              wv[part][0][e] = w2[0];
+              wv[part][NPL - 1][e] = w2[1];
+            }
+          } else {
 #pragma unroll
-              for (int e = 0; e < NW; ++e) {
-                uint32_t w3[3];
-                split_pair<NPL>(v[part][2 * e], v[part][2 * e + 1], w3);
+            for (int e = 0; e < NW; ++e) {
+              uint32_t w3[3];
+              split_pair<NPL>(v[part][2 * e], v[part][2 * e + 1], w3);
 #pragma unroll
-                for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = w3[pl];
-              }
+              for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = w3[pl];
             }
           }
-        } else if (GRAM) {
-          // A'(i, r) = conj(X[r, i]) for the 16 rows r of this half chunk: parts Re x and -Im x
-          int ldx = 0;
-          const float2* X = tc_buf(D, P.xbuf, p, ldx);   // sets ldx: the column offset is added after
-          X += (long long)i * ldx;
-          const int r0c = 32 * (c_begin + it) + 16 * hh;
-          const bool box = P.xbuf == BUF_Y;
-          // on one line of I_n the rows of the box buffer are consecutive too
-          const bool line = r0c + 15 < p.N && (r0c % (p.n + 1)) + 15 <= p.n;
-          const int rb = (box && line && vrow) ? map_row(r0c, p.n, p.d, p.n + 2, P.xshift) : r0c;
-          float v[2][16];
+        }
+      } else if (GRAM) {
+        // A'(i, r) = conj(X[r, i]) for the 16 rows r of this half chunk: parts Re x and -Im x
+        int ldx = 0;
+        const float2* X = tc_buf(D, P.xbuf, p, ldx);   // sets ldx: the column offset is added after
+        X += (long long)i * ldx;
+        const int r0c = 32 * (c_begin + it) + 16 * hh;
+        const bool box = P.xbuf == BUF_Y;
+        // on one line of I_n the rows of the box buffer are consecutive too
+        const bool line = r0c + 15 < p.N && (r0c % (p.n + 1)) + 15 <= p.n;
+        const int rb = (box && line && vrow) ? map_row(r0c, p.n, p.d, p.n + 2, P.xshift) : r0c;
+        float v[2][16];
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const int r = r0c + jj;
-            float2 x = make_float2(0.f, 0.f);
-            if (vrow && r < p.N) x = X[(!box || line) ? rb + jj : map_row(r, p.n, p.d, p.n + 2, P.xshift)];
-            v[0][jj] = x.x;
-            v[1][jj] = -x.y;
-          }
+        for (int jj = 0; jj < 16; ++jj) {
+          const int r = r0c + jj;
+          float2 x = make_float2(0.f, 0.f);
+          if (vrow && r < p.N) x = X[(!box || line) ? rb + jj : map_row(r, p.n, p.d, p.n + 2, P.xshift)];
+          v[0][jj] = x.x;
+          v[1][jj] = -x.y;
+        }
 #pragma unroll
-          for (int part = 0; part < 2; ++part) {
-            if (K::TF32) {
+        for (int part = 0; part < 2; ++part) {
+          if (K::TF32) {
 #pragma unroll
-              for (int e = 0; e < NW; ++e) {
-                uint32_t w2[2];
-                split_tf32(v[part][e], w2);
-                wv[part][0][e] = w2[0];
-                wv[part][NPL - 1][e] = w2[1];
-              }
-            } else {
+            for (int e = 0; e < NW; ++e) {
+              uint32_t w2[2];
+              split_tf32(v[part][e], w2);
+              wv[part][0][e] = w2[0];
+              wv[part][NPL - 1][e] = w2[1];
+            }
+          } else {
 #pragma unroll
-              for (int e = 0; e < NW; ++e) {
-                uint32_t w3[3];
-                split_pair<NPL>(v[part][2 * e], v[part][2 * e + 1], w3);
+            for (int e = 0; e < NW; ++e) {
+              uint32_t w3[3];
+              split_pair<NPL>(v[part][2 * e], v[part][2 * e + 1], w3);
 #pragma unroll
-                for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = w3[pl];
-              }
+              for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = w3[pl];
             }
           }
-        } else if (g0 >= 0) {
-          // the 16 points lie on one grid line
-          const int x = K::TF32 ? gk - g0 : gk + g0;
-          const uint32_t sh = (uint32_t)(x & 1) << 4;
+        }
+      } else if (g0 >= 0) {
+        // the 16 points lie on one grid line
+        const int x = K::TF32 ? gk - g0 : gk + g0;
+        const uint32_t sh = (uint32_t)(x & 1) << 4;
+#pragma unroll
+        for (int part = 0; part < 2; ++part)
+#pragma unroll
+          for (int pl = 0; pl < NPL; ++pl) {
+            const unsigned char* Tb = wtab + (size_t)(part * NPL + pl) * P.win_cap * EB;
+            if (FMT == TT_TF32) {              // point j at entry x - j
+#pragma unroll
+              for (int e = 0; e < NW; ++e) wv[part][pl][e] = ((const uint32_t*)Tb)[x - e];
+            } else if (FMT == TT_WIDE) {       // points (2e, 2e + 1): the word at entry x + 2e
+#pragma unroll
+              for (int e = 0; e < NW; ++e) wv[part][pl][e] = ((const uint32_t*)Tb)[x + 2 * e];
+            } else {                           // joined from two aligned words by a 16-bit funnel shift
+              const uint32_t* T = (const uint32_t*)Tb + (x >> 1);
+              uint32_t w[NW + 1];
+#pragma unroll
+              for (int e = 0; e <= NW; ++e) w[e] = T[e];
+#pragma unroll
+              for (int e = 0; e < NW; ++e) wv[part][pl][e] = __funnelshift_r(w[e], w[e + 1], sh);
+            }
+          }
+      } else {
+        // points on several grid lines: each point from its own entry; points past N take the last
+        // one's samples (B' is zero there)
+        const int h = min(32 * (c_begin + it) + 16 * hh + (lane & 15), p.N - 1);
+        int ghl = 0;                           // grid_of_h, with the division as a multiplication
+        {
+          unsigned rem = h;
+          int mul = 1;
+          for (int l = p.d - 1; l > 0; --l) {
+            unsigned qt = __umulhi(rem, inv_n1), dg = rem - qt * n1;
+            if (dg >= n1) { dg -= n1; ++qt; }
+            ghl += dg * mul;
+            rem = qt;
+            mul *= p.G;
+          }
+          ghl += rem * mul;
+        }
+        if (FMT == TT_WIDE) {
+#pragma unroll
+          for (int e = 0; e < NW; ++e) {
+            const int ga = __shfl_sync(0xffffffffu, ghl, 2 * e), gb = __shfl_sync(0xffffffffu, ghl, 2 * e + 1);
+            const uint32_t* T = (const uint32_t*)wtab + gk + ga;
+            if (gb == ga + 1) {                // both on one line (the same for every row)
+#pragma unroll
+              for (int part = 0; part < 2; ++part)
+#pragma unroll
+                for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = T[(part * NPL + pl) * P.win_cap];
+            } else {
+#pragma unroll
+              for (int part = 0; part < 2; ++part)
+#pragma unroll
+                for (int pl = 0; pl < NPL; ++pl)
+                  wv[part][pl][e] = __byte_perm(T[(part * NPL + pl) * P.win_cap], T[(part * NPL + pl) * P.win_cap + gb - ga], 0x5410);
+            }
+          }
+        } else {
+          int xs[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const int g = __shfl_sync(0xffffffffu, ghl, j);
+            xs[j] = K::TF32 ? gk - g : gk + g;
+          }
 #pragma unroll
           for (int part = 0; part < 2; ++part)
 #pragma unroll
             for (int pl = 0; pl < NPL; ++pl) {
               const unsigned char* Tb = wtab + (size_t)(part * NPL + pl) * P.win_cap * EB;
-              if (FMT == TT_TF32) {              // point j at entry x - j
 #pragma unroll
-                for (int e = 0; e < NW; ++e) wv[part][pl][e] = ((const uint32_t*)Tb)[x - e];
-              } else if (FMT == TT_WIDE) {       // points (2e, 2e + 1): the word at entry x + 2e
-#pragma unroll
-                for (int e = 0; e < NW; ++e) wv[part][pl][e] = ((const uint32_t*)Tb)[x + 2 * e];
-              } else {                           // joined from two aligned words by a 16-bit funnel shift
-                const uint32_t* T = (const uint32_t*)Tb + (x >> 1);
-                uint32_t w[NW + 1];
-#pragma unroll
-                for (int e = 0; e <= NW; ++e) w[e] = T[e];
-#pragma unroll
-                for (int e = 0; e < NW; ++e) wv[part][pl][e] = __funnelshift_r(w[e], w[e + 1], sh);
-              }
-            }
-        } else {
-          // points on several grid lines: each point from its own entry; points past N take the last
-          // one's samples (B' is zero there)
-          const int h = min(32 * (c_begin + it) + 16 * hh + (lane & 15), p.N - 1);
-          const int ghl = grid_of_h(h, p);
-          if (FMT == TT_WIDE) {
-#pragma unroll
-            for (int e = 0; e < NW; ++e) {
-              const int ga = __shfl_sync(0xffffffffu, ghl, 2 * e), gb = __shfl_sync(0xffffffffu, ghl, 2 * e + 1);
-              const uint32_t* T = (const uint32_t*)wtab + gk + ga;
-              if (gb == ga + 1) {                // both on one line (the same for every row)
-#pragma unroll
-                for (int part = 0; part < 2; ++part)
-#pragma unroll
-                  for (int pl = 0; pl < NPL; ++pl) wv[part][pl][e] = T[(part * NPL + pl) * P.win_cap];
-              } else {
-#pragma unroll
-                for (int part = 0; part < 2; ++part)
-#pragma unroll
-                  for (int pl = 0; pl < NPL; ++pl)
-                    wv[part][pl][e] = __byte_perm(T[(part * NPL + pl) * P.win_cap], T[(part * NPL + pl) * P.win_cap + gb - ga], 0x5410);
-              }
-            }
-          } else {
-            int xs[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int g = __shfl_sync(0xffffffffu, ghl, j);
-              xs[j] = K::TF32 ? gk - g : gk + g;
-            }
-#pragma unroll
-            for (int part = 0; part < 2; ++part)
-#pragma unroll
-              for (int pl = 0; pl < NPL; ++pl) {
-                const unsigned char* Tb = wtab + (size_t)(part * NPL + pl) * P.win_cap * EB;
-#pragma unroll
-                for (int e = 0; e < NW; ++e) {
-                  if (FMT == TT_TF32) {
-                    wv[part][pl][e] = ((const uint32_t*)Tb)[xs[e]];
-                  } else {
-                    const uint16_t* T = (const uint16_t*)Tb;
-                    wv[part][pl][e] = (uint32_t)T[xs[2 * e]] | (uint32_t)T[xs[2 * e + 1]] << 16;
-                  }
+              for (int e = 0; e < NW; ++e) {
+                if (FMT == TT_TF32) {
+                  wv[part][pl][e] = ((const uint32_t*)Tb)[xs[e]];
+                } else {
+                  const uint16_t* T = (const uint16_t*)Tb;
+                  wv[part][pl][e] = (uint32_t)T[xs[2 * e]] | (uint32_t)T[xs[2 * e + 1]] << 16;
                 }
               }
-          }
+            }
         }
-#pragma unroll
-        for (int part = 0; part < 2; ++part)
-#pragma unroll
-          for (int pl = 0; pl < NPL; ++pl) {
-            const uint32_t col = a0 + pl * K::PCOLS + part * (K::PCOLS / 2);
-            if (K::TF32) tmem_st_x16(col, wv[part][pl]);
-            else tmem_st_x8(col, wv[part][pl]);
-          }
       }
+      // (the words are ready before the stage is awaited: only the stores follow the MMAs that release it)
+      if (it >= SA && !__all_sync(0xffffffffu, mbar_wait_spin(&bar_aempty[s], ph ^ 1u, TC_SPIN))) {
+        s_err = 1;
+        break;
+      }
+      tc_fence_after();
+#pragma unroll
+      for (int part = 0; part < 2; ++part)
+#pragma unroll
+        for (int pl = 0; pl < NPL; ++pl) {
+          const uint32_t col = a0 + pl * K::PCOLS + part * (K::PCOLS / 2);
+          if (K::TF32) tmem_st_x16(col, wv[part][pl]);
+          else tmem_st_x8(col, wv[part][pl]);
+        }
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_full[s]);
-      if (++s == S) { s = 0; ph ^= 1u; }
+      if (lane == 0) mbar_arrive(&bar_afull[s]);
+      if (++s == SA) { s = 0; ph ^= 1u; }
     }
     // epilogue: D (TMEM) -> Y; the warps of a quadrant take alternate 16-column groups
-    constexpr int CSTEP = HALVES == 1 ? 32 : 16;
     const bool dready = idle || __all_sync(0xffffffffu, mbar_wait(&bar_d, 0, TC_SPIN));
     if (!dready) s_err = 1;
     int ldy;
@@ -720,7 +742,7 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
     if (job.nks == 1) {
       if (dready && !s_err) {
         tc_fence_after();
-        for (int c0 = 16 * hh0; c0 < NT; c0 += CSTEP) {
+        for (int c0 = 16 * hh; c0 < NT; c0 += 32) {
           float v[16];
           tc_load_acc<NPL>(tb + lane_off + c0, lay.stacked, NT, v);
           if (vrow) {
@@ -739,7 +761,7 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
       float* mine = P.part + (size_t)blockIdx.x * slot;
       const bool mine_ok = ws_ok(D, (long long)blockIdx.x - job.ks + job.nks <= P.part_jobs && job.ks < job.nks, 21);
       if (dready && !s_err && !idle) tc_fence_after();
-      for (int c0 = 16 * hh0; c0 < NT; c0 += CSTEP) {
+      for (int c0 = 16 * hh; c0 < NT; c0 += 32) {
         float v[16];
         if (dready && !s_err && !idle) {
           tc_load_acc<NPL>(tb + lane_off + c0, lay.stacked, NT, v);
@@ -764,7 +786,7 @@ __global__ void __launch_bounds__(32 * (2 + AW), AW == TC_APROD ? 1 : 2)
         __threadfence();
         const float* base = P.part + (size_t)first_job * slot;
         using Acc = typename std::conditional<GRAM, double, float>::type;
-        for (int c0 = 16 * hh0; c0 < NT; c0 += CSTEP) {
+        for (int c0 = 16 * hh; c0 < NT; c0 += 32) {
           Acc v[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) v[e] = (Acc)__ldcg(base + (size_t)(c0 + e) * TC_BM + i);
@@ -842,18 +864,18 @@ void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int 
   xb_prep(D, xbuf, xshift, wsel, xb, kind, prob_stride, -1, 0, 0, D.maxN, s);
 }
 
-template <int KIND, int MODE, int FMT = TT_TF32, int AW = TC_APROD>
+template <int KIND, int MODE, int FMT = TT_TF32, bool HALF = false>
 static cudaError_t launch_tc_kind(const Dev& D, const ToeplitzJob* jobs, int njobs, const TcParams& P, int* err,
                                   size_t sm, cudaStream_t s) {
   static size_t set = 0;
   if (sm > set) {
     // the attribute must cover this launch's dynamic shared memory (static + dynamic <= 227 KB)
     cudaError_t e =
-        cudaFuncSetAttribute(k_toeplitz_tc<KIND, MODE, AW, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(k_toeplitz_tc<KIND, MODE, FMT, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     set = sm;
   }
-  k_toeplitz_tc<KIND, MODE, AW, FMT><<<njobs, 32 * (2 + AW), sm, s>>>(D, jobs, P, err);
+  k_toeplitz_tc<KIND, MODE, FMT, HALF><<<njobs, 32 * (2 + TC_APROD), sm, s>>>(D, jobs, P, err);
   return cudaGetLastError();
 }
 
@@ -876,13 +898,13 @@ cudaError_t launch_toeplitz_tc(const Dev& D, const ToeplitzJob* jobs, int njobs,
   note_launch();
   constexpr int TCP = TC_PRODUCT;
   if (kind == PRONY_TF32X3)
-    return half ? launch_tc_kind<PRONY_TF32X3, TCP, TT_TF32, TC_APROD2>(D, jobs, njobs, P, err, sm, s)
+    return half ? launch_tc_kind<PRONY_TF32X3, TCP, TT_TF32, true>(D, jobs, njobs, P, err, sm, s)
                 : launch_tc_kind<PRONY_TF32X3, TCP, TT_TF32>(D, jobs, njobs, P, err, sm, s);
   if (kind == PRONY_BF16X3)
-    return half ? launch_tc_kind<PRONY_BF16X3, TCP, TT_WIDE, TC_APROD2>(D, jobs, njobs, P, err, sm, s)
+    return half ? launch_tc_kind<PRONY_BF16X3, TCP, TT_WIDE, true>(D, jobs, njobs, P, err, sm, s)
            : fmt == TT_WIDE ? launch_tc_kind<PRONY_BF16X3, TCP, TT_WIDE>(D, jobs, njobs, P, err, sm, s)
                             : launch_tc_kind<PRONY_BF16X3, TCP, TT_COMPACT>(D, jobs, njobs, P, err, sm, s);
-  return half ? launch_tc_kind<PRONY_BF16X2, TCP, TT_WIDE, TC_APROD2>(D, jobs, njobs, P, err, sm, s)
+  return half ? launch_tc_kind<PRONY_BF16X2, TCP, TT_WIDE, true>(D, jobs, njobs, P, err, sm, s)
          : fmt == TT_WIDE ? launch_tc_kind<PRONY_BF16X2, TCP, TT_WIDE>(D, jobs, njobs, P, err, sm, s)
                           : launch_tc_kind<PRONY_BF16X2, TCP, TT_COMPACT>(D, jobs, njobs, P, err, sm, s);
 }

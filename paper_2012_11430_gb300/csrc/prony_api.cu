@@ -451,7 +451,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     return need;
   };
   // wide tables where their windows fit at the same split (with the stages given, or two): a pair of points is one
-  // load instead of two and a shift (the same products: 14.7 -> 13.7 ms); a longer split would load more windows
+  // load instead of two and a shift (the same products: then 14.7 -> 13.7 ms); a longer split would load more windows
   if (bf16)
     for (int st = T.stages; st >= st_min; --st)
       if (win_cap_for(st, TT_WIDE) >= std::max(256, longest(TT_WIDE))) {
@@ -462,16 +462,15 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   T.win_cap = win_cap_for(T.stages, T.fmt);
   // Narrow blocks (at most 24 columns in BF16x3) of problems whose windows are short: two CTAs per SM, each with
   // half of its memories, so that one's set-up, window load and epilogue run under the other's
-  // chunks (the products of 4096 problems with n 7..31: 16.1 -> 14.7 ms a solve).  From four CTAs per SM on:
-  // below that a single one per SM has more producer warps on its chunks.  Wider accumulators leave
+  // chunks (the products of 4096 problems with n 7..31: 16.1 -> 14.7 ms a solve when it was made).  From four CTAs per SM on:
+  // below that every SM has a CTA of its own.  Wider accumulators leave
   // no tensor memory for it, longer windows no shared memory.
   {
     const size_t per = 228 * 1024 / 2 - 1024 - 6144;   // (1 KB reserved per CTA, static shared memory)
     const int need = longest(T.fmt);
     const int sa = tc_half_stages(prec, T.ntbox);
-    // (narrower problems of the batch have room for more A stages than the widest)
     int st = std::min(T.stages, 3);
-    while (st > std::max(1, sa) && tc_smem_bytes(prec, T.fmt, T.ntbox, st, need) > per) --st;
+    while (st > 1 && tc_smem_bytes(prec, T.fmt, T.ntbox, st, need) > per) --st;
     if (sa > 0 && T.fmt != TT_COMPACT && !getenv("PRONY_TC_BSTAGES") &&
         (long long)tiles_in * nks >= 4 * 152 && tc_smem_bytes(prec, T.fmt, T.ntbox, st, need) <= per) {
       T.half = 1;
