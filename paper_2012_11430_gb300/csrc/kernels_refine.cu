@@ -23,8 +23,9 @@
 // with |eps| < 0.1, the sum of c_j T in twice FP32 (error-free sums) from a table of the CTA, the sum of
 // c_j T eps in FP32, whose rounding is ten times smaller than that of the whole.
 // Measured at d = 2, n = 63 (16384 points), m = 20: a step took 195 us (143 in a one-CTA solve with three
-// barriers per column, 40 in the M sums over all points, 9 in a separate trial pass), now 41 us (k_lm_step
-// 23, k_lm_points 17): 50 steps 10.05 -> 2.15 ms.  Both kernels are latency chains on an almost idle GPU.
+// barriers per column, 40 in the M sums over all points, 9 in a separate trial pass), now 40 us (k_lm_step
+// 26, k_lm_points 16, their launches overlapped): 50 steps 10.05 -> 2.00 ms.  Both kernels are latency chains
+// on an almost idle GPU.
 #include "common.cuh"
 
 #include <algorithm>
@@ -38,6 +39,29 @@ constexpr int LM_EP = LM_TILE + 1;      // pitch of the exponentials (threads of
 constexpr int LM_NB = 16;               // column block of the Cholesky factorisation
 constexpr int LM_SOLVE_THREADS = 512;
 constexpr double TWO_PI = 6.283185307179586;
+
+// The steps are launched as a chain (programmatic dependent launch): a kernel's blocks become resident as soon as
+// every block of the one before has begun, and wait here until it has completed and its writes are visible; what
+// that saves is the launch latency between kernels of 16 to 26 us (50 steps: 2.25 -> 2.00 ms; the kernels of a solve,
+// launched from a graph, gained nothing by it).  Every kernel launched so begins with chain_begin().
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+void chain_launch(void (*k)(P...), int blocks, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(blocks);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
+}
 
 struct LmState {
   double lambda;
@@ -101,6 +125,7 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
                                                        long long K, int npt_blocks, const float2* y,
                                                        const LmState* st, const float4* circle, double* sets,
                                                        float2* vs, double* ls) {
+  chain_begin();
   extern __shared__ float4 lm_smem[];
   __shared__ uint64_t T[PRONY_MMAX * PRONY_DMAX];
   __shared__ float2 Tf[LM_SEG];
@@ -291,6 +316,7 @@ __global__ void __launch_bounds__(LM_SOLVE_THREADS) k_lm_step(double* t, double2
                                                               int d, LmState* st, double* sets, const float2* vs, const double* ls, int nblk,
                                                               double* hist, int step,
                                                               int solve) {
+  chain_begin();
   extern __shared__ __align__(16) float lm_f[];
   __shared__ int s_ok, s_cur;
   __shared__ float dinv[PRONY_LM_PMAX];
@@ -571,8 +597,8 @@ void launch_refine_lm(double* t, double2* c, int m, int d, const int* lo, const 
   k_lm_init<<<1, 256, 0, s>>>(st, lambda0, t, c, tc, cc, circle, m, d);
   for (int it = 0; it <= iters; ++it) {
     note_launch();
-    k_lm_points<<<npt + npair, LM_TILE, sp, s>>>(tc, cc, m, d, B, K, npt, y, st, circle, sets, vs, ls);
+    chain_launch(k_lm_points, npt + npair, LM_TILE, sp, s, tc, cc, m, d, B, K, npt, y, st, circle, sets, vs, ls);
     note_launch();
-    k_lm_step<<<1, LM_SOLVE_THREADS, ss, s>>>(t, c, tc, cc, m, d, st, sets, vs, ls, npt, hist, it, it < iters);
+    chain_launch(k_lm_step, 1, LM_SOLVE_THREADS, ss, s, t, c, tc, cc, m, d, st, sets, vs, ls, npt, hist, it, it < iters);
   }
 }
