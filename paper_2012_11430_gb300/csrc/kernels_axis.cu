@@ -95,12 +95,12 @@ __device__ __forceinline__ void ax_put(float2* grid, uint32_t* tab, int Gd4, int
   }
 }
 
-// F^(w; x') for four frequencies per thread, and the tables of T^* from them: the samples conj f(-x)
+// F^(w; x') for four frequencies per thread (or per `parts` threads, each summing a piece of the line), and the tables of T^* from them: the samples conj f(-x)
 // transform to conj F^(w; -x'), zero where -x' leaves the grid.  The difference x_0 = n + 1 occurs
 // in the products over the row box {0..n+1}^d only; `trim` leaves those samples out where a caller
 // asks for a product over I_n alone (whatever they hold, they do not enter it).
 template <int MODE, int FMT>
-__global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
+__global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim, int parts) {
   extern __shared__ float2 ax_tw[];
   const ProbDesc& p = D.P[blockIdx.y];
   const int G = p.G, Gs = p.Gd / G;
@@ -111,7 +111,13 @@ __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
   __syncthreads();
   const int groups = (G + 3) / 4;
   const long long total = (long long)Gs * groups;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total; q += (long long)gridDim.x * blockDim.x) {
+  const int part = threadIdx.x & (parts - 1), per_block = blockDim.x / parts;
+  const int last = trim ? G - 1 : G;
+  const int seg = (last + 8 * parts - 1) / (8 * parts) * 8, i_begin = min(part * seg, last), i_end = min(i_begin + seg, last);
+  // (the loop runs for whole warps: items past the end repeat the last one and write nothing)
+  for (long long q0 = blockIdx.x * (long long)per_block; q0 < total; q0 += (long long)gridDim.x * per_block) {
+    const long long q = min(q0 + threadIdx.x / parts, total - 1);
+    const bool mine = q0 + threadIdx.x / parts < total;
     const int x = (int)(q % Gs), w0 = 4 * (int)(q / Gs);
     const float2* f = D.gF + p.grid + x;
     float2 acc[2][4];                             // two interleaved partial sums per frequency
@@ -120,13 +126,12 @@ __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
     for (int u = 0; u < 4; ++u) {
       acc[0][u] = acc[1][u] = make_float2(0.f, 0.f);
       step[u] = min(w0 + u, G - 1);
-      at[u] = (int)((long long)step[u] * (G - p.n) % G);          // twiddle of x_0 = -n
+      at[u] = (int)((long long)step[u] * (G - p.n + i_begin) % G);          // twiddle of x_0 = -n + i_begin
     }
-    const int last = trim ? G - 1 : G;
-    for (int i0 = 0; i0 < last; i0 += 8) {        // eight loads in flight
+    for (int i0 = i_begin; i0 < i_end; i0 += 8) {  // eight loads in flight
       float2 v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = i0 + e < last ? f[(long long)(i0 + e) * Gs] : make_float2(0.f, 0.f);
+      for (int e = 0; e < 8; ++e) v[e] = i0 + e < i_end ? f[(long long)(i0 + e) * Gs] : make_float2(0.f, 0.f);
 #pragma unroll
       for (int e = 0; e < 8; ++e)
 #pragma unroll
@@ -151,9 +156,13 @@ __global__ void __launch_bounds__(64) k_axis_tables(Dev D, Dev S, int trim) {
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      if (w0 + u >= G) break;
+      float2 v = make_float2(acc[0][u].x + acc[1][u].x, acc[0][u].y + acc[1][u].y);
+      for (int o = 1; o < parts; o <<= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+      }
+      if (!mine || w0 + u >= G || (u & (parts - 1)) != part) continue;
       const ProbDesc& ps = S.P[p.sub + w0 + u];
-      const float2 v = make_float2(acc[0][u].x + acc[1][u].x, acc[0][u].y + acc[1][u].y);
       ax_put<MODE, FMT>(S.gF + ps.grid, S.tabF + ps.toff, ps.Gd4, x, v);
       ax_put<MODE, FMT>(S.gH + ps.grid, S.tabH + ps.toff, ps.Gd4, mvalid ? mir : x,
                    mvalid ? make_float2(v.x, -v.y) : make_float2(0.f, 0.f));
@@ -401,8 +410,12 @@ template <int MODE, int FMT>
 static cudaError_t axis_tables(const Dev& D, const Dev& S, int trim, cudaStream_t s) {
   const int G = 2 * max_axis_n(S) + 2;
   const long long items = (long long)S.maxGd * ((G + 3) / 4);
+  // eight threads a sum where that leaves at most two warps per scheduler: a single small problem has a few thousand
+  // sums of 2 n + 2 terms, each a chain of loads and twiddle steps (d = 2, n = 50: 44 -> 13 us)
+  const int parts = 8 * items * D.nprob <= 152LL * 256 ? 8 : 1;
   note_launch();
-  k_axis_tables<MODE, FMT><<<dim3(blocks_per_problem((items + 63) / 64, D.nprob), D.nprob), 64, sizeof(float2) * G, s>>>(D, S, trim);
+  k_axis_tables<MODE, FMT><<<dim3(blocks_per_problem((parts * items + 63) / 64, D.nprob), D.nprob), 64, sizeof(float2) * G, s>>>(
+      D, S, trim, parts);
   return cudaGetLastError();
 }
 
