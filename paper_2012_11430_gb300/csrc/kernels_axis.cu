@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256, 2) k_axis_in(Dev D, Dev S, int xbuf, int 
 // The inverse transform of one line (k', column j) by a lane, KB rows k_0 at a time:
 //   y[k] = (1/L) sum over the classes of P cos + i Q sin,  P = A + A', Q = A - A' for even k with
 // A = y^(w) + y^(w+H), A' = y^(-w) + y^(H-w), and the differences instead of the sums for odd k.
-template <int KB>
+template <int KB, int SP>
 __global__ void __launch_bounds__(256) k_axis_out(Dev D, Dev S, int wsel, int ybuf, int y_ext) {
   extern __shared__ float4 ax_tab[];              // [class][k_0] = (cos, cos, sin, sin)
   const ProbDesc& p = D.P[blockIdx.y];
@@ -352,17 +352,21 @@ __global__ void __launch_bounds__(256) k_axis_out(Dev D, Dev S, int wsel, int yb
   const float scale = 1.0f / (float)L;
   const int lane = threadIdx.x & 31;
   const long long items = (long long)nt * w * nblk;
-  for (long long it = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); it < items;
-       it += (long long)gridDim.x * (blockDim.x >> 5)) {
+  constexpr int PER = 8 / SP;                     // items of a block at a time
+  const int warp = threadIdx.x >> 5, sub = warp % SP;
+  for (long long it0 = blockIdx.x * (long long)PER; it0 < items; it0 += (long long)gridDim.x * PER) {
+    const bool mine = it0 + warp / SP < items;
+    if (SP == 1 && !mine) break;
+    const long long it = mine ? it0 + warp / SP : items - 1;
     const int blk = (int)(it % nblk), t = (int)(it / nblk % nt), j = (int)(it / nblk / nt);
     const int kp = 32 * t + lane, k0 = blk * KB;
-    const bool valid = kp < Np;
+    const bool valid = mine && kp < Np;
     const float2* src = src0 + (long long)j * Np + (valid ? kp : 0);
     u64 acc[KB];
 #pragma unroll
     for (int k = 0; k < KB; ++k) acc[k] = 0ull;
 #pragma unroll(KB <= 8 ? 4 : 2)
-    for (int c = 0; c < ncls; ++c) {
+    for (int c = sub; c < ncls; c += SP) {
       const bool four = c != 0 && 2 * c != H;
       const float2 zero = make_float2(0.f, 0.f);
       const float2 y0 = src[c * fstride], y2 = src[(c + H) * fstride];
@@ -381,7 +385,29 @@ __global__ void __launch_bounds__(256) k_axis_out(Dev D, Dev S, int wsel, int yb
         ax_fma(acc[k + 1], qo, t1.y);
       }
     }
-    if (valid) {
+    if (SP > 1) {                                 // the warps of an item: sums over their classes, in order
+      __shared__ u64 part[SP > 1 ? 8 : 1][SP > 1 ? KB : 1][32];
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < KB; ++k) part[warp][k][lane] = acc[k];
+      __syncthreads();
+      constexpr int OWN = KB / SP;
+      if (valid) {
+        float2* dst = Y + (long long)j * ldy + (long long)k0 * Np + kp;
+#pragma unroll
+        for (int e = 0; e < OWN; ++e) {
+          const int k = sub * OWN + e;
+          float2 v = ax_unpack(part[warp - sub][k][lane]);
+#pragma unroll
+          for (int g = 1; g < SP; ++g) {
+            const float2 u = ax_unpack(part[warp - sub + g][k][lane]);
+            v.x += u.x;
+            v.y += u.y;
+          }
+          if (k0 + k < K) dst[(long long)k * Np] = make_float2(v.x * scale, v.y * scale);
+        }
+      }
+    } else if (valid) {
       float2* dst = Y + (long long)j * ldy + (long long)k0 * Np + kp;
 #pragma unroll
       for (int k = 0; k < KB; ++k)
@@ -462,23 +488,27 @@ cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int w
   }
 }
 
-template <int KB>
+template <int KB, int SP>
 static cudaError_t axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s) {
   static size_t set = 0;
   const int H = max_axis_n(S) + 1, K = y_ext ? H + 1 : H, nblk = (K + KB - 1) / KB;
   // (H / 2 + 1) x Kt grows with n: the largest problem's table is the largest of the batch
   const size_t sm = sizeof(float4) * (size_t)(H / 2 + 1) * nblk * KB;
-  cudaError_t e = allow_smem(k_axis_out<KB>, sm, set);
+  cudaError_t e = allow_smem(k_axis_out<KB, SP>, sm, set);
   if (e != cudaSuccess) return e;
   const long long items = (long long)(((y_ext ? S.maxNext : S.maxN) + 31) / 32) * maxw * nblk;
   note_launch();
-  k_axis_out<KB><<<dim3(blocks_per_problem((items + 7) / 8, D.nprob), D.nprob), 256, sm, s>>>(D, S, wsel, ybuf, y_ext);
+  k_axis_out<KB, SP><<<dim3(blocks_per_problem((items * SP + 7) / 8, D.nprob), D.nprob), 256, sm, s>>>(D, S, wsel, ybuf, y_ext);
   return cudaGetLastError();
 }
 
 cudaError_t launch_axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s) {
   // 22 rows a pass re-read the sub-products least; few lines (a single small problem) take 8 rows a
-  // pass, which gives three times the warps
+  // pass, which gives three times the warps, and with fewer than eight warps per SM four warps share a line's
+  // classes (d = 2, n = 50, 37 columns: 25 -> 11 us; with 11 warps per SM, d = 3, n = 19, 40 columns, 3 us slower)
   const long long lines = (long long)(((y_ext ? S.maxNext : S.maxN) + 31) / 32) * maxw * D.nprob;
-  return lines >= 152LL * 16 ? axis_out<22>(D, S, wsel, ybuf, y_ext, maxw, s) : axis_out<8>(D, S, wsel, ybuf, y_ext, maxw, s);
+  if (lines >= 152LL * 16) return axis_out<22, 1>(D, S, wsel, ybuf, y_ext, maxw, s);
+  const int nblk = (max_axis_n(S) + (y_ext ? 2 : 1) + 7) / 8;
+  return lines * nblk < 152LL * 8 ? axis_out<8, 4>(D, S, wsel, ybuf, y_ext, maxw, s)
+                                  : axis_out<8, 1>(D, S, wsel, ybuf, y_ext, maxw, s);
 }

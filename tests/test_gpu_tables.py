@@ -71,3 +71,23 @@ def test_narrow_batches(ctx, prec, shapes):
         te, ce = W.match_to_truth(outs[k].t, outs[k].c, probs[i].t, probs[i].c)
         assert te <= tol and ce <= 20 * tol, (k, te, ce)
         assert np.array_equal(outs[k].t, outs[i].t) and np.array_equal(outs[k].c, outs[i].c)
+
+
+@pytest.mark.parametrize("prec", ["bf16x3", "fp32"])
+@pytest.mark.parametrize("d,n,r,ext", [(2, 47, 1, 1), (2, 63, 40, 0), (3, 15, 64, 1), (3, 19, 40, 0), (3, 15, 128, 1)])
+def test_transformed_products(ctx, monkeypatch, prec, d, n, r, ext):
+    """Products through the transform of the leading axis with few and with many lines, against FP64 FFTs: FP32 sums of
+    N terms, statistically well below N u of the result's norm."""
+    import torch
+    monkeypatch.setenv("PRONY_AXIS", "1")
+    rng = np.random.Generator(np.random.PCG64(600 + 10 * d + n))
+    L, N = n + (2 if ext else 1), (n + 1) ** d
+    grid = rng.standard_normal((2 * n + 2,) * d) + 1j * rng.standard_normal((2 * n + 2,) * d)
+    X = (rng.standard_normal((r, N)) + 1j * rng.standard_normal((r, N))).astype(np.complex64)
+    Y = torch.full((r, L ** d), float("nan"), dtype=torch.complex64, device="cuda")
+    ctx.toeplitz_mm_dev(torch.from_numpy(grid.reshape(-1)).cuda(), d, n, torch.from_numpy(X).cuda(), L, 0, prec, Y)
+    ax = tuple(range(1, d + 1))
+    G = np.fft.fftn(np.roll(grid, (-n,) * d, axis=tuple(range(d))))
+    ref = np.fft.ifftn(G * np.fft.fftn(X.reshape((r,) + (n + 1,) * d), s=G.shape, axes=ax), axes=ax)
+    ref = ref[(slice(None),) + (slice(0, L),) * d].reshape(r, -1)
+    assert np.linalg.norm(Y.cpu().numpy() - ref) <= 64 * U32 * np.sqrt(N) * np.linalg.norm(ref)
