@@ -93,7 +93,7 @@ def committed_counters(config: str, precision: str):
                 elif parts[0] == "tensor_pipe":
                     pipe = {"value": float(parts[3]), "unit": "% of active cycles",
                             "source": "ncu sm__pipe_tensor_cycles_active, time-weighted over the products of a "
-                                      "solve (profiles/toeplitz_tc_C3_batch8_bf16x3.md)"}
+                                      "solve (profiles/kernels_by_case.md)"}
     return traffic, pipe
 
 

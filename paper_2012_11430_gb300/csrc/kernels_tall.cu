@@ -145,9 +145,8 @@ __global__ void k_zero_small(Dev D, long long off, long long bytes) {
 }
 
 // ----------------------------------------------------------------------------- tall-skinny Gram
-// out[a][b] = sum_r conj(X[r, a]) Z[r, b] over a block of `chunk` rows (chosen by the launcher
-// so that the batch gives a few blocks per SM: few blocks per problem means few FP64 atomics on
-// the same output entries).
+// out[a][b] = sum_r conj(X[r, a]) Z[r, b] over a block of `chunk` rows (chosen by the launcher so that the
+// batch fills the resident blocks: few blocks per problem means few partial Grams to add).
 //
 // Rows are staged RS at a time through three shared-memory buffers filled by cp.async (two passes in flight while
 // one is multiplied; rows past the end are zeros).  A buffer holds the values as they are in memory, column-major,
@@ -156,7 +155,7 @@ __global__ void k_zero_small(Dev D, long long off, long long bytes) {
 // acc2 += (Re x Im z, Im x Re z), with conj(x) z = (acc1.lo + acc1.hi) + i (acc2.lo - acc2.hi) at the end, so that
 // nothing but a swap of z is rearranged.  What bounds a 4 x 4 tile is then shared memory and the FP32 pipe about
 // equally; values stored as the four floats of two paired operands took twice the loads (64 blocks of 8000 x 80:
-// 0.69 ms, now 0.45; a solve of 4096 problems with n 7..31: 5.3 -> 1.9 ms of Gram sums, with blocks of 128 threads).
+// 0.69 ms, now 0.39; a solve of 4096 problems with n 7..31: 5.3 -> 1.9 ms of Gram sums, with blocks of 128 threads).
 // Output ownership is interleaved: thread (ti, tj) owns the entries (ti + NA i, tj + NB j),
 // i, j < 4, so the threads of a warp read consecutive columns (different banks) or the same one
 // (broadcast).  When there are fewer 4x4 tiles than threads, threads split the staged row pairs into

@@ -8,7 +8,7 @@
 //   -> SVD(Q), S_l = U_Q^* (U^* Y_l) V_Q Sigma^{-1}  (Y_l = rows k + e_l of the last Y)
 //   -> C_mu, eig, z, t -> conj(A) f, Gram, c -> ||A^T c - f||.
 // Every kernel loops over the problems of the batch; problems that stopped skip work.
-// The host waits once per power iteration to read the "all stopped" flag.
+// A solve is one graph launch; the host waits once, for the results.
 #include "common.cuh"
 #include "../../include/prony.h"
 
