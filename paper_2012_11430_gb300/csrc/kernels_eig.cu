@@ -468,7 +468,8 @@ __global__ void __launch_bounds__(NT) k_svd_S(Dev D) {
     if (rank == 0 && s_rank[threadIdx.x] == b - 1) s_red[0] = mine;
     if (rank == 0 && s_rank[threadIdx.x] == 0) s_red[1] = mine;
   }
-  __syncthreads();
+  // (over the cluster: after an odd number of steps V lies in the first S_l slot, which the CTAs write below)
+  cl_sync<CL>();
   if (rank == 0 && threadIdx.x == 0) st.sigma_ratio = s_red[1] > 0.0 ? s_red[0] / s_red[1] : 0.0;
   // ---- U_Q = Q V_Q Sigma^{-1}, S_l = (U_Q^* M_l) V_Q Sigma^{-1}: this CTA takes the columns (of U_Q) and
   // rows (of S_l) i = rank mod CL, so no other CTA's results are needed

@@ -55,3 +55,32 @@ def test_batches_of_every_cluster_width(ctx, count, n, m):
         te, ce = W.match_to_truth(outs[k].t, outs[k].c, probs[i].t, probs[i].c)
         assert te <= 1e-6 and ce <= 1e-5, (k, te, ce)
         assert np.array_equal(outs[k].t, outs[i].t) and np.array_equal(outs[k].c, outs[i].c)
+
+
+def _close_pairs(m, a, gap):
+    """Q with pairs of singular values a relative `gap` apart, and M_l of known eigenvalues exp(-2 pi i t)."""
+    rng = np.random.Generator(np.random.PCG64(900 + m))
+    gauss = lambda *s: rng.standard_normal(s) + 1j * rng.standard_normal(s)  # noqa: E731
+    U0 = np.linalg.qr(gauss(a, m))[0]
+    V0 = np.linalg.qr(gauss(m, m))[0]
+    sigma = np.linspace(2.0, 1.0, m // 2).repeat(2)
+    sigma[1::2] *= 1 - gap
+    Wm = np.linalg.qr(gauss(m, m))[0] + 0.3 * gauss(m, m) / np.sqrt(m)
+    t = np.stack([(rng.permutation(m) + 0.5 + 0.2 * rng.uniform(-1, 1, m)) / m for _ in range(2)], 1)
+    S = [Wm @ np.diag(np.exp(-2j * np.pi * t[:, l])) @ np.linalg.inv(Wm) for l in range(2)]
+    Q = U0 @ np.diag(sigma) @ V0.conj().T
+    return Q, np.array([U0 @ S[l] @ np.diag(sigma) @ V0.conj().T for l in range(2)]), sigma, t
+
+
+CLOSE = [(m, a, gap) for m, a in ((12, 24), (32, 64), (40, 80), (64, 128)) for gap in (1e-3, 1e-4)]
+
+
+@pytest.mark.parametrize("m,a,gap", CLOSE)
+def test_close_singular_values_repeat(ctx, m, a, gap):
+    """Close singular values take three or more refinement steps, after an odd number of which V lies where
+    S_1 is written: every run gives the same bits."""
+    Q, M, _, _ = _close_pairs(m, a, gap)
+    first = ctx.small_steps(Q, M)
+    assert first[-1] == 0
+    for _ in range(30):
+        assert all(np.array_equal(x, y) for x, y in zip(first, ctx.small_steps(Q, M)))
