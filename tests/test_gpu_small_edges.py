@@ -84,3 +84,16 @@ def test_close_singular_values_repeat(ctx, m, a, gap):
     assert first[-1] == 0
     for _ in range(30):
         assert all(np.array_equal(x, y) for x, y in zip(first, ctx.small_steps(Q, M)))
+
+
+@pytest.mark.parametrize("m,a,gap", CLOSE)
+def test_close_singular_values_converge(ctx, m, a, gap):
+    """... and are refined until they converge: sigma to FP64 rounding, z (which no basis of a pair changes) as in
+    test_small_steps_sizes."""
+    Q, M, sigma, t = _close_pairs(m, a, gap)
+    sig, _, z, tg, status = ctx.small_steps(Q, M)
+    assert status == 0
+    sigma = np.sort(sigma)[::-1]
+    assert np.max(np.abs(sig - sigma) / sigma) <= 64 * 2.0 ** -53 * m
+    o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
+    assert np.max(np.abs(z[og] - np.exp(-2j * np.pi * t[o]))) <= 1e-11
