@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(NQ > 2 ? 512 : 256) k_chol(Dev D, int wsel, in
             t[r][q] = (k < w && k != pv) ? T[jj * LR + k] : make_float2(0.f, 0.f);
           }
         }
+        __syncwarp();                           // every lane has read T[j][pv] before one of them overwrites it
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           if (!go[r]) continue;

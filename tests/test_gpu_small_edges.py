@@ -97,3 +97,17 @@ def test_close_singular_values_converge(ctx, m, a, gap):
     assert np.max(np.abs(sig - sigma) / sigma) <= 64 * 2.0 ** -53 * m
     o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
     assert np.max(np.abs(z[og] - np.exp(-2j * np.pi * t[o]))) <= 1e-11
+
+
+@pytest.mark.parametrize("n,m", [(15, 10), (23, 30), (31, 45), (31, 64)])
+def test_pivoted_blocks_repeat(ctx, n, m):
+    """The pivoted elimination of blocks of 1 to 4 column groups (r0 = 2 m): equal problems of a call and of
+    repeated calls give the same bits."""
+    p = W.make_problem(f"pv{m}", 2, n, m, 7100 + m, snr_db=40.0)
+    runs = [ctx.solve_batched([p.grid] * 24, [2] * 24, [n] * 24, [m] * 24) for _ in range(3)]
+    first = runs[0][0][0]
+    te, ce = W.match_to_truth(first.t, first.c, p.t, p.c)
+    assert te <= 1e-2 / n and ce <= 0.1              # (noise of 40 dB)
+    for outs, rc in runs:
+        assert rc == 0
+        assert all(np.array_equal(o.t, first.t) and np.array_equal(o.c, first.c) for o in outs)
