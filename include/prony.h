@@ -258,6 +258,9 @@ typedef struct {
  *   PRONY_AXIS=0 / 1     the products of every problem directly / through a DFT of the leading axis
  *                        wherever that is possible (d >= 2, n <= 95; not PRONY_FFT32).  Default:
  *                        the transform for problems of at least 2048 points (n+1)^d where it costs less
+ *   PRONY_ALLOC_MAX=b    no single device buffer of more than b bytes: growing one beyond that is refused as
+ *                        a failed allocation is (a program that shares the device; the DFT products then
+ *                        give way to the direct ones where those fit)
  * The first three change launch configurations only, never the arithmetic beyond FP32 summation
  * order; the fourth changes how the X M products are rounded (both are FP32-accurate), the fifth
  * how the products are (FP32 transforms around shorter dot products in the chosen arithmetic).

@@ -52,6 +52,8 @@ int ensure(DBuf& b, size_t bytes) {
   b.p = nullptr;
   b.cap = 0;
   size_t want = bytes + bytes / 4;
+  if (const char* lim = getenv("PRONY_ALLOC_MAX"))
+    if (want > std::strtoull(lim, nullptr, 10)) return cuda_fail(cudaErrorMemoryAllocation, "PRONY_ALLOC_MAX");
   cudaError_t e = cudaMalloc(&b.p, want);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
   b.cap = want;
@@ -361,6 +363,7 @@ int tc_set_jobs(prony_ctx* ctx, Batch& B, int nks) {
 
 int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   TcConf& T = B.tc;
+  T = TcConf{};                                // (a set-up that ran out of memory may have chosen otherwise)
   T.on = true;
   T.kind = prec;
   const int npl = tc_planes(prec);
@@ -974,7 +977,12 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
     if (!rc) rc = setup_products(ctx, B, o.precision);
     if (rc && rc != PRONY_ENOMEM) return rc;
     B.ax.on = !rc;
-    if (rc) cudaGetLastError();
+    if (rc) {
+      cudaGetLastError();
+      B.part = nullptr;
+      B.cnt = nullptr;
+      B.part_jobs = 0;
+    }
   }
   if (!B.ax.on && (rc = setup_products(ctx, B, o.precision))) return rc;
   if (o.svd_method == 1 && fft_fits(B)) {

@@ -1,0 +1,45 @@
+"""Products through the transform of the leading axis give way to the direct ones when their buffers cannot be
+allocated (PRONY_ALLOC_MAX refuses the larger of the two)."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def ctx():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2012_11430_gb300 import Context
+    with Context(0) as c:
+        yield c
+
+
+def _solve(ctx, p, count, precision):
+    from paper_2012_11430_gb300 import default_opts
+    outs, rc = ctx.solve_batched([p.grid] * count, [p.d] * count, [p.n] * count, [p.m] * count, default_opts(precision=precision))
+    assert rc == 0
+    te, ce = W.match_to_truth(outs[0].t, outs[0].c, p.t, p.c)
+    assert te <= 1e-6 and ce <= 1e-5
+    return outs
+
+
+def _same(a, b):
+    return all(np.array_equal(x.t, y.t) and np.array_equal(x.c, y.c) for x, y in zip(a, b))
+
+
+def test_direct_products_after_a_refused_transform(ctx, monkeypatch):
+    """64 problems of n = 63, m = 5 take two CTAs per SM for the 8192 sub-products (a B' buffer of 252 MB) and one
+    for the direct ones (126 MB): between the two the call gives what the direct products give."""
+    monkeypatch.setenv("PRONY_TC_TUNE", "0")
+    p = W.make_problem("fb", 2, 63, 5, 7200)
+    monkeypatch.setenv("PRONY_ALLOC_MAX", str(160 << 20))
+    got = _solve(ctx, p, 64, "bf16x3")
+    monkeypatch.delenv("PRONY_ALLOC_MAX")
+    monkeypatch.setenv("PRONY_AXIS", "0")
+    assert _same(got, _solve(ctx, p, 64, "bf16x3"))
+    monkeypatch.delenv("PRONY_AXIS")
+    _solve(ctx, p, 64, "bf16x3")
