@@ -761,15 +761,18 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec) {
   }
   int rc;
   const size_t cap = ctx->axP.cap, tcap = ctx->axtw.cap;
-  if ((rc = ensure(ctx->axP, sizeof(ProbDesc) * sub))) return rc;
-  if ((rc = ensure(ctx->axtw, sizeof(float2) * twoff))) return rc;
+  rc = ensure(ctx->axP, sizeof(ProbDesc) * sub);
+  if (!rc) rc = ensure(ctx->axtw, sizeof(float2) * twoff);
+  // a buffer that moved holds nothing, also when a later allocation of this call fails
+  if (ctx->axP.cap != cap || ctx->axtw.cap != tcap) ctx->ax_sig.clear();
+  if (rc) return rc;
   if ((rc = ensure(ctx->axY, sizeof(float2) * std::max(xoff, yoff)))) return rc;
   if (prec == PRONY_FP32) {
     if ((rc = ensure(ctx->axX, sizeof(float2) * xoff))) return rc;
     if ((rc = ensure(ctx->axF, sizeof(float2) * grid))) return rc;
     if ((rc = ensure(ctx->axH, sizeof(float2) * grid))) return rc;
   }
-  if (ctx->axP.cap != cap || ctx->axtw.cap != tcap || sig != ctx->ax_sig) {
+  if (sig != ctx->ax_sig) {
     ctx->ax_sig.clear();
     // twiddles exp(2 pi i j / G) = (cos, sin), rounded from FP64
     std::vector<float2> tw;

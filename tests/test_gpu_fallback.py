@@ -43,3 +43,17 @@ def test_direct_products_after_a_refused_transform(ctx, monkeypatch):
     assert _same(got, _solve(ctx, p, 64, "bf16x3"))
     monkeypatch.delenv("PRONY_AXIS")
     _solve(ctx, p, 64, "bf16x3")
+
+
+def test_layout_known_before_a_refused_one(ctx, monkeypatch):
+    """A layout whose sub-problem descriptors are on the device, a larger one whose descriptors replace them but whose
+    blocks are refused (170 of 128 MB, the direct products' largest 87), then the first again."""
+    small, large = W.make_problem("kl", 2, 63, 5, 7201), W.make_problem("kl", 2, 63, 20, 7202)
+    first = _solve(ctx, small, 2, "fp32")
+    monkeypatch.setenv("PRONY_ALLOC_MAX", str(128 << 20))
+    got = _solve(ctx, large, 64, "fp32")
+    assert _same(_solve(ctx, small, 2, "fp32"), first)
+    monkeypatch.delenv("PRONY_ALLOC_MAX")
+    assert _same(_solve(ctx, small, 2, "fp32"), first)
+    monkeypatch.setenv("PRONY_AXIS", "0")
+    assert _same(got, _solve(ctx, large, 64, "fp32"))
