@@ -80,6 +80,8 @@ struct prony_ctx {
   // products by axis transform: sub-problem descriptors, twiddles, transformed blocks and samples
   DBuf axP, axtw, axX, axY, axF, axH;
   std::vector<int> ax_sig;              // (n, d, m, r0) of every problem axP was built for
+  std::vector<int> ax_refused;          // the last such layout whose transformed products did not fit the device,
+  int ax_refused_prec = -1;             // and in which arithmetic
   int* h_flag = nullptr;            // pinned: loop flag, body counters, error flags (see queue_flags)
   void* pin = nullptr;              // pinned staging of a call's results, grown on demand
   size_t pin_cap = 0;
@@ -723,14 +725,34 @@ bool axis_pays(const std::vector<ProbDesc>& P, int prec) {
   return e ? atoi(e) != 0 : axis < dense;
 }
 
+// What the transformed products of a batch are sized by (sizes only).
+std::vector<int> axis_signature(const std::vector<ProbDesc>& P) {
+  std::vector<int> sig;
+  sig.reserve(4 * P.size());
+  for (const auto& p : P)
+    for (const int v : {p.n, p.d, p.m, p.r0}) sig.push_back(v);
+  return sig;
+}
+
+// Gives back what an attempt at the transformed products allocated or grew.
+void release_axis(prony_ctx* ctx) {
+  DBuf* bufs[] = {&ctx->axP, &ctx->axtw, &ctx->axX, &ctx->axY, &ctx->axF, &ctx->axH, &ctx->xb, &ctx->tabF, &ctx->tabH,
+                  &ctx->tcjobs, &ctx->jobs, &ctx->part, &ctx->cnt};
+  for (DBuf* b : bufs) {
+    if (b->p) cudaFree(b->p);
+    *b = DBuf{};
+  }
+  ctx->ax_sig.clear();
+  ctx->tcjob_sig.clear();
+}
+
 // Sub-problems of the products by axis transform: problem i's G frequencies, each a problem of
 // d - 1 dimensions on the same n, with its own sample tables and blocks.
-int setup_axis(prony_ctx* ctx, Batch& B, int prec) {
+int setup_axis(prony_ctx* ctx, Batch& B, int prec, const std::vector<int>& sig) {
   auto& A = B.ax;
   A.rep.resize(B.P.size());
   long long grid = 0, xoff = 0, yoff = 0, toff = 0, twoff = 0;
   int sub = 0, maxn = 0, maxN = 0, maxNext = 0, maxGd = 0;
-  std::vector<int> sig;
   for (size_t i = 0; i < B.P.size(); ++i) {
     const ProbDesc& p = B.P[i];
     ProbDesc& q = A.rep[i];
@@ -757,7 +779,6 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec) {
     maxN = std::max(maxN, q.N);
     maxNext = std::max(maxNext, q.Next);
     maxGd = std::max(maxGd, q.Gd);
-    for (const int v : {p.n, p.d, p.m, p.r0}) sig.push_back(v);
   }
   int rc;
   const size_t cap = ctx->axP.cap, tcap = ctx->axtw.cap;
@@ -798,7 +819,7 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec) {
     }
     // synchronous with respect to this host copy (pageable memory); stream-ordered on the device
     CK(cudaMemcpyAsync(ctx->axP.p, all.data(), sizeof(ProbDesc) * all.size(), cudaMemcpyHostToDevice, ctx->stream));
-    ctx->ax_sig = std::move(sig);
+    ctx->ax_sig = sig;
   }
   Dev& S = A.S;
   S = B.D;
@@ -974,17 +995,25 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
     if ((rc = setup_fft(ctx, B))) return rc;
     return upload_problems(ctx, B.P);
   }
-  // a batch whose transformed blocks do not fit the device keeps the direct products
+  // A batch whose transformed blocks do not fit the device keeps the direct products.  The attempt's buffers go
+  // first (the direct ones may need their room), and the layout is remembered, so that its next call neither
+  // allocates nor frees.
   if (axis_pays(B.P, o.precision)) {
-    rc = setup_axis(ctx, B, o.precision);
-    if (!rc) rc = setup_products(ctx, B, o.precision);
-    if (rc && rc != PRONY_ENOMEM) return rc;
-    B.ax.on = !rc;
-    if (rc) {
-      cudaGetLastError();
-      B.part = nullptr;
-      B.cnt = nullptr;
-      B.part_jobs = 0;
+    const std::vector<int> sig = axis_signature(B.P);
+    if (o.precision != ctx->ax_refused_prec || sig != ctx->ax_refused) {
+      rc = setup_axis(ctx, B, o.precision, sig);
+      if (!rc) rc = setup_products(ctx, B, o.precision);
+      if (rc && rc != PRONY_ENOMEM) return rc;
+      B.ax.on = !rc;
+      if (rc) {
+        cudaGetLastError();
+        release_axis(ctx);
+        ctx->ax_refused = sig;
+        ctx->ax_refused_prec = o.precision;
+        B.part = nullptr;
+        B.cnt = nullptr;
+        B.part_jobs = 0;
+      }
     }
   }
   if (!B.ax.on && (rc = setup_products(ctx, B, o.precision))) return rc;

@@ -57,3 +57,32 @@ def test_layout_known_before_a_refused_one(ctx, monkeypatch):
     assert _same(_solve(ctx, small, 2, "fp32"), first)
     monkeypatch.setenv("PRONY_AXIS", "0")
     assert _same(got, _solve(ctx, large, 64, "fp32"))
+
+
+def test_refused_transform_keeps_no_memory(ctx, monkeypatch):
+    """After a refused attempt a context holds what the direct products hold (PRONY_AXIS=0 from the start), and further
+    calls of the layout change nothing."""
+    import torch
+    from paper_2012_11430_gb300 import Context
+    monkeypatch.setenv("PRONY_TC_TUNE", "0")
+    p = W.make_problem("km", 2, 63, 20, 7203)
+
+    def held(context, **env):
+        free = torch.cuda.mem_get_info()[0]
+        for k, v in env.items():
+            monkeypatch.setenv(k, v)
+        used = []
+        for _ in range(3):
+            _solve(context, p, 64, "bf16x3")
+            used.append(free - torch.cuda.mem_get_info()[0])
+        for k in env:
+            monkeypatch.delenv(k)
+        return used
+
+    _solve(ctx, p, 2, "bf16x3")                        # kernels and graph memory of the process
+    with Context(0) as direct:
+        a = held(direct, PRONY_AXIS="0")
+    with Context(0) as refused:                        # B' tiles: 629 MB transformed, 315 MB direct
+        b = held(refused, PRONY_ALLOC_MAX=str(512 << 20))
+    assert b[0] == b[1] == b[2]
+    assert abs(a[0] - b[0]) <= 32 << 20
