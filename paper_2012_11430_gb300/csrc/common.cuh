@@ -41,6 +41,7 @@ struct ProbDesc {
                               // a sub-problem: offset of its axis twiddles
   int st;                     // index of the problem's state (a sub-problem: of its parent's)
   int sub;                    // index of the problem's first sub-problem (products by axis transform)
+  long long xchunk;           // index of its first B' tile among those of the batch ((N + 31) / 32 K chunks each)
 };
 
 // Per-problem iteration state, device resident.
@@ -387,28 +388,29 @@ __host__ __device__ inline void tc_window(int fmt, int Gd4, int f_lo, int f_hi, 
 int tc_planes(int kind);
 size_t tc_stage_bytes(int kind, int ntbox);
 size_t tc_smem_bytes(int kind, int fmt, int ntbox, int stages, int win_cap);
-long long tc_prob_stride(int kind, int ntbox, int maxnc);
+// B' tiles (`xb`): those of a product or Gram lie at xb_stride = tc_stage_bytes(kind, ntbox) bytes per K chunk of the
+// batch (ProbDesc::xchunk), those of an X M product at xb_stride bytes per problem.
 // Split K workspace of the tensor-core products: tc_part_floats(ntbox) floats per job, one zeroed
 // counter per job.
 size_t tc_part_floats(int ntbox);
 void launch_split_tables(const Dev& D, int fmt, cudaStream_t s);
-void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long prob_stride,
+void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long xb_stride,
                     cudaStream_t s);
 cudaError_t launch_toeplitz_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int adjoint, int wsel, int ybuf,
                                int y_ext, int kind, int fmt, int ntbox, int win_cap, int stages, int half, const void* xb,
-                               long long prob_stride, float* part, int* cnt, long long part_jobs, int* err,
+                               long long xb_stride, float* part, int* cnt, long long part_jobs, int* err,
                                cudaStream_t s);
 // A stages of a product CTA that shares its SM with a second one (half: 256 columns of tensor memory);
 // 0: the stacked accumulator of ntbox columns per plane leaves no room
 int tc_half_stages(int kind, int ntbox);
 cudaError_t launch_gram_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int xbuf, int xshift, int xw, int zw,
-                           long long out_off, int out_ld, int ntbox, int stages, const void* xb, long long prob_stride,
+                           long long out_off, int out_ld, int ntbox, int stages, const void* xb, long long xb_stride,
                            float* part, int* cnt, long long part_jobs, int* err, cudaStream_t s);
 // OUT = X M (as launch_apply without Z and norm) on the tensor cores, three BF16 planes; jobs: one
 // per row tile of the N rows, nks = 1; OUT is not the box buffer Y.
 cudaError_t launch_apply_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int xbuf, int xw, int outw,
                             long long m_off, int m_double, int outbuf, int ntbox, int stages, void* xb,
-                            long long prob_stride, int* err, cudaStream_t s);
+                            long long xb_stride, int* err, cudaStream_t s);
 
 // kernels_axis.cu (products with the leading axis diagonalised by a DFT).  S: the Dev of the
 // sub-problems (S.P their descriptors, S.V / S.B2 / S.Y the transformed blocks).
@@ -416,7 +418,7 @@ enum AxisMode { AX_FP32 = 0, AX_BF16X3 = 1, AX_TF32X3 = 2, AX_BF16X2 = 3 };   //
 constexpr int AX_MAX_N = 95;          // largest n (twiddle table of (n + 3)/2 x (n + 1) float4 in shared memory)
 cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int fmt, int trim, cudaStream_t s);
 cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int wsel, int maxw, void* xb,
-                           long long prob_stride, cudaStream_t s);
+                           long long xb_stride, cudaStream_t s);
 cudaError_t launch_axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s);
 
 // kernels_refine.cu (Levenberg-Marquardt refinement of (t, c))

@@ -225,7 +225,7 @@ __device__ __forceinline__ void ax_emit(const Dev& S, const ProbDesc& ps, unsign
 // the warps: there the loads' latency counts.
 template <int MODE, int CL, int NC>
 __global__ void __launch_bounds__(256, 2) k_axis_in(Dev D, Dev S, int xbuf, int wsel, unsigned char* xb,
-                                                 long long prob_stride) {
+                                                 long long xb_stride) {
   extern __shared__ float4 ax_tab[];              // [class][h_0] = (cos, cos, sin, sin)
   const ProbDesc& p = D.P[blockIdx.y];
   const ProbState& st = D.st[p.st];
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(256, 2) k_axis_in(Dev D, Dev S, int xbuf, int 
   constexpr int NPL = MODE == AX_BF16X3 ? 3 : 2;
   constexpr int HU = CL * NC == 8 ? 2 : 8;        // h_0 per pass (their loads are in flight together)
   const size_t tile_bytes = (size_t)(MODE == AX_TF32X3 ? 2 : 1) * NPL * NT * 128;
-  const long long items = (long long)nc * ncol * ngrp;
+  const long long items = (long long)nc * ncol * ngrp, xchunk = S.P[p.sub].xchunk;
   for (long long it = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); it < items;
        it += (long long)gridDim.x * (blockDim.x >> 5)) {
     const int grp = (int)(it % ngrp), c = (int)(it / ngrp / ncol), j0 = NC * (int)(it / ngrp % ncol);
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(256, 2) k_axis_in(Dev D, Dev S, int xbuf, int 
         const float2 a = make_float2(ce.x + co.x, ce.y + co.y), b = make_float2(se.x + so.x, se.y + so.y);
         const float2 c2 = make_float2(ce.x - co.x, ce.y - co.y), d2 = make_float2(se.x - so.x, se.y - so.y);
         auto put = [&](int f, float2 v) {
-          ax_emit<MODE>(S, S.P[p.sub + f], xb + prob_stride * (p.sub + f) + (size_t)c * tile_bytes, NT, j0 + k, hp, valid,
+          ax_emit<MODE>(S, S.P[p.sub + f], xb + xb_stride * (xchunk + f * nc) + (size_t)c * tile_bytes, NT, j0 + k, hp, valid,
                         Np, lane, v);
         };
         put(cls, make_float2(a.x + b.y, a.y - b.x));              // cos - i sin
@@ -454,7 +454,7 @@ cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int fmt, in
 
 template <int MODE, int CL, int NC>
 static cudaError_t axis_in_as(const Dev& D, const Dev& S, int xbuf, int wsel, long long items, void* xb,
-                              long long prob_stride, cudaStream_t s) {
+                              long long xb_stride, cudaStream_t s) {
   static size_t set = 0;
   const int H = max_axis_n(S) + 1;
   const size_t sm = sizeof(float4) * (size_t)(H / 2 + 1) * (H + (H & 1));
@@ -463,28 +463,28 @@ static cudaError_t axis_in_as(const Dev& D, const Dev& S, int xbuf, int wsel, lo
   const long long per = items * D.nprob > 152LL * 64 ? 2 : 1;     // items per warp (one twiddle table per block)
   note_launch();
   k_axis_in<MODE, CL, NC><<<dim3(blocks_per_problem((items + 8 * per - 1) / (8 * per), D.nprob), D.nprob), 256, sm, s>>>(
-      D, S, xbuf, wsel, (unsigned char*)xb, prob_stride);
+      D, S, xbuf, wsel, (unsigned char*)xb, xb_stride);
   return cudaGetLastError();
 }
 
 template <int MODE>
-static cudaError_t axis_in(const Dev& D, const Dev& S, int xbuf, int wsel, int maxw, void* xb, long long prob_stride,
+static cudaError_t axis_in(const Dev& D, const Dev& S, int xbuf, int wsel, int maxw, void* xb, long long xb_stride,
                            cudaStream_t s) {
   // items of the largest problem; the wide form from about eight of its warps per SM on
   const int ncls = (max_axis_n(S) + 1) / 2 + 1;
   const long long lines = (long long)((S.maxN + 31) / 32) * ((2 * maxw + 15) / 16 * 8);
   if (lines * ncls / 8 * D.nprob >= 152LL * 8)
-    return axis_in_as<MODE, 4, 2>(D, S, xbuf, wsel, (lines + 1) / 2 * ((ncls + 3) / 4), xb, prob_stride, s);
-  return axis_in_as<MODE, 1, 1>(D, S, xbuf, wsel, lines * ncls, xb, prob_stride, s);
+    return axis_in_as<MODE, 4, 2>(D, S, xbuf, wsel, (lines + 1) / 2 * ((ncls + 3) / 4), xb, xb_stride, s);
+  return axis_in_as<MODE, 1, 1>(D, S, xbuf, wsel, lines * ncls, xb, xb_stride, s);
 }
 
 cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int wsel, int maxw, void* xb,
-                           long long prob_stride, cudaStream_t s) {
+                           long long xb_stride, cudaStream_t s) {
   switch (mode) {
-    case AX_FP32: return axis_in<AX_FP32>(D, S, xbuf, wsel, maxw, xb, prob_stride, s);
-    case AX_TF32X3: return axis_in<AX_TF32X3>(D, S, xbuf, wsel, maxw, xb, prob_stride, s);
-    case AX_BF16X2: return axis_in<AX_BF16X2>(D, S, xbuf, wsel, maxw, xb, prob_stride, s);
-    default: return axis_in<AX_BF16X3>(D, S, xbuf, wsel, maxw, xb, prob_stride, s);
+    case AX_FP32: return axis_in<AX_FP32>(D, S, xbuf, wsel, maxw, xb, xb_stride, s);
+    case AX_TF32X3: return axis_in<AX_TF32X3>(D, S, xbuf, wsel, maxw, xb, xb_stride, s);
+    case AX_BF16X2: return axis_in<AX_BF16X2>(D, S, xbuf, wsel, maxw, xb, xb_stride, s);
+    default: return axis_in<AX_BF16X3>(D, S, xbuf, wsel, maxw, xb, xb_stride, s);
   }
 }
 

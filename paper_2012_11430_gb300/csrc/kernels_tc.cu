@@ -113,7 +113,7 @@ __device__ __forceinline__ void mma_ts(bool tf32, uint32_t d, uint32_t a, uint64
 // byte offset m_off -- complex64 with leading dimension LDR, or complex128 (m_double, rounded to
 // complex64) with leading dimension LDM.
 template <int KIND>
-__global__ void k_xb_prep(Dev D, int xbuf, int xshift, int wsel, unsigned char* xb, long long prob_stride,
+__global__ void k_xb_prep(Dev D, int xbuf, int xshift, int wsel, unsigned char* xb, long long xb_stride,
                           long long m_off, int m_double, int asel) {
   using K = TcKind<KIND>;
   constexpr int NPL = K::NPL;
@@ -132,7 +132,7 @@ __global__ void k_xb_prep(Dev D, int xbuf, int xshift, int wsel, unsigned char* 
   int ldx = 0;
   const float2* X = msrc ? nullptr : tc_buf(D, xbuf, p, ldx);
   const unsigned char* Mb = (const unsigned char*)D.small + p.soff + (msrc ? m_off : 0);
-  unsigned char* out = xb + prob_stride * pi;
+  unsigned char* out = xb + xb_stride * (msrc ? pi : p.xchunk);
   const long long total = (long long)nc * NT * GPC;   // (chunk, row, group)
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
        q += (long long)gridDim.x * blockDim.x) {
@@ -245,7 +245,7 @@ __global__ void k_split_tables(Dev D, int fmt) {
 
 struct TcParams {
   const unsigned char* xb;        // B' tiles (k_xb_prep)
-  long long prob_stride;          // bytes of B' tiles per problem
+  long long xb_stride;            // bytes of B' tiles per K chunk of the batch (APPLY: per problem)
   int adjoint, wsel, ybuf, y_ext;
   int ntbox;                      // B' rows reserved per plane and problem (>= every NT)
   int win_cap;                    // window capacity (entries per table: BF16 a multiple of 8, TF32 of 4)
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_APROD), HALF ? 2 : 1)
                         gtab + 4LL * (GPL * part + pl) * p.Gd4 + (long long)wlo * EB, (uint32_t)(wlen * EB), &bar_win);
       }
       const uint32_t tile_bytes = (uint32_t)K::KHALVES * half_bytes;
-      const unsigned char* src0 = P.xb + P.prob_stride * job.prob + (size_t)c_begin * tile_bytes;
+      const unsigned char* src0 = P.xb + P.xb_stride * (APPLY ? job.prob : p.xchunk) + (size_t)c_begin * tile_bytes;
       int issued = 0;
       int s = 0;
       uint32_t ph = 0;                            // stage and round parity (no divisions in the loop)
@@ -836,10 +836,7 @@ void launch_split_tables(const Dev& D, int fmt, cudaStream_t s) {
   k_split_tables<<<g, 256, 0, s>>>(D, fmt);
 }
 
-// Bytes of B' tiles reserved per problem: every chunk at the widest tile of the batch.
-long long tc_prob_stride(int kind, int ntbox, int maxnc) { return (long long)maxnc * (long long)tc_stage_bytes(kind, ntbox); }
-
-static void xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long prob_stride,
+static void xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long xb_stride,
                     long long m_off, int m_double, int asel, long long src_rows, cudaStream_t s) {
   note_launch();
   // items (chunk, row, 16-byte group) of the largest problem, about four per thread
@@ -848,20 +845,20 @@ static void xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int 
   unsigned char* b = (unsigned char*)xb;
   switch (kind) {
     case PRONY_BF16X3:
-      k_xb_prep<PRONY_BF16X3><<<g, 256, 0, s>>>(D, xbuf, xshift, wsel, b, prob_stride, m_off, m_double, asel);
+      k_xb_prep<PRONY_BF16X3><<<g, 256, 0, s>>>(D, xbuf, xshift, wsel, b, xb_stride, m_off, m_double, asel);
       break;
     case PRONY_BF16X2:
-      k_xb_prep<PRONY_BF16X2><<<g, 256, 0, s>>>(D, xbuf, xshift, wsel, b, prob_stride, m_off, m_double, asel);
+      k_xb_prep<PRONY_BF16X2><<<g, 256, 0, s>>>(D, xbuf, xshift, wsel, b, xb_stride, m_off, m_double, asel);
       break;
     default:
-      k_xb_prep<PRONY_TF32X3><<<g, 256, 0, s>>>(D, xbuf, xshift, wsel, b, prob_stride, m_off, m_double, asel);
+      k_xb_prep<PRONY_TF32X3><<<g, 256, 0, s>>>(D, xbuf, xshift, wsel, b, xb_stride, m_off, m_double, asel);
       break;
   }
 }
 
-void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long prob_stride,
+void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int kind, long long xb_stride,
                     cudaStream_t s) {
-  xb_prep(D, xbuf, xshift, wsel, xb, kind, prob_stride, -1, 0, 0, D.maxN, s);
+  xb_prep(D, xbuf, xshift, wsel, xb, kind, xb_stride, -1, 0, 0, D.maxN, s);
 }
 
 template <int KIND, int MODE, int FMT = TT_TF32, bool HALF = false>
@@ -890,9 +887,9 @@ size_t tc_part_floats(int ntbox) { return (size_t)ntbox * TC_BM; }
 
 cudaError_t launch_toeplitz_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int adjoint, int wsel, int ybuf,
                                int y_ext, int kind, int fmt, int ntbox, int win_cap, int stages, int half, const void* xb,
-                               long long prob_stride, float* part, int* cnt, long long part_jobs, int* err,
+                               long long xb_stride, float* part, int* cnt, long long part_jobs, int* err,
                                cudaStream_t s) {
-  TcParams P{(const unsigned char*)xb, prob_stride, adjoint, wsel, ybuf, y_ext, ntbox, win_cap, stages, part, cnt,
+  TcParams P{(const unsigned char*)xb, xb_stride, adjoint, wsel, ybuf, y_ext, ntbox, win_cap, stages, part, cnt,
              part_jobs, 0, -1, 0, 0, 0};
   const size_t sm = tc_smem_bytes(kind, fmt, ntbox, stages, win_cap);
   note_launch();
@@ -912,9 +909,9 @@ cudaError_t launch_toeplitz_tc(const Dev& D, const ToeplitzJob* jobs, int njobs,
 // The Gram X^* Z of two tall blocks on the tensor cores in three BF16 planes (B' tiles of Z from
 // k_xb_prep at `xb`), one CTA per problem and K range (jobs: row tile 0).
 cudaError_t launch_gram_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int xbuf, int xshift, int xw, int zw,
-                           long long out_off, int out_ld, int ntbox, int stages, const void* xb, long long prob_stride,
+                           long long out_off, int out_ld, int ntbox, int stages, const void* xb, long long xb_stride,
                            float* part, int* cnt, long long part_jobs, int* err, cudaStream_t s) {
-  TcParams P{(const unsigned char*)xb, prob_stride, 0, zw, 0, 0, ntbox, 0, stages, part, cnt, part_jobs,
+  TcParams P{(const unsigned char*)xb, xb_stride, 0, zw, 0, 0, ntbox, 0, stages, part, cnt, part_jobs,
              xbuf, xshift, xw, out_off, out_ld};
   const size_t sm = tc_smem_bytes(PRONY_BF16X3, TT_WIDE, ntbox, stages, 0);
   note_launch();
@@ -925,9 +922,9 @@ cudaError_t launch_gram_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int
 // workspace at m_off) by k_xb_prep, then one CTA per row tile of N rows (jobs with nks = 1).
 cudaError_t launch_apply_tc(const Dev& D, const ToeplitzJob* jobs, int njobs, int xbuf, int xw, int outw,
                             long long m_off, int m_double, int outbuf, int ntbox, int stages, void* xb,
-                            long long prob_stride, int* err, cudaStream_t s) {
-  xb_prep(D, -1, -1, outw, xb, PRONY_BF16X3, prob_stride, m_off, m_double, xw, D.maxR0, s);
-  TcParams P{(const unsigned char*)xb, prob_stride, 0, outw, outbuf, 0, ntbox, 0, stages, nullptr, nullptr, 0,
+                            long long xb_stride, int* err, cudaStream_t s) {
+  xb_prep(D, -1, -1, outw, xb, PRONY_BF16X3, xb_stride, m_off, m_double, xw, D.maxR0, s);
+  TcParams P{(const unsigned char*)xb, xb_stride, 0, outw, outbuf, 0, ntbox, 0, stages, nullptr, nullptr, 0,
              xbuf, -1, xw, 0, 0};
   // at least half the shared memory of an SM, so that one CTA holds an SM (and all of its tensor
   // memory) at a time

@@ -148,7 +148,7 @@ struct TcConf {
   int kind = PRONY_BF16X3, ntbox = 16, stages = 2, win_cap = 0, nks = 1;
   int half = 0;                       // two CTAs per SM
   int fmt = 0;                        // TcTable format of the sample tables
-  long long prob_stride = 0;          // bytes of B' tiles per problem
+  long long xb_stride = 0;          // bytes of a B' tile
   int njobs_ext = 0, njobs_in = 0;
   ToeplitzJob* jobs_ext = nullptr;
   ToeplitzJob* jobs_in = nullptr;
@@ -156,7 +156,7 @@ struct TcConf {
   // tall-skinny Grams on the tensor cores (three BF16 planes): one CTA per problem and K range
   bool gram = false;
   int nks_gram = 1, gram_stages = 2, njobs_gram = 0;
-  long long gram_stride = 0;          // bytes of the Gram's B' tiles per problem
+  long long gram_stride = 0;          // bytes of a B' tile of the Grams
   ToeplitzJob* jobs_gram = nullptr;
   // X M products of the tall blocks on the tensor cores (three BF16 planes): one CTA per row tile
   bool apply = false;
@@ -371,13 +371,12 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   const int npl = tc_planes(prec);
   T.ntbox = ((2 * maxw + 15) / 16) * 16;
   const std::vector<ProbDesc>& Q = B.shapes();
-  int maxnc = 0, maxrows = 0, tiles_ext = 0, tiles_in = 0, nprod = 0;
+  int maxnc = 0, maxrows = 0, tiles_ext = 0, tiles_in = 0;
   for (size_t i = 0; i < Q.size(); ++i) {
     maxnc = std::max(maxnc, (Q[i].N + 31) / 32);
     maxrows = std::max(maxrows, B.P[i].N);
     tiles_ext += B.copies(i) * ((Q[i].Next + 127) / 128);
     tiles_in += B.copies(i) * ((Q[i].N + 127) / 128);
-    nprod += B.copies(i);
   }
   const size_t stage = tc_stage_bytes(prec, T.ntbox);
   const size_t avail = 227 * 1024 - 2048 - 4608;   // static shared memory of the kernel (chunk table)
@@ -484,7 +483,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     }
   }
   T.nks_min = nks;
-  T.prob_stride = tc_prob_stride(prec, T.ntbox, maxnc);
+  T.xb_stride = (long long)stage;
   // Grams of the tall blocks on the tensor cores, on request only (PRONY_TC_GRAM=1): the FP32
   // accumulator in tensor memory rounds once per MMA, and the Grams of CholeskyQR2, of Q = U^* T V
   // and of U^* T_l V need FP32-level accuracy: with them on the tensor cores the power iteration's
@@ -501,7 +500,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     T.nks_gram = std::max(T.nks_gram, (gnc + 63) / 64);         // at most 64 K chunks per CTA
     const size_t gstage = tc_stage_bytes(PRONY_BF16X3, T.ntbox);
     T.gram_stages = (int)std::max<size_t>(1, std::min<size_t>(4, (avail - 1024) / gstage));
-    T.gram_stride = tc_prob_stride(PRONY_BF16X3, T.ntbox, gnc);
+    T.gram_stride = (long long)gstage;
   }
   // X M products of the tall blocks (CholeskyQR2, the final U and V) on the tensor cores in three
   // BF16 planes, FP32-exact operands: the inner dimension is at most r0 <= 128 (four K chunks), so
@@ -516,7 +515,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     const int maxac = (maxw + 31) / 32;
     const size_t astage = tc_stage_bytes(PRONY_BF16X3, T.ntbox);
     T.apply_stages = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::min(4, maxac), (avail - 1024) / astage));
-    T.apply_stride = tc_prob_stride(PRONY_BF16X3, T.ntbox, maxac);
+    T.apply_stride = maxac * (long long)astage;
   }
   // batch shape signature for the tuning cache
   T.key = std::to_string(prec) + (B.ax.on ? "a" : "") + (T.half ? "h" : "") + std::to_string(T.fmt) + ":" + std::to_string(B.P.size()) + ":" + std::to_string(maxw) + ":" +
@@ -539,10 +538,11 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   DT.tabF = (uint32_t*)ctx->tabF.p;
   DT.tabH = (uint32_t*)ctx->tabH.p;
   // B' tiles of the products and (three BF16 planes) of the Grams share one buffer
-  if ((rc = ensure(ctx->xb, std::max((size_t)nprod * (size_t)T.prob_stride,
-                                     B.P.size() * (size_t)std::max(T.gram ? T.gram_stride : 0LL,
-                                                                   T.apply ? T.apply_stride : 0LL)))))
-    return rc;
+  auto chunks = [&](const ProbDesc& last, int copies) { return last.xchunk + copies * ((last.N + 31LL) / 32); };
+  const long long xb_bytes = std::max(chunks(Q.back(), B.copies(Q.size() - 1)) * T.xb_stride,
+                                      std::max(T.gram ? chunks(B.P.back(), 1) * T.gram_stride : 0LL,
+                                               T.apply ? (long long)B.P.size() * T.apply_stride : 0LL));
+  if ((rc = ensure(ctx->xb, (size_t)xb_bytes))) return rc;
   // (zeroed when allocated and after an error)
   if (!ctx->tcerr.p) {
     if ((rc = ensure(ctx->tcerr, 256))) return rc;
@@ -595,10 +595,10 @@ void toeplitz_product(prony_ctx* ctx, const Batch& B, const Dev& D, int ext, int
     const TcConf& T = B.tc;
     const Dev& S = B.ax.S;
     const int sbuf = ext ? BUF_Y : BUF_B2;
-    cudaError_t e = launch_axis_in(D, S, prec, xbuf, wsel, B.maxw, ctx->xb.p, T.prob_stride, s);
+    cudaError_t e = launch_axis_in(D, S, prec, xbuf, wsel, B.maxw, ctx->xb.p, T.xb_stride, s);
     if (e == cudaSuccess && T.on)
       e = launch_toeplitz_tc(S, ext ? T.jobs_ext : T.jobs_in, ext ? T.njobs_ext : T.njobs_in, adjoint, wsel, sbuf, ext,
-                             T.kind, T.fmt, T.ntbox, T.win_cap, T.stages, T.half, ctx->xb.p, T.prob_stride, (float*)B.part, B.cnt,
+                             T.kind, T.fmt, T.ntbox, T.win_cap, T.stages, T.half, ctx->xb.p, T.xb_stride, (float*)B.part, B.cnt,
                              B.part_jobs, T.err, s);
     else if (e == cudaSuccess)
       launch_toeplitz(S, ext ? B.jobs_ext : B.jobs_in, ext ? B.njobs_ext : B.njobs_in, adjoint, BUF_V, wsel, sbuf, ext,
@@ -607,10 +607,10 @@ void toeplitz_product(prony_ctx* ctx, const Batch& B, const Dev& D, int ext, int
     if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
   } else if (B.tc.on) {
     const TcConf& T = B.tc;
-    launch_xb_prep(D, xbuf, -1, wsel, ctx->xb.p, T.kind, T.prob_stride, s);
+    launch_xb_prep(D, xbuf, -1, wsel, ctx->xb.p, T.kind, T.xb_stride, s);
     cudaError_t e = launch_toeplitz_tc(D, ext ? T.jobs_ext : T.jobs_in, ext ? T.njobs_ext : T.njobs_in, adjoint,
                                        wsel, ybuf, ext, T.kind, T.fmt, T.ntbox, T.win_cap, T.stages, T.half, ctx->xb.p,
-                                       T.prob_stride, (float*)B.part, B.cnt, B.part_jobs, T.err, s);
+                                       T.xb_stride, (float*)B.part, B.cnt, B.part_jobs, T.err, s);
     if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
   } else {
     launch_toeplitz(D, ext ? B.jobs_ext : B.jobs_in, ext ? B.njobs_ext : B.njobs_in, adjoint, xbuf, wsel, ybuf, ext,
@@ -751,7 +751,7 @@ void release_axis(prony_ctx* ctx) {
 int setup_axis(prony_ctx* ctx, Batch& B, int prec, const std::vector<int>& sig) {
   auto& A = B.ax;
   A.rep.resize(B.P.size());
-  long long grid = 0, xoff = 0, yoff = 0, toff = 0, twoff = 0;
+  long long grid = 0, xoff = 0, yoff = 0, toff = 0, twoff = 0, xchunk = 0;
   int sub = 0, maxn = 0, maxN = 0, maxNext = 0, maxGd = 0;
   for (size_t i = 0; i < B.P.size(); ++i) {
     const ProbDesc& p = B.P[i];
@@ -767,6 +767,7 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec, const std::vector<int>& sig) 
     q.yoff = yoff;
     q.toff = toff;
     q.foff = twoff;
+    q.xchunk = xchunk;
     q.st = (int)i;
     q.sub = -1;
     sub += p.G;                                  // = p.sub of the next problem
@@ -775,6 +776,7 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec, const std::vector<int>& sig) 
     yoff += (long long)p.G * q.Next * q.r0;
     toff += 6LL * p.G * q.Gd4;
     twoff += p.G;
+    xchunk += (long long)p.G * ((q.N + 31) / 32);
     maxn = std::max(maxn, p.n);
     maxN = std::max(maxN, q.N);
     maxNext = std::max(maxNext, q.Next);
@@ -815,6 +817,7 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec, const std::vector<int>& sig) 
         q.xoff += (long long)q.N * q.r0;
         q.yoff += (long long)q.Next * q.r0;
         q.toff += 6LL * q.Gd4;
+        q.xchunk += (q.N + 31) / 32;
       }
     }
     // synchronous with respect to this host copy (pageable memory); stream-ordered on the device
@@ -889,7 +892,7 @@ int setup_products(prony_ctx* ctx, Batch& B, int prec) {
 int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opts& o, Batch& B, bool product_only = false) {
   const int np = (int)hp.size();
   B.P.resize(np);
-  long long goff = 0, xoff = 0, yoff = 0, toff = 0;
+  long long goff = 0, xoff = 0, yoff = 0, toff = 0, xchunk = 0;
   int sub = 0;
   int maxN = 0, maxNext = 0, maxGd = 0, maxR0 = 0, maxM = 0, maxD = 0;
   long long tiles_ext = 0, tiles_in = 0;
@@ -919,6 +922,8 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
     p.Gd4 = (p.Gd + 3) & ~3;
     p.toff = toff;
     toff += 6LL * p.Gd4;
+    p.xchunk = xchunk;
+    xchunk += (p.N + 31) / 32;
     goff += p.Gd;
     xoff += (long long)p.N * p.r0;
     yoff += (long long)p.Next * p.r0;
@@ -1065,7 +1070,7 @@ std::string loop_graph_key(const Batch& B, const void* xb, const int* dflag, int
   put(B.P.data(), sizeof(ProbDesc) * B.P.size());
   const TcConf& T = B.tc;
   const long long tc[] = {T.on, T.half, T.fmt, T.kind, T.ntbox, T.stages, T.win_cap, T.nks, (long long)(size_t)B.part,
-                          (long long)(size_t)B.cnt, B.part_jobs, T.prob_stride, T.njobs_ext,
+                          (long long)(size_t)B.cnt, B.part_jobs, T.xb_stride, T.njobs_ext,
                           T.njobs_in, (long long)(size_t)T.jobs_ext, (long long)(size_t)T.jobs_in,
                           (long long)(size_t)T.err, B.fft.on, B.fft.lz, B.fft.maxpts, B.njobs_ext, B.njobs_in, B.nks,
                           B.maxw, (long long)(size_t)B.jobs_ext, (long long)(size_t)B.jobs_in,

@@ -86,3 +86,27 @@ def test_refused_transform_keeps_no_memory(ctx, monkeypatch):
         b = held(refused, PRONY_ALLOC_MAX=str(512 << 20))
     assert b[0] == b[1] == b[2]
     assert abs(a[0] - b[0]) <= 32 << 20
+
+
+def test_mixed_batch_memory(ctx, monkeypatch):
+    """200 problems of d = 2 beside one of d = 3, whose sub-products have 13 K chunks instead of 2: the transformed
+    products hold about twice the blocks of the direct ones (2 (n + 1) (n + 2)^(d - 1) rows for (n + 2)^d), whatever
+    the widest sub-product of the batch."""
+    import torch
+    from paper_2012_11430_gb300 import Context, default_opts
+    monkeypatch.setenv("PRONY_TC_TUNE", "0")
+    p2, p3 = W.make_problem("mb2", 2, 63, 6, 7204), W.make_problem("mb3", 3, 19, 6, 7205)
+    ps = [p2] * 200 + [p3]
+    used = {}
+    for axis in ("0", "1"):
+        monkeypatch.setenv("PRONY_AXIS", axis)
+        with Context(0) as c:
+            free = torch.cuda.mem_get_info()[0]
+            outs, rc = c.solve_batched([p.grid for p in ps], [p.d for p in ps], [p.n for p in ps], [p.m for p in ps],
+                                       default_opts(precision="bf16x3"))
+            used[axis] = free - torch.cuda.mem_get_info()[0]
+        assert rc == 0
+        for o, p in ((outs[0], p2), (outs[199], p2), (outs[200], p3)):
+            te, ce = W.match_to_truth(o.t, o.c, p.t, p.c)
+            assert te <= 1e-6 and ce <= 1e-5
+    assert used["1"] <= 3 * used["0"]
