@@ -287,7 +287,7 @@ __device__ void svd_jacobi(const Dev& D, ProbState& st, const double2* Q, int a,
 
 // ----------------------------------------------------------------------------- SVD of Q and S_l
 template <int CL, int NT>
-__global__ void __launch_bounds__(NT) k_svd_S(Dev D) {
+__global__ void __launch_bounds__(NT) k_svd_S(Dev D, int cols) {
   extern __shared__ double2 zsm[];
   __shared__ double s_red[32];
   __shared__ double s_lam[PRONY_MMAX], s_inv[PRONY_MMAX];
@@ -477,24 +477,31 @@ __global__ void __launch_bounds__(NT) k_svd_S(Dev D) {
   // ---- U_Q = Q V_Q Sigma^{-1}, S_l = (U_Q^* M_l) V_Q Sigma^{-1}: this CTA takes the columns (of U_Q) and
   // rows (of S_l) i = rank mod CL, so no other CTA's results are needed
   const int ni = (b - rank + CL - 1) / CL;       // how many
-  double2* sU = sA + (size_t)a * b;              // a x ni
-  double2* sP = sU + (size_t)a * ((b + CL - 1) / CL);   // ni x b
+  // `cols` of them at a time where shared memory does not hold all (a = 128, b = 64 and narrow clusters)
+  const int cw = min(cols, (b + CL - 1) / CL);
+  double2* sU = sA + (size_t)max(a, b) * b;      // a x cw
+  double2* sP = sU + (size_t)a * cw;             // cw x b
   double2* UQ = (double2*)(sb + D.L.uq);
   for (int e = threadIdx.x; e < a * ni; e += NT) {
     const int r = e / ni, c = e % ni, i = rank + c * CL;
     const double2 u = cscale(zdot<false>(sA + r * b, 1, sVQ + i, b, b), s_inv[i]);
-    sU[e] = u;
+    if (ni <= cw) sU[e] = u;
     UQ[r * LM + i] = u;
   }
   for (int l = 0; l < p.d; ++l) {
     __syncthreads();
     stage(sA, (const double2*)(sb + D.L.mproj) + (size_t)l * D.L.LDR * LM, LM, a, b);
-    __syncthreads();
-    for (int e = threadIdx.x; e < ni * b; e += NT) sP[e] = zdot<true>(sU + e / b, ni, sA + e % b, b, a);
-    __syncthreads();
     double2* S = (double2*)(sb + D.L.S) + (size_t)l * LM * LM;
-    for (int e = threadIdx.x; e < ni * b; e += NT)
-      S[(rank + e / b * CL) * LM + e % b] = cscale(zdot<false>(sP + (e / b) * b, 1, sVQ + e % b, b, b), s_inv[e % b]);
+    for (int c0 = 0; c0 < ni; c0 += cw) {
+      const int nc = min(cw, ni - c0);
+      if (ni > cw)                               // (this CTA's own columns, written above)
+        for (int e = threadIdx.x; e < a * nc; e += NT) sU[e] = UQ[(e / nc) * LM + rank + (c0 + e % nc) * CL];
+      __syncthreads();
+      for (int e = threadIdx.x; e < nc * b; e += NT) sP[e] = zdot<true>(sU + e / b, nc, sA + e % b, b, a);
+      __syncthreads();
+      for (int e = threadIdx.x; e < nc * b; e += NT)
+        S[(rank + (c0 + e / b) * CL) * LM + e % b] = cscale(zdot<false>(sP + (e / b) * b, 1, sVQ + e % b, b, b), s_inv[e % b]);
+    }
   }
 }
 
@@ -1037,17 +1044,21 @@ cudaError_t launch_cluster(void (*kernel)(Args...), int cl, int threads, size_t 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Shared memory of k_svd_S: V_Q, an a x b operand, columns of U_Q and rows of P (the Jacobi columns, FP32, fit as well).
+constexpr size_t SVD_SMEM = 227 * 1024 - 2560;   // what a block may have, less the kernel's static part
 template <int CL, int NT>
 void run_svd(const Dev& D, cudaStream_t s) {
   static size_t set = 0;
-  const size_t a = D.L.LDR, b = D.L.LDM, own = (b + CL - 1) / CL;
-  // V_Q, an a x b operand, own columns of U_Q, own rows of P; the Jacobi columns (FP32) fit as well
-  const size_t sm = sizeof(double2) * (b * b + std::max(a, b) * b + a * own + own * b);
+  const size_t a = std::max(D.L.LDR, D.L.LDM), b = D.L.LDM;
+  // as many of the CTA's columns of U_Q as fit: all of them but for a >= 98 (CL = 1) to 124 (CL = 4), r0 = 2 m; at
+  // least ten (a = 128, b = 64)
+  const size_t fixed = b * b + a * b, cols = std::min((b + CL - 1) / CL, (SVD_SMEM / sizeof(double2) - fixed) / (a + b));
+  const size_t sm = sizeof(double2) * (fixed + (a + b) * cols);
   if (sm > set) {
     cudaFuncSetAttribute(k_svd_S<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     set = sm;
   }
-  launch_cluster(k_svd_S<CL, NT>, CL, NT, sm, D.nprob, s, D);
+  launch_cluster(k_svd_S<CL, NT>, CL, NT, sm, D.nprob, s, D, (int)cols);
 }
 
 template <int CL, int NT>

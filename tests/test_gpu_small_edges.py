@@ -111,3 +111,29 @@ def test_pivoted_blocks_repeat(ctx, n, m):
     for outs, rc in runs:
         assert rc == 0
         assert all(np.array_equal(o.t, first.t) and np.array_equal(o.c, first.c) for o in outs)
+
+
+@pytest.mark.parametrize("count", [40, 80, 160])
+@pytest.mark.parametrize("n,m", [(23, 50), (27, 58), (31, 64)])
+def test_wide_problems_in_batches(ctx, count, n, m):
+    """The widest blocks (r0 = 2 m up to 128) in batches for which a problem gets four, two or one CTAs: its columns of
+    U_Q are then taken a few at a time."""
+    probs = [W.make_problem(f"wd{i}", 2, n, m, 7300 + m + i) for i in range(3)]
+    outs, rc = ctx.solve_batched([probs[i % 3].grid for i in range(count)], [2] * count, [n] * count, [m] * count)
+    assert rc == 0
+    for k in range(count):
+        p = probs[k % 3]
+        te, ce = W.match_to_truth(outs[k].t, outs[k].c, p.t, p.c)
+        assert te <= 1e-6 and ce <= 1e-5, (k, te, ce)
+        assert np.array_equal(outs[k].t, outs[k % 3].t) and np.array_equal(outs[k].c, outs[k % 3].c)
+
+
+def test_one_wide_problem_among_many(ctx):
+    """The block sizes of a call are those of its widest problem."""
+    wide, narrow = W.make_problem("wm", 2, 31, 64, 7400), W.make_problem("wn", 2, 9, 3, 7401)
+    ps = [narrow] * 199 + [wide]
+    outs, rc = ctx.solve_batched([p.grid for p in ps], [p.d for p in ps], [p.n for p in ps], [p.m for p in ps])
+    assert rc == 0
+    for o, p in zip(outs, ps):
+        te, ce = W.match_to_truth(o.t, o.c, p.t, p.c)
+        assert te <= 1e-6 and ce <= 1e-5
