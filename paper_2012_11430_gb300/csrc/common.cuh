@@ -448,9 +448,9 @@ void launch_lz_all_done(const Dev& D, int* flag, cudaStream_t s);
 // kernels_small.cu
 enum QrMode { QR_PLAIN = 0, QR_DROP = 1, QR_RANK = 2, QR_AUTO = 3 };   // AUTO: RANK on a problem's first iteration
 void launch_chol(const Dev& D, int wsel, int target, int mode, double tol, int rank_mode, cudaStream_t s);
-void launch_svd_S(const Dev& D, cudaStream_t s);
+cudaError_t launch_svd_S(const Dev& D, cudaStream_t s);
 void launch_canon(const Dev& D, cudaStream_t s);
-void launch_eig_t(const Dev& D, unsigned long long seed, cudaStream_t s);
+cudaError_t launch_eig_t(const Dev& D, unsigned long long seed, cudaStream_t s);
 void launch_solve_c(const Dev& D, cudaStream_t s);
 void launch_check(const Dev& D, double tol_power, int max_iter, int* all_done, cudaStream_t s);
 void launch_reset_done(const Dev& D, cudaStream_t s);

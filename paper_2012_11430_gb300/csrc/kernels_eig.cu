@@ -1047,7 +1047,7 @@ cudaError_t launch_cluster(void (*kernel)(Args...), int cl, int threads, size_t 
 // Shared memory of k_svd_S: V_Q, an a x b operand, columns of U_Q and rows of P (the Jacobi columns, FP32, fit as well).
 constexpr size_t SVD_SMEM = 227 * 1024 - 2560;   // what a block may have, less the kernel's static part
 template <int CL, int NT>
-void run_svd(const Dev& D, cudaStream_t s) {
+cudaError_t run_svd(const Dev& D, cudaStream_t s) {
   static size_t set = 0;
   const size_t a = std::max(D.L.LDR, D.L.LDM), b = D.L.LDM;
   // as many of the CTA's columns of U_Q as fit: all of them but for a >= 98 (CL = 1) to 124 (CL = 4), r0 = 2 m; at
@@ -1055,24 +1055,26 @@ void run_svd(const Dev& D, cudaStream_t s) {
   const size_t fixed = b * b + a * b, cols = std::min((b + CL - 1) / CL, (SVD_SMEM / sizeof(double2) - fixed) / (a + b));
   const size_t sm = sizeof(double2) * (fixed + (a + b) * cols);
   if (sm > set) {
-    cudaFuncSetAttribute(k_svd_S<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(k_svd_S<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
     set = sm;
   }
-  launch_cluster(k_svd_S<CL, NT>, CL, NT, sm, D.nprob, s, D, (int)cols);
+  return launch_cluster(k_svd_S<CL, NT>, CL, NT, sm, D.nprob, s, D, (int)cols);
 }
 
 template <int CL, int NT>
-void run_eig(const Dev& D, const MuTable& mu, cudaStream_t s) {
+cudaError_t run_eig(const Dev& D, const MuTable& mu, cudaStream_t s) {
   static size_t set = 0;
   const size_t m = D.L.LDM, own = (m + CL - 1) / CL;
   // W and two more m x m operands (the correction's FP32 blocks fit in those); the FP32 iterations' three
   const size_t sm = std::max(sizeof(double2) * (m * m + std::max(2 * m * m, (m * m + 3 * m * own + 1) / 2)),
                              sizeof(float2) * 3 * m * (NT > 512 ? 65 : 33));
   if (sm > set) {
-    cudaFuncSetAttribute(k_eig_t<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(k_eig_t<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
     set = sm;
   }
-  launch_cluster(k_eig_t<CL, NT>, CL, NT, sm, D.nprob, s, D, mu);
+  return launch_cluster(k_eig_t<CL, NT>, CL, NT, sm, D.nprob, s, D, mu);
 }
 }  // namespace
 
@@ -1084,21 +1086,21 @@ static int cluster_of(const Dev& D) {
   return want >= 8 && fit >= 8 ? 8 : want >= 4 && fit >= 4 ? 4 : want >= 4 && fit >= 2 ? 2 : 1;
 }
 
-void launch_svd_S(const Dev& D, cudaStream_t s) {
+cudaError_t launch_svd_S(const Dev& D, cudaStream_t s) {
   const int cl = cluster_of(D);
   if (D.L.LDM > 32) {
-    if (cl == 8) run_svd<8, 640>(D, s);
-    else if (cl == 4) run_svd<4, 640>(D, s);
-    else if (cl == 2) run_svd<2, 640>(D, s);
-    else run_svd<1, 640>(D, s);
+    if (cl == 8) return run_svd<8, 640>(D, s);
+    if (cl == 4) return run_svd<4, 640>(D, s);
+    if (cl == 2) return run_svd<2, 640>(D, s);
+    return run_svd<1, 640>(D, s);
   } else if (D.L.LDM > 16) {
-    if (cl == 4) run_svd<4, 512>(D, s);
-    else if (cl == 2) run_svd<2, 512>(D, s);
-    else run_svd<1, 512>(D, s);
+    if (cl == 4) return run_svd<4, 512>(D, s);
+    if (cl == 2) return run_svd<2, 512>(D, s);
+    return run_svd<1, 512>(D, s);
   } else {
-    if (cl == 4) run_svd<4, 128>(D, s);
-    else if (cl == 2) run_svd<2, 128>(D, s);
-    else run_svd<1, 128>(D, s);
+    if (cl == 4) return run_svd<4, 128>(D, s);
+    if (cl == 2) return run_svd<2, 128>(D, s);
+    return run_svd<1, 128>(D, s);
   }
 }
 
@@ -1107,7 +1109,7 @@ void launch_canon(const Dev& D, cudaStream_t s) {
   k_canon<<<D.nprob, 256, 0, s>>>(D);
 }
 
-void launch_eig_t(const Dev& D, unsigned long long seed, cudaStream_t s) {
+cudaError_t launch_eig_t(const Dev& D, unsigned long long seed, cudaStream_t s) {
   double2 g[PRONY_DMAX];                         // complex normals (the draw convention of Philox above)
   for (int l = 0; l < PRONY_DMAX; ++l) {
     uint64_t c[4] = {(uint64_t)l, 0, 0, 0};
@@ -1123,17 +1125,17 @@ void launch_eig_t(const Dev& D, unsigned long long seed, cudaStream_t s) {
   }
   const int cl = cluster_of(D);
   if (D.L.LDM > 32) {
-    if (cl == 8) run_eig<8, 640>(D, mu, s);
-    else if (cl == 4) run_eig<4, 640>(D, mu, s);
-    else if (cl == 2) run_eig<2, 640>(D, mu, s);
-    else run_eig<1, 640>(D, mu, s);
+    if (cl == 8) return run_eig<8, 640>(D, mu, s);
+    if (cl == 4) return run_eig<4, 640>(D, mu, s);
+    if (cl == 2) return run_eig<2, 640>(D, mu, s);
+    return run_eig<1, 640>(D, mu, s);
   } else if (D.L.LDM > 16) {
-    if (cl == 4) run_eig<4, 512>(D, mu, s);
-    else if (cl == 2) run_eig<2, 512>(D, mu, s);
-    else run_eig<1, 512>(D, mu, s);
+    if (cl == 4) return run_eig<4, 512>(D, mu, s);
+    if (cl == 2) return run_eig<2, 512>(D, mu, s);
+    return run_eig<1, 512>(D, mu, s);
   } else {
-    if (cl == 4) run_eig<4, 128>(D, mu, s);
-    else if (cl == 2) run_eig<2, 128>(D, mu, s);
-    else run_eig<1, 128>(D, mu, s);
+    if (cl == 4) return run_eig<4, 128>(D, mu, s);
+    if (cl == 2) return run_eig<2, 128>(D, mu, s);
+    return run_eig<1, 128>(D, mu, s);
   }
 }

@@ -96,7 +96,7 @@ struct prony_ctx {
   std::vector<std::vector<ProbState>> snaps;
   prony_stats stats{};
   long long launch_base = 0;
-  cudaError_t launch_err = cudaSuccess;   // first failed tensor-core launch of the current call
+  cudaError_t launch_err = cudaSuccess;   // first failed launch of the current call
   std::map<std::string, int> tc_tuned;   // batch shape -> K split
   // the tensor-core job list on the device: (nks, P, then n and d of every problem) it was
   // built for, and its ext / in counts (a repeated batch layout skips the rebuild and the upload)
@@ -552,7 +552,9 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
   return tc_set_jobs(ctx, B, nks0);
 }
 
-// One Toeplitz block product for every live problem of the batch.
+void note_launch_error(prony_ctx* ctx, cudaError_t e) {
+  if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+}
 
 // The Gram X^* Z of two tall blocks (N rows) for every live problem: out (FP64, small workspace at
 // out_off, leading dimension out_ld) = sum over the rows r in I_n of conj(X[r, a]) Z[r, b]; on the
@@ -564,7 +566,7 @@ void gram(prony_ctx* ctx, const Batch& B, const Dev& D, int xbuf, int xshift, in
     launch_xb_prep(D, zbuf, zshift, zw, ctx->xb.p, PRONY_BF16X3, T.gram_stride, s);
     cudaError_t e = launch_gram_tc(D, T.jobs_gram, T.njobs_gram, xbuf, xshift, xw, zw, out_off, out_ld, T.ntbox,
                                    T.gram_stages, ctx->xb.p, T.gram_stride, (float*)B.part, B.cnt, B.part_jobs, T.err, s);
-    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+    note_launch_error(ctx, e);
   } else {
     launch_gram(D, xbuf, xshift, xw, zbuf, zshift, zw, out_off, out_ld, s);
   }
@@ -579,7 +581,7 @@ void apply(prony_ctx* ctx, const Batch& B, const Dev& D, int xbuf, int xw, int o
   if (T.on && T.apply && outbuf != BUF_Y) {
     cudaError_t e = launch_apply_tc(D, T.jobs_apply, T.njobs_apply, xbuf, xw, outw, m_off, m_double, outbuf, T.ntbox,
                                     T.apply_stages, ctx->xb.p, T.apply_stride, T.err, s);
-    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+    note_launch_error(ctx, e);
   } else {
     launch_apply(D, xbuf, xw, outw, m_off, m_double, -1, outbuf, 0, s);
   }
@@ -604,14 +606,14 @@ void toeplitz_product(prony_ctx* ctx, const Batch& B, const Dev& D, int ext, int
       launch_toeplitz(S, ext ? B.jobs_ext : B.jobs_in, ext ? B.njobs_ext : B.njobs_in, adjoint, BUF_V, wsel, sbuf, ext,
                       B.maxw, B.part, B.cnt, B.part_jobs, s);
     if (e == cudaSuccess) e = launch_axis_out(D, S, wsel, ybuf, ext, B.maxw, s);
-    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+    note_launch_error(ctx, e);
   } else if (B.tc.on) {
     const TcConf& T = B.tc;
     launch_xb_prep(D, xbuf, -1, wsel, ctx->xb.p, T.kind, T.xb_stride, s);
     cudaError_t e = launch_toeplitz_tc(D, ext ? T.jobs_ext : T.jobs_in, ext ? T.njobs_ext : T.njobs_in, adjoint,
                                        wsel, ybuf, ext, T.kind, T.fmt, T.ntbox, T.win_cap, T.stages, T.half, ctx->xb.p,
                                        T.xb_stride, (float*)B.part, B.cnt, B.part_jobs, T.err, s);
-    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+    note_launch_error(ctx, e);
   } else {
     launch_toeplitz(D, ext ? B.jobs_ext : B.jobs_in, ext ? B.njobs_ext : B.njobs_in, adjoint, xbuf, wsel, ybuf, ext,
                     B.maxw, B.part, B.cnt, B.part_jobs, s);
@@ -846,7 +848,7 @@ int setup_axis(prony_ctx* ctx, Batch& B, int prec, const std::vector<int>& sig) 
 void product_tables(prony_ctx* ctx, const Batch& B, int prec, int trim, cudaStream_t s) {
   if (B.ax.on) {
     const cudaError_t e = launch_axis_tables(B.D, B.ax.S, prec, B.tc.fmt, trim, s);
-    if (e != cudaSuccess && ctx->launch_err == cudaSuccess) ctx->launch_err = e;
+    note_launch_error(ctx, e);
   } else if (B.tc.on) {
     launch_split_tables(B.D, B.tc.fmt, s);
   }
@@ -891,6 +893,7 @@ int setup_products(prony_ctx* ctx, Batch& B, int prec) {
 // (host or device, per problem sample_off) into the packed grid64 buffer.
 int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opts& o, Batch& B, bool product_only = false) {
   const int np = (int)hp.size();
+  ctx->launch_err = cudaSuccess;
   B.P.resize(np);
   long long goff = 0, xoff = 0, yoff = 0, toff = 0, xchunk = 0;
   int sub = 0;
@@ -1116,6 +1119,16 @@ int build_solve_graph(prony_ctx* ctx, const std::vector<Seg>& segs, int* dflag, 
   cudaGraph_t g;
   CK(cudaGraphCreate(&g, 0));
   cudaGraphNode_t prev = nullptr;
+  cudaGetLastError();
+  // the segment's own failure, or that of any launch in it: a graph without a kernel is never kept
+  auto enqueue = [&](const Seg& seg) {
+    const int rc = seg.fn();
+    note_launch_error(ctx, cudaGetLastError());
+    if (rc || ctx->launch_err == cudaSuccess) return rc;
+    const cudaError_t e = ctx->launch_err;
+    ctx->launch_err = cudaSuccess;
+    return cuda_fail(e, "kernel launch");
+  };
   for (const Seg& seg : segs) {
     const long long before = g_launches.load();
     if (!seg.loop) {
@@ -1124,7 +1137,7 @@ int build_solve_graph(prony_ctx* ctx, const std::vector<Seg>& segs, int* dflag, 
         cudaGraphDestroy(g);
         return cuda_fail(be, "cudaStreamBeginCapture");
       }
-      const int rc = seg.fn();
+      const int rc = enqueue(seg);
       cudaGraph_t child = nullptr;
       const cudaError_t ce = cudaStreamEndCapture(s, &child);
       const long long n = g_launches.load() - before;
@@ -1172,7 +1185,7 @@ int build_solve_graph(prony_ctx* ctx, const std::vector<Seg>& segs, int* dflag, 
       cudaGraphDestroy(g);
       return cuda_fail(e, "solve graph loop node");
     }
-    const int rc = seg.fn();
+    const int rc = enqueue(seg);
     launch_loop_cond(h, dflag, count, seg.cap, s);
     cudaGraph_t body;
     const cudaError_t ce = cudaStreamEndCapture(s, &body);
@@ -1330,7 +1343,7 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
     // M_l = U^* Y_l  with Y_l the rows k + e_l of the last product Y = T V
     for (int l = 0; l < D.maxD; ++l)
       gram(ctx, B, D, BUF_U, -1, W_U, BUF_Y, l, W_V, D.L.mproj + 16LL * l * D.L.LDR * D.L.LDM, D.L.LDM, s);
-    launch_svd_S(D, s);
+    note_launch_error(ctx, launch_svd_S(D, s));
     if (ro.want_S) {
       // phase-canonical basis: argmax over V V_Q, then rotate U_Q, V_Q, S_l
       apply(ctx, B, D, BUF_V, W_V, W_V, D.L.vq, 1, BUF_B1, s);
@@ -1340,7 +1353,7 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
       apply(ctx, B, D, BUF_V, W_V, W_V, D.L.vq, 1, BUF_B1, s);   // V_final
       apply(ctx, B, D, BUF_U, W_U, W_V, D.L.uq, 1, BUF_B2, s);   // U_final
     }
-    launch_eig_t(D, o.seed, s);
+    note_launch_error(ctx, launch_eig_t(D, o.seed, s));
     launch_powers(D, s);
     launch_rhs(D, 0, s);
     launch_solve_c(D, s);
@@ -1823,9 +1836,8 @@ int prony_small_steps(prony_ctx* ctx, int d, int m, int a, const prony_c128* Q, 
   D.L = L;
   D.cap_jacobi = jacobi_cap;
   D.cap_eigqr = eigqr_cap;
-  launch_svd_S(D, s);
-  launch_eig_t(D, seed, s);
-  CK(cudaGetLastError());
+  CK(launch_svd_S(D, s));
+  CK(launch_eig_t(D, seed, s));
   std::vector<char> h(L.bytes);
   CK(cudaMemcpyAsync(h.data(), sb, L.bytes, cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&st, ctx->st.p, sizeof(ProbState), cudaMemcpyDeviceToHost, s));

@@ -110,3 +110,18 @@ def test_mixed_batch_memory(ctx, monkeypatch):
             te, ce = W.match_to_truth(o.t, o.c, p.t, p.c)
             assert te <= 1e-6 and ce <= 1e-5
     assert used["1"] <= 3 * used["0"]
+
+
+def test_failed_launch_is_reported_every_time(ctx):
+    """65536 problems are one more than a grid's second dimension holds: the call that captures the solve reports the
+    failed launch, and so does a repeated one (no graph without those kernels is kept); other calls go on."""
+    from paper_2012_11430_gb300 import PronyError, default_opts
+    from paper_2012_11430_gb300.binding import PRONY_ECUDA
+    P = 65536
+    grid = np.ones(4, dtype=np.complex128)
+    o = default_opts(precision="fp32")
+    for _ in range(2):
+        with pytest.raises(PronyError) as e:
+            ctx.solve_batched([grid] * P, [1] * P, [1] * P, [1] * P, o)
+        assert e.value.code == PRONY_ECUDA
+    _solve(ctx, W.make_problem("fl", 2, 15, 5, 7206), 3, "fp32")
