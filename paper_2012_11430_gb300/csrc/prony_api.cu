@@ -97,6 +97,7 @@ struct prony_ctx {
   prony_stats stats{};
   long long launch_base = 0;
   cudaError_t launch_err = cudaSuccess;   // first failed launch of the current call
+  bool unchecked = false;                 // a call queued work whose error flags no one has looked at (clear_flags)
   std::map<std::string, int> tc_tuned;   // batch shape -> K split
   // the tensor-core job list on the device: (nks, P, then n and d of every problem) it was
   // built for, and its ext / in counts (a repeated batch layout skips the rebuild and the upload)
@@ -254,6 +255,14 @@ int wait_for(prony_ctx* ctx, cudaStream_t user) {
   if (!user) return PRONY_OK;
   CK(cudaEventRecord(ctx->order, user));
   CK(cudaStreamWaitEvent(ctx->stream, ctx->order, 0));
+  return PRONY_OK;
+}
+
+// The kernels' error flags and the counters that a kernel with an error may leave behind.
+int clear_flags(prony_ctx* ctx) {
+  DBuf* bufs[] = {&ctx->oob, &ctx->tcerr, &ctx->cnt, &ctx->rcnt};
+  for (DBuf* b : bufs)
+    if (b->p) CK(cudaMemsetAsync(b->p, 0, b->cap, ctx->stream));
   return PRONY_OK;
 }
 
@@ -543,7 +552,7 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
                                       std::max(T.gram ? chunks(B.P.back(), 1) * T.gram_stride : 0LL,
                                                T.apply ? (long long)B.P.size() * T.apply_stride : 0LL));
   if ((rc = ensure(ctx->xb, (size_t)xb_bytes))) return rc;
-  // (zeroed when allocated and after an error)
+  // (zeroed when allocated and by clear_flags)
   if (!ctx->tcerr.p) {
     if ((rc = ensure(ctx->tcerr, 256))) return rc;
     CK(cudaMemsetAsync(ctx->tcerr.p, 0, sizeof(int), ctx->stream));
@@ -894,6 +903,11 @@ int setup_products(prony_ctx* ctx, Batch& B, int prec) {
 int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opts& o, Batch& B, bool product_only = false) {
   const int np = (int)hp.size();
   ctx->launch_err = cudaSuccess;
+  if (ctx->unchecked) {                        // (a call that ended before its results were read)
+    const int rc = clear_flags(ctx);
+    if (rc) return rc;
+  }
+  ctx->unchecked = true;
   B.P.resize(np);
   long long goff = 0, xoff = 0, yoff = 0, toff = 0, xchunk = 0;
   int sub = 0;
@@ -1517,24 +1531,25 @@ int queue_results(prony_ctx* ctx, const Batch& B, const double* tdev, const doub
 // bounded waits or window overflow.
 int check_flags(prony_ctx* ctx) {
   count_graph_launches(ctx);
-  if (const int oob = ctx->h_flag[3]) {
-    CK(cudaMemsetAsync(ctx->oob.p, 0, sizeof(int), ctx->stream));
-    if (ctx->cnt.p) CK(cudaMemsetAsync(ctx->cnt.p, 0, ctx->cnt.cap, ctx->stream));
-    if (ctx->rcnt.p) CK(cudaMemsetAsync(ctx->rcnt.p, 0, ctx->rcnt.cap, ctx->stream));
+  const int oob = ctx->h_flag[3], tc = ctx->h_flag[4];
+  const cudaError_t launch = ctx->launch_err;
+  ctx->launch_err = cudaSuccess;
+  if (oob || tc) {
+    const int rc = clear_flags(ctx);
+    if (rc) return rc;
     CK(cudaStreamSynchronize(ctx->stream));
+  }
+  ctx->unchecked = false;
+  if (oob) {
     g_err = "internal workspace bound check failed at site " + std::to_string(oob);
     return PRONY_ECUDA;
   }
-  if (ctx->launch_err != cudaSuccess) {
-    const cudaError_t e = ctx->launch_err;
-    ctx->launch_err = cudaSuccess;
-    g_err = std::string("Toeplitz product launch: ") + cudaGetErrorString(e);
+  if (launch != cudaSuccess) {
+    g_err = std::string("kernel launch: ") + cudaGetErrorString(launch);
     return PRONY_ECUDA;
   }
-  if (const int h = ctx->h_flag[4]) {
-    CK(cudaMemsetAsync(ctx->tcerr.p, 0, sizeof(int), ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    g_err = "tensor-core Toeplitz kernel reported error " + std::to_string(h);
+  if (tc) {
+    g_err = "tensor-core Toeplitz kernel reported error " + std::to_string(tc);
     return PRONY_ECUDA;
   }
   return PRONY_OK;
