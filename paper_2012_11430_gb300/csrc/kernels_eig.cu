@@ -187,10 +187,31 @@ __device__ void svd_jacobi(const Dev& D, ProbState& st, const double2* Q, int a,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
   float2* Qc = fsm;                                             // [b][a] columns
   float2* Vc = fsm + (size_t)a * b;                             // [b][b] columns
+  // Q times the power of two that takes its largest entry to [2^24, 2^25): the squares and fourth powers below then
+  // stay in range whatever the unit of the samples (V does not depend on the factor), columns down to 1e-15 of
+  // the largest included.  On the exponent bits: FP64 operations and conversions are slow here.
+  if (threadIdx.x == 0) s_rot = 0;
+  __syncthreads();
+  {
+    int e = 0;
+    for (int idx = threadIdx.x; idx < a * b; idx += blockDim.x) {
+      const double2 q = Q[idx / b * LM + idx % b];
+      e = max(e, max((__double2hiint(q.x) >> 20) & 0x7FF, (__double2hiint(q.y) >> 20) & 0x7FF));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) atomicMax(&s_rot, e);
+  }
+  __syncthreads();
+  const int shift = 1023 + 24 - s_rot;
+  auto scaled = [&](double v) {                  // v 2^shift; v itself where not finite
+    const int hi = __double2hiint(v), e = (hi >> 20) & 0x7FF;
+    if (e == 0x7FF) return (float)v;
+    return e == 0 || e + shift <= 0 ? 0.f : (float)__hiloint2double(hi + shift * (1 << 20), __double2loint(v));
+  };
   for (int idx = threadIdx.x; idx < a * b; idx += blockDim.x) {
     const int i = idx / b, j = idx % b;
     const double2 q = Q[i * LM + j];
-    Qc[j * a + i] = fc((float)q.x, (float)q.y);
+    Qc[j * a + i] = fc(scaled(q.x), scaled(q.y));
   }
   for (int idx = threadIdx.x; idx < b * b; idx += blockDim.x) {
     const int i = idx % b, j = idx / b;
@@ -241,9 +262,10 @@ __device__ void svd_jacobi(const Dev& D, ProbState& st, const double2* Q, int a,
           ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
         }
         const float ag2 = fabs2(ga);
+        // (|gamma| below 3e-19, where the square of the largest column is above 2e14: nothing to rotate)
         if (!(ag2 > jtol2 * fmaxf(al * be, 0.f)) || ag2 < 1e-37f) continue;
         const float ri = rsqrtf(ag2), ag = ag2 * ri;             // 1 / |gamma|, |gamma|
-        const float zeta = (be - al) * 0.5f * ri, z1 = fmaf(zeta, zeta, 1.f);
+        const float zeta = fminf(fmaxf((be - al) * 0.5f * ri, -1e18f), 1e18f), z1 = fmaf(zeta, zeta, 1.f);
         const float tt = copysignf(__fdividef(1.f, fabsf(zeta) + z1 * rsqrtf(z1)), zeta);
         const float c = rsqrt_n(fmaf(tt, tt, 1.f)), s = c * tt;
         const float rn = rsqrt_n(ag2);

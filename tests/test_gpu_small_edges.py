@@ -137,3 +137,16 @@ def test_one_wide_problem_among_many(ctx):
     for o, p in zip(outs, ps):
         te, ce = W.match_to_truth(o.t, o.c, p.t, p.c)
         assert te <= 1e-6 and ce <= 1e-5
+
+
+@pytest.mark.parametrize("unit", [1e-30, 1e-12, 1e-11, 1e8, 1e30])
+@pytest.mark.parametrize("m,a", [(5, 10), (20, 40), (40, 80)])
+def test_small_steps_in_any_unit(ctx, m, a, unit):
+    """Q and M_l in another unit: sigma in that unit, S_l and z unchanged, as accurate as in test_small_steps_sizes."""
+    Q, M, sigma, t = _close_pairs(m + m % 2, a, 1e-2)
+    sig, S, z, tg, status = ctx.small_steps(unit * Q, unit * M)
+    assert status == 0
+    sigma = np.sort(sigma)[::-1] * unit
+    assert np.max(np.abs(sig - sigma) / sigma) <= 64 * 2.0 ** -53 * len(sigma)
+    o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
+    assert np.max(np.abs(z[og] - np.exp(-2j * np.pi * t[o]))) <= 1e-11
