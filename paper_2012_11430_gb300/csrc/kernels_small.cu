@@ -156,7 +156,10 @@ __global__ void __launch_bounds__(NQ > 2 ? 512 : 256) k_chol(Dev D, int wsel, in
     }
     if (warp == 0) {
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) d[q] -= (lk[q].x * lk[q].x + lk[q].y * lk[q].y) * inv2;
+      for (int q = 0; q < NQ; ++q) {            // (scaled before they are squared: the Gram's unit is the samples' squared)
+        const float x = lk[q].x * inv, y = lk[q].y * inv;
+        d[q] -= x * x + y * y;
+      }
       if (lane == 0) {
         perm[i] = pv;
         dinv[i] = inv;

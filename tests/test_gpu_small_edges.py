@@ -150,3 +150,15 @@ def test_small_steps_in_any_unit(ctx, m, a, unit):
     assert np.max(np.abs(sig - sigma) / sigma) <= 64 * 2.0 ** -53 * len(sigma)
     o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
     assert np.max(np.abs(z[og] - np.exp(-2j * np.pi * t[o]))) <= 1e-11
+
+
+@pytest.mark.parametrize("prec", ["bf16x3", "fp32", "fft32"])
+@pytest.mark.parametrize("n,m", [(15, 5), (31, 20)])
+def test_solve_in_any_unit(ctx, prec, n, m):
+    """A noise-free solve with samples of any size: the same nodes, coefficients in the samples' unit."""
+    from paper_2012_11430_gb300 import default_opts
+    p = W.make_problem(f"un{m}", 2, n, m, 7500 + m)
+    for unit in (1e-12, 1e-11, 1.0, 1e8):
+        r = ctx.solve(unit * p.grid, 2, n, m, default_opts(precision=prec))
+        te, ce = W.match_to_truth(r.t, r.c / unit, p.t, p.c)
+        assert r.info["status"] == 0 and te <= 1e-6 and ce <= 1e-5, (unit, te, ce)
