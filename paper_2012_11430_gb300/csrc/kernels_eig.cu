@@ -573,10 +573,10 @@ __device__ __forceinline__ void bar4() { asm volatile("bar.sync 1, 128;" ::: "me
 
 // Eigenvectors W of the m x m matrix H (m <= 32 NQ; shared memory, pitch 32 NQ + 1, zero beyond m) and X ~ W^{-1}, both FP32 values, to
 // global memory in FP64.  The whole block (at least 128 threads).
-// (FP32 copies Wf, Xf, packed, and the eigenvalues lamf beside them).
+// (FP32 copies Wf, Xf, packed, and the eigenvalues lamf, times `unit`, beside them).
 template <int NQ>
 __device__ void eig_w(const Dev& D, ProbState& st, int m, float2* H, float2* Z, float2* Y, double2* Wd, double2* Xd,
-                      int LM, float2* Wf, float2* Xf, float2* lamf) {
+                      int LM, float2* Wf, float2* Xf, float2* lamf, float unit) {
   constexpr int LD = 32 * NQ + 1;
   __shared__ float2 hv[PRONY_MMAX];
   __shared__ float4 rot[PRONY_MMAX];             // rotations of a sweep: c, Re s, Im s
@@ -790,7 +790,7 @@ __device__ void eig_w(const Dev& D, ProbState& st, int m, float2* H, float2* Z, 
     hn = 0.f;
     for (int w = 0; w < nwarp; ++w) hn = fmaxf(hn, s_red[w]);
     const float small = fmaxf(hn, 1e-30f) * 5.9604645e-8f;
-    for (int k = threadIdx.x; k < m; k += blockDim.x) lamf[k] = H[k * LD + k];
+    for (int k = threadIdx.x; k < m; k += blockDim.x) lamf[k] = fscale(H[k * LD + k], unit);
     for (int k = warp; k < m; k += nwarp) {
       const float2 lamk = H[k * LD + k];
       float2 acc[NQ], rd[NQ];
@@ -912,13 +912,30 @@ __global__ void __launch_bounds__(NT) k_eig_t(Dev D, MuTable mu) {
     float2* H = (float2*)zsm;                    // m x m each, pitch LD
     float2* Z = H + m * LD;
     float2* Y = Z + m * LD;
+    __shared__ int s_big;
+    if (threadIdx.x == 0) s_big = 0;
+    __syncthreads();
+    int big = 0;                                 // bits of the largest entry
     for (int q = threadIdx.x; q < m * LD; q += NT) {
       const int i = q / LD, j = q % LD;
-      H[q] = j < m ? __ldcg(Cm + i * m + j) : fc(0.f, 0.f);
+      const float2 c = j < m ? __ldcg(Cm + i * m + j) : fc(0.f, 0.f);
+      big = max(big, max(__float_as_int(fabsf(c.x)), __float_as_int(fabsf(c.y))));
+      H[q] = c;
       Z[q] = fc(i == j ? 1.f : 0.f, 0.f);
     }
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_big, big);
     __syncthreads();
-    eig_w<NQ>(D, st, m, H, Z, Y, Wd, Xd, LM, Wf, Xf, lamf);
+    // the QR iteration forms fourth powers of the entries: a matrix whose largest lies outside 2^-8..2^8 is
+    // scaled by a power of two (its eigenvectors stay the same)
+    const int e = s_big >> 23;
+    const bool scale = e > 0 && e < 254 && (e < 127 - 8 || e > 127 + 8);
+    if (scale) {
+      const float f = __int_as_float((254 - e) << 23);
+      for (int q = threadIdx.x; q < m * LD; q += NT) H[q] = fscale(H[q], f);
+      __syncthreads();
+    }
+    eig_w<NQ>(D, st, m, H, Z, Y, Wd, Xd, LM, Wf, Xf, lamf, scale ? __int_as_float(e << 23) : 1.f);
     if (threadIdx.x == 0) st.rank_used = m;
   }
   cl_sync<CL>();

@@ -162,3 +162,15 @@ def test_solve_in_any_unit(ctx, prec, n, m):
         r = ctx.solve(unit * p.grid, 2, n, m, default_opts(precision=prec))
         te, ce = W.match_to_truth(r.t, r.c / unit, p.t, p.c)
         assert r.info["status"] == 0 and te <= 1e-6 and ce <= 1e-5, (unit, te, ce)
+
+
+@pytest.mark.parametrize("unit", [1e-20, 1e-12, 1e-8, 1e6, 1e12, 1e20])
+@pytest.mark.parametrize("m,a", [(5, 10), (20, 40), (40, 80)])
+def test_small_steps_eigenvalues_of_any_size(ctx, m, a, unit):
+    """M_l in another unit than Q: z in the unit of M_l, t unchanged, as accurate as in test_small_steps_sizes."""
+    Q, M, sigma, t = _close_pairs(m + m % 2, a, 1e-2)
+    _, _, z, tg, status = ctx.small_steps(Q, unit * M)
+    assert status == 0
+    o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
+    assert np.max(np.abs(z[og] / unit - np.exp(-2j * np.pi * t[o]))) <= 1e-11
+    assert np.max(W.torus_dist(tg[og], t[o])) <= 2e-12
