@@ -43,7 +43,8 @@ typedef enum {
   PRONY_OK = 0,
   PRONY_EINVAL = -1,    /* bad argument (sizes, NULL pointer, unsupported precision) */
   PRONY_ERANK = -2,     /* detected numerical rank of T is below m (outputs still filled) */
-  PRONY_ENOCONV = -3,   /* an iteration hit its cap (power method, eigen-QR, Jacobi) */
+  PRONY_ENOCONV = -3,   /* an iteration hit its cap (power method, eigen-QR, Jacobi), or the eigenvectors
+                           of C_mu have no inverse in FP32 */
   PRONY_ENAN = -4,      /* non-finite input samples or intermediate results */
   PRONY_ECUDA = -5,     /* CUDA runtime error (message: prony_last_error) */
   PRONY_ENOMEM = -6     /* device allocation failed */

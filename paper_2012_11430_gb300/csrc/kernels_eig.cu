@@ -1009,11 +1009,13 @@ __global__ void __launch_bounds__(NT) k_eig_t(Dev D, MuTable mu) {
   }
   cl_sync<CL>();
   // ---- Newton-Schulz steps X <- 2X - X (W X) until ||I - W X||_max before the last is below 1e-8 (two,
-  // unless the correction of W was large)
+  // unless the correction of W was large).  A step squares the deviation: a W singular to FP32 leaves one that does
+  // not fall, and the steps end after two; what then stays above 1e-8 is PRONY_ENOCONV.
   __shared__ float s_dev[32];
   __shared__ int s_more;
   float* devs = (float*)(lamf + m);              // one slot per CTA and parity of the step
   stage(sW, Wc, LM, m, m);
+  float last = 0.f;                              // (thread 0) the deviation before
   for (int it = 0; it < 6; ++it) {
     stage(sX, Xd, LM, m, m);
     __syncthreads();
@@ -1022,7 +1024,8 @@ __global__ void __launch_bounds__(NT) k_eig_t(Dev D, MuTable mu) {
       const int j = rank + e / m * CL, c = e % m;
       const double2 r = zdot<false>(sW + j * m, 1, sX + c, m, m);
       Rd[j * LM + c] = r;
-      dev = fmaxf(dev, fabsf((float)(r.x - (c == j ? 1.0 : 0.0))) + fabsf((float)r.y));
+      const float q = fabsf((float)(r.x - (c == j ? 1.0 : 0.0))) + fabsf((float)r.y);
+      dev = fmaxf(dev, q < 1e30f ? q : 1e30f);   // (NaN among the large)
     }
     for (int o = 16; o > 0; o >>= 1) dev = fmaxf(dev, __shfl_xor_sync(0xffffffffu, dev, o));
     if ((threadIdx.x & 31) == 0) s_dev[threadIdx.x >> 5] = dev;
@@ -1036,7 +1039,9 @@ __global__ void __launch_bounds__(NT) k_eig_t(Dev D, MuTable mu) {
     if (threadIdx.x == 0) {
       dev = 0.f;
       for (int r = 0; r < CL; ++r) dev = fmaxf(dev, __ldcg(devs + (it & 1) * CL + r));
-      s_more = dev > 1e-8f && it < 5;
+      s_more = dev > 1e-8f && it < 5 && (it == 0 || dev < last);
+      last = dev;
+      if (!s_more && rank == 0 && dev > 1e-4f) set_status_e(st, ST_ENOCONV);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < nj * m; e += NT) {

@@ -174,3 +174,13 @@ def test_small_steps_eigenvalues_of_any_size(ctx, m, a, unit):
     o, og = np.lexsort(t.T[::-1]), np.lexsort(tg.T[::-1])
     assert np.max(np.abs(z[og] / unit - np.exp(-2j * np.pi * t[o]))) <= 1e-11
     assert np.max(W.torus_dist(tg[og], t[o])) <= 2e-12
+
+
+@pytest.mark.parametrize("m", [16, 40])
+def test_defective_matrix_reports_enoconv(ctx, m):
+    """C_mu a single Jordan block: no eigenvector basis, W singular to FP32, its inverse does not converge."""
+    from paper_2012_11430_gb300 import PRONY_ENOCONV
+    J = np.exp(-0.7j) * np.eye(m) + np.eye(m, k=1)
+    sig, S, z, t, status = ctx.small_steps(np.eye(m), J[None])
+    assert status == PRONY_ENOCONV
+    assert np.all(np.isfinite(sig)) and np.all(np.isfinite(S))
