@@ -300,6 +300,13 @@ inline int blocks_per_problem(long long want, int nprob) {
 }
 // Message returned by prony_last_error() on this host thread.
 void set_last_error(const char* msg);
+// Dynamic shared memory that a kernel may be launched with on the current device: raised when `bytes` is more than
+// any launch asked for so far, never lowered (another thread may be about to launch with the larger size).
+cudaError_t allow_smem_of(const void* kernel, size_t bytes);
+template <typename F>
+cudaError_t allow_smem(F* kernel, size_t bytes) {
+  return allow_smem_of((const void*)kernel, bytes);
+}
 
 // Column counts of the tall blocks, selected per problem: r0, the current U / V widths, m, the
 // pending X -> X M product, a single column, and the Lanczos basis sizes k and k + 1.

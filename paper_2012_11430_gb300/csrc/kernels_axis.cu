@@ -422,14 +422,6 @@ __global__ void __launch_bounds__(256) k_axis_out(Dev D, Dev S, int wsel, int yb
 // S.fLT holds the largest n of the batch, S.maxN / S.maxNext / S.maxGd its largest sub-problem.
 inline int max_axis_n(const Dev& S) { return S.fLT; }
 
-template <typename F>
-cudaError_t allow_smem(F* kernel, size_t bytes, size_t& set) {
-  if (bytes <= set) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) set = bytes;
-  return e;
-}
-
 }  // namespace
 
 template <int MODE, int FMT>
@@ -455,10 +447,9 @@ cudaError_t launch_axis_tables(const Dev& D, const Dev& S, int mode, int fmt, in
 template <int MODE, int CL, int NC>
 static cudaError_t axis_in_as(const Dev& D, const Dev& S, int xbuf, int wsel, long long items, void* xb,
                               long long xb_stride, cudaStream_t s) {
-  static size_t set = 0;
   const int H = max_axis_n(S) + 1;
   const size_t sm = sizeof(float4) * (size_t)(H / 2 + 1) * (H + (H & 1));
-  cudaError_t e = allow_smem(k_axis_in<MODE, CL, NC>, sm, set);
+  cudaError_t e = allow_smem(k_axis_in<MODE, CL, NC>, sm);
   if (e != cudaSuccess) return e;
   const long long per = items * D.nprob > 152LL * 64 ? 2 : 1;     // items per warp (one twiddle table per block)
   note_launch();
@@ -490,11 +481,10 @@ cudaError_t launch_axis_in(const Dev& D, const Dev& S, int mode, int xbuf, int w
 
 template <int KB, int SP>
 static cudaError_t axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s) {
-  static size_t set = 0;
   const int H = max_axis_n(S) + 1, K = y_ext ? H + 1 : H, nblk = (K + KB - 1) / KB;
   // (H / 2 + 1) x Kt grows with n: the largest problem's table is the largest of the batch
   const size_t sm = sizeof(float4) * (size_t)(H / 2 + 1) * nblk * KB;
-  cudaError_t e = allow_smem(k_axis_out<KB, SP>, sm, set);
+  cudaError_t e = allow_smem(k_axis_out<KB, SP>, sm);
   if (e != cudaSuccess) return e;
   const long long items = (long long)(((y_ext ? S.maxNext : S.maxN) + 31) / 32) * maxw * nblk;
   note_launch();

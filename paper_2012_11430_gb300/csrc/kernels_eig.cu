@@ -1092,32 +1092,24 @@ cudaError_t launch_cluster(void (*kernel)(Args...), int cl, int threads, size_t 
 constexpr size_t SVD_SMEM = 227 * 1024 - 2560;   // what a block may have, less the kernel's static part
 template <int CL, int NT>
 cudaError_t run_svd(const Dev& D, cudaStream_t s) {
-  static size_t set = 0;
   const size_t a = std::max(D.L.LDR, D.L.LDM), b = D.L.LDM;
   // as many of the CTA's columns of U_Q as fit: all of them but for a >= 98 (CL = 1) to 124 (CL = 4), r0 = 2 m; at
   // least ten (a = 128, b = 64)
   const size_t fixed = b * b + a * b, cols = std::min((b + CL - 1) / CL, (SVD_SMEM / sizeof(double2) - fixed) / (a + b));
   const size_t sm = sizeof(double2) * (fixed + (a + b) * cols);
-  if (sm > set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_svd_S<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    set = sm;
-  }
+  const cudaError_t e = allow_smem(k_svd_S<CL, NT>, sm);
+  if (e != cudaSuccess) return e;
   return launch_cluster(k_svd_S<CL, NT>, CL, NT, sm, D.nprob, s, D, (int)cols);
 }
 
 template <int CL, int NT>
 cudaError_t run_eig(const Dev& D, const MuTable& mu, cudaStream_t s) {
-  static size_t set = 0;
   const size_t m = D.L.LDM, own = (m + CL - 1) / CL;
   // W and two more m x m operands (the correction's FP32 blocks fit in those); the FP32 iterations' three
   const size_t sm = std::max(sizeof(double2) * (m * m + std::max(2 * m * m, (m * m + 3 * m * own + 1) / 2)),
                              sizeof(float2) * 3 * m * (NT > 512 ? 65 : 33));
-  if (sm > set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_eig_t<CL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    set = sm;
-  }
+  const cudaError_t e = allow_smem(k_eig_t<CL, NT>, sm);
+  if (e != cudaSuccess) return e;
   return launch_cluster(k_eig_t<CL, NT>, CL, NT, sm, D.nprob, s, D, mu);
 }
 }  // namespace

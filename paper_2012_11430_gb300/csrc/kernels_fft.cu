@@ -381,7 +381,7 @@ void launch_fft_tables(const Dev& D, int maxpts, cudaStream_t s) {
   note_launch();
   k_fft_twiddles<<<(D.fLT + 255) / 256, 256, 0, s>>>(D.ftw, D.fLT);
   const size_t sm = sizeof(float2) * ((size_t)maxpts + D.fLT);
-  cudaFuncSetAttribute(k_fft_table, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  allow_smem(k_fft_table, sm);
   note_launch();
   k_fft_table<<<D.nprob, fft_threads(maxpts), sm, s>>>(D);
 }
@@ -389,11 +389,7 @@ void launch_fft_tables(const Dev& D, int maxpts, cudaStream_t s) {
 void launch_toeplitz_fft(const Dev& D, int maxpts, int maxw, int adjoint, int xbuf, int wsel, int ybuf, int y_ext,
                          cudaStream_t s) {
   const size_t sm = sizeof(float2) * ((size_t)maxpts + D.fLT);
-  static size_t set = 0;
-  if (sm > set) {
-    cudaFuncSetAttribute(k_toeplitz_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    set = sm;
-  }
+  allow_smem(k_toeplitz_fft, sm);
   note_launch();
   k_toeplitz_fft<<<dim3(maxw, D.nprob), fft_threads(maxpts), sm, s>>>(D, adjoint, xbuf, wsel, ybuf, y_ext);
 }

@@ -567,16 +567,8 @@ long long lm_workspace_bytes(int m, int d) {
 
 // Dynamic shared-memory limits of the refinement kernels.
 cudaError_t lm_set_attributes(int m, int d) {
-  static size_t set_p = 0, set_s = 0;
-  const size_t sp = lm_points_smem(m, d), ss = lm_step_smem(m, d);
-  cudaError_t e = cudaSuccess;
-  if (sp > set_p &&
-      (e = cudaFuncSetAttribute(k_lm_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp)) == cudaSuccess)
-    set_p = sp;
-  if (e == cudaSuccess && ss > set_s &&
-      (e = cudaFuncSetAttribute(k_lm_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss)) == cudaSuccess)
-    set_s = ss;
-  return e;
+  const cudaError_t e = allow_smem(k_lm_points, lm_points_smem(m, d));
+  return e == cudaSuccess ? allow_smem(k_lm_step, lm_step_smem(m, d)) : e;
 }
 
 // The whole refinement, enqueued on `s`: 2 iters + 3 launches (the host stays ahead of the device,

@@ -414,11 +414,7 @@ void launch_reset_done(const Dev& D, cudaStream_t s) { note_launch(); k_reset_do
 
 template <int NQ>
 static void run_chol(const Dev& D, int wsel, int target, int mode, double tol, int rank_mode, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_chol<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float2) * 1024 * NQ * NQ));
-    attr = true;
-  }
+  allow_smem(k_chol<NQ>, sizeof(float2) * 1024 * NQ * NQ);   // (a failure shows in the launch)
   note_launch();
   k_chol<NQ><<<D.nprob, NQ > 2 ? 512 : 256, sizeof(float2) * D.L.LDR * D.L.LDR, s>>>(D, wsel, target, mode, tol, rank_mode);
 }
@@ -433,12 +429,8 @@ void launch_chol(const Dev& D, int wsel, int target, int mode, double tol, int r
 }
 
 void launch_solve_c(const Dev& D, cudaStream_t s) {
-  static bool attr = false;
-  size_t sm = sizeof(double2) * PRONY_MMAX * PRONY_MMAX;
-  if (!attr) {
-    cudaFuncSetAttribute(k_solve_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  const size_t sm = sizeof(double2) * PRONY_MMAX * PRONY_MMAX;
+  allow_smem(k_solve_c, sm);
   note_launch();
   k_solve_c<<<D.nprob, 256, sm, s>>>(D);
 }

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <map>
+#include <mutex>
 
 namespace {
 
@@ -984,38 +985,33 @@ void launch_zero_small(const Dev& D, long long off, long long bytes, cudaStream_
   k_zero_small<<<g, 256, 0, s>>>(D, off, bytes);
 }
 
-// The dynamic shared memory attribute of k_gram only ever grows (a launch needs it to cover its
-// own size; lowering it for a smaller batch would make a later larger launch fail).
-static size_t g_gram_attr = 0;
-static void gram_attr(size_t sm) {
-  if (sm > g_gram_attr) {
-    cudaFuncSetAttribute(k_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    g_gram_attr = sm;
+// Blocks of k_gram resident on the current device with `sm` bytes of shared memory each.
+static int gram_slots(int nthr, size_t sm) {
+  static std::mutex lock;
+  static std::map<std::pair<int, size_t>, int> known;   // (device, shared memory)
+  int dev = 0, occ = 1, sms = 1;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> hold(lock);
+  int& slots = known[{dev, sm}];
+  if (slots) return slots;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  allow_smem(k_gram, sm);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gram, nthr, sm) != cudaSuccess) {
+    cudaGetLastError();
+    occ = 2;
   }
+  return slots = std::max(1, occ) * sms;
 }
 
 // Launch geometry of k_gram for a batch: dynamic shared memory, rows per block and blocks per
 // problem (the batch fills the resident blocks once or twice, at least RS rows per block).
 static void gram_geometry(const Dev& D, size_t& sm, int& chunk, int& nblk) {
-  static std::map<size_t, int> slots_for;      // shared memory size -> resident blocks on the GPU
   // the staging buffers (float2 per value); afterwards the same space holds the sums of the row groups, at most
   // one thread's per thread
   const int RS = gram_rows(D.L.LDR), nthr = gram_threads(D.L.LDR);
   sm = sizeof(float2) * std::max<size_t>((size_t)GRAM_STAGES * gram_buf_elems(D.L.LDR), (size_t)nthr * GRAM_RED);
-  auto it = slots_for.find(sm);
-  if (it == slots_for.end()) {
-    int occ = 1, dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    gram_attr(sm);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gram, nthr, sm) != cudaSuccess) {
-      cudaGetLastError();
-      occ = 2;
-    }
-    it = slots_for.emplace(sm, std::max(1, occ) * sms).first;
-  }
   // at most 64 blocks per problem: the last block of a problem adds every block's partial Gram
-  const int np = std::max(1, D.nprob), slots = it->second;
+  const int np = std::max(1, D.nprob), slots = gram_slots(nthr, sm);
   int per_prob = std::max(1, std::min(64, slots / np));
   // (a whole number per problem that leaves over a tenth of the resident blocks empty: two rounds of half the rows)
   if ((long long)np * per_prob * 10 < 9LL * slots && per_prob < 64) per_prob = std::min(64, 2 * slots / np);
@@ -1050,7 +1046,7 @@ void launch_gram(const Dev& D, int xbuf, int xshift, int xw, int zbuf, int zshif
   size_t sm;
   int chunk, nblk;
   gram_geometry(D, sm, chunk, nblk);
-  gram_attr(sm);
+  allow_smem(k_gram, sm);
   dim3 g(nblk, D.nprob);
   note_launch();
   const int own_sum = nblk <= 8;                 // few partials: the last block adds them
@@ -1063,13 +1059,9 @@ void launch_gram(const Dev& D, int xbuf, int xshift, int xw, int zbuf, int zshif
 
 void launch_apply(const Dev& D, int xbuf, int xw, int outw, long long m_off, int m_double, int zbuf, int outbuf,
                   int norm_only, cudaStream_t s) {
-  static size_t set = 0;
   const int rows = D.L.LDR <= 64 ? 128 : 64;
   const size_t sm = sizeof(float2) * ((size_t)D.L.LDR * ((D.L.LDR + 3) & ~3) + (size_t)D.L.LDR * rows);
-  if (sm > set) {
-    cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    set = sm;
-  }
+  allow_smem(k_apply, sm);
   dim3 g((D.maxN + rows - 1) / rows, D.nprob);
   note_launch();
   k_apply<<<g, 256, sm, s>>>(D, xbuf, xw, outw, m_off, m_double, zbuf, outbuf, norm_only, rows);
@@ -1135,12 +1127,8 @@ cudaError_t launch_eval_points(const double* t, const double2* c, int m, int d, 
     return cudaGetLastError();
   }
   const size_t sm = eval_table_bytes(m);
-  static size_t set = 0;
-  if (sm > set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_eval_many, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    set = sm;
-  }
+  const cudaError_t e = allow_smem(k_eval_many, sm);
+  if (e != cudaSuccess) return e;
   note_launch();
   k_eval_tables<<<(m * EV_HI + EV_MID + 63) / 64, 64, 0, s>>>(c, m, tab);
   note_launch();

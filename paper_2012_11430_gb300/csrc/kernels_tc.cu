@@ -864,14 +864,8 @@ void launch_xb_prep(const Dev& D, int xbuf, int xshift, int wsel, void* xb, int 
 template <int KIND, int MODE, int FMT = TT_TF32, bool HALF = false>
 static cudaError_t launch_tc_kind(const Dev& D, const ToeplitzJob* jobs, int njobs, const TcParams& P, int* err,
                                   size_t sm, cudaStream_t s) {
-  static size_t set = 0;
-  if (sm > set) {
-    // the attribute must cover this launch's dynamic shared memory (static + dynamic <= 227 KB)
-    cudaError_t e =
-        cudaFuncSetAttribute(k_toeplitz_tc<KIND, MODE, FMT, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    set = sm;
-  }
+  const cudaError_t e = allow_smem(k_toeplitz_tc<KIND, MODE, FMT, HALF>, sm);   // (static + dynamic <= 227 KB)
+  if (e != cudaSuccess) return e;
   k_toeplitz_tc<KIND, MODE, FMT, HALF><<<njobs, 32 * (2 + TC_APROD), sm, s>>>(D, jobs, P, err);
   return cudaGetLastError();
 }
