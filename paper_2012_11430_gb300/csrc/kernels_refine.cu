@@ -34,7 +34,8 @@ namespace {
 
 constexpr int LM_TILE = 128;            // points per CTA (= threads) in the point pass
 constexpr int LM_SEG_BITS = 5, LM_SEG = 1 << LM_SEG_BITS;   // table points of the unit circle
-constexpr int LM_MAXCTA = 304;          // point CTAs at most (two per SM)
+constexpr int LM_CTA = 304;             // point CTAs (two per SM) of fewer than 32 tiles each,
+constexpr int LM_MAXCTA = 608;          // and of more (lm_point_ctas)
 constexpr int LM_EP = LM_TILE + 1;      // pitch of the exponentials (threads of different terms: different banks)
 constexpr int LM_NB = 16;               // column block of the Cholesky factorisation
 constexpr int LM_SOLVE_THREADS = 512;
@@ -108,6 +109,16 @@ __host__ __device__ inline int lm_ld(int P) {
   return 4 * (g | 1);
 }
 
+// Axes of more than 4096 points (32 FP32 terms per thread) are summed as S pieces' starts times a piece of S points:
+// 2 sqrt(len) terms.  The one CTA of a pair of terms would otherwise be bound by its own loop (one axis of 2^22 points,
+// m = 1: 2324 us a step, now 300; of 65536: 55, now 26); up to 4096 points the loop hides under the points' pass.
+__device__ inline int lm_axis_split(int len) {
+  if (len <= 32 * LM_TILE) return 0;
+  int s = 6;
+  while ((1LL << 2 * s) < len) ++s;
+  return 1 << s;
+}
+
 __device__ inline double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
@@ -133,7 +144,7 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
   const int P = m * (d + 2);
   double* H = sets + (1 - st->cur) * lm_set_elems(m, d);
   if ((int)blockIdx.x >= npt_blocks) {
-    __shared__ double axis_sum[LM_TILE / 32][PRONY_DMAX][6];
+    __shared__ double axis_sum[LM_TILE / 32][PRONY_DMAX][3][6];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int pair = (int)blockIdx.x - npt_blocks;                // a (a + 1) / 2 + b
     int a = (int)((sqrtf(8.f * pair + 1.f) - 1.f) * 0.5f);
@@ -143,14 +154,14 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
     for (int l = threadIdx.x; l < d; l += LM_TILE)                // conj(e_a) e_b = exp(-2 pi i (t_b - t_a) x)
       T[l] = frac64(t[b * d + l]) - frac64(t[a * d + l]);
     __syncthreads();
-    for (int l = 0; l < d; ++l) {
-      const uint64_t dt = T[l];
+    // the warps' sums of x^p q^x (p = 0, 1, 2; re, im) over x = x0 + i step, i < n, at most 2^16
+    auto powers = [&](uint64_t dt, int x0, int step, int n, double (&out)[LM_TILE / 32][PRONY_DMAX][3][6], int l, int which) {
       double tot = 0.0;                                           // lane z < 6: the z-th sum of the warp
-      for (int i0 = 0; i0 < B.len[l]; i0 += 32 * LM_TILE) {       // at most 32 FP32 terms per thread, then FP64
+      for (int i0 = 0; i0 < n; i0 += 32 * LM_TILE) {              // at most 32 FP32 terms per thread, then FP64
         float s[6] = {};
-        const int i1 = min(B.len[l], i0 + 32 * LM_TILE);
+        const int i1 = min(n, i0 + 32 * LM_TILE);
         for (int i = i0 + threadIdx.x; i < i1; i += LM_TILE) {
-          const int x = B.lo[l] + i;
+          const int x = x0 + i * step;
           const float u = (float)(int)((dt * (uint64_t)(long long)x) >> 32) * 2.3283064365386963e-10f;
           float sn, cn;
           sincospif(2.0f * u, &sn, &cn);
@@ -170,21 +181,51 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
         }
         tot += (double)mine;
       }
-      if (lane < 6) axis_sum[warp][l][lane] = tot;
+      if (lane < 6) out[warp][l][which][lane] = tot;
+    };
+    for (int l = 0; l < d; ++l) {
+      const int len = B.len[l], S = lm_axis_split(len);
+      if (S == 0) {
+        powers(T[l], B.lo[l], 1, len, axis_sum, l, 0);
+      } else {
+        const int U = len / S;
+        powers(T[l], 0, 1, S, axis_sum, l, 0);
+        powers(T[l], B.lo[l], S, U, axis_sum, l, 1);
+        powers(T[l], B.lo[l] + U * S, 1, len - U * S, axis_sum, l, 2);
+      }
+    }
+    __syncthreads();
+    for (int z = threadIdx.x; z < 18 * d; z += LM_TILE) {         // the warps' sums, in order
+      const int l = z / 18, w = z / 6 % 3, e = z % 6;
+      if (w == 0 || lm_axis_split(B.len[l]))
+        axis_sum[0][l][w][e] += axis_sum[1][l][w][e] + axis_sum[2][l][w][e] + axis_sum[3][l][w][e];
+    }
+    __syncthreads();
+    if (threadIdx.x < d && lm_axis_split(B.len[threadIdx.x])) {
+      // sum_u sum_v (X_u + v)^p q^(X_u + v), X_u = lo + S u, from V_k = sum v^k q^v and X_k = sum X_u^k q^X_u; and
+      // the last len - U S terms
+      double(&g)[3][6] = axis_sum[0][threadIdx.x];
+      const double2 v0 = make_double2(g[0][0], g[0][1]), v1 = make_double2(g[0][2], g[0][3]), v2 = make_double2(g[0][4], g[0][5]);
+      const double2 x0 = make_double2(g[1][0], g[1][1]), x1 = make_double2(g[1][2], g[1][3]), x2 = make_double2(g[1][4], g[1][5]);
+      const double2 r0 = cmul(x0, v0), r1 = cadd(cmul(x1, v0), cmul(x0, v1));
+      const double2 r2 = cadd(cadd(cmul(x2, v0), cscale(cmul(x1, v1), 2.0)), cmul(x0, v2));
+      g[0][0] = r0.x + g[2][0];
+      g[0][1] = r0.y + g[2][1];
+      g[0][2] = r1.x + g[2][2];
+      g[0][3] = r1.y + g[2][3];
+      g[0][4] = r2.x + g[2][4];
+      g[0][5] = r2.y + g[2][5];
     }
     __syncthreads();
     const int al = threadIdx.x / (d + 2), be = threadIdx.x % (d + 2);
     const int p = a * (d + 2) + al, q = b * (d + 2) + be;
-    for (int z = threadIdx.x; z < 6 * d; z += LM_TILE)            // the warps' sums, in order
-      axis_sum[0][z / 6][z % 6] += axis_sum[1][z / 6][z % 6] + axis_sum[2][z / 6][z % 6] + axis_sum[3][z / 6][z % 6];
-    __syncthreads();
     if (al < d + 2 && q <= p) {
       int wa, wb;
       const double2 sa = sigma_of(al, d, c[a], wa), sb = sigma_of(be, d, c[b], wb);
       double2 v = make_double2(sa.x * sb.x + sa.y * sb.y, sa.x * sb.y - sa.y * sb.x);   // conj(sa) sb M_ab
       for (int l = 0; l < d; ++l) {
         const int pw = 2 * ((wa == l + 1) + (wb == l + 1));
-        v = cmul(v, make_double2(axis_sum[0][l][pw], axis_sum[0][l][pw + 1]));
+        v = cmul(v, make_double2(axis_sum[0][l][0][pw], axis_sum[0][l][0][pw + 1]));
       }
       H[(long long)p * P + q] = v.x;
     }
@@ -548,6 +589,13 @@ __global__ void k_lm_init(LmState* st, double lambda0, const double* t, const do
   for (int q = threadIdx.x; q < m; q += blockDim.x) cc[q] = c[q];
 }
 
+// Every point CTA adds a slot to the sums of k_lm_step, one CTA's work, so there are few; from 32 tiles each (1.2
+// million points) the pass over the points outweighs that, and four CTAs per SM hide more of its latency (2^22
+// points on one axis: m = 1 428 -> 300 us a step, m = 20 942 -> 617).
+inline int lm_point_ctas(long long K) {
+  const long long tiles = (K + LM_TILE - 1) / LM_TILE;
+  return (int)std::min<long long>(tiles, tiles < 32 * LM_CTA ? LM_CTA : LM_MAXCTA);
+}
 size_t lm_points_smem(int m, int d) {
   return sizeof(float4) * (size_t)m * LM_SEG + sizeof(float2) * ((size_t)m * LM_EP + 2 * LM_TILE) +
          sizeof(float) * (size_t)d * LM_TILE;
@@ -584,7 +632,7 @@ void launch_refine_lm(double* t, double2* c, int m, int d, const int* lo, const 
   LmState* st = (LmState*)(sets + 2 * lm_set_elems(m, d));
   const Box B = make_box(d, lo, len);
   const size_t sp = lm_points_smem(m, d), ss = lm_step_smem(m, d);
-  const int npt = (int)std::min<long long>(LM_MAXCTA, (K + LM_TILE - 1) / LM_TILE), npair = m * (m + 1) / 2;
+  const int npt = lm_point_ctas(K), npair = m * (m + 1) / 2;
   note_launch();
   k_lm_init<<<1, 256, 0, s>>>(st, lambda0, t, c, tc, cc, circle, m, d);
   for (int it = 0; it <= iters; ++it) {

@@ -224,3 +224,28 @@ def test_lm_reproducible(ctx):
         a = refine_lm(*args, ctx, lo, length, steps=8)
         b = refine_lm(*args, ctx, lo, length, steps=8)
         assert all(torch.equal(x, y) for x, y in zip(a, b)), (d, n)
+
+
+@pytest.mark.parametrize("d,lo,length,m", [
+    (1, [0], [4097], 2), (1, [5], [65535], 4), (1, [-2 ** 19], [2 ** 20 + 7], 3), (2, [-3, -20000], [5, 40001], 2),
+    (2, [-5000, 1], [10000, 9], 3),
+])
+def test_lm_long_axes(ctx, d, lo, length, m):
+    """Axes of more than 4096 points, whose sums are formed from pieces: one point more, a piece short of a square,
+    a last piece of few points, beside a short axis; bounds as in test_lm_steps_match_fp64_iteration."""
+    import torch
+    from paper_2012_11430_gb300.refine import refine_lm
+    rng = np.random.default_rng(60 + m)
+    k = O.box_set(length, d) + np.array(lo)
+    t = np.stack([(rng.permutation(m) + 0.5 + 0.2 * rng.uniform(-1, 1, m)) / m for _ in range(d)], 1)
+    c = (0.5 + rng.random(m)) * np.exp(2j * np.pi * rng.random(m))
+    y = (O.expsum(t, c, k) + 0.01 * (rng.standard_normal(len(k)) + 1j * rng.standard_normal(len(k)))).astype(np.complex64)
+    t0 = np.mod(t + 0.02 * rng.uniform(-1, 1, t.shape) / np.array(length), 1.0)
+    c0 = c * (1 + 0.02 * rng.standard_normal(m))
+    for steps in (1, 3):
+        tr, cr, Lr = _lm64(t0.copy(), c0.copy(), k, y.astype(np.complex128), steps)
+        tg, cg, Lg = refine_lm(_dev(t0, torch.float64), _dev(c0, torch.complex128), torch.from_numpy(y).cuda(), ctx, lo,
+                               length, steps=steps)
+        assert np.max(W.torus_dist(tg.cpu().numpy(), tr) * np.array(length)) <= 1e-5
+        assert np.linalg.norm(cg.cpu().numpy() - cr) <= 1e-4 * np.linalg.norm(cr)
+        assert abs(Lg[0].item() - Lr[0]) <= 1e-6 * Lr[0]
