@@ -915,6 +915,7 @@ __global__ void k_eval_points(const double* t, const double2* c, int m, int d, c
 // term.  65536 points, m = 40: 338 us with sincospi per term, now 109 us and 3.5 us for the tables (the
 // FP64 pipe's floor for 14 operations a term is about 60 us), the whole host call 408 -> 179 us.
 constexpr int EV_HI = 64, EV_MID = 256;
+constexpr int EV_MANY = 12;           // terms from which the tables serve few points too
 // tab: c_j exp(-2 pi i q / 64) at j * 64 + q, then exp(-2 pi i q / 2^14), q < 256
 __global__ void k_eval_tables(const double2* c, int m, double2* tab) {
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < m * EV_HI + EV_MID; q += gridDim.x * blockDim.x) {
@@ -1117,11 +1118,13 @@ void launch_expsum_bwd_finish(const double* acc, int m, int d, double* gt, float
 
 size_t eval_table_bytes(int m) { return sizeof(double2) * ((size_t)m * EV_HI + EV_MID); }
 
-// tab: eval_table_bytes(m) of scratch.  The tables cost one launch more and m * 64 exponentials, so
-// few points keep the direct kernel (up to a few exponentials per table entry).
+// tab: eval_table_bytes(m) of scratch.  The tables cost a launch more, m * 64 exponentials and their copy into shared
+// memory, 5 to 8 us in all; what they save is half of the FP64 work and, for many terms, a chain of m exponentials per
+// point.  Few terms therefore take them from 65536 exponentials on (K = 65536, m = 1: 111 us directly, 105 with
+// tables; half as many points: 74 and 77), twelve and more from 8192 (K = 512, m = 16: 66 and 52 us).
 cudaError_t launch_eval_points(const double* t, const double2* c, int m, int d, const int* k, int K, double2* f,
                                double2* tab, cudaStream_t s) {
-  if ((long long)K * m < 8192) {
+  if ((long long)K * m < (m >= EV_MANY ? 8192 : 65536)) {
     note_launch();
     k_eval_points<<<blocks_for(K, 128), 128, 0, s>>>(t, c, m, d, k, K, f);
     return cudaGetLastError();

@@ -28,3 +28,11 @@ def test_eval_many_points(ctx, d, m, K, reach):
     ph = (T[None] * k.astype(np.int64).astype(np.uint64)[:, None, :]).sum(-1, dtype=np.uint64)   # exact mod 2^64
     e = np.exp(-2j * np.pi * (ph.astype(np.int64).astype(np.float64) * 2.0 ** -64))
     assert np.max(np.abs(ctx.eval(t, c, k) - e @ c)) <= 8 * 2.0 ** -53 * (m + 8) * np.sum(np.abs(c)) / m ** 0.5
+
+
+@pytest.mark.parametrize("d,m,K,reach", [(1, 1, 65535, 300), (1, 1, 65536, 300), (2, 11, 5957, 64), (2, 11, 5958, 64),
+                                         (3, 12, 682, 64), (3, 12, 683, 64)])
+def test_eval_sides_of_the_size_rule(ctx, d, m, K, reach):
+    """Few terms take the tables from 65536 exponentials on, twelve from 8192: the bound of test_eval_many_points on
+    both sides."""
+    test_eval_many_points(ctx, d, m, K, reach)
