@@ -894,11 +894,11 @@ __global__ void k_expsum_bwd_finish(const double* acc, int m, int d, double* gt,
 }
 
 __global__ void k_eval_points(const double* t, const double2* c, int m, int d, const int* k, int K, double2* f) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < K; q += gridDim.x * blockDim.x) {
+  for (long long q = blockIdx.x * blockDim.x + threadIdx.x; q < K; q += gridDim.x * blockDim.x) {   // (K up to 2^31 - 1)
     double2 acc = make_double2(0.0, 0.0);
     for (int j = 0; j < m; ++j) {
       uint64_t a = 0;
-      for (int l = 0; l < d; ++l) a += frac64(t[j * d + l]) * (uint64_t)(long long)k[(long long)q * d + l];
+      for (int l = 0; l < d; ++l) a += frac64(t[j * d + l]) * (uint64_t)(long long)k[q * d + l];
       double u = (double)(long long)a * 5.421010862427522e-20;   // 2^-64
       double sn, cn;
       sincospi(2.0 * u, &sn, &cn);
@@ -934,10 +934,10 @@ __global__ void __launch_bounds__(128) k_eval_many(const double* t, const double
   for (int q = threadIdx.x; q < m * d; q += blockDim.x) T[q] = frac64(t[q]);
   __syncthreads();
   const double2* mid = ev_tab + m * EV_HI;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < K; q += gridDim.x * blockDim.x) {
+  for (long long q = blockIdx.x * blockDim.x + threadIdx.x; q < K; q += gridDim.x * blockDim.x) {
     uint64_t kq[PRONY_DMAX];
 #pragma unroll
-    for (int l = 0; l < PRONY_DMAX; ++l) kq[l] = l < d ? (uint64_t)(long long)k[(long long)q * d + l] : 0;
+    for (int l = 0; l < PRONY_DMAX; ++l) kq[l] = l < d ? (uint64_t)(long long)k[q * d + l] : 0;
     double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};   // even and odd terms
 #pragma unroll 2
     for (int j = 0; j < m; ++j) {
@@ -1135,6 +1135,6 @@ cudaError_t launch_eval_points(const double* t, const double2* c, int m, int d, 
   note_launch();
   k_eval_tables<<<(m * EV_HI + EV_MID + 63) / 64, 64, 0, s>>>(c, m, tab);
   note_launch();
-  k_eval_many<<<std::min((K + 127) / 128, 4 * 152), 128, sm, s>>>(t, tab, m, d, k, K, f);
+  k_eval_many<<<std::min(blocks_for(K, 128), 4 * 152), 128, sm, s>>>(t, tab, m, d, k, K, f);
   return cudaGetLastError();
 }
