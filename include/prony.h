@@ -60,6 +60,10 @@ typedef enum {
  *   PRONY_TF32X3 : FP32 operands split into TF32 hi+lo, three tensor-core
  *                  products (tcgen05.mma kind::tf32), FP32 accumulation.
  *   PRONY_BF16X2 : BF16 hi+lo split, three tensor-core products.
+ *                  The three tensor-core forms hold the samples of a row tile and a range of columns in
+ *                  shared memory: sizes of which not even 32 columns fit are PRONY_EINVAL (by the width and the
+ *                  form: directly d = 3 from n = 37 to 82 on and d = 4 from n = 8 to 14 on, through the DFT
+ *                  d = 3 with n > 95 and d = 4 from n = 37 on).
  *   PRONY_FFT32  : no dense product: T embedded in a circulant of L^d points (L the power of
  *                  two >= 2n+2), FP32 FFTs in shared memory, O(L^d log L) per column instead
  *                  of O(N^2).  Needs d <= 3 and L^(d-1) (L+1) + L <= 128 * 130 for every

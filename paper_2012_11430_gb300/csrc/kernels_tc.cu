@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_APROD), HALF ? 2 : 1)
   const int nc = APPLY ? (aw + 31) / 32 : (p.N + 31) / 32;
   const int cper = (nc + job.nks - 1) / job.nks;
   const int c_begin = job.ks * cper, c_end = min(nc, c_begin + cper);
-  const int nchunks = max(0, c_end - c_begin);
+  int nchunks = max(0, c_end - c_begin);
   const int NT = ((2 * w + 15) / 16) * 16;
   const TcLayout lay = tc_layout<KIND>(NT, TMEM_COLS);
   // Two rings of K chunks: B' tiles in shared memory (filled by the loader's bulk copies) and A' tiles in
@@ -384,6 +384,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_APROD), HALF ? 2 : 1)
     if (wlen > P.win_cap) {
       if (threadIdx.x == 0) atomicExch(err, 3);
       idle = true;
+      nchunks = 0;                              // nothing below reads a window that is not there
     }
   }
   if (idle && job.nks == 1) return;             // no partial to contribute
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_APROD), HALF ? 2 : 1)
   } else {
     // ------------------------------------------------------------- A' producers + epilogue
     // Warps 2..: quadrant q = warp & 3 (TMEM lanes 32q..32q+31 = tile rows), half hh of every
-    // K chunk (input points 32c + 16hh .. +15), or both halves in turn.
+    // K chunk (input points 32c + 16hh .. +15).
     const int q = warp & 3;
     const int hh = (warp - 2) >> 2;
     const int i = 32 * q + lane;                // row within the tile

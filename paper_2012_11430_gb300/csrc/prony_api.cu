@@ -255,6 +255,28 @@ int max_window(const ProbDesc& p, int L, int nks, int fmt) {
   return mx;
 }
 
+// The two parts of a window: the most grid indices that a 128-row tile spans, and that a K range of nks does.  The
+// longest window is one longer than their sum, plus what tc_window rounds (window_bounds).
+int row_span(const ProbDesc& p, int L) {
+  const int rows = (int)ipow(L, p.d);
+  int mx = 0;
+  for (int r0 = 0; r0 < rows; r0 += 128)
+    mx = std::max(mx, h_grid_of_row(std::min(rows, r0 + 128) - 1, L, p) - h_grid_of_row(r0, L, p));
+  return mx;
+}
+int k_span(const ProbDesc& p, int nks) {
+  const int nc = (p.N + 31) / 32, cper = (nc + nks - 1) / nks;
+  int mx = 0;
+  for (int cb = 0; cb < nc; cb += cper)
+    mx = std::max(mx, h_grid_of_h(std::min(p.N, 32 * (cb + cper)) - 1, p) - h_grid_of_h(32 * cb, p));
+  return mx;
+}
+void window_bounds(int span, int fmt, int& lo, int& hi) {
+  const int a = fmt == TT_COMPACT ? 8 : 4, spare = fmt == TT_COMPACT ? 8 : 0;
+  lo = (span + a - 1) / a * a + spare;
+  hi = (span + 2 * a - 2) / a * a + spare;
+}
+
 // Problem descriptors to the device, unless it holds these already (a repeated batch layout).
 int upload_problems(prony_ctx* ctx, const std::vector<ProbDesc>& P) {
   const size_t bytes = sizeof(ProbDesc) * P.size();
@@ -439,17 +461,35 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
     wmemo.emplace(key, wl);
     return wl;
   };
-  auto split_for = [&](int cap, int fmt) {
-    int nks = nks_lo;
-    for (;; ++nks) {
-      bool fits = true;
-      for (const auto& sh : shapes) {
-        const ProbDesc& p = Q[sh.second];
-        nks = std::min(nks, std::max(1, (p.N + 31) / 32));
-        if (window_of(sh.second, nks, 1, fmt) > cap || window_of(sh.second, nks, 0, fmt) > cap) fits = false;
+  // whether every window of a split fits `cap` entries (by its bounds where these decide)
+  std::map<std::pair<int, int>, int> rspan, kspan;
+  auto span_of = [&](int i, int nks, int ext) {
+    auto r = rspan.find({i, ext});
+    if (r == rspan.end()) r = rspan.emplace(std::make_pair(i, ext), row_span(Q[i], ext ? Q[i].n + 2 : Q[i].n + 1)).first;
+    auto k = kspan.find({i, nks});
+    if (k == kspan.end()) k = kspan.emplace(std::make_pair(i, nks), k_span(Q[i], nks)).first;
+    return r->second + k->second + 1;
+  };
+  auto split_fits = [&](int nks, int cap, int fmt) {
+    for (const auto& sh : shapes) {
+      const int i = sh.second, nc = (Q[i].N + 31) / 32;
+      if ((nc + nks - 1) / nks > max_chunks) return false;
+      for (int ext = 0; ext < 2; ++ext) {
+        int lo, hi;
+        window_bounds(span_of(i, nks, ext), fmt, lo, hi);
+        if (lo > cap || (hi > cap && window_of(i, nks, ext, fmt) > cap)) return false;
       }
-      if (fits || nks >= maxnc) break;
     }
+    return true;
+  };
+  // the smallest split whose windows fit, from the fewest chunks of a problem of the batch on (longer splits leave the
+  // small problems' CTAs without work); INT_MAX: none does
+  int minnc = maxnc;
+  for (const auto& sh : shapes) minnc = std::min(minnc, std::max(1, (Q[sh.second].N + 31) / 32));
+  auto split_for = [&](int cap, int fmt) {
+    if (!split_fits(maxnc, cap, fmt)) return INT_MAX;
+    int nks = std::min(nks_lo, minnc);
+    while (!split_fits(nks, cap, fmt)) ++nks;
     return nks;
   };
   // Fewer B stages leave room for a longer window and so may allow a smaller split: fewer CTAs,
@@ -471,7 +511,15 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
       T.stages = st;
     }
   }
-  if (nks == INT_MAX) return PRONY_EINVAL;
+  // (one stage leaves the most room)
+  if (nks == INT_MAX && st_min > 1 && win_cap_for(1, T.fmt) >= 256) {
+    nks = split_for(win_cap_for(1, T.fmt), T.fmt);
+    T.stages = st_min = 1;
+  }
+  if (nks == INT_MAX) {
+    g_err = "no K split of the tensor-core products has sample windows that fit shared memory";
+    return PRONY_EINVAL;
+  }
   auto longest = [&](int fmt) {
     int need = 0;
     for (const auto& sh : shapes)
