@@ -51,9 +51,13 @@ typedef enum {
 } prony_status;
 
 /* Arithmetic of the Toeplitz block products (the small steps are FP64 always).
- * For d >= 2 and at least 2048 points a product may first diagonalise the leading axis by an FP32 DFT and
- * run one product of d - 1 dimensions per frequency in the arithmetic below (a sample that is not
- * finite then spoils every row of the product).
+ * For d >= 2 and at least 2048 points (2500 for d > 2 in a tensor-core form) a product may first diagonalise the
+ * leading axis by an FP32 DFT and run one product of d - 1 dimensions per frequency in the arithmetic
+ * below.  Its error then is one of FP32 rounding of whole lines along that axis, not of each entry's own sum:
+ * against the norm of the product it is no larger, but where samples or columns decay strongly along the first
+ * axis, or are nearly all zero, small entries of the product lose relative accuracy, intermediate values are up to
+ * (2n+2)(n+1) times the largest product of a sample and an entry, and a sample that is not finite spoils every
+ * row.  (PRONY_AXIS=0, below, keeps the direct products.)
  *   PRONY_FP32   : complex64 operands, FP32 FMA on the CUDA cores.
  *   PRONY_BF16X3 : FP32 operands split into three BF16 parts, six tensor-core
  *                  products (tcgen05.mma kind::f16), FP32 accumulation.
@@ -262,7 +266,7 @@ typedef struct {
  *                        the FP32 CUDA cores instead of the tensor cores (three BF16 planes)
  *   PRONY_AXIS=0 / 1     the products of every problem directly / through a DFT of the leading axis
  *                        wherever that is possible (d >= 2, n <= 95; not PRONY_FFT32).  Default:
- *                        the transform for problems of at least 2048 points (n+1)^d where it costs less
+ *                        the transform for problems of at least 2048 (2500) points (n+1)^d where it costs less
  *   PRONY_ALLOC_MAX=b    no single device buffer of more than b bytes: growing one beyond that is refused as
  *                        a failed allocation is (a program that shares the device; the DFT products then
  *                        give way to the direct ones where those fit)

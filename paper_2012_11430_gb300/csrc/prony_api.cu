@@ -782,16 +782,19 @@ int setup_fft(prony_ctx* ctx, Batch& B) {
 // multiply-adds, for two more kernels and the traffic of the transformed blocks.  Costs in
 // units of one K chunk of a 128-row tile (about 1.1 us of an SM on the tensor cores): a CTA's
 // set-up and epilogue weigh about five chunks, the transforms 1e-3 per transformed value.
-// Below 2048 points the direct product's FP32 sums are short and round less than the transforms
-// do (relative error at N = 1331: 1.9e-7 direct, 2.4e-7 transformed; at N = 2601: 3.6e-7 and
-// 2.6e-7; at N = 8000: 3.4e-6 and 7e-7, BF16x3), so small problems keep it whatever the cost.
+// Where the direct product's FP32 sums are short they round less than the transforms do, so small problems keep it
+// whatever the cost (relative error against FP64 of random blocks, direct and transformed):
+//   N = 1331 (d = 3)  BF16x3 1.9e-7, 2.4e-7        N = 2197 (d = 3)  TF32x3 7.8e-7, 8.4e-7   FP32 4.3e-7, 2.7e-7
+//   N = 2116 (d = 2)  BF16x3 3.0e-7, 1.9e-7        N = 2401 (d = 4)  BF16x3 3.0e-7, 6.4e-7   FP32 4.5e-7, 3.0e-7
+//   N = 2744 (d = 3)  BF16x3 4.2e-7, 3.6e-7        N = 8000 (d = 3)  BF16x3 3.4e-6, 7.4e-7
+// The sub-products of d >= 3 are longer than those of d = 2 at the same N, hence two limits for the tensor-core forms.
 // PRONY_AXIS=0 / 1 overrides the size and cost rules.
 bool axis_pays(const std::vector<ProbDesc>& P, int prec) {
   if (prec != PRONY_FP32 && !is_tc(prec)) return false;
   const char* e = getenv("PRONY_AXIS");
   double dense = 0.0, axis = 0.0;
   for (const auto& p : P) {
-    if (p.d < 2 || p.n > AX_MAX_N || (!e && p.N < 2048)) return false;
+    if (p.d < 2 || p.n > AX_MAX_N || (!e && p.N < (p.d > 2 && is_tc(prec) ? 2500 : 2048))) return false;
     const double H = p.n + 1, Ns = p.N / H, Rs = p.Next / (H + 1);
     dense += std::ceil(p.Next / 128.0) * (std::ceil(p.N / 32.0) + 5);
     axis += 2 * H * (std::ceil(Rs / 128.0) * (std::ceil(Ns / 32.0) + 5) + 1e-3 * Ns * p.r0);
