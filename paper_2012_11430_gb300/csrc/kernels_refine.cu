@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
   const int P = m * (d + 2);
   double* H = sets + (1 - st->cur) * lm_set_elems(m, d);
   if ((int)blockIdx.x >= npt_blocks) {
-    __shared__ double axis_sum[LM_TILE / 32][PRONY_DMAX][3][6];
+    __shared__ double axis_sum[LM_TILE / 32][3][PRONY_DMAX][6];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int pair = (int)blockIdx.x - npt_blocks;                // a (a + 1) / 2 + b
     int a = (int)((sqrtf(8.f * pair + 1.f) - 1.f) * 0.5f);
@@ -154,78 +154,74 @@ __global__ void __launch_bounds__(LM_TILE) k_lm_points(const double* t, const do
     for (int l = threadIdx.x; l < d; l += LM_TILE)                // conj(e_a) e_b = exp(-2 pi i (t_b - t_a) x)
       T[l] = frac64(t[b * d + l]) - frac64(t[a * d + l]);
     __syncthreads();
-    // the warps' sums of x^p q^x (p = 0, 1, 2; re, im) over x = x0 + i step, i < n, at most 2^16
-    auto powers = [&](uint64_t dt, int x0, int step, int n, double (&out)[LM_TILE / 32][PRONY_DMAX][3][6], int l, int which) {
-      double tot = 0.0;                                           // lane z < 6: the z-th sum of the warp
-      for (int i0 = 0; i0 < n; i0 += 32 * LM_TILE) {              // at most 32 FP32 terms per thread, then FP64
-        float s[6] = {};
-        const int i1 = min(n, i0 + 32 * LM_TILE);
-        for (int i = i0 + threadIdx.x; i < i1; i += LM_TILE) {
-          const int x = x0 + i * step;
-          const float u = (float)(int)((dt * (uint64_t)(long long)x) >> 32) * 2.3283064365386963e-10f;
-          float sn, cn;
-          sincospif(2.0f * u, &sn, &cn);
-          const float xf = (float)x, x2 = xf * xf;
-          s[0] += cn;
-          s[1] -= sn;
-          s[2] += xf * cn;
-          s[3] -= xf * sn;
-          s[4] += x2 * cn;
-          s[5] -= x2 * sn;
-        }
-        float mine = 0.f;
-#pragma unroll
-        for (int z = 0; z < 6; ++z) {                             // FP32 over a warp, FP64 beyond
-          for (int o = 16; o > 0; o >>= 1) s[z] += __shfl_xor_sync(0xffffffffu, s[z], o);
-          if (lane == z) mine = s[z];
-        }
-        tot += (double)mine;
-      }
-      if (lane < 6) out[warp][l][which][lane] = tot;
-    };
+    // the warps' sums of x^p q^x (p = 0, 1, 2; re, im) over an axis, or over its pieces' starts, a piece and the rest
+    bool split = false;
     for (int l = 0; l < d; ++l) {
-      const int len = B.len[l], S = lm_axis_split(len);
-      if (S == 0) {
-        powers(T[l], B.lo[l], 1, len, axis_sum, l, 0);
-      } else {
-        const int U = len / S;
-        powers(T[l], 0, 1, S, axis_sum, l, 0);
-        powers(T[l], B.lo[l], S, U, axis_sum, l, 1);
-        powers(T[l], B.lo[l] + U * S, 1, len - U * S, axis_sum, l, 2);
+      const uint64_t dt = T[l];
+      const int len = B.len[l], S = lm_axis_split(len), U = S ? len / S : 0;
+      if (S) split = true;
+      for (int w = 0; w < (S ? 3 : 1); ++w) {
+        const int n = S == 0 ? len : w == 0 ? S : w == 1 ? U : len - U * S;             // at most 2^16
+        const int x0 = S == 0 || w == 1 ? B.lo[l] : w == 0 ? 0 : B.lo[l] + U * S, step = w == 1 ? S : 1;
+        double tot = 0.0;                                         // lane z < 6: the z-th sum of the warp
+        for (int i0 = 0; i0 < n; i0 += 32 * LM_TILE) {            // at most 32 FP32 terms per thread, then FP64
+          float s[6] = {};
+          const int i1 = min(n, i0 + 32 * LM_TILE);
+          for (int i = i0 + threadIdx.x; i < i1; i += LM_TILE) {
+            const int x = x0 + i * step;
+            const float u = (float)(int)((dt * (uint64_t)(long long)x) >> 32) * 2.3283064365386963e-10f;
+            float sn, cn;
+            sincospif(2.0f * u, &sn, &cn);
+            const float xf = (float)x, x2 = xf * xf;
+            s[0] += cn;
+            s[1] -= sn;
+            s[2] += xf * cn;
+            s[3] -= xf * sn;
+            s[4] += x2 * cn;
+            s[5] -= x2 * sn;
+          }
+          float mine = 0.f;
+#pragma unroll
+          for (int z = 0; z < 6; ++z) {                           // FP32 over a warp, FP64 beyond
+            for (int o = 16; o > 0; o >>= 1) s[z] += __shfl_xor_sync(0xffffffffu, s[z], o);
+            if (lane == z) mine = s[z];
+          }
+          tot += (double)mine;
+        }
+        if (lane < 6) axis_sum[warp][w][l][lane] = tot;
       }
-    }
-    __syncthreads();
-    for (int z = threadIdx.x; z < 18 * d; z += LM_TILE) {         // the warps' sums, in order
-      const int l = z / 18, w = z / 6 % 3, e = z % 6;
-      if (w == 0 || lm_axis_split(B.len[l]))
-        axis_sum[0][l][w][e] += axis_sum[1][l][w][e] + axis_sum[2][l][w][e] + axis_sum[3][l][w][e];
-    }
-    __syncthreads();
-    if (threadIdx.x < d && lm_axis_split(B.len[threadIdx.x])) {
-      // sum_u sum_v (X_u + v)^p q^(X_u + v), X_u = lo + S u, from V_k = sum v^k q^v and X_k = sum X_u^k q^X_u; and
-      // the last len - U S terms
-      double(&g)[3][6] = axis_sum[0][threadIdx.x];
-      const double2 v0 = make_double2(g[0][0], g[0][1]), v1 = make_double2(g[0][2], g[0][3]), v2 = make_double2(g[0][4], g[0][5]);
-      const double2 x0 = make_double2(g[1][0], g[1][1]), x1 = make_double2(g[1][2], g[1][3]), x2 = make_double2(g[1][4], g[1][5]);
-      const double2 r0 = cmul(x0, v0), r1 = cadd(cmul(x1, v0), cmul(x0, v1));
-      const double2 r2 = cadd(cadd(cmul(x2, v0), cscale(cmul(x1, v1), 2.0)), cmul(x0, v2));
-      g[0][0] = r0.x + g[2][0];
-      g[0][1] = r0.y + g[2][1];
-      g[0][2] = r1.x + g[2][2];
-      g[0][3] = r1.y + g[2][3];
-      g[0][4] = r2.x + g[2][4];
-      g[0][5] = r2.y + g[2][5];
     }
     __syncthreads();
     const int al = threadIdx.x / (d + 2), be = threadIdx.x % (d + 2);
     const int p = a * (d + 2) + al, q = b * (d + 2) + be;
+    for (int z = threadIdx.x; z < 6 * d; z += LM_TILE)            // the warps' sums, in order
+      for (int w = 0; w < (lm_axis_split(B.len[z / 6]) ? 3 : 1); ++w)
+        axis_sum[0][w][z / 6][z % 6] += axis_sum[1][w][z / 6][z % 6] + axis_sum[2][w][z / 6][z % 6] + axis_sum[3][w][z / 6][z % 6];
+    __syncthreads();
+    if (split) {
+      if (threadIdx.x < d && lm_axis_split(B.len[threadIdx.x])) {
+        // sum_u sum_v (X_u + v)^p q^(X_u + v), X_u = lo + S u, from V_k = sum v^k q^v and X_k = sum X_u^k q^X_u; and
+        // the last len - U S terms
+        auto sum = [&](int w, int k) { return make_double2(axis_sum[0][w][threadIdx.x][2 * k], axis_sum[0][w][threadIdx.x][2 * k + 1]); };
+        const double2 v0 = sum(0, 0), v1 = sum(0, 1), v2 = sum(0, 2), x0 = sum(1, 0), x1 = sum(1, 1), x2 = sum(1, 2);
+        const double2 r[3] = {cmul(x0, v0), cadd(cmul(x1, v0), cmul(x0, v1)),
+                              cadd(cadd(cmul(x2, v0), cscale(cmul(x1, v1), 2.0)), cmul(x0, v2))};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const double2 t = cadd(r[k], sum(2, k));
+          axis_sum[0][0][threadIdx.x][2 * k] = t.x;
+          axis_sum[0][0][threadIdx.x][2 * k + 1] = t.y;
+        }
+      }
+      __syncthreads();
+    }
     if (al < d + 2 && q <= p) {
       int wa, wb;
       const double2 sa = sigma_of(al, d, c[a], wa), sb = sigma_of(be, d, c[b], wb);
       double2 v = make_double2(sa.x * sb.x + sa.y * sb.y, sa.x * sb.y - sa.y * sb.x);   // conj(sa) sb M_ab
       for (int l = 0; l < d; ++l) {
         const int pw = 2 * ((wa == l + 1) + (wb == l + 1));
-        v = cmul(v, make_double2(axis_sum[0][l][0][pw], axis_sum[0][l][0][pw + 1]));
+        v = cmul(v, make_double2(axis_sum[0][0][l][pw], axis_sum[0][0][l][pw + 1]));
       }
       H[(long long)p * P + q] = v.x;
     }
