@@ -115,8 +115,8 @@ int prony_ctx_create(prony_ctx** ctx, int device);
 int prony_ctx_destroy(prony_ctx* ctx);
 
 /* Algorithm 1 for one problem.  samples: (2n+2)^d grid (see above).  d >= 1,
- * n >= 1, 1 <= m <= (n+1)^d, m <= 64, d m (n+1) <= 6144 (the phase tables of the right-hand
- * side), (n+1)^d <= 2e8, else PRONY_EINVAL.  opts may be NULL (defaults).
+ * n >= 1, 1 <= m <= (n+1)^d, m <= 64, d m (n+1) <= 6144 (96 KB of powers of its
+ * nodes), (n+1)^d <= 2e8, else PRONY_EINVAL.  opts may be NULL (defaults).
  * Outputs: t_out[m*d] (row j = t_j, components in [0,1)), c_out[m]; the pairs
  * are sorted lexicographically by t.  info may be NULL. */
 int prony_solve(prony_ctx* ctx, const prony_c128* samples, int d, int n, int m,
@@ -198,8 +198,10 @@ int prony_expsum_bwd_dev(prony_ctx* ctx, const double* t_dev, const void* c_dev,
  * y_dev: prod(len) complex64 samples, loss_dev: iters+1 float64 or NULL (the loss before each
  * step and after the last).  Each step: one FP32 Cholesky solve of the Jacobi-scaled damped
  * system (Marquardt damping lambda, initial value lambda0 > 0), one pass over the points at the
- * candidate for its loss, J^* J and J^* r (FP32 per block, FP64 accumulators); the step is taken if
- * the loss decreased (lambda / 3), else refused (lambda * 4).
+ * candidate for its loss, J^* J and J^* r; the step is taken if the loss decreased (lambda / 3), else
+ * refused (lambda * 4).  The model is evaluated beyond FP32 and the loss summed in FP64.  J^* J (sums over
+ * the axes) and J^* r (over the points) are FP32 over at most 128 terms and FP64 within a block of the GPU;
+ * the blocks' J^* r are then rounded to FP32 and added without further error.  All sums have a fixed order.
  * m * (d + 2) <= 160, else PRONY_EINVAL.  Runs on `stream` (NULL: the context stream) and
  * returns when the refined (t, c) are written. */
 int prony_refine_lm_dev(prony_ctx* ctx, double* t_dev, prony_c128* c_dev, int m, int d,
@@ -259,7 +261,7 @@ typedef struct {
 
 /* Tuning overrides of the tensor-core products, read from the environment at every call:
  *   PRONY_TC_BSTAGES=s   exactly s B' stages in shared memory (default: the most stages, from
- *                        4 down to 2, that reach the smallest K split whose windows fit)
+ *                        4 down to 2, that reach the smallest K split whose windows fit; one where only that fits)
  *   PRONY_TC_KSPLIT=k    a K split of at least k (no autotuning)
  *   PRONY_TC_TUNE=0      no autotuning: the smallest K split
  *   PRONY_TC_APPLY=0     the X M products of the tall blocks (CholeskyQR2, the final U and V) on
@@ -268,8 +270,9 @@ typedef struct {
  *                        wherever that is possible (d >= 2, n <= 95; not PRONY_FFT32).  Default:
  *                        the transform for problems of at least 2048 (2500) points (n+1)^d where it costs less
  *   PRONY_ALLOC_MAX=b    no single device buffer of more than b bytes: growing one beyond that is refused as
- *                        a failed allocation is (a program that shares the device; the DFT products then
- *                        give way to the direct ones where those fit)
+ *                        a failed allocation is (a program that shares the device).  DFT products whose buffers
+ *                        are refused, so or by the device, give way to the direct ones where those fit; the
+ *                        context keeps to that for this layout of sizes until another layout is refused
  * The first three change launch configurations only, never the arithmetic beyond FP32 summation
  * order; the fourth changes how the X M products are rounded (both are FP32-accurate), the fifth
  * how the products are (FP32 transforms around shorter dot products in the chosen arithmetic).

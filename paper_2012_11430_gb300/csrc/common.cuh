@@ -124,9 +124,9 @@ struct Dev {
   const double2* grid64;
   float2* gF;
   float2* gH;
-  // Split BF16 planes of the samples for the tensor-core path (Section 1 samples, split once):
-  // table a = part * 3 + plane (part 0: Re, 1: Im) of problem p at toff + a * Gd4; word x holds
-  // plane(F[x]) in its low half and plane(F[x - 1]) in its high half (F = gF for tabF, gH for tabH).
+  // Split planes of the samples for the tensor-core path (Section 1 samples, split once per solve), of gF in tabF
+  // and gH in tabH: table a = part * planes + plane (part 0: Re, 1: Im; three BF16 planes, two TF32) of problem p at
+  // word toff + a * Gd4, in one of the formats of TcTable below.
   uint32_t* tabF;
   uint32_t* tabH;
   float2* V;

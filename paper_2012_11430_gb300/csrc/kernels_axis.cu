@@ -493,8 +493,9 @@ static cudaError_t axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int 
 }
 
 cudaError_t launch_axis_out(const Dev& D, const Dev& S, int wsel, int ybuf, int y_ext, int maxw, cudaStream_t s) {
-  // 22 rows a pass re-read the sub-products least; few lines (a single small problem) take 8 rows a
-  // pass, which gives three times the warps, and with fewer than eight warps per SM four warps share a line's
+  // 22 rows a pass re-read the sub-products least: the most that leave two blocks of 256 threads per SM (109 registers,
+  // 24 rows take 146).  A last pass computes rows past the end: none at n = 19, a fifth of the work at n = 50.  Few lines (a
+  // single small problem) take 8 rows a pass, which gives three times the warps, and with fewer than eight warps per SM four warps share a line's
   // classes (d = 2, n = 50, 37 columns: 25 -> 11 us; with 11 warps per SM, d = 3, n = 19, 40 columns, 3 us slower)
   const long long lines = (long long)(((y_ext ? S.maxNext : S.maxN) + 31) / 32) * maxw * D.nprob;
   if (lines >= 152LL * 16) return axis_out<22, 1>(D, S, wsel, ybuf, y_ext, maxw, s);

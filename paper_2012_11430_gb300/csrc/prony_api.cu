@@ -145,7 +145,7 @@ int validate(const HostProb& h) {
   if (h.d < 1 || h.d > PRONY_DMAX || h.n < 1 || h.m < 1 || h.m > PRONY_MMAX) return PRONY_EINVAL;
   double N = std::pow((double)(h.n + 1), h.d);
   if (N > 2.0e8 || h.m > N) return PRONY_EINVAL;
-  if ((long long)h.d * h.m * (h.n + 1) > 6144) return PRONY_EINVAL;   // phase tables of the RHS kernel
+  if ((long long)h.d * h.m * (h.n + 1) > 6144) return PRONY_EINVAL;   // documented: 96 KB of powers (zpow) per problem
   return PRONY_OK;
 }
 
@@ -526,8 +526,11 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
       need = std::max(need, std::max(window_of(sh.second, nks, 1, fmt), window_of(sh.second, nks, 0, fmt)));
     return need;
   };
-  // wide tables where their windows fit at the same split (with the stages given, or two): a pair of points is one
-  // load instead of two and a shift (the same products: then 14.7 -> 13.7 ms); a longer split would load more windows
+  // Wide tables where their windows fit at the same split (with the stages given, or two): a pair of points is one
+  // load instead of two and a shift, and two CTAs per SM, below, need them.  The products of 4096 problems with n
+  // 7..31 take 11.9 ms a solve with both; at one CTA per SM, with the loads hidden under the MMAs, 16.4 ms with wide
+  // tables and 15.8 with compact ones (64 problems of d = 3, n = 19: 10.5 and 10.3).  A longer split would load more
+  // windows.
   if (bf16)
     for (int st = T.stages; st >= st_min; --st)
       if (win_cap_for(st, TT_WIDE) >= std::max(256, longest(TT_WIDE))) {
@@ -537,10 +540,9 @@ int setup_tc(prony_ctx* ctx, Batch& B, int prec, int maxw) {
       }
   T.win_cap = win_cap_for(T.stages, T.fmt);
   // Narrow blocks (at most 24 columns in BF16x3) of problems whose windows are short: two CTAs per SM, each with
-  // half of its memories, so that one's set-up, window load and epilogue run under the other's
-  // chunks (the products of 4096 problems with n 7..31: 16.1 -> 14.7 ms a solve when it was made).  From four CTAs per SM on:
-  // below that every SM has a CTA of its own.  Wider accumulators leave
-  // no tensor memory for it, longer windows no shared memory.
+  // half of its memories, so that one's set-up, window load and epilogue run under the other's chunks (the
+  // products above: 15.8 -> 11.9 ms a solve).  From four CTAs per SM on: below that every SM has a CTA of its own.
+  // Wider accumulators leave no tensor memory for it, longer windows no shared memory.
   {
     const size_t per = 228 * 1024 / 2 - 1024 - 6144;   // (1 KB reserved per CTA, static shared memory)
     const int need = longest(T.fmt);
@@ -978,7 +980,6 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
   long long goff = 0, xoff = 0, yoff = 0, toff = 0, xchunk = 0;
   int sub = 0;
   int maxN = 0, maxNext = 0, maxGd = 0, maxR0 = 0, maxM = 0, maxD = 0;
-  long long tiles_ext = 0, tiles_in = 0;
   for (int i = 0; i < np; ++i) {
     const HostProb& h = hp[i];
     ProbDesc& p = B.P[i];
@@ -1016,8 +1017,6 @@ int setup_batch(prony_ctx* ctx, const std::vector<HostProb>& hp, const prony_opt
     maxR0 = std::max(maxR0, p.r0);
     maxM = std::max(maxM, p.m);
     maxD = std::max(maxD, p.d);
-    tiles_ext += (p.Next + 63) / 64;
-    tiles_in += (p.N + 63) / 64;
   }
   SmallLay L = make_small_lay((maxR0 + 1) / 2 * 2, maxM, maxD);
   for (int i = 0; i < np; ++i) B.P[i].soff = (long long)i * L.bytes;
