@@ -246,6 +246,8 @@ int prony_toeplitz_mm_static(const prony_c128* grid_dev, int d, int n, const voi
  * stream; its algorithmic work is accumulated: flops = 8 * rows * N * width per live
  * problem (one complex multiply-add = 8 real flops), bytes = samples read
  * (8 (2n+2)^d) + X read (8 N width) + Y written (8 rows width) at complex64.
+ * Products by FFT or through the DFT of the leading axis count the flops of their transforms and
+ * sub-products instead.
  * launches counts every kernel the library launched (all kernels, all contexts)
  * since the last reset. */
 typedef struct {

@@ -24,7 +24,7 @@
 // c_j T eps in FP32, whose rounding is ten times smaller than that of the whole.
 // Measured at d = 2, n = 63 (16384 points), m = 20: a step took 195 us (143 in a one-CTA solve with three
 // barriers per column, 40 in the M sums over all points, 9 in a separate trial pass), now 40 us (k_lm_step
-// 26, k_lm_points 16, their launches overlapped): 50 steps 10.05 -> 2.00 ms.  Both kernels are latency chains
+// 26, k_lm_points 16, their launches overlapped): 50 steps 10.05 -> 1.98 ms.  Both kernels are latency chains
 // on an almost idle GPU.
 #include "common.cuh"
 
@@ -43,7 +43,7 @@ constexpr double TWO_PI = 6.283185307179586;
 
 // The steps are launched as a chain (programmatic dependent launch): a kernel's blocks become resident as soon as
 // every block of the one before has begun, and wait here until it has completed and its writes are visible; what
-// that saves is the launch latency between kernels of 16 to 26 us (50 steps: 2.25 -> 2.00 ms; the kernels of a solve,
+// that saves is the launch latency between kernels of 16 to 26 us (50 steps: 2.25 -> 1.98 ms; the kernels of a solve,
 // launched from a graph, gained nothing by it).  Every kernel launched so begins with chain_begin().
 __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
