@@ -1462,7 +1462,10 @@ int run_batch(prony_ctx* ctx, Batch& B, const prony_opts& o, const RunOut& ro) {
     CK(cudaGetLastError());
     return PRONY_OK;
   }
-  prefix();
+  if ((rc = prefix())) return rc;
+  // (before anything works on what a failed launch did not write, and before the autotuner skips candidates by launch_err)
+  note_launch_error(ctx, cudaGetLastError());
+  if (ctx->launch_err != cudaSuccess) return cuda_fail(ctx->launch_err, "kernel launch");
   if (lanczos) {
     for (int step = 0; step < lz_cap; ++step) {
       if ((rc = lz_step())) return rc;

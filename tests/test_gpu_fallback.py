@@ -125,3 +125,16 @@ def test_failed_launch_is_reported_every_time(ctx):
             ctx.solve_batched([grid] * P, [1] * P, [1] * P, [1] * P, o)
         assert e.value.code == PRONY_ECUDA
     _solve(ctx, W.make_problem("fl", 2, 15, 5, 7206), 3, "fp32")
+
+
+def test_failed_launch_before_the_autotuner(ctx):
+    """... and where the first call of a batch shape runs step by step from the host (tensor-core products not tuned yet)."""
+    from paper_2012_11430_gb300 import PronyError, default_opts
+    from paper_2012_11430_gb300.binding import PRONY_ECUDA
+    P = 65536
+    grid = np.ones(4, dtype=np.complex128)
+    for _ in range(2):
+        with pytest.raises(PronyError) as e:
+            ctx.solve_batched([grid] * P, [1] * P, [1] * P, [1] * P, default_opts(precision="bf16x3"))
+        assert e.value.code == PRONY_ECUDA
+    _solve(ctx, W.make_problem("fl", 2, 15, 5, 7207), 3, "bf16x3")
