@@ -116,7 +116,7 @@ int prony_ctx_destroy(prony_ctx* ctx);
 
 /* Algorithm 1 for one problem.  samples: (2n+2)^d grid (see above).  d >= 1,
  * n >= 1, 1 <= m <= (n+1)^d, m <= 64, d m (n+1) <= 6144 (96 KB of powers of its
- * nodes), (n+1)^d <= 2e8, else PRONY_EINVAL.  opts may be NULL (defaults).
+ * nodes), (n+1)^d <= 2e8, (2n+2)^d < 2^31, else PRONY_EINVAL.  opts may be NULL (defaults).
  * Outputs: t_out[m*d] (row j = t_j, components in [0,1)), c_out[m]; the pairs
  * are sorted lexicographically by t.  info may be NULL. */
 int prony_solve(prony_ctx* ctx, const prony_c128* samples, int d, int n, int m,

@@ -141,10 +141,12 @@ double default_tol_power(int prec) {
   return 1e-6;
 }
 
+// Points and samples of a problem within the kernels' 32-bit indices ((2n+2)^d passes 2^31 at d = 4, n = 107 first).
+bool size_ok(int d, int n) { return std::pow((double)n + 1, d) <= 2.0e8 && std::pow(2.0 * n + 2, d) < 2147483648.0; }
+
 int validate(const HostProb& h) {
   if (h.d < 1 || h.d > PRONY_DMAX || h.n < 1 || h.m < 1 || h.m > PRONY_MMAX) return PRONY_EINVAL;
-  double N = std::pow((double)(h.n + 1), h.d);
-  if (N > 2.0e8 || h.m > N) return PRONY_EINVAL;
+  if (!size_ok(h.d, h.n) || h.m > std::pow((double)h.n + 1, h.d)) return PRONY_EINVAL;
   if ((long long)h.d * h.m * (h.n + 1) > 6144) return PRONY_EINVAL;   // documented: 96 KB of powers (zpow) per problem
   return PRONY_OK;
 }
@@ -2041,7 +2043,7 @@ int prony_toeplitz_mm_dev(prony_ctx* ctx, const prony_c128* grid_dev, int d, int
   if (check_precision(precision)) return PRONY_EINVAL;
   CK(cudaSetDevice(ctx->device));
   std::vector<HostProb> hp = {{d, n, 1, 0, 0}};
-  if (std::pow((double)(n + 1), d) > 2.0e8 || r > (long long)ipow(n + 1, d)) return PRONY_EINVAL;
+  if (!size_ok(d, n) || r > ipow(n + 1, d)) return PRONY_EINVAL;
   prony_opts o;
   prony_default_opts(&o);
   o.oversample_p = r - 1;

@@ -61,3 +61,22 @@ def test_windows_that_do_not_fit_are_refused(ctx, monkeypatch, d, n, r, prec, fi
     Z = Z[(slice(None),) + (slice(L),) * d].reshape(r, -1)
     # the accumulator truncates once per MMA: 64 chunks of 24 MMAs at most, 2^-23 each of a partial sum
     assert (Y - Z).abs().square().sum().sqrt() <= 64 * 24 * 2.0 ** -23 * Z.abs().square().sum().sqrt()
+
+
+def test_sample_counts_beyond_32_bits_are_refused(ctx):
+    """d = 4, n = 107: (n + 1)^4 is within the limit on points, (2n + 2)^4 is not below 2^31.  Refused before anything is
+    read or allocated."""
+    import ctypes
+
+    import torch
+    from paper_2012_11430_gb300 import PronyError
+    from paper_2012_11430_gb300.binding import PRONY_EINVAL
+    x = torch.zeros((1, 8), dtype=torch.complex64, device="cuda")
+    g = torch.zeros(8, dtype=torch.complex128, device="cuda")
+    for prec in ("fp32", "bf16x3"):
+        with pytest.raises(PronyError) as e:
+            ctx.toeplitz_mm_dev(g, 4, 107, x, 108, 0, prec, x)
+        assert e.value.code == PRONY_EINVAL
+    z = np.zeros(16)
+    ptr = z.ctypes.data_as(ctypes.c_void_p)
+    assert ctx._lib.prony_solve(ctx._h, ptr, 4, 107, 1, None, ptr, ptr, None) == PRONY_EINVAL
